@@ -5,14 +5,17 @@
 // rows the sparse loops read (code * scale + offset with one binary32 rounding, then one rounding to the storage
 // type), so that the cache at rest is the packed form and the bf16 rows are a transient working copy of one layer.
 // HBM-bound kernels, 16-byte accesses, bit-exact arithmetic (binary32, directed fp16 roundings of the metadata).
-#include "fl_internal.cuh"
+#include "codec.cuh"
 
 namespace {
+
+using namespace fl_codec;
 
 struct BaseArgs {
   const void* k; const void* v;        // quantize: inputs [L, d]; dequantize: unused
   void* k_out; void* v_out;            // dequantize: outputs [L, d]; quantize: unused
   const void* k_tail; const void* v_tail;   // dequantize: rows Lq .. L-1 in the storage type
+  void* k_tail_out; void* v_tail_out;       // quantize: receive them
   int L;
   uint8_t* k_codes; __half* k_scale; __half* k_zero;
   uint8_t* v_codes; __half* v_scale; __half* v_zero;
@@ -20,212 +23,332 @@ struct BaseArgs {
   int Lq, d, group, dh, mask_words;
 };
 
-template <int BITS>
-__device__ __forceinline__ void store_codes8(uint8_t* row, int elem, const float (&q)[8]) {
-  uint32_t c[8];
+// Eight consecutive elements of a row as loaded, their minimum / maximum against another eight, and as pairs.
+template <typename T>
+struct Raw8;
+template <>
+struct Raw8<__nv_bfloat16> {
+  uint4 r;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { r = __ldg(reinterpret_cast<const uint4*>(p)); }
+  __device__ __forceinline__ void pairs(f32x2 (&x)[4]) const { unpack_bf16(r, x); }
+  __device__ __forceinline__ void store(__nv_bfloat16* p) const { *reinterpret_cast<uint4*>(p) = r; }
+  static __device__ __forceinline__ uint32_t lo2(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 v = __hmin2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  static __device__ __forceinline__ uint32_t hi2(uint32_t a, uint32_t b) {
+    const __nv_bfloat162 v = __hmax2(*reinterpret_cast<__nv_bfloat162*>(&a), *reinterpret_cast<__nv_bfloat162*>(&b));
+    return *reinterpret_cast<const uint32_t*>(&v);
+  }
+  __device__ __forceinline__ void take_min(const Raw8& o) { r.x = lo2(r.x, o.r.x); r.y = lo2(r.y, o.r.y); r.z = lo2(r.z, o.r.z); r.w = lo2(r.w, o.r.w); }
+  __device__ __forceinline__ void take_max(const Raw8& o) { r.x = hi2(r.x, o.r.x); r.y = hi2(r.y, o.r.y); r.z = hi2(r.z, o.r.z); r.w = hi2(r.w, o.r.w); }
+  __device__ __forceinline__ void range(float& mn, float& mx) const {
+    const uint32_t a = lo2(lo2(r.x, r.y), lo2(r.z, r.w)), b = hi2(hi2(r.x, r.y), hi2(r.z, r.w));
+    mn = fminf(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u));
+    mx = fmaxf(__uint_as_float(b << 16), __uint_as_float(b & 0xffff0000u));
+  }
+};
+template <>
+struct Raw8<float> {
+  float4 a, b;
+  __device__ __forceinline__ void load(const float* p) {
+    a = __ldg(reinterpret_cast<const float4*>(p));
+    b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+  }
+  __device__ __forceinline__ void pairs(f32x2 (&x)[4]) const {
+    x[0] = pair(a.x, a.y); x[1] = pair(a.z, a.w); x[2] = pair(b.x, b.y); x[3] = pair(b.z, b.w);
+  }
+  __device__ __forceinline__ void store(float* p) const { reinterpret_cast<float4*>(p)[0] = a; reinterpret_cast<float4*>(p)[1] = b; }
+  __device__ __forceinline__ void take_min(const Raw8& o) {
+    a = make_float4(fminf(a.x, o.a.x), fminf(a.y, o.a.y), fminf(a.z, o.a.z), fminf(a.w, o.a.w));
+    b = make_float4(fminf(b.x, o.b.x), fminf(b.y, o.b.y), fminf(b.z, o.b.z), fminf(b.w, o.b.w));
+  }
+  __device__ __forceinline__ void take_max(const Raw8& o) {
+    a = make_float4(fmaxf(a.x, o.a.x), fmaxf(a.y, o.a.y), fmaxf(a.z, o.a.z), fmaxf(a.w, o.a.w));
+    b = make_float4(fmaxf(b.x, o.b.x), fmaxf(b.y, o.b.y), fmaxf(b.z, o.b.z), fmaxf(b.w, o.b.w));
+  }
+  __device__ __forceinline__ void range(float& mn, float& mx) const {
+    mn = fminf(fminf(fminf(a.x, a.y), fminf(a.z, a.w)), fminf(fminf(b.x, b.y), fminf(b.z, b.w)));
+    mx = fmaxf(fmaxf(fmaxf(a.x, a.y), fmaxf(a.z, a.w)), fmaxf(fmaxf(b.x, b.y), fmaxf(b.z, b.w)));
+  }
+};
+// Two consecutive elements in shared memory and their running extrema.
+template <typename T>
+struct Pair2;
+template <>
+struct Pair2<__nv_bfloat16> {
+  uint32_t v;
+  __device__ __forceinline__ void load(const __nv_bfloat16* p) { v = *reinterpret_cast<const uint32_t*>(p); }
+  __device__ __forceinline__ void take_min(const __nv_bfloat16* p) { v = Raw8<__nv_bfloat16>::lo2(v, *reinterpret_cast<const uint32_t*>(p)); }
+  __device__ __forceinline__ void take_max(const __nv_bfloat16* p) { v = Raw8<__nv_bfloat16>::hi2(v, *reinterpret_cast<const uint32_t*>(p)); }
+  __device__ __forceinline__ float2 floats() const { return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u)); }
+};
+template <>
+struct Pair2<float> {
+  float2 v;
+  __device__ __forceinline__ void load(const float* p) { v = *reinterpret_cast<const float2*>(p); }
+  __device__ __forceinline__ void take_min(const float* p) { v = make_float2(fminf(v.x, p[0]), fminf(v.y, p[1])); }
+  __device__ __forceinline__ void take_max(const float* p) { v = make_float2(fmaxf(v.x, p[0]), fmaxf(v.y, p[1])); }
+  __device__ __forceinline__ float2 floats() const { return v; }
+};
+
+// Packing of K and V. Bound by HBM (read once, codes written once); what it has to avoid is reading a key twice, a
+// dependent walk over the group's rows, and more than ~8 instructions an element (two passes of 64 dependent rows per
+// thread and a division per element took 129 us for the keys and 76 us for the values of 20 k rows of 2048, 0.8 TB/s).
+//
+// Keys: a CTA owns 256 channels of one token group, 32 pieces of 8 channels by ROWL row lanes; a thread loads its rows
+// at once, keeps them in registers, and after the group's minimum and maximum per channel have been joined in shared
+// memory encodes them from there. The CTAs past k_ctas copy the tail rows.
+template <typename T>
+constexpr int kBqRows = sizeof(T) == 2 ? 4 : 8;        // rows of a token group per thread
+constexpr int kBqCh = 256;                             // channels of a key CTA
+
+template <typename T, int BITS, int ROWL>
+__global__ void __launch_bounds__(32 * ROWL, (sizeof(T) == 2 ? 1024 : 512) / (32 * ROWL))
+base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas) {
+  constexpr int kThreads = 32 * ROWL;
+  __shared__ __align__(16) T red[2][ROWL][kBqCh];
+  __shared__ __align__(16) float meta[3][kBqCh];       // offset (negated), scale, reciprocal
+  fl_grid_wait();
+  fl_grid_release();
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (blockIdx.x < (unsigned)k_ctas) {
+    const int slabs = a.d / kBqCh;
+    const int g = blockIdx.x / slabs, c0 = (blockIdx.x - g * slabs) * kBqCh;
+    const int elem = c0 + lane * 8, rl = tid >> 5;
+    const int t0 = g * a.group + rl, t1 = min(a.Lq, (g + 1) * a.group);
+    const T* k = static_cast<const T*>(a.k) + elem;
+    Raw8<T> raw[kBqRows<T>];
 #pragma unroll
-  for (int i = 0; i < 8; ++i) c[i] = (uint32_t)q[i];
-  if (BITS == 8) {
-    *reinterpret_cast<uint2*>(row + elem) = make_uint2(c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24),
-                                                       c[4] | (c[5] << 8) | (c[6] << 16) | (c[7] << 24));
-  } else if (BITS == 4) {
-    uint32_t w = 0;
+    for (int i = 0; i < kBqRows<T>; ++i) {             // a short last group repeats its first row (changes no extremum)
+      const int t = t0 + i * ROWL < t1 ? t0 + i * ROWL : g * a.group;
+      raw[i].load(k + (size_t)t * a.d);
+    }
+    Raw8<T> mn = raw[0], mx = raw[0];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) w |= c[i] << (4 * i);
-    *reinterpret_cast<uint32_t*>(row + elem / 2) = w;
+    for (int i = 1; i < kBqRows<T>; ++i) { mn.take_min(raw[i]); mx.take_max(raw[i]); }
+    mn.store(&red[0][rl][lane * 8]);
+    mx.store(&red[1][rl][lane * 8]);
+    __syncthreads();
+    for (int ch = tid * 2; ch < kBqCh; ch += kThreads * 2) {     // two channels per thread
+      Pair2<T> lo, hi;
+      lo.load(&red[0][0][ch]);
+      hi.load(&red[1][0][ch]);
+#pragma unroll
+      for (int r = 1; r < ROWL; ++r) { lo.take_min(&red[0][r][ch]); hi.take_max(&red[1][r][ch]); }
+      const float2 l2 = lo.floats(), h2 = hi.floats();
+      __half zh[2], sh[2];
+      group_meta<BITS>(l2.x, h2.x, zh[0], sh[0]);
+      group_meta<BITS>(l2.y, h2.y, zh[1], sh[1]);
+      *reinterpret_cast<__half2*>(a.k_zero + (size_t)g * a.d + c0 + ch) = __halves2half2(zh[0], zh[1]);
+      *reinterpret_cast<__half2*>(a.k_scale + (size_t)g * a.d + c0 + ch) = __halves2half2(sh[0], sh[1]);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        const float s = __half2float(sh[e]);
+        meta[0][ch + e] = -__half2float(zh[e]);
+        meta[1][ch + e] = s;
+        meta[2][ch + e] = scale_rcp(s);
+      }
+    }
+    __syncthreads();
+    f32x2 nz[4], inv[4], ninv[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      nz[e] = *reinterpret_cast<const f32x2*>(&meta[0][lane * 8 + 2 * e]);
+      inv[e] = *reinterpret_cast<const f32x2*>(&meta[2][lane * 8 + 2 * e]);
+      ninv[e] = inv[e] ^ 0x8000000080000000ull;
+    }
+    uint8_t* dst = a.k_codes + ((size_t)t0 * a.d + elem) * BITS / 8;
+#pragma unroll
+    for (int i = 0; i < kBqRows<T>; ++i) {
+      if (t0 + i * ROWL >= t1) break;
+      f32x2 x[4], q[4];
+      raw[i].pairs(x);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) x[e] = add2(x[e], nz[e]);
+      quotients<BITS, 4>(x, inv, ninv, [&](int e) { return *reinterpret_cast<const f32x2*>(&meta[1][lane * 8 + 2 * e]); }, q);
+      store_codes<BITS, 4>(dst, q);
+      dst += (size_t)ROWL * a.d * BITS / 8;
+    }
   } else {
-    uint32_t w = 0;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) w |= c[i] << (2 * i);
-    *reinterpret_cast<uint16_t*>(row + elem / 4) = (uint16_t)w;
-  }
-}
-
-// scale and offset of one group from its minimum and maximum: offset rounded down, scale rounded up (fp16)
-template <int BITS>
-__device__ __forceinline__ void group_meta(float mn, float mx, __half& zh, __half& sh) {
-  zh = __float2half_rd(mn);
-  const float range = __fsub_rn(mx, __half2float(zh));
-  sh = range == 0.f ? __float2half_rn(0.f) : __float2half_ru(__fdiv_rn(range, (float)((1 << BITS) - 1)));
-}
-
-template <int BITS>
-__device__ __forceinline__ float code_of(float x, float zf, float sf) {
-  if (sf == 0.f) return 0.f;
-  const float q = rintf(__fdiv_rn(__fsub_rn(x, zf), sf));          // round half to even
-  return fminf(fmaxf(q, 0.f), (float)((1 << BITS) - 1));
-}
-
-// Keys: one CTA per group of `group` consecutive positions, one thread per 8 channels. Two passes over the
-// group's rows (the second finds them in L2): minimum and maximum per channel, then the codes.
-template <typename T, int BITS>
-__global__ void __launch_bounds__(256) base_quant_k_kernel(const __grid_constant__ BaseArgs a) {
-  const int g = blockIdx.x;
-  const int t0 = g * a.group, t1 = min(a.Lq, t0 + a.group);
-  const T* k = static_cast<const T*>(a.k);
-  for (int elem = (blockIdx.y * blockDim.x + threadIdx.x) * 8; elem < a.d; elem += gridDim.y * blockDim.x * 8) {
-    float mn[8], mx[8], x[8];
-    load8<T>(k + (size_t)t0 * a.d + elem, mn);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) mx[i] = mn[i];
-    for (int t = t0 + 1; t < t1; ++t) {
-      load8<T>(k + (size_t)t * a.d + elem, x);
-#pragma unroll
-      for (int i = 0; i < 8; ++i) { mn[i] = fminf(mn[i], x[i]); mx[i] = fmaxf(mx[i], x[i]); }
-    }
-    __align__(16) __half zh[8];
-    __align__(16) __half sh[8];
-    float zf[8], sf[8];
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      group_meta<BITS>(mn[i], mx[i], zh[i], sh[i]);
-      zf[i] = __half2float(zh[i]);
-      sf[i] = __half2float(sh[i]);
-    }
-    *reinterpret_cast<uint4*>(a.k_zero + (size_t)g * a.d + elem) = *reinterpret_cast<const uint4*>(zh);
-    *reinterpret_cast<uint4*>(a.k_scale + (size_t)g * a.d + elem) = *reinterpret_cast<const uint4*>(sh);
-    for (int t = t0; t < t1; ++t) {
-      load8<T>(k + (size_t)t * a.d + elem, x);
-      float q[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) q[i] = code_of<BITS>(x[i], zf[i], sf[i]);
-      store_codes8<BITS>(a.k_codes + (size_t)t * (a.d * BITS / 8), elem, q);
+    // tail rows, as they are
+    const int64_t n_vec = (int64_t)(a.L - a.Lq) * a.d * sizeof(T) / 16;
+    const int64_t step = (int64_t)(gridDim.x - k_ctas) * kThreads;
+    const uint4* k = reinterpret_cast<const uint4*>(static_cast<const T*>(a.k) + (size_t)a.Lq * a.d);
+    const uint4* v = reinterpret_cast<const uint4*>(static_cast<const T*>(a.v) + (size_t)a.Lq * a.d);
+    for (int64_t i = (int64_t)(blockIdx.x - k_ctas) * kThreads + tid; i < n_vec; i += step) {
+      reinterpret_cast<uint4*>(a.k_tail_out)[i] = __ldg(k + i);
+      reinterpret_cast<uint4*>(a.v_tail_out)[i] = __ldg(v + i);
     }
   }
 }
 
-// Values: one thread per 8 consecutive channels of a position; the group's minimum and maximum by shuffles over
-// the group / 8 lanes that share it. blockDim.x * 8 divides d or is a multiple of it in whole rows (host).
+// Values: pieces of 16 elements, their index running over the whole matrix (no row arithmetic: code and metadata offsets
+// follow from it); two pieces per thread are in flight, minima and maxima by shuffles over the lanes of a group.
+constexpr int kBvThreads = 256;
+
 template <typename T, int BITS>
-__global__ void __launch_bounds__(256) base_quant_v_kernel(const __grid_constant__ BaseArgs a) {
-  const int per_row = a.d >> 3;
-  const int lanes_per_group = a.group >> 3;
-  const int64_t total = (int64_t)a.Lq * per_row;      // a multiple of 32: d % 256 == 0
+__global__ void __launch_bounds__(kBvThreads) base_quant_v_kernel(const __grid_constant__ BaseArgs a) {
+  constexpr int U = 2;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int lanes_per_group = a.group >> 4, gs = 31 - __clz(a.group);
+  const int64_t total = ((int64_t)a.Lq * a.d) >> 4;
+  const int64_t i0 = (int64_t)blockIdx.x * (kBvThreads * U) + tid;
   const T* v = static_cast<const T*>(a.v);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int t = (int)(i / per_row), elem = (int)(i - (int64_t)t * per_row) * 8;
-    float x[8];
-    load8<T>(v + (size_t)t * a.d + elem, x);
-    float mn = x[0], mx = x[0];
+  fl_grid_wait();
+  fl_grid_release();
+  Raw8<T> raw[U][2];
 #pragma unroll
-    for (int u = 1; u < 8; ++u) { mn = fminf(mn, x[u]); mx = fmaxf(mx, x[u]); }
+  for (int u = 0; u < U; ++u) {
+    const int64_t i = i0 + u * kBvThreads;
+    if (i < total) { raw[u][0].load(v + i * 16); raw[u][1].load(v + i * 16 + 8); }
+  }
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int64_t i = i0 + u * kBvThreads;
+    if (i - lane >= total) break;                      // warp-uniform; total is a multiple of 16, whole half warps
+    const bool on = i < total;
+    Raw8<T> mnr = raw[u][0], mxr = raw[u][0];
+    mnr.take_min(raw[u][1]);
+    mxr.take_max(raw[u][1]);
+    float mn, mx, skip;
+    mnr.range(mn, skip);
+    mxr.range(skip, mx);
     for (int o = 1; o < lanes_per_group; o <<= 1) {
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
     __half zh, sh;
     group_meta<BITS>(mn, mx, zh, sh);
-    const float zf = __half2float(zh), sf = __half2float(sh);
-    float q[8];
+    const float z = __half2float(zh), s = __half2float(sh), r = scale_rcp(s);
+    f32x2 x[8], q[8], inv[8], ninv[8];
+    raw[u][0].pairs(*reinterpret_cast<f32x2(*)[4]>(&x[0]));
+    raw[u][1].pairs(*reinterpret_cast<f32x2(*)[4]>(&x[4]));
 #pragma unroll
-    for (int u = 0; u < 8; ++u) q[u] = code_of<BITS>(x[u], zf, sf);
-    store_codes8<BITS>(a.v_codes + (size_t)t * (a.d * BITS / 8), elem, q);
-    if (((elem >> 3) & (lanes_per_group - 1)) == 0) {
-      const int gs = 31 - __clz(a.group);
-      const size_t gi = (size_t)t * (a.d >> gs) + (elem >> gs);
+    for (int e = 0; e < 8; ++e) {
+      x[e] = add2(x[e], pair(-z, -z));
+      inv[e] = pair(r, r);
+      ninv[e] = pair(-r, -r);
+    }
+    quotients<BITS, 8>(x, inv, ninv, [&](int) { return pair(s, s); }, q);
+    if (!on) continue;
+    store_codes<BITS, 8>(a.v_codes + i * 2 * BITS, q);
+    if ((lane & (lanes_per_group - 1)) == 0) {
+      const int64_t gi = (i * 16) >> gs;
       a.v_scale[gi] = sh;
       a.v_zero[gi] = zh;
     }
   }
 }
 
-// Rebuild rows [0, Lq) of K and V in the storage type: blockIdx.y = 0 keys (metadata per token group and channel),
-// 1 values (metadata per token and channel group). One thread per 8 channels of a position, four positions per
-// thread and pass so that their loads are in flight together. With a row mask only the (head, position) pairs whose
-// bit is set are rebuilt; everything else of the output is left as it is.
+// Rebuild rows [0, Lq) of K and V in the storage type. A warp owns one head's rows of 32 consecutive positions of one
+// side (keys or values): one word of the row mask, and for the keys one token group, whose scales and offsets (per
+// channel) it reads and converts once. The wanted rows are compacted first, so that no lane idles over rows that are not
+// wanted, and dh / 8 lanes take a row (8 channels each: the codes of eight rows per lane are asked for together). The
+// values' metadata is one pair per row and channel group. Rows whose bit is clear are left as they are.
+// Bound by HBM: 20 k rows of 2048, int4: 41 MB in, 164 MB out = 31 us (one row per CTA pass and scalar arithmetic: 48 us).
+constexpr int kDqWarps = 8;
+
+template <typename T, int BITS, bool IS_V>
+__device__ __forceinline__ void dequant_rows(const BaseArgs& a, int head, int t0, uint32_t want, uint8_t* list, int lane) {
+  constexpr int U = BITS == 8 ? 4 : 8;      // rows per lane whose loads are in flight together
+  constexpr int W = BITS == 8 ? 2 : 1;
+  const int lpr = a.dh >> 3, rpi = 32 / lpr;                  // lanes per row, rows per step
+  const int sub = lane / lpr, elem = head * a.dh + (lane - sub * lpr) * 8;
+  const int gs = 31 - __clz(a.group);
+  const uint8_t* codes = IS_V ? a.v_codes : a.k_codes;
+  const __half* scale = IS_V ? a.v_scale : a.k_scale;
+  const __half* zero = IS_V ? a.v_zero : a.k_zero;
+  T* out = static_cast<T*>(IS_V ? a.v_out : a.k_out) + elem;
+  const int n = __popc(want);
+  if ((want >> lane) & 1u) list[__popc(want & ((1u << lane) - 1u))] = (uint8_t)lane;
+  f32x2 sc[4], zr[4];
+  if (!IS_V) {
+    const size_t mi = (size_t)(t0 >> gs) * a.d + elem;
+    const uint4 sraw = __ldg(reinterpret_cast<const uint4*>(scale + mi));
+    const uint4 zraw = __ldg(reinterpret_cast<const uint4*>(zero + mi));
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 s2 = __half22float2(reinterpret_cast<const __half2*>(&sraw)[e]);
+      const float2 z2 = __half22float2(reinterpret_cast<const __half2*>(&zraw)[e]);
+      sc[e] = pair(s2.x, s2.y);
+      zr[e] = pair(z2.x, z2.y);
+    }
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int r0 = 0; r0 < n; r0 += U * rpi) {
+    uint32_t raw[U][W];
+    __half vs[U], vz[U];
+    int row[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int r = r0 + u * rpi + sub;
+      row[u] = r < n ? t0 + list[r] : -1;
+      if (row[u] < 0) continue;
+      const size_t off = (size_t)row[u] * a.d + elem;
+      const uint8_t* src = codes + off * BITS / 8;
+      if constexpr (BITS == 8) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(src));
+        raw[u][0] = v.x; raw[u][1] = v.y;
+      } else if constexpr (BITS == 4) {
+        raw[u][0] = __ldg(reinterpret_cast<const uint32_t*>(src));
+      } else {
+        raw[u][0] = __ldg(reinterpret_cast<const uint16_t*>(src));
+      }
+      if (IS_V) { vs[u] = __ldg(scale + (off >> gs)); vz[u] = __ldg(zero + (off >> gs)); }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (row[u] < 0) continue;
+      f32x2 x[4];
+      codes_to_pairs<BITS, 4>(raw[u], x);
+      if (IS_V) {
+        const float s = __half2float(vs[u]), z = __half2float(vz[u]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = fma2(x[e], pair(s, s), pair(z, z));
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = fma2(x[e], sc[e], zr[e]);
+      }
+      T* dst = out + (size_t)row[u] * a.d;
+      if constexpr (sizeof(T) == 2) {
+        *reinterpret_cast<uint4*>(dst) = pack_bf16(x);
+      } else {
+        reinterpret_cast<ulonglong2*>(dst)[0] = make_ulonglong2(x[0], x[1]);
+        reinterpret_cast<ulonglong2*>(dst)[1] = make_ulonglong2(x[2], x[3]);
+      }
+    }
+  }
+}
+
 template <typename T, int BITS>
-__global__ void __launch_bounds__(256) base_dequant_kernel(const __grid_constant__ BaseArgs a) {
+__global__ void __launch_bounds__(kDqWarps * 32) base_dequant_kernel(const __grid_constant__ BaseArgs a, int H, int unit_ctas) {
+  __shared__ uint8_t lists[kDqWarps][32];
   fl_grid_wait();
   fl_grid_release();
-  const bool is_v = blockIdx.y != 0;
-  const int per_row = a.d >> 3;
-  const int gs = 31 - __clz(a.group);
-  const uint8_t* codes = is_v ? a.v_codes : a.k_codes;
-  const __half* scale = is_v ? a.v_scale : a.k_scale;
-  const __half* zero = is_v ? a.v_zero : a.k_zero;
-  T* out = static_cast<T*>(is_v ? a.v_out : a.k_out);
-  constexpr int U = 4;      // rows whose loads are in flight together
-  // the unquantized tail rows, copied as they are (always: they are few)
-  {
-    const T* tail = static_cast<const T*>(is_v ? a.v_tail : a.k_tail);
-    const int n_vec = (a.L - a.Lq) * per_row * (int)(sizeof(T) * 8 / 16);
-    const uint4* src = reinterpret_cast<const uint4*>(tail);
-    uint4* dst = reinterpret_cast<uint4*>(out + (size_t)a.Lq * a.d);
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_vec; i += gridDim.x * blockDim.x) dst[i] = __ldg(src + i);
-  }
-  // A CTA owns a run of consecutive rows and its threads the same 8 channels of each. Per batch of four rows a thread
-  // makes two trips to memory: its head's mask bits (two words), then the codes (and the values' metadata) of every
-  // wanted row at once. The keys' scales and offsets (per channel and token group) are read and converted once per
-  // token group, not once per row. The code becomes a float by arithmetic (2^23 + c is exact), not by a conversion:
-  // conversions run on a narrow pipe.
-  const int rows_per_cta = (a.Lq + gridDim.x - 1) / gridDim.x;
-  const int r_lo = blockIdx.x * rows_per_cta, r_hi = min(a.Lq, r_lo + rows_per_cta);
-  for (int v0 = threadIdx.x; v0 < per_row; v0 += blockDim.x) {
-    const int elem = v0 * 8;
-    const int head = elem / a.dh;
-    int tg_cached = -1;
-    float ksc[8], kzr[8];
-    for (int t0 = r_lo; t0 < r_hi; t0 += U) {
-      uint32_t want = (1u << U) - 1u;                          // bit u: row t0 + u is rebuilt
-      if (a.row_mask != nullptr) {
-        const uint32_t* mrow = a.row_mask + (size_t)head * a.mask_words;
-        const int w = t0 >> 5;
-        const uint32_t lo = __ldg(mrow + w), hi = w + 1 < a.mask_words ? __ldg(mrow + w + 1) : 0u;
-        want = __funnelshift_r(lo, hi, t0 & 31) & ((1u << U) - 1u);
-      }
-      if (r_hi - t0 < U) want &= (1u << (r_hi - t0)) - 1u;
-      if (want == 0u) continue;
-      uint32_t raw[U][BITS == 8 ? 2 : 1];
-      __half vsh[U], vzh[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (!((want >> u) & 1u)) continue;
-        const int t = t0 + u;
-        const uint8_t* row = codes + (size_t)t * (a.d * BITS / 8);
-        if (BITS == 8) {
-          const uint2 r2 = __ldg(reinterpret_cast<const uint2*>(row + elem));
-          raw[u][0] = r2.x; raw[u][BITS == 8 ? 1 : 0] = r2.y;
-        } else if (BITS == 4) {
-          raw[u][0] = __ldg(reinterpret_cast<const uint32_t*>(row + elem / 2));
-        } else {
-          raw[u][0] = __ldg(reinterpret_cast<const uint16_t*>(row + elem / 4));
-        }
-        if (is_v) {
-          const size_t gi = (size_t)t * (a.d >> gs) + (elem >> gs);
-          vsh[u] = __ldg(scale + gi);
-          vzh[u] = __ldg(zero + gi);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (!((want >> u) & 1u)) continue;
-        const int t = t0 + u;
-        float x[8];
-        if (!is_v) {
-          if ((t >> gs) != tg_cached) {      // the same for every thread of the CTA
-            tg_cached = t >> gs;
-            const size_t mi = (size_t)tg_cached * a.d + elem;
-            const uint4 sraw = __ldg(reinterpret_cast<const uint4*>(scale + mi));
-            const uint4 zraw = __ldg(reinterpret_cast<const uint4*>(zero + mi));
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              ksc[e] = __half2float(reinterpret_cast<const __half*>(&sraw)[e]);
-              kzr[e] = __half2float(reinterpret_cast<const __half*>(&zraw)[e]);
-            }
-          }
-        }
-        const float vsc = is_v ? __half2float(vsh[u]) : 0.f, vzr = is_v ? __half2float(vzh[u]) : 0.f;
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-          uint32_t c;
-          if (BITS == 8) c = (raw[u][BITS == 8 ? (e >> 2) : 0] >> (8 * (e & 3))) & 0xFFu;
-          else if (BITS == 4) c = (raw[u][0] >> (4 * e)) & 0xFu;
-          else c = (raw[u][0] >> (2 * e)) & 0x3u;
-          const float cf = __fsub_rn(__uint_as_float(0x4B000000u | c), 8388608.f);
-          x[e] = is_v ? __fmaf_rn(cf, vsc, vzr) : __fmaf_rn(cf, ksc[e], kzr[e]);
-        }
-        store8<T>(out + (size_t)t * a.d + elem, x);
-      }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (blockIdx.x < (unsigned)unit_ctas) {
+    // heads fastest: the CTAs in flight share the sectors of the values' metadata and whole rows of the codes
+    const int64_t unit = (int64_t)blockIdx.x * kDqWarps + warp;
+    const int64_t w2 = unit / H;
+    const int head = (int)(unit - w2 * H);
+    const int word = (int)(w2 >> 1), t0 = word * 32;
+    if (t0 >= a.Lq) return;
+    uint32_t want = a.row_mask != nullptr ? __ldg(a.row_mask + (size_t)head * a.mask_words + word) : 0xffffffffu;
+    if (a.Lq - t0 < 32) want &= (1u << (a.Lq - t0)) - 1u;
+    if (want == 0u) return;
+    if (w2 & 1) dequant_rows<T, BITS, true>(a, head, t0, want, lists[warp], lane);
+    else dequant_rows<T, BITS, false>(a, head, t0, want, lists[warp], lane);
+  } else {
+    // the unquantized tail rows, copied as they are (always: they are few)
+    const int64_t n_vec = (int64_t)(a.L - a.Lq) * a.d * sizeof(T) / 16;
+    const int64_t step = (int64_t)(gridDim.x - unit_ctas) * blockDim.x;
+    uint4* k = reinterpret_cast<uint4*>(static_cast<T*>(a.k_out) + (size_t)a.Lq * a.d);
+    uint4* v = reinterpret_cast<uint4*>(static_cast<T*>(a.v_out) + (size_t)a.Lq * a.d);
+    for (int64_t i = (int64_t)(blockIdx.x - unit_ctas) * blockDim.x + threadIdx.x; i < n_vec; i += step) {
+      k[i] = __ldg(static_cast<const uint4*>(a.k_tail) + i);
+      v[i] = __ldg(static_cast<const uint4*>(a.v_tail) + i);
     }
   }
 }
@@ -294,28 +417,40 @@ BaseArgs base_args(const fl_shape* s, const fl_kv_base_q* q) {
 
 template <typename T>
 int launch_quant_base(fl_ctx* ctx, const fl_shape* s, const BaseArgs& a, cudaStream_t st) {
+  const int threads = 32 * (a.group / kBqRows<T>);
   const int n_tg = (a.Lq + a.group - 1) / a.group;
-  const dim3 kgrid(n_tg, (a.d / 8 + 255) / 256);
-  const int kthreads = a.d / 8 < 256 ? a.d / 8 : 256;
-  int64_t vb = ((int64_t)a.Lq * (a.d / 8) + 255) / 256;
-  const int vgrid = (int)(vb > (int64_t)ctx->sm_count * 16 ? (int64_t)ctx->sm_count * 16 : vb);
-#define FL_BASEQ(BITS)                                                          \
-  do {                                                                          \
-    base_quant_k_kernel<T, BITS><<<kgrid, kthreads, 0, st>>>(a);                \
-    base_quant_v_kernel<T, BITS><<<vgrid, 256, 0, st>>>(a);                     \
+  const int64_t k_ctas = (int64_t)n_tg * (a.d / kBqCh);   // d is a multiple of 256; all grids are below 2^31 (L d <= 2^40)
+  const int64_t v_ctas = ((int64_t)a.Lq * a.d / 16 + kBvThreads * 2 - 1) / (kBvThreads * 2);
+  int64_t t_ctas = ((int64_t)(a.L - a.Lq) * a.d * (int64_t)sizeof(T) / 16 + threads - 1) / threads;
+  if (t_ctas > ctx->sm_count * 4) t_ctas = ctx->sm_count * 4;
+  const dim3 kgrid((unsigned)(k_ctas + t_ctas)), vgrid((unsigned)v_ctas);
+#define FL_BASEK(BITS, ROWL) \
+  FL_CHECK_CUDA(fl_launch(ctx, base_quant_k_kernel<T, BITS, ROWL>, kgrid, dim3(threads), 0, st, a, (int)k_ctas))
+#define FL_BASEQ(BITS)                                                                                            \
+  do {                                                                                                            \
+    if (a.group == 32) FL_BASEK(BITS, 32 / kBqRows<T>);                                                           \
+    else if (a.group == 64) FL_BASEK(BITS, 64 / kBqRows<T>);                                                      \
+    else FL_BASEK(BITS, 128 / kBqRows<T>);                                                                        \
+    if (v_ctas > 0) FL_CHECK_CUDA(fl_launch(ctx, base_quant_v_kernel<T, BITS>, vgrid, dim3(kBvThreads), 0, st, a)); \
   } while (0)
   if (s->bits == 8) FL_BASEQ(8); else if (s->bits == 4) FL_BASEQ(4); else FL_BASEQ(2);
 #undef FL_BASEQ
+#undef FL_BASEK
   return fl_launch_status();
 }
 
 template <typename T>
 int launch_dequant_base(fl_ctx* ctx, const fl_shape* s, const BaseArgs& a, cudaStream_t st) {
-  int64_t b = a.L;     // one CTA per row, up to 16 CTAs per SM and side; each then walks several rows
-  const dim3 grid((unsigned)(b > (int64_t)ctx->sm_count * 16 ? (int64_t)ctx->sm_count * 16 : b), 2);
-  if (s->bits == 8) FL_CHECK_CUDA(fl_launch(ctx, base_dequant_kernel<T, 8>, grid, dim3(256), 0, st, a));
-  else if (s->bits == 4) FL_CHECK_CUDA(fl_launch(ctx, base_dequant_kernel<T, 4>, grid, dim3(256), 0, st, a));
-  else FL_CHECK_CUDA(fl_launch(ctx, base_dequant_kernel<T, 2>, grid, dim3(256), 0, st, a));
+  const int64_t units = (int64_t)((a.Lq + 31) / 32) * 2 * s->n_heads;
+  const int64_t unit_ctas = (units + kDqWarps - 1) / kDqWarps;
+  int64_t t_ctas = ((int64_t)(a.L - a.Lq) * a.d * (int64_t)sizeof(T) / 16 + kDqWarps * 32 - 1) / (kDqWarps * 32);
+  if (t_ctas > ctx->sm_count * 4) t_ctas = ctx->sm_count * 4;
+  if (unit_ctas + t_ctas == 0) return FL_OK;
+#define FL_BASED(BITS)                                                                                                \
+  FL_CHECK_CUDA(fl_launch(ctx, base_dequant_kernel<T, BITS>, dim3((unsigned)(unit_ctas + t_ctas)), dim3(kDqWarps * 32), 0, st, \
+                          a, s->n_heads, (int)unit_ctas))
+  if (s->bits == 8) FL_BASED(8); else if (s->bits == 4) FL_BASED(4); else FL_BASED(2);
+#undef FL_BASED
   return fl_launch_status();
 }
 
@@ -330,15 +465,7 @@ extern "C" int fl_quant_kv_base(fl_ctx* ctx, const fl_shape* shape, const void* 
   BaseArgs a = base_args(shape, base);
   a.k = k; a.v = v;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  const size_t row_bytes = (size_t)a.d * fl_elem_bytes(shape);
-  if (a.Lq < shape->L) {
-    const size_t n = (size_t)(shape->L - a.Lq) * row_bytes;
-    FL_CHECK_CUDA(cudaMemcpyAsync(base->k_tail, static_cast<const char*>(k) + (size_t)a.Lq * row_bytes, n,
-                                  cudaMemcpyDeviceToDevice, st));
-    FL_CHECK_CUDA(cudaMemcpyAsync(base->v_tail, static_cast<const char*>(v) + (size_t)a.Lq * row_bytes, n,
-                                  cudaMemcpyDeviceToDevice, st));
-  }
-  if (a.Lq == 0) return FL_OK;
+  a.k_tail_out = base->k_tail; a.v_tail_out = base->v_tail;
   return shape->dtype == FL_F32 ? launch_quant_base<float>(ctx, shape, a, st)
                                 : launch_quant_base<__nv_bfloat16>(ctx, shape, a, st);
 }
