@@ -3,8 +3,10 @@
 // selected column subset and cached mass; nothing is shared between queries, so the work is a gather of the selected
 // K/V rows, rebuilt on the way from the base and the residual streams (Eq. 8 chain, dequantize-and-add in
 // registers), two dot products and two weighted sums per column: bound by the bytes of the selected rows.
-// One CTA per (query, head); a group of dh/8 lanes owns a column at a time (16-byte loads, 8 elements per lane).
+// Two kernels: tensor-core tiles for bf16 rows of 128 (below), and for everything else one CTA per (query, head) in
+// which a group of dh/8 lanes owns a column at a time (16-byte loads, 8 elements per lane).
 #include "attn_simt.cuh"
+#include "codec.cuh"
 
 namespace {
 
@@ -149,161 +151,542 @@ __global__ void __launch_bounds__(kDecThreads) decode_attn_kernel(const __grid_c
   decode_merge<T, DH, G>(a, qh, cnt, g, ch, lse_p, mass, m_run, l_run, acc_o, acc_n, acc_o_s, acc_n_s, stat_s, logit_s);
 }
 
-// The same for bf16 storage, head dimension 128 and at most four residual streams (NS = loop_r - 1), with the
-// dependent lookups taken out of the main loop: the column list and, per stream, the slot of every selected column
-// are staged in shared memory first (two rounds of independent loads for the whole problem), so that an iteration's
-// loads (base rows and payloads of two columns per lane group) depend on nothing but shared memory and the hardware
-// keeps several iterations' bytes in flight. Without this every iteration is three dependent trips to memory.
+// ------------------------------------------------------------------------------------------------------------
+// The same for bf16 storage, head dimension 128 and at most four residual streams (NS = loop_r - 1), on tensor cores.
+//
+// What bounds it: the selected rows are 256-byte pieces scattered over the whole K/V base, 512 bytes a column, so the
+// floor is the HBM time of those bytes. Sixteen lanes per column with every element unpacked, rebuilt, rounded and
+// multiplied in registers took ~250 warp instructions per two columns, more than the issue slots the HBM time leaves,
+// and kept 32 KB per SM in flight. Here a warp takes 16 columns at a time: their K and V rows come by 16-byte
+// asynchronous copies into a double buffer of its own (8 KB a stage, no registers held while they fly), the logits of
+// both terms are 8 mma (A = the 16 K rows, B = q_old | q_new), and the weighted sums 8 mma (A = V transposed, B = the
+// probabilities): ~15 instructions a column. Nothing is rounded on the way: K, V and q are bf16 in storage and their
+// products exact; a probability (binary32) goes in as three bf16 pieces (hi + mid + lo = 24 bits) in three of the
+// eight columns that the instruction has anyway: [old hi, mid, lo, new hi, mid, lo, 0, 0].
+// The columns are split into those without any payload (plain rows, as above) and those with one, which are rebuilt
+// in registers (Eq. 8 chain) as the rows before and after the loop's own residual and go through two tile pairs.
+// A problem is split over a cluster of SPLIT CTAs (distributed shared memory joins their results): few queries would
+// leave most SMs idle otherwise, and a CTA with at most 512 columns has lists short enough for three CTAs per SM.
+// ------------------------------------------------------------------------------------------------------------
+constexpr int kMmaWarps = 4;
+constexpr int kMmaThreads = kMmaWarps * 32;
+constexpr int kMmaTile = 16;                               // columns of a tile
+constexpr int kMmaTileBytes = kMmaTile * 256;              // K or V rows of a tile
+constexpr int kMmaStages = 2;
+constexpr int kMmaStageBytes = 2 * kMmaTileBytes;          // K | V
+constexpr int kMmaMaxSplit = 8;                            // portable cluster size
+
+struct DecMmaCtl {
+  float acc[kMmaWarps][2][128];      // per warp: old and new weighted sums
+  float stat[kMmaWarps][3];          // mass, reference, row sum
+  float out[2][128];                 // the CTA's sums (new: against its own reference), read by the cluster
+  float cta_stat[3];
+  int warp_cnt[kMmaWarps][2];
+};
+
+__host__ __device__ constexpr size_t decode_mma_smem(int per_cta) {
+  // tiles, control block, then per column: position, logit, index in the piece
+  return 128 + (size_t)kMmaWarps * kMmaStages * kMmaStageBytes + sizeof(DecMmaCtl) + (size_t)per_cta * (4 + 4 + 2);
+}
+
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t addr, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+// byte offset of 16-byte piece `ch` (0..15) of row `row` in a tile: pieces are XOR-swizzled by the row so that the
+// eight rows of an 8x8 matrix lie in different banks
+__device__ __forceinline__ uint32_t tile_off(int row, int ch) { return (uint32_t)(row * 256 + ((ch ^ (row & 7)) << 4)); }
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ float dsmem_ld(const float* p, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  float v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
+  return v;
+}
+
+// One stream's payload of eight elements added to their pairs (BITS 16: the stored row takes their place).
+template <int BITS>
+__device__ __forceinline__ void dec_payload(const Payload8<__nv_bfloat16, BITS>& p, fl_codec::f32x2 (&x)[4]) {
+  if constexpr (BITS == 16) {
+    fl_codec::unpack_bf16(p.raw, x);
+  } else {
+    const float sc = __half2float(p.sc), zr = __half2float(p.zr);
+    const uint32_t w[2] = {p.raw.x, p.raw.y};
+    fl_codec::f32x2 c[4];
+    fl_codec::codes_to_pairs<BITS, 4>(w, c);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = fl_codec::add2(x[i], fl_codec::fma2(c[i], fl_codec::pair(sc, sc), fl_codec::pair(zr, zr)));
+  }
+}
+
+// Running state of a warp: both terms' weighted sums as D[dim][variant] tiles, the old term's mass, the new term's
+// reference and sum (mass and sum as per-lane partials of the lanes that hold logits).
+struct DecMmaState {
+  float acc[8][4];
+  float mass, l, ref;
+};
+
+// One tile: logits from k_old / k_new (the same address for plain columns), probabilities, weighted sums of v_old /
+// v_new. `n_valid` columns count; `lu` is the local index of the lane's column pair (valid in lanes t == 0).
+__device__ __forceinline__ void dec_tile(DecMmaState& st, const uint32_t (&bq)[8][2], uint32_t k_old, uint32_t k_new,
+                                         uint32_t v_old, uint32_t v_new, bool two, int n_valid, float scale, float lse_p,
+                                         const uint16_t* ord_u, float* logit_s, int lane) {
+  const int g = lane >> 2, t = lane & 3;
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  {
+    const int row = lane & 15, half = lane >> 4;
+    float e[4] = {0.f, 0.f, 0.f, 0.f};      // two chains: an mma waits for the one before it in its chain
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      uint32_t a[4];
+      ldsm4(k_old + tile_off(row, kk * 2 + half), a);
+      mma_16816((kk & 1) ? e : s, a, bq[kk][0], bq[kk][1]);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] += e[i];
+    if (two) {                       // the new term's logits come from the rows after the loop's residual
+      float s2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int kk = 0; kk < 8; ++kk) {
+        uint32_t a[4];
+        ldsm4(k_new + tile_off(row, kk * 2 + half), a);
+        mma_16816(s2, a, bq[kk][0], bq[kk][1]);
+      }
+      s[1] = s2[1];
+      s[3] = s2[3];
+    }
+  }
+  // lanes t == 0 hold (old, new) logits of columns g and g + 8
+  const bool on0 = t == 0 && g < n_valid, on1 = t == 0 && g + 8 < n_valid;
+  const float sn0 = s[1] * scale, sn1 = s[3] * scale;
+  if (on0) logit_s[ord_u[g]] = sn0;
+  if (on1) logit_s[ord_u[g + 8]] = sn1;
+  float mx = fmaxf(on0 ? sn0 : -INFINITY, on1 ? sn1 : -INFINITY);
+#pragma unroll
+  for (int o = 16; o >= 4; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  mx = __shfl_sync(0xffffffffu, mx, 0);
+  if (mx > st.ref) {                 // warp-uniform: the new term moves to a larger reference
+    const float f = expf(st.ref - mx);                  // 0 the first time (ref = -inf)
+    st.ref = mx;
+    st.l *= f;
+    const float f0 = t >= 2 ? f : 1.f, f1 = t >= 1 ? f : 1.f;   // variants 3, 4, 5 belong to the new term
+#pragma unroll
+    for (int m = 0; m < 8; ++m) { st.acc[m][0] *= f0; st.acc[m][1] *= f1; st.acc[m][2] *= f0; st.acc[m][3] *= f1; }
+  }
+  float p[4] = {0.f, 0.f, 0.f, 0.f};
+  if (on0) { p[0] = expf(s[0] * scale - lse_p); p[1] = expf(sn0 - st.ref); }
+  if (on1) { p[2] = expf(s[2] * scale - lse_p); p[3] = expf(sn1 - st.ref); }
+  st.mass += p[0] + p[2];
+  st.l += p[1] + p[3];
+  // B operand of the weighted sums: lane (g, t) needs variant g of columns 2t, 2t+1, 2t+8, 2t+9
+  uint32_t bo[2] = {0u, 0u}, bn[2] = {0u, 0u};
+#pragma unroll
+  for (int hf = 0; hf < 2; ++hf) {
+    float v[2];
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float po = __shfl_sync(0xffffffffu, p[2 * hf], 4 * (2 * t + e));
+      const float pn = __shfl_sync(0xffffffffu, p[2 * hf + 1], 4 * (2 * t + e));
+      v[e] = g < 3 ? po : pn;
+    }
+    const int piece = g < 3 ? g : g - 3;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const float hi = __bfloat162float(__float2bfloat16_rn(v[e]));
+      const float r1 = v[e] - hi;
+      const float mid = __bfloat162float(__float2bfloat16_rn(r1));
+      v[e] = g >= 6 ? 0.f : (piece == 0 ? hi : (piece == 1 ? mid : r1 - mid));
+    }
+    const uint32_t w = bf16_pair(v[0], v[1]);
+    if (!two || g < 3) bo[hf] = w;
+    if (two && g >= 3) bn[hf] = w;
+  }
+  {
+    const int col = (lane & 7) + ((lane >> 4) << 3), half = (lane >> 3) & 1;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+      uint32_t a[4];
+      ldsm4_t(v_old + tile_off(col, m * 2 + half), a);
+      mma_16816(st.acc[m], a, bo[0], bo[1]);
+    }
+    if (two) {
+#pragma unroll
+      for (int m = 0; m < 8; ++m) {
+        uint32_t a[4];
+        ldsm4_t(v_new + tile_off(col, m * 2 + half), a);
+        mma_16816(st.acc[m], a, bn[0], bn[1]);
+      }
+    }
+  }
+}
+
 template <int BITS, int NS>
-__global__ void __launch_bounds__(kDecThreads) decode_attn_staged_kernel(const __grid_constant__ DecodeArgs a) {
+__global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const __grid_constant__ DecodeArgs a, int split,
+                                                                         int per_cta) {
   using T = __nv_bfloat16;
-  constexpr int DH = 128, LPC = 16, CPW = 2, G = kDecWarps * CPW, UN = 2;
-  extern __shared__ __align__(16) float smem[];
-  float* acc_o_s = smem;
-  float* acc_n_s = acc_o_s + G * DH;
-  float* stat_s = acc_n_s + G * DH;
-  float* logit_s = stat_s + 3 * G;
-  int32_t* col_s = reinterpret_cast<int32_t*>(logit_s + a.c);          // [c]
-  int32_t* slot_s = col_s + a.c;                                       // [NS][c]
+  constexpr int DH = 128;
+  extern __shared__ __align__(16) uint8_t dyn[];
+  uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn) + 127) & ~uintptr_t(127));
+  DecMmaCtl& ctl = *reinterpret_cast<DecMmaCtl*>(tiles + kMmaWarps * kMmaStages * kMmaStageBytes);
+  int32_t* ord_col = reinterpret_cast<int32_t*>(&ctl + 1);      // [per_cta] positions: plain columns, then the others
+  float* logit_s = reinterpret_cast<float*>(ord_col + per_cta);   // [per_cta] by index in the CTA's piece of the list
+  uint16_t* ord_u = reinterpret_cast<uint16_t*>(logit_s + per_cta);   // [per_cta] index in the piece of an ordered column
   fl_grid_wait();
   fl_grid_release();
-  const int t = blockIdx.x, h = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int sub = lane / LPC, ch = lane % LPC;
-  const int g = warp * CPW + sub;
-  const size_t qh = (size_t)t * a.H + h;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int part = split > 1 ? (int)cluster_rank() : 0;
+  const int prob = blockIdx.x / split;                          // (query, head)
+  const int h = prob % a.H;
+  const size_t qh = (size_t)prob;
   const int cnt = min(__ldg(a.col_cnt + qh), a.c);
-  const int32_t* cols = a.col_idx + qh * a.c;
-  for (int u = threadIdx.x; u < cnt; u += kDecThreads) {
-    const int j = __ldg(cols + u);
-    col_s[u] = j;
-#pragma unroll
-    for (int s_ = 0; s_ < NS; ++s_) slot_s[s_ * a.c + u] = __ldg(a.k.s[s_].slot + j);
-  }
-  const int elem = h * DH + ch * 8;
-  float qo[8], qn[8];
-  load8<T>(static_cast<const T*>(a.q_old) + qh * DH + ch * 8, qo);
-  load8<T>(static_cast<const T*>(a.q_new) + qh * DH + ch * 8, qn);
+  const int u_lo = min(cnt, part * per_cta), n = min(cnt, (part + 1) * per_cta) - u_lo;
+  const int32_t* cols = a.col_idx + qh * a.c + u_lo;
   const float lse_p = a.lse_prev[qh];
-  float mass = 0.f, m_run = -INFINITY, l_run = 0.f, acc_o[8], acc_n[8];
+
+  // B operand of the logits: column 0 = q_old, column 1 = q_new, the other six zero
+  uint32_t bq[8][2];
+  {
+    const int g = lane >> 2, t = lane & 3;
+    const T* q = static_cast<const T*>(g == 0 ? a.q_old : a.q_new) + qh * DH;
 #pragma unroll
-  for (int i = 0; i < 8; ++i) acc_o[i] = acc_n[i] = 0.f;
-  __syncthreads();
+    for (int kk = 0; kk < 8; ++kk)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf)
+        bq[kk][hf] = g < 2 ? __ldg(reinterpret_cast<const uint32_t*>(q + kk * 16 + hf * 8 + t * 2)) : 0u;
+  }
+  // ---- partition: a warp owns a contiguous span of the piece; columns without a payload first --------------------
+  int n_plain;
+  {
+    int32_t* raw = reinterpret_cast<int32_t*>(tiles);    // staged in the idle tiles: position, complemented with a payload
+    const int span = ((n + kMmaWarps - 1) / kMmaWarps + 31) & ~31;
+    const int beg = warp * span, end = min(n, beg + span);
+    int n0 = 0, n1 = 0;
+#pragma unroll 1
+    for (int base = beg; base < end; base += 128) {      // four columns per lane and step in flight
+      int j[4];
+      bool pay[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int u = base + e * 32 + lane;
+        j[e] = u < end ? __ldg(cols + u) : -1;
+        pay[e] = false;
+      }
+#pragma unroll
+      for (int s = 0; s < NS; ++s) {
+        int sl[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sl[e] = j[e] >= 0 ? __ldg(a.k.s[s].slot + j[e]) : -1;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) pay[e] |= sl[e] >= 0;
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int u = base + e * 32 + lane;
+        n0 += __popc(__ballot_sync(0xffffffffu, u < end && !pay[e]));
+        n1 += __popc(__ballot_sync(0xffffffffu, u < end && pay[e]));
+        if (u < end) raw[u] = pay[e] ? ~j[e] : j[e];
+      }
+    }
+    if (lane == 0) { ctl.warp_cnt[warp][0] = n0; ctl.warp_cnt[warp][1] = n1; }
+    __syncthreads();
+    int tot0 = 0, before0 = 0, before1 = 0;
+#pragma unroll
+    for (int w = 0; w < kMmaWarps; ++w) {
+      tot0 += ctl.warp_cnt[w][0];
+      if (w < warp) { before0 += ctl.warp_cnt[w][0]; before1 += ctl.warp_cnt[w][1]; }
+    }
+    n_plain = tot0;
+    const uint32_t lt = (1u << lane) - 1;
+#pragma unroll 1
+    for (int base = beg; base < end; base += 32) {
+      const int u = base + lane;
+      const int r = u < end ? raw[u] : 0;
+      const bool pay = u < end && r < 0, plain = u < end && r >= 0;
+      const uint32_t m0 = __ballot_sync(0xffffffffu, plain), m1 = __ballot_sync(0xffffffffu, pay);
+      if (u < end) {
+        const int dst = pay ? tot0 + before1 + __popc(m1 & lt) : before0 + __popc(m0 & lt);
+        ord_col[dst] = pay ? ~r : r;
+        ord_u[dst] = (uint16_t)u;
+      }
+      before0 += __popc(m0);
+      before1 += __popc(m1);
+    }
+    __syncthreads();
+  }
+  DecMmaState st;
+  st.mass = st.l = 0.f;
+  st.ref = -INFINITY;
+#pragma unroll
+  for (int m = 0; m < 8; ++m)
+#pragma unroll
+    for (int i = 0; i < 4; ++i) st.acc[m][i] = 0.f;
+  uint8_t* my_tiles = tiles + warp * kMmaStages * kMmaStageBytes;
+  const uint32_t my_addr = (uint32_t)__cvta_generic_to_shared(my_tiles);
+  const int ch = lane & 15, rsub = lane >> 4;
+  const int elem = h * DH + ch * 8;
   const T* kb = static_cast<const T*>(a.k.base) + elem;
   const T* vb = static_cast<const T*>(a.v.base) + elem;
-  for (int u0 = 0; u0 < cnt; u0 += G * UN) {
-    // every load of the two columns first
-    uint4 rk[UN], rv[UN];
-    Payload8<T, BITS> pk[UN][NS], pv[UN][NS];
-    int sl[UN][NS];
-    bool on[UN];
+
+  // The warp's tiles: plain ones first (dealt round robin from warp 0), then those of columns with a payload (from the
+  // last warp down). Base rows come by asynchronous copies, one tile ahead; a payload tile needs the other stage for
+  // its second pair of tiles, so the tile after it is asked for when it is done.
+  const int plain_tiles = (n_plain + kMmaTile - 1) / kMmaTile, pay_tiles = (n - n_plain + kMmaTile - 1) / kMmaTile;
+  const int my_plain = plain_tiles > warp ? (plain_tiles - warp + kMmaWarps - 1) / kMmaWarps : 0;
+  const int pw = kMmaWarps - 1 - warp;
+  const int my_tiles_n = my_plain + (pay_tiles > pw ? (pay_tiles - pw + kMmaWarps - 1) / kMmaWarps : 0);
+  // first ordered column of the warp's tile i, and the end of its class
+  auto tile_first = [&](int i) { return i < my_plain ? (i * kMmaWarps + warp) * kMmaTile
+                                                     : n_plain + ((i - my_plain) * kMmaWarps + pw) * kMmaTile; };
+  auto issue = [&](int i, int stage) {
+    const int first = tile_first(i), last = (i < my_plain ? n_plain : n) - 1;
+    const uint32_t dst = my_addr + stage * kMmaStageBytes;
 #pragma unroll
-    for (int q = 0; q < UN; ++q) {
-      const int u = u0 + q * G + g;
-      on[q] = u < cnt;
-      const int j = on[q] ? col_s[u] : 0;
-      rk[q] = on[q] ? __ldg(reinterpret_cast<const uint4*>(kb + (size_t)j * a.d)) : make_uint4(0, 0, 0, 0);
-      rv[q] = on[q] ? __ldg(reinterpret_cast<const uint4*>(vb + (size_t)j * a.d)) : make_uint4(0, 0, 0, 0);
-#pragma unroll
-      for (int s_ = 0; s_ < NS; ++s_) {
-        sl[q][s_] = on[q] ? slot_s[s_ * a.c + u] : -1;
-        if (sl[q][s_] >= 0) {
-          payload_load<T, BITS>(a.k.s[s_], sl[q][s_], elem, a.d, a.group, pk[q][s_]);
-          payload_load<T, BITS>(a.v.s[s_], sl[q][s_], elem, a.d, a.group, pv[q][s_]);
-        }
-      }
+    for (int q = 0; q < 8; ++q) {
+      const int row = q * 2 + rsub;
+      const size_t off = (size_t)ord_col[min(first + row, last)] * a.d;   // past the end: any row (its weight is zero)
+      const uint32_t o = dst + tile_off(row, ch);
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o), "l"(kb + off) : "memory");
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o + kMmaTileBytes), "l"(vb + off) : "memory");
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  if (my_tiles_n > 0) issue(0, 0);
+  int stage = 0;
+#pragma unroll 1
+  for (int i = 0; i < my_tiles_n; ++i) {
+    const int first = tile_first(i);
+    const uint32_t kt = my_addr + stage * kMmaStageBytes, vt = kt + kMmaTileBytes;
+    if (i < my_plain) {
+      if (i + 1 < my_tiles_n) {
+        issue(i + 1, stage ^ 1);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+      } else {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+      }
+      __syncwarp();
+      dec_tile(st, bq, kt, kt, vt, vt, false, n_plain - first, a.scale, lse_p, ord_u + first, logit_s, lane);
+      __syncwarp();
+    } else {
+      // Xhat^(r-1) takes the place of the base rows, Xhat^(r) goes to the other stage; each lane rebuilds the pieces it
+      // copied itself. The lanes of a half warp look up one stream row each and hand it on.
+      const int n_valid = min(kMmaTile, n - first);
+      const int jl = ord_col[min(first + (lane & 15), n - 1)];
+      int slot[NS];
 #pragma unroll
-    for (int q = 0; q < UN; ++q) {
-      float ko[8], kn[8], vo[8], vn[8];
-      {
-        const __nv_bfloat162* hk = reinterpret_cast<const __nv_bfloat162*>(&rk[q]);
-        const __nv_bfloat162* hv = reinterpret_cast<const __nv_bfloat162*>(&rv[q]);
+      for (int s = 0; s < NS; ++s) slot[s] = __ldg(a.k.s[s].slot + jl);
+      uint8_t* t_old = my_tiles + stage * kMmaStageBytes;
+      uint8_t* t_new = my_tiles + (stage ^ 1) * kMmaStageBytes;
+      const uint32_t kn = my_addr + (stage ^ 1) * kMmaStageBytes;
+      bool landed = false;
+      constexpr int E = (NS == 1 || (NS == 2 && BITS <= 4)) ? 4 : 2;   // columns per half warp whose payloads fit the registers
+#pragma unroll 1
+      for (int q0 = 0; q0 < 8; q0 += E) {
+        Payload8<T, BITS> pk[E][NS], pv[E][NS];
+        int sl[E][NS];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 fk = __bfloat1622float2(hk[i]), fv = __bfloat1622float2(hv[i]);
-          kn[2 * i] = fk.x; kn[2 * i + 1] = fk.y;
-          vn[2 * i] = fv.x; vn[2 * i + 1] = fv.y;
+        for (int e = 0; e < E; ++e)
+#pragma unroll
+          for (int s = 0; s < NS; ++s) {
+            sl[e][s] = __shfl_sync(0xffffffffu, slot[s], (q0 + e) * 2 + rsub);
+            if (sl[e][s] >= 0) {
+              payload_load<T, BITS>(a.k.s[s], sl[e][s], elem, a.d, a.group, pk[e][s]);
+              payload_load<T, BITS>(a.v.s[s], sl[e][s], elem, a.d, a.group, pv[e][s]);
+            }
+          }
+        if (!landed) { asm volatile("cp.async.wait_group 0;" ::: "memory"); landed = true; }
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const uint32_t o = tile_off((q0 + e) * 2 + rsub, ch);
+#pragma unroll
+          for (int kv = 0; kv < 2; ++kv) {
+            uint4* old_p = reinterpret_cast<uint4*>(t_old + o + kv * kMmaTileBytes);
+            fl_codec::f32x2 x[4];
+            fl_codec::unpack_bf16(*old_p, x);
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+              // Xhat^(r-1), rounded to the storage type as attention consumes it
+              if (s == NS - 1 && NS > 1) *old_p = fl_codec::pack_bf16(x);
+              if (sl[e][s] >= 0) dec_payload<BITS>(kv ? pv[e][s] : pk[e][s], x);
+            }
+            *reinterpret_cast<uint4*>(t_new + o + kv * kMmaTileBytes) = fl_codec::pack_bf16(x);
+          }
         }
       }
-      // Eq. 8 chain in loop order; the state before the loop's own stream is Xhat^(r-1)
-#pragma unroll
-      for (int s_ = 0; s_ < NS; ++s_) {
-        if (s_ == NS - 1) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) { ko[i] = kn[i]; vo[i] = vn[i]; }
-        }
-        if (sl[q][s_] >= 0) {
-          payload_apply<T, BITS>(pk[q][s_], kn);
-          payload_apply<T, BITS>(pv[q][s_], vn);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        ko[i] = to_float<T>(from_float<T>(ko[i])); kn[i] = to_float<T>(from_float<T>(kn[i]));
-        vo[i] = to_float<T>(from_float<T>(vo[i])); vn[i] = to_float<T>(from_float<T>(vn[i]));
-      }
-      float so = 0.f, sn = 0.f;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) { so = fmaf(qo[i], ko[i], so); sn = fmaf(qn[i], kn[i], sn); }
-#pragma unroll
-      for (int o = 1; o < LPC; o <<= 1) {
-        so += __shfl_xor_sync(0xffffffffu, so, o);
-        sn += __shfl_xor_sync(0xffffffffu, sn, o);
-      }
-      if (on[q]) {
-        const int u = u0 + q * G + g;
-        const float po = expf(so * a.scale - lse_p);
-        mass += po;
-        const float sv = sn * a.scale;
-        if (ch == 0) logit_s[u] = sv;
-        const float m_new = fmaxf(m_run, sv);
-        const float corr = expf(m_run - m_new);
-        const float pn = expf(sv - m_new);
-        l_run = l_run * corr + pn;
-        m_run = m_new;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-          acc_o[i] = fmaf(po, vo[i], acc_o[i]);
-          acc_n[i] = fmaf(pn, vn[i], acc_n[i] * corr);
-        }
-      }
+      __syncwarp();
+      dec_tile(st, bq, kt, kn, vt, kn + kMmaTileBytes, true, n_valid, a.scale, lse_p, ord_u + first, logit_s, lane);
+      __syncwarp();
+      if (i + 1 < my_tiles_n) issue(i + 1, stage ^ 1);
     }
+    stage ^= 1;
   }
-  decode_merge<T, DH, G>(a, qh, cnt, g, ch, lse_p, mass, m_run, l_run, acc_o, acc_n, acc_o_s, acc_n_s, stat_s, logit_s);
+  // ---- warps, then CTAs of the cluster, in a fixed order -------------------------------------------------------------
+  {
+    const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+    for (int m = 0; m < 8; ++m)
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {
+        const float c0 = st.acc[m][2 * hf], c1 = st.acc[m][2 * hf + 1];
+        // t = 0: old hi, mid; t = 1: old lo, new hi; t = 2: new mid, lo
+        const float from1_old = __shfl_sync(0xffffffffu, c0, (lane & ~3) + 1);
+        const float from1_new = __shfl_sync(0xffffffffu, c1, (lane & ~3) + 1);
+        const int dim = m * 16 + hf * 8 + g;
+        if (t == 0) ctl.acc[warp][0][dim] = (c0 + c1) + from1_old;
+        if (t == 2) ctl.acc[warp][1][dim] = from1_new + (c0 + c1);
+      }
+    float mass = st.mass, l = st.l;
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) {
+      mass += __shfl_xor_sync(0xffffffffu, mass, o);
+      l += __shfl_xor_sync(0xffffffffu, l, o);
+    }
+    if (lane == 0) { ctl.stat[warp][0] = mass; ctl.stat[warp][1] = st.ref; ctl.stat[warp][2] = l; }
+  }
+  __syncthreads();
+  {
+    float ref = -INFINITY, mass = 0.f, l = 0.f, f[kMmaWarps];
+#pragma unroll
+    for (int w = 0; w < kMmaWarps; ++w) { ref = fmaxf(ref, ctl.stat[w][1]); mass += ctl.stat[w][0]; }
+#pragma unroll
+    for (int w = 0; w < kMmaWarps; ++w) {
+      f[w] = ctl.stat[w][1] > -INFINITY ? expf(ctl.stat[w][1] - ref) : 0.f;
+      l += ctl.stat[w][2] * f[w];
+    }
+    float so = 0.f, sn = 0.f;
+#pragma unroll
+    for (int w = 0; w < kMmaWarps; ++w) { so += ctl.acc[w][0][tid]; sn += ctl.acc[w][1][tid] * f[w]; }
+    ctl.out[0][tid] = so;
+    ctl.out[1][tid] = sn;
+    if (tid == 0) { ctl.cta_stat[0] = mass; ctl.cta_stat[1] = ref; ctl.cta_stat[2] = l; }
+  }
+  if (split > 1) cluster_sync(); else __syncthreads();
+  float m_tot = -INFINITY, mass_tot = 0.f, l_tot = 0.f, so = 0.f, sn = 0.f;
+  if (split > 1) {
+    float rr[kMmaMaxSplit];
+#pragma unroll
+    for (int p = 0; p < kMmaMaxSplit; ++p)
+      if (p < split) {
+        rr[p] = dsmem_ld(&ctl.cta_stat[1], p);
+        m_tot = fmaxf(m_tot, rr[p]);
+        mass_tot += dsmem_ld(&ctl.cta_stat[0], p);
+      }
+#pragma unroll
+    for (int p = 0; p < kMmaMaxSplit; ++p)
+      if (p < split) {
+        const float f = rr[p] > -INFINITY ? expf(rr[p] - m_tot) : 0.f;
+        l_tot += dsmem_ld(&ctl.cta_stat[2], p) * f;
+        if (part == 0) {
+          so += dsmem_ld(&ctl.out[0][tid], p);
+          sn += dsmem_ld(&ctl.out[1][tid], p) * f;
+        }
+      }
+  } else {
+    m_tot = ctl.cta_stat[1]; mass_tot = ctl.cta_stat[0]; l_tot = ctl.cta_stat[2];
+    so = ctl.out[0][tid]; sn = ctl.out[1][tid];
+  }
+  const bool has = cnt > 0 && m_tot > -INFINITY && mass_tot > 0.f;
+  const float w = has ? mass_tot / l_tot : 0.f;
+  if (part == 0) {
+    const T* op = static_cast<const T*>(a.o_prev) + qh * DH;
+    T* oo = static_cast<T*>(a.o_out) + qh * DH;
+    const float prev = __bfloat162float(op[tid]);
+    oo[tid] = has ? __float2bfloat16_rn(prev - so + w * sn) : op[tid];
+    if (tid == 0) a.lse_out[qh] = has ? m_tot + logf(l_tot) - logf(mass_tot) : lse_p;
+  }
+  if (a.p_new_out != nullptr) {
+    float* po = a.p_new_out + qh * a.c + part * per_cta;
+    const int lim = min(a.c - part * per_cta, per_cta);
+    for (int u = tid; u < lim; u += kMmaThreads) po[u] = (has && u < n) ? w * expf(logit_s[u] - m_tot) : 0.f;
+  }
+  if (split > 1) cluster_sync();     // nobody leaves while another CTA still reads its shared memory
 }
 
 template <int BITS>
-int launch_decode_staged(const fl_ctx* ctx, const DecodeArgs& a, int n_streams, dim3 grid, size_t smem, cudaStream_t st) {
-#define FL_DECS(NS)                                                                                       \
-  do {                                                                                                    \
-    auto kern = decode_attn_staged_kernel<BITS, NS>;                                                      \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));    \
-    FL_CHECK_CUDA(fl_launch(ctx, kern, grid, dim3(kDecThreads), smem, st, a));                            \
-  } while (0)
-  switch (n_streams) {
-    case 1: FL_DECS(1); break;
-    case 2: FL_DECS(2); break;
-    case 3: FL_DECS(3); break;
-    default: FL_DECS(4); break;
+int launch_decode_mma(const fl_ctx* ctx, const DecodeArgs& a, int n_problems, cudaStream_t st) {
+  // Split of a problem: until a CTA has at most 512 columns (lists of ~10 KB, three CTAs per SM), and further while
+  // the grid does not fill two CTAs per SM and a CTA keeps a tile for each of its warps.
+  int split = 1;
+  while (split < kMmaMaxSplit && ((a.c + split - 1) / split > 512 ||
+                                  ((int64_t)n_problems * split < 2 * ctx->sm_count && a.c >= 2 * split * kMmaWarps * kMmaTile)))
+    split *= 2;
+  const int per_cta = ((a.c + split - 1) / split + kMmaTile - 1) / kMmaTile * kMmaTile;
+  const int ns = a.n_old + 1;
+  const size_t smem = decode_mma_smem(per_cta);
+  // the partition stages the positions in the tiles; indices are 16 bits wide (implied)
+  if ((size_t)per_cta * 4 > (size_t)kMmaWarps * kMmaStages * kMmaStageBytes || smem > (size_t)ctx->max_smem_optin)
+    return FL_ERR_UNSUPPORTED;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(n_problems * split));
+  cfg.blockDim = dim3(kMmaThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  int n_attr = 0;
+  if (split > 1) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+    attr[n_attr].val.clusterDim.x = (unsigned)split;
+    attr[n_attr].val.clusterDim.y = attr[n_attr].val.clusterDim.z = 1;
+    ++n_attr;
   }
-#undef FL_DECS
+  if (ctx->pdl) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
+    ++n_attr;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n_attr;
+#define FL_DECM(NS)                                                                                        \
+  do {                                                                                                     \
+    auto kern = decode_attn_mma_kernel<BITS, NS>;                                                          \
+    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));     \
+    FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, a, split, per_cta));                                      \
+  } while (0)
+  switch (ns) {
+    case 1: FL_DECM(1); break;
+    case 2: FL_DECM(2); break;
+    case 3: FL_DECM(3); break;
+    default: FL_DECM(4); break;
+  }
+#undef FL_DECM
   return fl_launch_status();
 }
 
 template <typename T, int DH>
 int launch_decode(const fl_ctx* ctx, const fl_shape* s, const DecodeArgs& a, int n_queries, cudaStream_t st) {
   const dim3 grid(n_queries, s->n_heads);
-  if (sizeof(T) == 2 && DH == 128 && a.n_old + 1 <= 4) {
-    const size_t staged = decode_smem<128>(a.c) + sizeof(int32_t) * (size_t)a.c * (a.n_old + 2);
-    if (staged <= (size_t)ctx->max_smem_optin) {
-      switch (s->bits) {
-        case 2: return launch_decode_staged<2>(ctx, a, a.n_old + 1, grid, staged, st);
-        case 4: return launch_decode_staged<4>(ctx, a, a.n_old + 1, grid, staged, st);
-        case 8: return launch_decode_staged<8>(ctx, a, a.n_old + 1, grid, staged, st);
-        default: return launch_decode_staged<16>(ctx, a, a.n_old + 1, grid, staged, st);
-      }
+  if (sizeof(T) == 2 && DH == 128 && a.n_old + 1 <= 4 && (int64_t)n_queries * s->n_heads * kMmaMaxSplit < INT32_MAX) {
+    int rc;
+    const int n_problems = n_queries * s->n_heads;
+    switch (s->bits) {
+      case 2: rc = launch_decode_mma<2>(ctx, a, n_problems, st); break;
+      case 4: rc = launch_decode_mma<4>(ctx, a, n_problems, st); break;
+      case 8: rc = launch_decode_mma<8>(ctx, a, n_problems, st); break;
+      default: rc = launch_decode_mma<16>(ctx, a, n_problems, st); break;
     }
+    if (rc != FL_ERR_UNSUPPORTED) return rc;
   }
   const size_t smem = decode_smem<DH>(a.c);
 #define FL_DEC(BITS)                                                                                      \
