@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "flashloop.h"
 
 struct fl_ctx {
@@ -134,6 +136,40 @@ inline cudaError_t fl_launch(const fl_ctx* ctx, void (*kernel)(KArgs...), dim3 g
   cfg.numAttrs = (ctx != nullptr && ctx->pdl) ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
+
+// Cluster dimension and (unless FL_NO_PDL) programmatic serialization of a launch; attr has room for two.
+static inline void fl_cluster_attrs(const fl_ctx* ctx, int n_ctas, cudaLaunchAttribute* attr, cudaLaunchConfig_t* cfg) {
+  int n = 0;
+  if (n_ctas > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)n_ctas;
+    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
+  if (ctx->pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n].val.programmaticStreamSerializationAllowed = 1;
+    ++n;
+  }
+  cfg->attrs = attr;
+  cfg->numAttrs = n;
+}
+
+// Launch attributes of a kernel, set once per device and not before every launch (each call is about a microsecond of
+// host time): the dynamic shared memory it may ask for, and on request the largest carve-out (two CTAs per SM that share
+// all of it). One flag word per place of use, i.e. per kernel instance.
+#define FL_FUNC_ATTR_ONCE(ctx, kern, bytes, max_carveout)                                                                 \
+  do {                                                                                                                     \
+    static std::atomic<uint64_t> done__{0};                                                                                \
+    const uint64_t bit__ = 1ull << ((ctx)->device & 63);                                                                   \
+    if (!(done__.load(std::memory_order_acquire) & bit__)) {                                                               \
+      FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes)));                \
+      if (max_carveout)                                                                                                    \
+        FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                           \
+                                           (int)cudaSharedmemCarveoutMaxShared));                                          \
+      done__.fetch_or(bit__, std::memory_order_release);                                                                   \
+    }                                                                                                                      \
+  } while (0)
 
 // ---- 8-element vector access in storage type ---------------------------------------------------
 template <typename T>

@@ -3,8 +3,6 @@
 // reduction). Selection is an exact radix select on the order-preserving integer image of the float
 // scores, followed by an index-ordered compaction, so the result equals a full sort with the total
 // order (score descending, index ascending) and comes out ascending.
-#include <cstdlib>
-
 #include "fl_internal.cuh"
 
 namespace {
@@ -15,7 +13,11 @@ namespace {
 template <typename T>
 __global__ void __launch_bounds__(256) token_score_kernel(const T* __restrict__ h_prev, const T* __restrict__ h_cur,
                                                           const int32_t* __restrict__ cand, int n_cand, int d, float eps,
-                                                          float* __restrict__ scores) {
+                                                          float* __restrict__ scores, int32_t* __restrict__ slot_of_pos, int L) {
+  fl_grid_wait();
+  fl_grid_release();
+  // the slot map starts as "not active"; the selection that follows enters the active rows
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < L; i += gridDim.x * blockDim.x) slot_of_pos[i] = -1;
   const int lane = threadIdx.x & 31;
   const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (t >= n_cand) return;
@@ -176,38 +178,19 @@ __device__ void block_topk_ascending(const float* __restrict__ vals, int n, int 
   __syncthreads();
 }
 
-__global__ void __launch_bounds__(kSelThreads) token_select_kernel(const float* __restrict__ scores,
-                                                                   const int32_t* __restrict__ cand, int n_cand, int k,
-                                                                   int32_t* __restrict__ active_idx,
-                                                                   int32_t* __restrict__ slot_of_pos) {
-  __shared__ SelectSmem sm;
-  block_topk_ascending(scores, n_cand, k, sm, [&](int rank, int i) {
-    const int pos = cand != nullptr ? __ldg(cand + i) : i;
-    active_idx[rank] = pos;
-    slot_of_pos[pos] = rank;
-  });
-}
-
 // ------------------------------------------------------------------------------------------
-// The same selection with the keys staged in shared memory (problems of up to kSelCap candidates): the
-// scores are read from global memory once; the radix passes run on shared memory and, as soon as the bin
-// that holds the k-th largest key is small, on a compacted list of that bin's keys only.
+// Radix passes of up to 11 bits by a whole CTA: thread t owns bins 2 t and 2 t + 1 of 2048.
 // ------------------------------------------------------------------------------------------
-constexpr int kSelCap = 49152;    // 192 KB of keys
-constexpr int kSelSmall = 2048;
+constexpr int kBins = 2048;
 
-struct SelectSmem2 {
-  uint32_t hist12[4096];
+struct RadixCtl {
   uint32_t warp_tot[32];
-  uint32_t hist[256];
-  uint32_t warp_gt[32], warp_eq[32];
-  uint32_t prefix, k_rem, bin_cnt, n_small;
-  uint32_t small[kSelSmall];
+  uint32_t bin, rank, bin_cnt;
 };
 
-// Adds the warp's keys that are `on` to the histogram: lanes that share the digit of the first matching lane
-// are counted with one atomic (scores cluster in a few exponent bins, runs of equal scores are common), the
-// rest add themselves.
+// Adds the warp's digits that are `on` to the histogram: lanes that share the digit of the first matching lane are
+// counted with one atomic (scores cluster in a few exponent bins, runs of equal scores are common), the rest add
+// themselves.
 __device__ __forceinline__ void hist_add(uint32_t* hist, bool on, uint32_t digit, int lane) {
   const uint32_t active = __ballot_sync(0xffffffffu, on);
   if (active == 0) return;
@@ -218,280 +201,213 @@ __device__ __forceinline__ void hist_add(uint32_t* hist, bool on, uint32_t digit
   else if (on && digit != d0) atomicAdd(&hist[digit], 1u);
 }
 
-// one radix pass (`bits` <= 8 bits at `shift`) over list[0..m4*4): histogram of the keys that match `prefix`
-// above the digit. Four keys per thread and step: the four dependent chains (load, vote, atomic) overlap.
-__device__ __forceinline__ void radix_hist_pass(const uint32_t* list, int m4, int shift, int bits, uint32_t prefix,
-                                                uint32_t* hist) {
-  const int tid = threadIdx.x, lane = tid & 31;
-  const uint32_t hi_mask = shift + bits >= 32 ? 0u : (0xFFFFFFFFu << (shift + bits));
-  const uint32_t dmask = (1u << bits) - 1u;
-  const uint4* l4 = reinterpret_cast<const uint4*>(list);
-  for (int base = 0; base < m4; base += kSelThreads) {
-    const int i = base + tid;
-    const bool in = i < m4;
-    const uint4 kv = in ? l4[i] : make_uint4(0, 0, 0, 0);
-    hist_add(hist, in && (kv.x & hi_mask) == prefix, (kv.x >> shift) & dmask, lane);
-    hist_add(hist, in && (kv.y & hi_mask) == prefix, (kv.y >> shift) & dmask, lane);
-    hist_add(hist, in && (kv.z & hi_mask) == prefix, (kv.z >> shift) & dmask, lane);
-    hist_add(hist, in && (kv.w & hi_mask) == prefix, (kv.w >> shift) & dmask, lane);
+// The bin that holds the `rank`-th largest key (1-based), given the counts of the thread's two bins: ctl.bin, the rank
+// that is left inside it, and its count. All kSelThreads threads call it; two barriers.
+__device__ __forceinline__ void find_bin(uint32_t c0, uint32_t c1, uint32_t rank, RadixCtl& ctl) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const uint32_t sum = c0 + c1;
+  uint32_t incl = sum;                       // inclusive suffix sum over the lanes (higher lanes = larger digits)
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_down_sync(0xffffffffu, incl, o);
+    if (lane + o < 32) incl += v;
   }
+  if (lane == 0) ctl.warp_tot[warp] = incl;
+  __syncthreads();
+  uint32_t tot = ctl.warp_tot[lane];
+  const uint32_t own = tot;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_down_sync(0xffffffffu, tot, o);
+    if (lane + o < 32) tot += v;
+  }
+  const uint32_t above = __shfl_sync(0xffffffffu, tot - own, warp) + incl - sum;
+  if (above < rank && rank <= above + sum) {
+    const bool hi = rank <= above + c1;
+    ctl.bin = 2 * tid + (hi ? 1 : 0);
+    ctl.rank = rank - above - (hi ? 0 : c1);
+    ctl.bin_cnt = hi ? c1 : c0;
+  }
+  __syncthreads();
 }
 
-// First level: 12-bit digit (sign, exponent, three mantissa bits) counted while the keys are staged. A warp whose
-// 32 keys share the digit adds them with one atomic; otherwise every lane adds itself (a handful of lanes per bin).
-__device__ __forceinline__ void hist12_add(uint32_t* hist12, uint32_t key, int lane) {
-  const uint32_t d = key >> 20;
-  int all_same;
-  __match_all_sync(0xffffffffu, d, &all_same);
-  if (all_same) { if (lane == 0) atomicAdd(&hist12[d], 32u); }
-  else atomicAdd(&hist12[d], 1u);
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint2 dsmem_ld2(const uint32_t* p, uint32_t rank) {
+  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
+  uint2 v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(r) : "memory");
+  return v;
 }
 
-__global__ void __launch_bounds__(kSelThreads, 1) column_select_smem_kernel(const float* __restrict__ col_scores,
-                                                                            const int32_t* __restrict__ cand_cols,
-                                                                            const int32_t* __restrict__ cand_cnt, int stride,
-                                                                            int c, int L, int q_block, int nb, int vec_ok,
-                                                                            int32_t* __restrict__ col_idx,
-                                                                            int32_t* __restrict__ col_cnt) {
-  extern __shared__ __align__(16) uint32_t keys[];   // [n rounded up to 4], padded with key 0 (below every real key)
-  __shared__ SelectSmem2 sm;
+// Token selection by a cluster of CTAs. A single CTA that walks the scores in global memory five times is bound by its
+// latency (53 us for 32 k candidates, 254 us for 128 k); here every CTA of a cluster of `n_ctas` keeps the keys of its
+// piece in shared memory, three radix passes at most find the threshold (the leading bits that all keys share are
+// skipped), histograms and counts are joined through distributed shared memory, and every CTA emits its own piece.
+constexpr int kTokCluster = 8;
+struct TokSmem {
+  uint32_t hist[3][kBins];           // one per pass: a pass needs no barrier before it clears the next one
+  uint32_t range[2];                 // smallest and largest key of the piece
+  uint32_t count[2];                 // keys above / equal to the threshold in the piece
+  uint32_t warp_gt[32], warp_eq[32];
+  uint32_t warp_lo[32], warp_hi[32];
+  RadixCtl ctl;
+};
+
+__global__ void __launch_bounds__(kSelThreads, 1) token_select_cluster_kernel(const float* __restrict__ scores,
+                                                                              const int32_t* __restrict__ cand, int n, int k,
+                                                                              int n_ctas, int piece,
+                                                                              int32_t* __restrict__ active_idx,
+                                                                              int32_t* __restrict__ slot_of_pos) {
+  extern __shared__ __align__(16) uint32_t dyn_smem[];
+  TokSmem& sm = *reinterpret_cast<TokSmem*>(dyn_smem);
+  uint32_t* keys = dyn_smem + (sizeof(TokSmem) + 15) / 16 * 4;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < 3 * kBins; i += kSelThreads) sm.hist[0][i] = 0;
   fl_grid_wait();
   fl_grid_release();
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // later blocks have more candidates (causal prefix): they are dispatched first, the short ones fill the tail
-  const int h = blockIdx.x, b = gridDim.y - 1 - blockIdx.y;
-  const size_t prob = (size_t)h * nb + b;
-  const float* vals = col_scores + prob * stride;
-  const int32_t* cols = cand_cols != nullptr ? cand_cols + prob * stride : nullptr;
-  int n = cand_cols != nullptr ? __ldg(cand_cnt + prob) : min(L, (b + 1) * q_block);
-  n = max(0, min(n, stride));
-  const int k = min(c, n);
-  int32_t* out = col_idx + prob * c;
-  for (int i = k + tid; i < c; i += kSelThreads) out[i] = -1;
-  if (tid == 0) col_cnt[prob] = k;
-  if (k == 0) return;
-  const int n4 = (n + 3) >> 2;
-  // ---- stage the order-preserving keys, counting their 12-bit digits on the way -----------------------------
-  for (int i = tid; i < 4096; i += kSelThreads) sm.hist12[i] = 0;
-  __syncthreads();
-  {
-    const float4* v4 = reinterpret_cast<const float4*>(vals);
-    uint4* k4 = reinterpret_cast<uint4*>(keys);
-    // four steps' loads are issued before the first is consumed: the staging is bound by memory latency otherwise
-    // (whole warps run every step: padding keys are 0, bin 0)
-    for (int base0 = 0; base0 < n4; base0 += 4 * kSelThreads) {
-      float4 v[4];
+  const int rank = n_ctas > 1 ? (int)cluster_rank() : 0;
+  const int base = rank * piece, m = max(0, min(piece, n - base));
+  auto join = [&]() { if (n_ctas > 1) cluster_sync(); else __syncthreads(); };
+  uint32_t lo = 0xffffffffu, hi = 0u;
+  for (int i0 = 0; i0 < m; i0 += 4 * kSelThreads) {      // four loads in flight per thread
+    float v[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = base0 + q * kSelThreads + tid;
-        v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (i < n4) {
-          if (vec_ok && i * 4 + 3 < n) {
-            v[q] = __ldg(v4 + i);
-          } else {
-            if (i * 4 + 0 < n) v[q].x = __ldg(vals + i * 4 + 0);
-            if (i * 4 + 1 < n) v[q].y = __ldg(vals + i * 4 + 1);
-            if (i * 4 + 2 < n) v[q].z = __ldg(vals + i * 4 + 2);
-            if (i * 4 + 3 < n) v[q].w = __ldg(vals + i * 4 + 3);
-          }
-        }
-      }
+    for (int e = 0; e < 4; ++e) {
+      const int i = i0 + e * kSelThreads + tid;
+      v[e] = i < m ? __ldg(scores + base + i) : 0.f;
+    }
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = base0 + q * kSelThreads + tid;
-        if (base0 + q * kSelThreads >= n4) break;   // CTA-uniform
-        uint4 kv = make_uint4(0, 0, 0, 0);
-        if (i < n4) {
-          if (i * 4 + 0 < n) kv.x = ordered_key(v[q].x);
-          if (i * 4 + 1 < n) kv.y = ordered_key(v[q].y);
-          if (i * 4 + 2 < n) kv.z = ordered_key(v[q].z);
-          if (i * 4 + 3 < n) kv.w = ordered_key(v[q].w);
-          k4[i] = kv;
-        }
-        hist12_add(sm.hist12, kv.x, lane);
-        hist12_add(sm.hist12, kv.y, lane);
-        hist12_add(sm.hist12, kv.z, lane);
-        hist12_add(sm.hist12, kv.w, lane);
+    for (int e = 0; e < 4; ++e) {
+      const int i = i0 + e * kSelThreads + tid;
+      if (i < m) {
+        const uint32_t key = ordered_key(v[e]);
+        keys[i] = key;
+        lo = min(lo, key);
+        hi = max(hi, key);
       }
     }
   }
-  __syncthreads();
-  uint32_t prefix = 0, k_rem = 0;
+  uint32_t thr = 0, k_rem = 0;
   const bool take_all = k >= n;
   if (!take_all) {
-    // ---- first level: the 12-bit bin that holds the k-th largest key (thread t owns bins 4t .. 4t+3) -------
-    {
-      uint32_t loc[4], sum = 0;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) { loc[j] = sm.hist12[tid * 4 + j]; sum += loc[j]; }
-      uint32_t incl = sum;                       // inclusive suffix sum over the warp (higher lanes = larger keys)
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_down_sync(0xffffffffu, incl, o);
-        if (lane + o < 32) incl += v;
-      }
-      if (lane == 0) sm.warp_tot[warp] = incl;
-      __syncthreads();
-      uint32_t above = incl - sum;               // keys in bins above this thread's
-      for (int w2 = warp + 1; w2 < 32; ++w2) above += sm.warp_tot[w2];
-      if (above < (uint32_t)k && (uint32_t)k <= above + sum) {
-        uint32_t acc = above;
-        for (int j = 3; j >= 0; --j) {
-          if ((uint32_t)k <= acc + loc[j]) {
-            sm.prefix = (uint32_t)(tid * 4 + j) << 20;
-            sm.k_rem = (uint32_t)k - acc;
-            sm.bin_cnt = loc[j];
-            break;
-          }
-          acc += loc[j];
-        }
-      }
-      if (tid == 0) sm.n_small = 0;
-      __syncthreads();
-      prefix = sm.prefix;
-      k_rem = sm.k_rem;
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if (lane == 0) { sm.warp_lo[warp] = lo; sm.warp_hi[warp] = hi; }
+    __syncthreads();
+    if (warp == 0) {
+      lo = __reduce_min_sync(0xffffffffu, sm.warp_lo[lane]);
+      hi = __reduce_max_sync(0xffffffffu, sm.warp_hi[lane]);
+      if (lane == 0) { sm.range[0] = lo; sm.range[1] = hi; }
     }
-    const uint32_t* list = keys;
-    int m4 = n4;
-    int fixed = 12;                              // leading bits of the threshold found so far
-    for (int pass = 0; pass < 4; ++pass) {
-      // pass 0 only tries the compaction; passes 1-3 resolve 8, 8 and 4 more bits
-      if (pass > 0) {
-        const int bits = pass == 3 ? 4 : 8;
-        const int shift = 32 - fixed - bits;
-        for (int i = tid; i < 256; i += kSelThreads) sm.hist[i] = 0;
-        __syncthreads();
-        radix_hist_pass(list, m4, shift, bits, prefix, sm.hist);
-        __syncthreads();
-        if (warp == 0) {
-          // lane owns digits [8*lane, 8*lane+8); find the digit holding the k_rem-th largest
-          uint32_t local[8], sum = 0;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) { local[j] = sm.hist[lane * 8 + j]; sum += local[j]; }
-          uint32_t incl = sum;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t v = __shfl_down_sync(0xffffffffu, incl, o);
-            if (lane + o < 32) incl += v;
-          }
-          const uint32_t above = incl - sum;
-          if (above < k_rem && k_rem <= above + sum) {
-            uint32_t acc = above;
-            for (int j = 7; j >= 0; --j) {
-              if (k_rem <= acc + local[j]) {
-                sm.prefix = prefix | ((uint32_t)(lane * 8 + j) << shift);
-                sm.k_rem = k_rem - acc;
-                sm.bin_cnt = local[j];
-                break;
-              }
-              acc += local[j];
-            }
-          }
-          if (lane == 0) sm.n_small = 0;
-        }
-        __syncthreads();
-        prefix = sm.prefix;
-        k_rem = sm.k_rem;
-        fixed += bits;
-      }
-      const uint32_t bin_cnt = sm.bin_cnt;
-      if (fixed < 32 && list == keys && bin_cnt <= (uint32_t)(kSelSmall - 4)) {
-        // the k-th largest key lies in a small bin: finish on that bin's keys alone
-        const uint32_t hi_mask = 0xFFFFFFFFu << (32 - fixed);
-        const int n_pad = n4 * 4;
-        for (int base = warp * 128; base < n_pad; base += kSelThreads * 4) {   // 128 keys per warp and step
-          uint32_t kk[4], m[4];
-          uint32_t total = 0;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const int i = base + j * 32 + lane;
-            kk[j] = i < n_pad ? keys[i] : 0u;
-            m[j] = __ballot_sync(0xffffffffu, i < n_pad && (kk[j] & hi_mask) == prefix);
-            total += __popc(m[j]);
-          }
-          if (total == 0) continue;
-          uint32_t off = 0;
-          if (lane == 0) off = atomicAdd(&sm.n_small, total);
-          off = __shfl_sync(0xffffffffu, off, 0);
-          const uint32_t lt = (1u << lane) - 1;
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            if ((m[j] >> lane) & 1u) sm.small[off + __popc(m[j] & lt)] = kk[j];
-            off += __popc(m[j]);
-          }
-        }
-        __syncthreads();
-        // pad the list to a multiple of four with keys that cannot match the prefix of any later pass
-        if (tid < 4) {
-          const uint32_t m = sm.n_small;
-          if (m + tid < ((m + 3) & ~3u)) sm.small[m + tid] = ~prefix;
-        }
-        list = sm.small;
-        m4 = (int)((bin_cnt + 3) >> 2);
-      }
-      __syncthreads();
+    join();
+    lo = 0xffffffffu; hi = 0u;
+    for (int r = 0; r < n_ctas; ++r) {
+      const uint2 v = n_ctas > 1 ? dsmem_ld2(sm.range, r) : make_uint2(sm.range[0], sm.range[1]);
+      lo = min(lo, v.x);
+      hi = max(hi, v.y);
     }
+    // bits below the common prefix of all keys, taken 11 at a time from the top
+    int left = 32 - __clz(lo ^ hi);          // 0: all keys are equal
+    uint32_t prefix = left == 32 ? 0u : (left == 0 ? lo : (lo >> left) << left);
+    k_rem = (uint32_t)k;
+    for (int pass = 0; left > 0; ++pass) {
+      const int bits = min(11, left), shift = left - bits;
+      const uint32_t hi_mask = left == 32 ? 0u : 0xffffffffu << left, dmask = (1u << bits) - 1u;
+      for (int i0 = 0; i0 < m; i0 += kSelThreads) {      // whole warps vote
+        const int i = i0 + tid;
+        const uint32_t key = i < m ? keys[i] : 0u;
+        hist_add(sm.hist[pass], i < m && (key & hi_mask) == prefix, (key >> shift) & dmask, lane);
+      }
+      join();
+      uint32_t c0 = 0, c1 = 0;
+      if (n_ctas > 1) {
+        uint2 v[kTokCluster];
+#pragma unroll
+        for (int r = 0; r < kTokCluster; ++r) v[r] = r < n_ctas ? dsmem_ld2(&sm.hist[pass][2 * tid], r) : make_uint2(0, 0);
+#pragma unroll
+        for (int r = 0; r < kTokCluster; ++r) { c0 += v[r].x; c1 += v[r].y; }
+      } else {
+        c0 = sm.hist[pass][2 * tid];
+        c1 = sm.hist[pass][2 * tid + 1];
+      }
+      find_bin(c0, c1, k_rem, sm.ctl);
+      prefix |= sm.ctl.bin << shift;
+      k_rem = sm.ctl.rank;
+      left = shift;
+      if (sm.ctl.bin_cnt == k_rem && left > 0) {   // the whole bin is selected: everything at or above it, no ties
+        prefix -= 1;                               // prefix > 0: a selected lowest bin would mean k >= n
+        k_rem = 0;
+        break;
+      }
+    }
+    thr = prefix;
   }
-  const uint32_t thr = prefix;
-  // ---- index-ordered compaction from the staged keys: each warp owns a contiguous span, walked 128 keys at a
-  // time (lane l holds keys l, 32 + l, 64 + l, 96 + l of the step: votes give every key its place in index order)
-  const int span = ((n + 31) / 32 + 127) / 128 * 128;
-  const int beg = warp * span, end = min(n, beg + span);
+  // ---- index-ordered emission: each warp owns a contiguous span of the piece --------------------------------
+  const int span = ((m + 31) / 32 + 31) / 32 * 32;
+  const int beg = warp * span, end = min(m, beg + span);
   uint32_t gt = 0, eq = 0;
   for (int i = beg + lane; i < end; i += 32) {
     const uint32_t key = keys[i];
     gt += (take_all || key > thr) ? 1u : 0u;
     eq += (!take_all && key == thr) ? 1u : 0u;
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    gt += __shfl_xor_sync(0xffffffffu, gt, o);
-    eq += __shfl_xor_sync(0xffffffffu, eq, o);
-  }
+  gt = __reduce_add_sync(0xffffffffu, gt);
+  eq = __reduce_add_sync(0xffffffffu, eq);
   if (lane == 0) { sm.warp_gt[warp] = gt; sm.warp_eq[warp] = eq; }
   __syncthreads();
-  uint32_t gt_before = 0, eq_before = 0;
-  for (int w = 0; w < warp; ++w) { gt_before += sm.warp_gt[w]; eq_before += sm.warp_eq[w]; }
-  const uint32_t lt = (1u << lane) - 1;
-  for (int base = beg; base < end; base += 128) {
-    uint32_t kk[4], mg[4];
-    bool any_eq_lane = false;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int i = base + j * 32 + lane;
-      kk[j] = i < end ? keys[i] : 0u;
-      mg[j] = __ballot_sync(0xffffffffu, i < end && (take_all || kk[j] > thr));
-      any_eq_lane |= i < end && !take_all && kk[j] == thr;
-    }
-    if (!__any_sync(0xffffffffu, any_eq_lane)) {
-      // no key of the step ties with the threshold: the selected ones are the greater ones, in index order
-      uint32_t off = gt_before + min(eq_before, k_rem);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if ((mg[j] >> lane) & 1u) {
-          const int i = base + j * 32 + lane;
-          out[off + __popc(mg[j] & lt)] = cols != nullptr ? __ldg(cols + i) : i;
-        }
-        off += __popc(mg[j]);
-      }
-      gt_before += __popc(mg[0]) + __popc(mg[1]) + __popc(mg[2]) + __popc(mg[3]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int i = base + j * 32 + lane;
-        const bool is_gt = (mg[j] >> lane) & 1u;
-        const bool is_eq = i < end && !take_all && kk[j] == thr;
-        const uint32_t me = __ballot_sync(0xffffffffu, is_eq);
-        const uint32_t my_gt = gt_before + __popc(mg[j] & lt), my_eq = eq_before + __popc(me & lt);
-        int rank = -1;
-        if (is_gt) rank = (int)(my_gt + min(my_eq, k_rem));
-        else if (is_eq && my_eq < k_rem) rank = (int)(my_gt + my_eq);
-        if (rank >= 0) out[rank] = cols != nullptr ? __ldg(cols + i) : i;
-        gt_before += __popc(mg[j]);
-        eq_before += __popc(me);
-      }
+  uint32_t wg = sm.warp_gt[lane], we = sm.warp_eq[lane];
+  const uint32_t tot_gt = __reduce_add_sync(0xffffffffu, wg), tot_eq = __reduce_add_sync(0xffffffffu, we);
+  uint32_t gt_before = __reduce_add_sync(0xffffffffu, lane < warp ? wg : 0u);
+  uint32_t eq_before = __reduce_add_sync(0xffffffffu, lane < warp ? we : 0u);
+  if (n_ctas > 1) {
+    if (tid == 0) { sm.count[0] = tot_gt; sm.count[1] = tot_eq; }
+    cluster_sync();
+    for (int r = 0; r < rank; ++r) {
+      const uint2 v = dsmem_ld2(sm.count, r);
+      gt_before += v.x;
+      eq_before += v.y;
     }
   }
+  const uint32_t lt = (1u << lane) - 1;
+  for (int i0 = beg; i0 < end; i0 += 32) {
+    const int i = i0 + lane;
+    const uint32_t key = i < end ? keys[i] : 0u;
+    const bool is_gt = i < end && (take_all || key > thr), is_eq = i < end && !take_all && key == thr;
+    const uint32_t m_gt = __ballot_sync(0xffffffffu, is_gt), m_eq = __ballot_sync(0xffffffffu, is_eq);
+    const uint32_t my_gt = gt_before + __popc(m_gt & lt), my_eq = eq_before + __popc(m_eq & lt);
+    if (is_gt || (is_eq && my_eq < k_rem)) {
+      const int at = (int)(my_gt + (is_gt ? min(my_eq, k_rem) : my_eq));
+      const int pos = cand != nullptr ? __ldg(cand + base + i) : base + i;
+      active_idx[at] = pos;
+      slot_of_pos[pos] = at;
+    }
+    gt_before += __popc(m_gt);
+    eq_before += __popc(m_eq);
+  }
+  if (n_ctas > 1) cluster_sync();   // nobody leaves while another CTA still reads its shared memory
+}
+
+// More candidates than the cluster's shared memory holds: one CTA over global memory.
+__global__ void __launch_bounds__(kSelThreads) token_select_kernel(const float* __restrict__ scores,
+                                                                   const int32_t* __restrict__ cand, int n_cand, int k,
+                                                                   int32_t* __restrict__ active_idx,
+                                                                   int32_t* __restrict__ slot_of_pos) {
+  __shared__ SelectSmem sm;
+  fl_grid_wait();
+  fl_grid_release();
+  block_topk_ascending(scores, n_cand, k, sm, [&](int rank, int i) {
+    const int pos = cand != nullptr ? __ldg(cand + i) : i;
+    active_idx[rank] = pos;
+    slot_of_pos[pos] = rank;
+  });
 }
 
 // ------------------------------------------------------------------------------------------
@@ -511,69 +427,38 @@ constexpr int kBitmapWords = 8192;     // positions a problem may have: 32 * kBi
 
 struct SampledSmem {
   SelectSmem generic;                  // fallback: radix select over all keys
-  uint32_t hist[256];
-  uint32_t prefix, rank, n_eq;
+  uint32_t hist[3][kBins];
+  RadixCtl ctl;
   uint32_t n_cand, n_tie;
   uint32_t warp_sum[32];
   int32_t tie_idx[kTieCap];
 };
 
-// `rank`-th largest (1-based) of the keys the threads hold (KPT per thread, `valid` marks the real ones), by four
-// 8-bit radix passes with warp-aggregated shared-memory histograms. Returns the key; *rank_in_eq = how many of the
-// keys equal to it belong to the `rank` largest, *n_eq = how many keys equal it. Only the first kpt_used slots of a
-// thread are looked at (the same number in every thread). All kSelThreads threads call it.
+// `rank`-th largest (1-based) of the keys the threads hold (KPT per thread, `valid` marks the real ones), by radix passes
+// of 11, 11 and 10 bits into the histograms first, first + 1, first + 2 (modulo 3, all zero on entry); n_pass = 2 leaves
+// the low 10 bits zero, a lower bound. Returns the key; afterwards sm.ctl.rank = how many of the keys equal to it belong
+// to the `rank` largest, sm.ctl.bin_cnt = how many keys equal it. Only the first kpt_used slots of a thread are looked at
+// (the same number in every thread). All kSelThreads threads call it.
 template <int KPT>
 __device__ uint32_t block_kth_largest(const uint32_t (&key)[KPT], const bool (&valid)[KPT], int kpt_used, uint32_t rank,
-                                      SampledSmem& sm, uint32_t* rank_in_eq, uint32_t* n_eq) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  uint32_t prefix = 0;
-  for (int shift = 24; shift >= 0; shift -= 8) {
-    for (int i = tid; i < 256; i += kSelThreads) sm.hist[i] = 0;
-    __syncthreads();
-    const uint32_t hi_mask = shift == 24 ? 0u : (0xFFFFFFFFu << (shift + 8));
+                                      SampledSmem& sm, int first, int n_pass) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  uint32_t prefix = 0, hi_mask = 0;
+  for (int pass = 0; pass < n_pass; ++pass) {
+    uint32_t* hist = sm.hist[(first + pass) % 3];
+    const int shift = pass == 0 ? 21 : (pass == 1 ? 10 : 0);
+    const uint32_t dmask = pass == 2 ? 1023u : 2047u;
 #pragma unroll
     for (int q = 0; q < KPT; ++q) {
       if (q >= kpt_used) break;               // CTA-uniform: the slots beyond it hold no key in any thread
-      const bool on = valid[q] && (key[q] & hi_mask) == prefix;
-      const uint32_t digit = (key[q] >> shift) & 0xFFu;
-      const uint32_t active = __ballot_sync(0xffffffffu, on);
-      if (on) {
-        const uint32_t peers = __match_any_sync(active, digit);
-        if ((peers & ((1u << lane) - 1)) == 0) atomicAdd(&sm.hist[digit], (uint32_t)__popc(peers));
-      }
+      hist_add(hist, valid[q] && (key[q] & hi_mask) == prefix, (key[q] >> shift) & dmask, lane);
     }
     __syncthreads();
-    if (warp == 0) {
-      uint32_t local[8], sum = 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) { local[j] = sm.hist[lane * 8 + j]; sum += local[j]; }
-      uint32_t incl = sum;                    // inclusive suffix sum over the lanes (higher lanes = larger digits)
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_down_sync(0xffffffffu, incl, o);
-        if (lane + o < 32) incl += v;
-      }
-      const uint32_t above = incl - sum;
-      if (above < rank && rank <= above + sum) {
-        uint32_t acc = above;
-        for (int j = 7; j >= 0; --j) {
-          if (rank <= acc + local[j]) {
-            sm.prefix = prefix | ((uint32_t)(lane * 8 + j) << shift);
-            sm.rank = rank - acc;
-            sm.n_eq = local[j];
-            break;
-          }
-          acc += local[j];
-        }
-      }
-    }
-    __syncthreads();
-    prefix = sm.prefix;
-    rank = sm.rank;
+    find_bin(hist[2 * tid], hist[2 * tid + 1], rank, sm.ctl);
+    prefix |= sm.ctl.bin << shift;
+    rank = sm.ctl.rank;
+    hi_mask = 0xffffffffu << shift;
   }
-  *rank_in_eq = rank;
-  *n_eq = sm.n_eq;
-  __syncthreads();
   return prefix;
 }
 
@@ -608,6 +493,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) column_select_sampled_kernel(c
     for (int i = tid; i < n; i += kSelThreads) out[i] = cols != nullptr ? __ldg(cols + i) : i;
     return;
   }
+  for (int i = tid; i < 3 * kBins; i += kSelThreads) sm.hist[0][i] = 0u;
+  __syncthreads();
   // ---- a value below the k-th largest key: from a regular sample when the problem is too long to list whole ----
   uint32_t thr_lo = 0;                                  // n <= kCandCap: every key is a candidate
   if (n > kCandCap) {
@@ -619,8 +506,8 @@ __global__ void __launch_bounds__(kSelThreads, 2) column_select_sampled_kernel(c
     const uint64_t target = (uint64_t)k + (uint64_t)k / 2 + 256;
     uint32_t r_s = (uint32_t)((target * kSample + n - 1) / n);
     r_s = min(max(r_s, 1u), (uint32_t)kSample);
-    uint32_t dummy0, dummy1;
-    thr_lo = block_kth_largest<1>(skey, sval, 1, r_s, sm, &dummy0, &dummy1);
+    thr_lo = block_kth_largest<1>(skey, sval, 1, r_s, sm, 0, 2);
+    for (int i = tid; i < 2 * kBins; i += kSelThreads) sm.hist[0][i] = 0u;   // (every thread has read its bins)
   }
   if (tid == 0) { sm.n_cand = 0; sm.n_tie = 0; }
   const int n_words = (n + 31) >> 5;
@@ -630,41 +517,43 @@ __global__ void __launch_bounds__(kSelThreads, 2) column_select_sampled_kernel(c
   {
     const float4* v4 = reinterpret_cast<const float4*>(vals);
     const int n4 = (n + 3) >> 2;
-    for (int base = 0; base < n4; base += kSelThreads) {
-      const int i = base + tid;
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (i < n4) {
-        if (vec_ok && i * 4 + 3 < n) v = __ldg(v4 + i);
-        else {
-          if (i * 4 + 0 < n) v.x = __ldg(vals + i * 4 + 0);
-          if (i * 4 + 1 < n) v.y = __ldg(vals + i * 4 + 1);
-          if (i * 4 + 2 < n) v.z = __ldg(vals + i * 4 + 2);
-          if (i * 4 + 3 < n) v.w = __ldg(vals + i * 4 + 3);
+    const uint32_t lt = (1u << lane) - 1u;
+    for (int base = 0; base < n4; base += 2 * kSelThreads) {
+      float4 v[2];                                      // two loads in flight
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const int i = base + q * kSelThreads + tid;
+        v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (vec_ok && i * 4 + 3 < n) v[q] = __ldg(v4 + i);
+        else if (i < n4) {
+          if (i * 4 + 0 < n) v[q].x = __ldg(vals + i * 4 + 0);
+          if (i * 4 + 1 < n) v[q].y = __ldg(vals + i * 4 + 1);
+          if (i * 4 + 2 < n) v[q].z = __ldg(vals + i * 4 + 2);
+          if (i * 4 + 3 < n) v[q].w = __ldg(vals + i * 4 + 3);
         }
       }
-      const uint32_t kk[4] = {ordered_key(v.x), ordered_key(v.y), ordered_key(v.z), ordered_key(v.w)};
-      bool on[4];
-      int mine = 0;
 #pragma unroll
-      for (int e = 0; e < 4; ++e) { on[e] = i < n4 && i * 4 + e < n && kk[e] >= thr_lo; mine += on[e] ? 1 : 0; }
-      // one atomic per warp and step: lanes take consecutive places behind it
-      int incl = mine;
+      for (int q = 0; q < 2; ++q) {
+        const int i4 = (base + q * kSelThreads + tid) * 4;
+        const uint32_t kk[4] = {ordered_key(v[q].x), ordered_key(v[q].y), ordered_key(v[q].z), ordered_key(v[q].w)};
+        // one atomic per warp and step: the hits take consecutive places behind it
+        uint32_t on[4], total = 0;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      if (total == 0) continue;
-      uint32_t at = 0;
-      if (lane == 31) at = atomicAdd(&sm.n_cand, (uint32_t)total);
-      at = __shfl_sync(0xffffffffu, at, 31) + (uint32_t)(incl - mine);
-#pragma unroll
-      for (int e = 0; e < 4; ++e)
-        if (on[e]) {
-          if (at < (uint32_t)kCandCap) { cand_key[at] = kk[e]; cand_idx[at] = i * 4 + e; }
-          ++at;
+        for (int e = 0; e < 4; ++e) {
+          on[e] = __ballot_sync(0xffffffffu, i4 + e < n && kk[e] >= thr_lo);
+          total += __popc(on[e]);
         }
+        if (total == 0) continue;
+        uint32_t at = 0;
+        if (lane == 0) at = atomicAdd(&sm.n_cand, total);
+        at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const uint32_t my = at + __popc(on[e] & lt);
+          if (((on[e] >> lane) & 1u) && my < (uint32_t)kCandCap) { cand_key[my] = kk[e]; cand_idx[my] = i4 + e; }
+          at += __popc(on[e]);
+        }
+      }
     }
   }
   __syncthreads();
@@ -682,9 +571,10 @@ __global__ void __launch_bounds__(kSelThreads, 2) column_select_sampled_kernel(c
       valid[q] = u < n_cand;
       key[q] = valid[q] ? cand_key[u] : 0u;
     }
-    uint32_t n_eq;
     const int kpt_used = (int)((n_cand + kSelThreads - 1) / kSelThreads);
-    thr = block_kth_largest<KPT>(key, valid, kpt_used, (uint32_t)k, sm, &take_eq, &n_eq);
+    thr = block_kth_largest<KPT>(key, valid, kpt_used, (uint32_t)k, sm, 2, 3);
+    take_eq = sm.ctl.rank;
+    const uint32_t n_eq = sm.ctl.bin_cnt;
     // ties with the threshold: all of them, or the take_eq lowest positions
     const bool rank_ties = take_eq < n_eq;
     if (rank_ties && n_eq > (uint32_t)kTieCap) fallback = true;            // CTA-uniform (n_eq is)
@@ -747,6 +637,8 @@ __global__ void __launch_bounds__(kSelThreads) column_select_kernel(const float*
                                                                     int32_t* __restrict__ col_idx,
                                                                     int32_t* __restrict__ col_cnt) {
   __shared__ SelectSmem sm;
+  fl_grid_wait();
+  fl_grid_release();
   // later blocks have more candidates (causal prefix): they are dispatched first, the short ones fill the tail
   const int h = blockIdx.x, b = gridDim.y - 1 - blockIdx.y;
   const size_t prob = (size_t)h * nb + b;
@@ -789,20 +681,34 @@ extern "C" int fl_select_tokens(fl_ctx* ctx, const fl_shape* shape, int loop_r, 
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int warps = 8;
-  const int grid = (n_cand + warps - 1) / warps;
+  const dim3 grid((n_cand + warps - 1) / warps);
   if (shape->dtype == FL_F32)
-    token_score_kernel<float><<<grid, warps * 32, 0, st>>>(static_cast<const float*>(h_prev),
-                                                           static_cast<const float*>(h_cur), cand, n_cand, d,
-                                                           shape->eps, scores);
+    FL_CHECK_CUDA(fl_launch(ctx, token_score_kernel<float>, grid, dim3(warps * 32), 0, st, static_cast<const float*>(h_prev),
+                            static_cast<const float*>(h_cur), cand, n_cand, d, shape->eps, scores, slot_of_pos, shape->L));
   else
-    token_score_kernel<__nv_bfloat16><<<grid, warps * 32, 0, st>>>(static_cast<const __nv_bfloat16*>(h_prev),
-                                                                   static_cast<const __nv_bfloat16*>(h_cur), cand,
-                                                                   n_cand, d, shape->eps, scores);
-  rc = fl_launch_status();
-  if (rc != FL_OK) return rc;
-  FL_CHECK_CUDA(cudaMemsetAsync(slot_of_pos, 0xFF, sizeof(int32_t) * (size_t)shape->L, st));
+    FL_CHECK_CUDA(fl_launch(ctx, token_score_kernel<__nv_bfloat16>, grid, dim3(warps * 32), 0, st,
+                            static_cast<const __nv_bfloat16*>(h_prev), static_cast<const __nv_bfloat16*>(h_cur), cand, n_cand,
+                            d, shape->eps, scores, slot_of_pos, shape->L));
   const int k_eff = k < n_cand ? k : n_cand;
-  token_select_kernel<<<1, kSelThreads, 0, st>>>(scores, cand, n_cand, k_eff, active_idx, slot_of_pos);
+  // one CTA while its threads have at most four keys each, a cluster beyond (joining it costs ~2 us a pass)
+  const int n_ctas = n_cand <= 4 * kSelThreads ? 1 : kTokCluster;
+  const int piece = (n_cand + n_ctas - 1) / n_ctas;
+  const size_t smem = (sizeof(TokSmem) + 15) / 16 * 16 + sizeof(uint32_t) * (size_t)piece;
+  if (smem > (size_t)ctx->max_smem_optin) {
+    FL_CHECK_CUDA(fl_launch(ctx, token_select_kernel, dim3(1), dim3(kSelThreads), 0, st, scores, cand, n_cand, k_eff,
+                            active_idx, slot_of_pos));
+    return fl_launch_status();
+  }
+  FL_FUNC_ATTR_ONCE(ctx, token_select_cluster_kernel, ctx->max_smem_optin, false);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(n_ctas);
+  cfg.blockDim = dim3(kSelThreads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  fl_cluster_attrs(ctx, n_ctas, attr, &cfg);
+  FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, token_select_cluster_kernel, scores, cand, (int)n_cand, k_eff, n_ctas, piece,
+                                   active_idx, slot_of_pos));
   return fl_launch_status();
 }
 
@@ -824,27 +730,18 @@ extern "C" int fl_select_columns(fl_ctx* ctx, const fl_shape* shape, const float
     if (rc != FL_OK) return rc;
   }
   dim3 grid(shape->n_heads, nb);
-  const size_t key_bytes = sizeof(uint32_t) * (((size_t)n_cand + 3) & ~(size_t)3);
   const int vec_ok = (fl_aligned16(col_scores) && n_cand % 4 == 0) ? 1 : 0;
-  const char* staged = std::getenv("FL_SELECT_STAGED");
-  if (n_cand <= 32 * kBitmapWords && !(staged != nullptr && staged[0] == '1')) {
+  if (n_cand <= 32 * kBitmapWords) {
     // sampled pre-threshold, candidate list, bit map over the positions (exact; falls back inside the kernel)
     const size_t dyn_bytes = sizeof(uint32_t) * (2 * (size_t)kCandCap + ((size_t)n_cand + 31) / 32);
-    FL_CHECK_CUDA(cudaFuncSetAttribute(column_select_sampled_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)dyn_bytes));
+    constexpr size_t kMaxDyn = sizeof(uint32_t) * (2 * (size_t)kCandCap + kBitmapWords);
+    FL_FUNC_ATTR_ONCE(ctx, column_select_sampled_kernel, kMaxDyn, true);
     FL_CHECK_CUDA(fl_launch(ctx, column_select_sampled_kernel, grid, dim3(kSelThreads), dyn_bytes,
                             static_cast<cudaStream_t>(stream), col_scores, cand_cols, cand_cnt, n_cand, c, shape->L,
                             shape->q_block, nb, vec_ok, col_idx, col_cnt));
-  } else if (n_cand <= kSelCap && key_bytes + 32768 <= (size_t)ctx->max_smem_optin) {
-    // keys staged in shared memory: the scores are read from global memory once
-    FL_CHECK_CUDA(cudaFuncSetAttribute(column_select_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)key_bytes));
-    FL_CHECK_CUDA(fl_launch(ctx, column_select_smem_kernel, grid, dim3(kSelThreads), key_bytes,
-                            static_cast<cudaStream_t>(stream), col_scores, cand_cols, cand_cnt, n_cand, c, shape->L,
-                            shape->q_block, nb, vec_ok, col_idx, col_cnt));
   } else {
-    column_select_kernel<<<grid, kSelThreads, 0, static_cast<cudaStream_t>(stream)>>>(
-        col_scores, cand_cols, cand_cnt, n_cand, c, shape->L, shape->q_block, nb, col_idx, col_cnt);
+    FL_CHECK_CUDA(fl_launch(ctx, column_select_kernel, grid, dim3(kSelThreads), 0, static_cast<cudaStream_t>(stream),
+                            col_scores, cand_cols, cand_cnt, n_cand, c, shape->L, shape->q_block, nb, col_idx, col_cnt));
   }
   return fl_launch_status();
 }
