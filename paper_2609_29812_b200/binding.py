@@ -115,17 +115,25 @@ def status_string(status: int) -> str:
 
 def _ptr(x) -> Optional[int]:
     """Device (or host) address of a tensor-like, an int address, or None."""
-    if x is None:
-        return None
-    if isinstance(x, int):
+    if x is None or isinstance(x, int):
         return x
-    return int(x.data_ptr())
+    return x.data_ptr()
+
+
+_current_stream = None   # () -> raw handle of torch's current stream
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return int(torch.cuda.current_stream().cuda_stream) or None
+        global _current_stream
+        if _current_stream is None:
+            import torch
+            torch.cuda.current_stream()       # initialises CUDA
+            raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+            # the stream object of the public call costs 3 us, as much as a kernel launch; the handle alone 0.2 us
+            _current_stream = ((lambda: raw(dev())) if raw is not None and dev is not None
+                               else (lambda: int(torch.cuda.current_stream().cuda_stream)))
+        return _current_stream() or None
     if isinstance(stream, int):
         return stream or None
     return int(stream.cuda_stream) or None
@@ -142,6 +150,12 @@ def make_shape(L, n_heads, head_dim, dtype, q_block, bits, group, eps, sm_scale)
                    float(eps), float(sm_scale))
 
 
+def _stream_struct(s: dict) -> FlKvStream:
+    get = s.get
+    return FlKvStream(_ptr(get("codes")), _ptr(get("scale")), _ptr(get("zero")), _ptr(get("slot_of_pos")),
+                      _ptr(get("rows_prev")), _ptr(get("rows_cur")), int(s["n_rows"]), 0)
+
+
 def make_store(k_base, v_base, k_streams: Sequence[dict] = (), v_streams: Sequence[dict] = ()) -> FlKvStore:
     """Builds the host-side store struct.  Each stream is a dict with codes, scale, zero, slot_of_pos
     (tensors or addresses), n_rows and optionally rows_prev / rows_cur (the transient workspace for the loop's
@@ -151,13 +165,7 @@ def make_store(k_base, v_base, k_streams: Sequence[dict] = (), v_streams: Sequen
     assert len(k_streams) == len(v_streams) <= FL_MAX_LOOPS
     for dst, src in ((st.k_res, k_streams), (st.v_res, v_streams)):
         for i, s in enumerate(src):
-            dst[i].codes = _ptr(s.get("codes"))
-            dst[i].scale = _ptr(s.get("scale"))
-            dst[i].zero = _ptr(s.get("zero"))
-            dst[i].slot_of_pos = _ptr(s.get("slot_of_pos"))
-            dst[i].rows_prev = _ptr(s.get("rows_prev"))
-            dst[i].rows_cur = _ptr(s.get("rows_cur"))
-            dst[i].n_rows = int(s["n_rows"])
+            dst[i] = _stream_struct(s)
     st.n_streams = len(k_streams)
     return st
 
@@ -169,6 +177,7 @@ class Context:
         h = C.c_void_p()
         _check("fl_create", lib.fl_create(C.byref(h), int(device)), True)
         self.handle = h
+        self._lent = None      # (address, bytes) of the workspace the context holds, as last set through this object
 
     def close(self):
         if self.handle:
@@ -209,6 +218,8 @@ def fl_loop_attention_workspace_bytes(ctx, shape) -> int:
 
 def fl_set_workspace(ctx, workspace, nbytes, stream=None, check=True) -> int:
     rc = lib.fl_set_workspace(_h(ctx), _ptr(workspace), int(nbytes), _stream(stream))
+    if isinstance(ctx, Context):
+        ctx._lent = (_ptr(workspace), int(nbytes)) if rc == FL_OK and workspace is not None else None
     return _check("fl_set_workspace", rc, check)
 
 

@@ -644,24 +644,11 @@ int launch_decode_mma(const fl_ctx* ctx, const DecodeArgs& a, int n_problems, cu
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
-  int n_attr = 0;
-  if (split > 1) {
-    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
-    attr[n_attr].val.clusterDim.x = (unsigned)split;
-    attr[n_attr].val.clusterDim.y = attr[n_attr].val.clusterDim.z = 1;
-    ++n_attr;
-  }
-  if (ctx->pdl) {
-    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
-    ++n_attr;
-  }
-  cfg.attrs = attr;
-  cfg.numAttrs = n_attr;
+  fl_cluster_attrs(ctx, split, attr, &cfg);
 #define FL_DECM(NS)                                                                                        \
   do {                                                                                                     \
     auto kern = decode_attn_mma_kernel<BITS, NS>;                                                          \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));     \
+    FL_FUNC_ATTR_ONCE(ctx, kern, ctx->max_smem_optin, true);                                               \
     FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, a, split, per_cta));                                      \
   } while (0)
   switch (ns) {
@@ -692,7 +679,7 @@ int launch_decode(const fl_ctx* ctx, const fl_shape* s, const DecodeArgs& a, int
 #define FL_DEC(BITS)                                                                                      \
   do {                                                                                                    \
     auto kern = decode_attn_kernel<T, DH, BITS>;                                                          \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));    \
+    FL_FUNC_ATTR_ONCE(ctx, kern, ctx->max_smem_optin, false);                                             \
     FL_CHECK_CUDA(fl_launch(ctx, kern, grid, dim3(kDecThreads), smem, st, a));                            \
   } while (0)
   switch (s->bits) {

@@ -220,11 +220,11 @@ constexpr size_t colscore_smem() {
 }
 
 template <typename T, int DH>
-int launch_dense(const fl_shape* s, const void* q, const void* k, const void* v, void* o, float* lse, float* col_scores,
+int launch_dense(const fl_ctx* ctx, const fl_shape* s, const void* q, const void* k, const void* v, void* o, float* lse, float* col_scores,
                  cudaStream_t st) {
   const int tiles = (s->L + kQTile - 1) / kQTile;
   auto kern = dense_attn_kernel<T, DH>;
-  FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dense_smem<DH>()));
+  FL_FUNC_ATTR_ONCE(ctx, kern, dense_smem<DH>(), false);
   kern<<<dim3(tiles, s->n_heads), kAttnThreads, dense_smem<DH>(), st>>>(
       static_cast<const T*>(q), static_cast<const T*>(k), static_cast<const T*>(v), static_cast<T*>(o), lse, s->L,
       s->n_heads, s->sm_scale);
@@ -238,7 +238,7 @@ int launch_dense(const fl_shape* s, const void* q, const void* k, const void* v,
   a.L = s->L; a.H = s->n_heads; a.q_block = s->q_block; a.nb = fl_n_blocks(s); a.d = s->n_heads * DH;
   a.group = s->group; a.scale = s->sm_scale;
   auto ck = colscore_kernel<T, DH, 16, false>;
-  FL_CHECK_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)colscore_smem<DH>()));
+  FL_FUNC_ATTR_ONCE(ctx, ck, colscore_smem<DH>(), false);
   const int col_groups = (s->L + kAttnWarps * kChunk - 1) / (kAttnWarps * kChunk);
   ck<<<dim3(col_groups, a.nb, s->n_heads), kAttnThreads, colscore_smem<DH>(), st>>>(a);
   return fl_launch_status();
@@ -247,7 +247,7 @@ int launch_dense(const fl_shape* s, const void* q, const void* k, const void* v,
 }  // namespace
 
 // Used by the sparse loop to emit next-loop column scores (defined here to share the kernel).
-int fl_launch_sparse_colscore(const fl_shape* s, const void* q_new, const int32_t* active_idx, int n_active,
+int fl_launch_sparse_colscore(const fl_ctx* ctx, const fl_shape* s, const void* q_new, const int32_t* active_idx, int n_active,
                               const DevSide& kside, int n_use, const int32_t* col_idx, const int32_t* col_cnt, int c,
                               const float* lse, float* out, cudaStream_t st) {
   ColScoreArgs a{};
@@ -262,7 +262,7 @@ int fl_launch_sparse_colscore(const fl_shape* s, const void* q_new, const int32_
 #define FL_CS_LAUNCH(T, DH, BITS)                                                                                  \
   do {                                                                                                             \
     auto ck = colscore_kernel<T, DH, BITS, true>;                                                                  \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(ck, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)colscore_smem<DH>())); \
+    FL_FUNC_ATTR_ONCE(ctx, ck, colscore_smem<DH>(), false);                                                        \
     ck<<<grid, kAttnThreads, colscore_smem<DH>(), st>>>(a);                                                        \
   } while (0)
 #define FL_CS_BITS(T, DH)                          \
@@ -299,8 +299,8 @@ extern "C" int fl_dense_loop_attention(fl_ctx* ctx, const fl_shape* shape, const
   rc = fl_launch_dense_tc(ctx, shape, q, k, v, o, lse, col_scores, status, st);
   if (rc != FL_ERR_UNSUPPORTED) return rc;
   if (shape->dtype == FL_F32)
-    return shape->head_dim == 64 ? launch_dense<float, 64>(shape, q, k, v, o, lse, col_scores, st)
-                                 : launch_dense<float, 128>(shape, q, k, v, o, lse, col_scores, st);
-  return shape->head_dim == 64 ? launch_dense<__nv_bfloat16, 64>(shape, q, k, v, o, lse, col_scores, st)
-                               : launch_dense<__nv_bfloat16, 128>(shape, q, k, v, o, lse, col_scores, st);
+    return shape->head_dim == 64 ? launch_dense<float, 64>(ctx, shape, q, k, v, o, lse, col_scores, st)
+                                 : launch_dense<float, 128>(ctx, shape, q, k, v, o, lse, col_scores, st);
+  return shape->head_dim == 64 ? launch_dense<__nv_bfloat16, 64>(ctx, shape, q, k, v, o, lse, col_scores, st)
+                               : launch_dense<__nv_bfloat16, 128>(ctx, shape, q, k, v, o, lse, col_scores, st);
 }

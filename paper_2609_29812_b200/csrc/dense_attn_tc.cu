@@ -670,16 +670,12 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
   a.L = s->L; a.H = s->n_heads; a.d = (int)d_row; a.q_block = s->q_block; a.nb = fl_n_blocks(s);
   a.scale = s->sm_scale;
   const int n_tiles = (s->L + kM - 1) / kM;
-  FL_CHECK_CUDA(cudaFuncSetAttribute(dense_flash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFlashSmem));
-  FL_CHECK_CUDA(cudaFuncSetAttribute(dense_flash_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared));
+  FL_FUNC_ATTR_ONCE(ctx, dense_flash_kernel, kFlashSmem, true);
   dense_flash_kernel<<<dim3(n_tiles * s->n_heads), kThreads, kFlashSmem, st>>>(a);
   int rc = fl_launch_status();
   if (rc != FL_OK || col_scores == nullptr) return rc;
   if (!fl_tile_tmap(ctx, k, s->L, d_row, kM, &a.k_map)) return FL_ERR_CUDA;
-  FL_CHECK_CUDA(cudaFuncSetAttribute(dense_colsum_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kColsumSmem));
-  FL_CHECK_CUDA(cudaFuncSetAttribute(dense_colsum_kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                     (int)cudaSharedmemCarveoutMaxShared));
+  FL_FUNC_ATTR_ONCE(ctx, dense_colsum_kernel, kColsumSmem, true);
   dense_colsum_kernel<<<dim3(n_tiles, a.nb, s->n_heads), kThreads, kColsumSmem, st>>>(a);
   return fl_launch_status();
 }
@@ -707,9 +703,7 @@ int fl_launch_sparse_colsum_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const
 #define FL_SC(BITS)                                                                                               \
   do {                                                                                                            \
     auto kern = sparse_colsum_kernel<BITS>;                                                                       \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSpColsumSmem));  \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                     \
-                                       (int)cudaSharedmemCarveoutMaxShared));                                    \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kSpColsumSmem, true);                                                              \
     kern<<<grid, kThreads, kSpColsumSmem, st>>>(a);                                                               \
   } while (0)
   switch (s->bits) {

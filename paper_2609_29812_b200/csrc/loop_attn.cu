@@ -3,7 +3,7 @@
 // head dimension) and the entry point, which dispatches to the tensor-core kernel when it applies.
 #include "attn_simt.cuh"
 
-int fl_launch_sparse_colscore(const fl_shape* s, const void* q_new, const int32_t* active_idx, int n_active,
+int fl_launch_sparse_colscore(const fl_ctx* ctx, const fl_shape* s, const void* q_new, const int32_t* active_idx, int n_active,
                               const DevSide& kside, int n_use, const int32_t* col_idx, const int32_t* col_cnt, int c,
                               const float* lse, float* out, cudaStream_t st);
 
@@ -203,12 +203,12 @@ __global__ void __launch_bounds__(kAttnThreads) loop_attn_kernel(const __grid_co
 }
 
 template <typename T, int DH>
-int launch_loop(const fl_shape* s, const LoopAttnArgs& a, int max_tiles, cudaStream_t st) {
+int launch_loop(const fl_ctx* ctx, const fl_shape* s, const LoopAttnArgs& a, int max_tiles, cudaStream_t st) {
   const dim3 grid(max_tiles, a.nb, s->n_heads);
 #define FL_LA(BITS)                                                                                               \
   do {                                                                                                            \
     auto kern = loop_attn_kernel<T, DH, BITS>;                                                                    \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)loop_smem<DH>())); \
+    FL_FUNC_ATTR_ONCE(ctx, kern, loop_smem<DH>(), false);                                                         \
     kern<<<grid, kAttnThreads, loop_smem<DH>(), st>>>(a);                                                         \
   } while (0)
   switch (s->bits) {
@@ -276,11 +276,11 @@ extern "C" int fl_loop_attention(fl_ctx* ctx, const fl_shape* shape, int loop_r,
   const int per_block = shape->q_block < n_active ? shape->q_block : n_active;
   const int max_tiles = (per_block + kQTile - 1) / kQTile;
   if (shape->dtype == FL_F32)
-    rc = shape->head_dim == 64 ? launch_loop<float, 64>(shape, a, max_tiles, st)
-                               : launch_loop<float, 128>(shape, a, max_tiles, st);
+    rc = shape->head_dim == 64 ? launch_loop<float, 64>(ctx, shape, a, max_tiles, st)
+                               : launch_loop<float, 128>(ctx, shape, a, max_tiles, st);
   else
-    rc = shape->head_dim == 64 ? launch_loop<__nv_bfloat16, 64>(shape, a, max_tiles, st)
-                               : launch_loop<__nv_bfloat16, 128>(shape, a, max_tiles, st);
+    rc = shape->head_dim == 64 ? launch_loop<__nv_bfloat16, 64>(ctx, shape, a, max_tiles, st)
+                               : launch_loop<__nv_bfloat16, 128>(ctx, shape, a, max_tiles, st);
   if (rc != FL_OK || col_scores_next == nullptr) return rc;
   // column scores that prepare a pruned selection for loop r+1 (Eq. 6 with a sparse source loop)
   return fl_next_col_scores(ctx, shape, loop_r, q_new, active_idx, n_active, store, col_idx, col_cnt, c, lse_out,
@@ -377,5 +377,5 @@ static int fl_next_col_scores(fl_ctx* ctx, const fl_shape* s, int loop_r, const 
   if (rc != FL_ERR_UNSUPPORTED) return rc;
   DevSide kside;
   fl_dev_side(store, true, &kside);
-  return fl_launch_sparse_colscore(s, q_new, active_idx, n_active, kside, loop_r - 1, col_idx, col_cnt, c, lse, out, st);
+  return fl_launch_sparse_colscore(ctx, s, q_new, active_idx, n_active, kside, loop_r - 1, col_idx, col_cnt, c, lse, out, st);
 }

@@ -639,10 +639,8 @@ int launch_mode(fl_ctx* ctx, int bits, dim3 grid, const StArgs& a, cudaStream_t 
 #define FL_ST(BITS)                                                                                              \
   do {                                                                                                           \
     auto kern = loop_attn_stream_kernel<BITS, MODE>;                                                             \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStSmemBytes));  \
     /* two CTAs per SM need the SM's whole shared memory: ask for the largest carve-out */                      \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,                    \
-                                       (int)cudaSharedmemCarveoutMaxShared));                                   \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kStSmemBytes, true);                                                            \
     FL_CHECK_CUDA(fl_launch(ctx, kern, grid, dim3(kThreads), kStSmemBytes, st, a));                             \
   } while (0)
   switch (bits) {

@@ -1021,7 +1021,7 @@ int fl_launch_loop_attn_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const voi
 #define FL_TC2(BITS, IDX, ECON)                                                                                  \
   do {                                                                                                           \
     auto kern = loop_attn_tc_kernel<BITS, IDX, ECON>;                                                            \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemBytes));  \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kTcSmemBytes, false);                                                           \
     FL_CHECK_CUDA(fl_launch(ctx, kern, grid, dim3(kThreads), kTcSmemBytes, st, a));                             \
   } while (0)
 #define FL_TC(BITS)                                   \

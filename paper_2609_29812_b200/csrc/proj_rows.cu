@@ -411,7 +411,7 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
 #define FL_PROJ(G, BN)                                                                                              \
   do {                                                                                                              \
     auto kern = proj_rows_kernel<G, BN, 0>;                                                                          \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProjSmem));         \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kProjSmem, false);                                                                 \
     FL_CHECK_CUDA(fl_launch(ctx, kern, dim3(grid), dim3(kThreads), kProjSmem, st, a));                              \
   } while (0)
   if (gather) {
@@ -491,7 +491,7 @@ extern "C" int fl_project_qkv_quant(fl_ctx* ctx, const fl_shape* shape, int loop
 #define FL_PROJQ(BITS)                                                                                              \
   do {                                                                                                              \
     auto kern = proj_rows_kernel<true, 256, BITS>;                                                                  \
-    FL_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kProjSmem));         \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kProjSmem, false);                                                                 \
     FL_CHECK_CUDA(fl_launch(ctx, kern, dim3(grid), dim3(kThreads), kProjSmem, st, a));                              \
   } while (0)
   if (shape->bits == 8) FL_PROJQ(8); else if (shape->bits == 4) FL_PROJQ(4); else FL_PROJQ(2);

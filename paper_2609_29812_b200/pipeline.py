@@ -11,6 +11,7 @@ Per-layer state carried across loops (all caller-owned device tensors):
 """
 from __future__ import annotations
 
+import itertools
 from dataclasses import dataclass
 from typing import List, Optional
 
@@ -68,6 +69,22 @@ def rows_workspace(dev, n: int, d: int):
     return ws
 
 
+_STATUS: dict = {}     # (device, stream) -> (zeroed words, counter of the words handed out)
+
+
+def status_word(dev):
+    """A zeroed int32 device word of its own: one of a block of 1024 that is cleared once, on the stream that will use it
+    (a fill kernel per word costs more host time than the call whose errors it collects). A block lives as long as
+    any word of it; words are not handed out again."""
+    key = (dev, B._stream(None))
+    while True:
+        block = _STATUS.get(key)
+        i = next(block[1]) if block is not None else 1024
+        if i < 1024:
+            return block[0][i:i + 1]
+        _STATUS[key] = (torch.zeros(1024, dtype=torch.int32, device=dev), itertools.count())
+
+
 def lend_workspace(ctx, shape, dev) -> int:
     """Hands the context the workspace with which the attention launch splits the problems of its last, partly empty
     wave over two CTAs each (a scheduling aid; 0 bytes when the shape cannot profit).  The tensor stays referenced
@@ -77,7 +94,9 @@ def lend_workspace(ctx, shape, dev) -> int:
         ws = getattr(ctx, "_workspace", None)
         if ws is None or ws.numel() < need:
             ws = torch.empty(need, dtype=torch.uint8, device=dev)
-        B.fl_set_workspace(ctx, ws, ws.numel())
+        # a context that holds this workspace already keeps it: every launch leaves its counters cleared
+        if getattr(ctx, "_lent", None) != (ws.data_ptr(), ws.numel()):
+            B.fl_set_workspace(ctx, ws, ws.numel())
         ctx._workspace = ws
     return need
 
@@ -106,7 +125,7 @@ class LayerState:
         self.col_scores = None
         self.lse = None
         self.store = None
-        self.status = torch.zeros(1, dtype=torch.int32, device=self.dev)   # asynchronous device-side errors
+        self.status = status_word(self.dev)   # asynchronous device-side errors
 
     # ---- loop 1 -------------------------------------------------------------------------------
     def dense_loop(self, q, k, v, want_col_scores=True):
@@ -186,9 +205,11 @@ class LayerState:
         def one(side):
             st = {"slot_of_pos": sel.slot_of_pos, "n_rows": n}
             if ws is not None:
-                st["rows_cur"] = ws[side][1][:n]
+                prev, cur = ws[side]
+                whole = cur.shape[0] == n
+                st["rows_cur"] = cur if whole else cur[:n]
                 if rows != "cur":    # rows="cur": a loop that reuses the carried old term reads nothing else
-                    st["rows_prev"] = ws[side][0][:n]
+                    st["rows_prev"] = prev if whole else prev[:n]
             if self.bits == 16:
                 st.update(codes=torch.empty(max(n, 1), d, dtype=self.dt, device=self.dev), scale=None, zero=None)
             else:
@@ -226,8 +247,9 @@ class LayerState:
     def carry_buffers(self):
         """Buffers of the old-term economy, allocated on first use: background rows [L, H, dh] and mass [H, L]."""
         if getattr(self, "bg_store", None) is None:
-            self.bg_store = torch.zeros_like(self.o_store)
-            self.mass = torch.zeros(self.w.n_heads, self.w.L, dtype=torch.float32, device=self.dev)
+            # rows of positions that were never active are neither written nor read
+            self.bg_store = torch.empty_like(self.o_store)
+            self.mass = torch.empty(self.w.n_heads, self.w.L, dtype=torch.float32, device=self.dev)
         return self.bg_store, self.mass
 
     def attention_indexed(self, loop_r, q_new, sel: TokenSelection, col_scores_next=None, check=True,
