@@ -84,6 +84,22 @@ int fl_launch_status();  // maps cudaGetLastError() to a status
 
 static inline int fl_elem_bytes(const fl_shape* s) { return s->dtype == FL_F32 ? 4 : 2; }
 static inline int fl_n_blocks(const fl_shape* s) { return (s->L + s->q_block - 1) / s->q_block; }
+// CTAs that share the 128-row tiles of a (query block, head) problem in the tensor-path attention: one for all of them,
+// or one for each. One CTA per problem makes a grid of few, long jobs, as long as the fullest block (a block of 1024 rows
+// with 90% of them active: 8 tiles in a row); one per tile pays the column list again (about an eighth of a tile's time
+// at 2048 columns). The shorter of the two in whole waves over the chip's CTA slots is taken, the fullest block counted
+// as 1.4 times the average (the active rows are not spread evenly) and the last tile of a block as half a tile.
+static inline int fl_attn_row_shares(const fl_shape* s, int n_active, int slots) {
+  const int64_t span = s->q_block < s->L ? s->q_block : s->L;
+  const int64_t rows = ((int64_t)n_active * span + s->L - 1) / s->L;             // of an average block
+  if (rows <= 128) return 1;
+  const int64_t full = rows * 7 / 5 < span ? rows * 7 / 5 : span;
+  const int64_t tiles = (full + 127) / 128, jobs = (int64_t)fl_n_blocks(s) * s->n_heads;
+  const int64_t tile_jobs = (jobs * (rows + 64) + 127) / 128;
+  const int64_t whole = (jobs + slots - 1) / slots * (8 * tiles + 1);
+  const int64_t shared = (tile_jobs + slots - 1) / slots * (8 + 1);
+  return shared < whole ? (int)tiles : 1;
+}
 
 // ---------------------------------------------------------------------------------------------
 // Device view of one side (K or V) of a store: base rows and the residual streams in loop order.

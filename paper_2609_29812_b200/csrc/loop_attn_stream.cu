@@ -70,6 +70,7 @@ struct alignas(64) StArgs {
   int c;
   int32_t* status;
   int L, H, q_block, nb, d, group;
+  int n_share;                         // CTAs that take the row tiles of a problem in turn
   float scale;
 };
 
@@ -110,7 +111,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // problem (query block b, head h): every chunk of a first-block problem needs the causal mask, which makes them the
   // longest jobs: they come first
-  const int item = blockIdx.x;
+  const int share = blockIdx.x % a.n_share, row_step = a.n_share * kM;   // row tiles share, share + n_share, ...
+  const int item = blockIdx.x / a.n_share;
   int b, h;
   if (a.nb == 1) { b = 0; h = item; }
   else if (item < a.H) { b = 0; h = item; }
@@ -190,8 +192,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   tc::tc_fence_after();
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
-  const int q_lo = ctl.q_lo, q_hi = ctl.q_hi;
-  if (q_hi > q_lo) {   // CTA-uniform: blocks without active rows only release the tensor memory
+  const int q_lo = ctl.q_lo + share * kM, q_hi = ctl.q_hi;
+  if (q_hi > q_lo) {   // CTA-uniform: without active rows the CTA only releases the tensor memory
   {
     // causal prefix, stable partition into plain / patched columns: every warp owns a contiguous span
     const int i_last = ctl.i_last;
@@ -252,7 +254,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   int g = 0;                    // chunks issued so far (all tiles): buffers = g & 1, one phase of their barriers per use
   uint32_t dirty_par_cta = 0;   // per-slot phase parity of the patched[] barriers (they only see dirty chunks)
 
-  for (int s0 = q_lo, tile = 0; s0 < q_hi; s0 += kM, ++tile) {
+  for (int s0 = q_lo, tile = 0; s0 < q_hi; s0 += row_step, ++tile) {
   const int n_rows = min(kM, q_hi - s0);
   const int g0 = g;
   const uint32_t dirty_par0 = dirty_par_cta;
@@ -478,10 +480,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
         if (MODE == kNewPass) {
           // running reference: taken from the first columns that show a finite logit and moved (with a rescale of
           // the accumulator row) only when a maximum beats it by more than the threshold
-          float cm = -INFINITY;
-#pragma unroll
-          for (int u = 0; u < 32; u += 2) cm = fmaxf(cm, fmaxf(__uint_as_float(r[u]), __uint_as_float(r[u + 1])));
-          cm *= c2;                                        // c2 > 0: scaling commutes with the maximum
+          const float cm = max32(r) * c2;                                        // c2 > 0: scaling commutes with the maximum
           const bool first = ref == -INFINITY && cm > -INFINITY;
           const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
           if (first) ref = cm;                             // accumulator row is still zero: nothing to rescale
@@ -521,16 +520,10 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
           }
           sub = ref == -INFINITY ? 0.f : ref;
         }
-        float sum = 0.f;
-#pragma unroll
-        for (int u = 0; u < 32; u += 2) {
-          const float p0 = tc::ex2(fmaf(__uint_as_float(r[u]), c2, -sub));
-          const float p1 = tc::ex2(fmaf(__uint_as_float(r[u + 1]), c2, -sub));
-          sum += p0 + p1;
-          r[u >> 1] = tc::pack_bf16(p0, p1);
-        }
+        uint32_t pk[16];
+        const float sum = exp32(r, c2, sub, pk);
         ell += sum;
-        tc::tmem_st16(sp_addr + hf * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
+        tc::tmem_st16(sp_addr + hf * 16, pk);
       }
       if (!ok) break;
       tc::tmem_wait_st();
@@ -607,7 +600,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     }
   }
   // every role is done with this tile: accumulator, Q tile and the ring bookkeeping move on together
-  if (s0 + kM < q_hi) {   // CTA-uniform: another row tile of the block follows
+  if (s0 + row_step < q_hi) {   // CTA-uniform: another row tile of the block follows
     for (int ci = 0; ci < n_chunks; ++ci)
       if (chunk_dirty(chunk_info(ci, n_plain, n_patch))) dirty_par_cta ^= 1u << ((g + ci) & 1);
     g += n_chunks;
@@ -691,7 +684,8 @@ int fl_launch_loop_attn_stream(fl_ctx* ctx, const fl_shape* s, int loop_r, const
   a.L = s->L; a.H = s->n_heads; a.q_block = s->q_block; a.nb = fl_n_blocks(s);
   a.d = s->n_heads * s->head_dim; a.group = s->group; a.scale = s->sm_scale;
   a.mass = carry->mass;
-  const dim3 grid(a.nb * s->n_heads);
+  a.n_share = fl_attn_row_shares(s, n_active, 2 * ctx->sm_count);
+  const dim3 grid(a.n_share * a.nb * s->n_heads);
   if (!carry->reuse) {
     if (!fl_tile_tmap(ctx, ks.rows_prev, n_active, d_row, 1, &a.k_rows_map) ||
         !fl_tile_tmap(ctx, vs.rows_prev, n_active, d_row, 1, &a.v_rows_map) ||

@@ -30,6 +30,8 @@
 // Shared memory: Q_old, Q_new tiles (64 KB) + a ring of four 32 KB operand slots (K tile | V tile); a chunk of
 // the first kind takes one slot, of the second kind two. Tensor memory (512 columns): acc_old 0-127,
 // acc_new 128-255, S_old / P_old 256-383 (two buffers), S_new / P_new 384-511.
+// Blocks of several 128-row tiles: the tiles are dealt to as many CTAs where that shortens the launch (one CTA walking all
+// tiles took as long as the fullest block: 775 us per loop at 8192 rows, 90 - 20% active, 2048 - 256 columns, 690 us shared).
 // One CTA per problem, except that the problems of a partly empty last wave are given to pairs of CTAs when the
 // caller has lent a workspace: each CTA of a pair takes half of the chunks, the one that completes first leaves its
 // accumulators and row statistics in the workspace and the other merges them into its own before the epilogue.
@@ -92,6 +94,7 @@ struct alignas(64) TcArgs {
   int n_old;
   int use_rows;                      // columns active in this loop are gathered from the materialized rows
   int n_full;                        // CTAs 0 .. n_full-1 take one problem each; the rest are pairs sharing one
+  int n_share;                       // > 1: that many CTAs take the row tiles of each problem in turn (no pairs then)
   int32_t* part_cnt;                 // [kMaxSplit] arrival counters of the pairs (zero between launches)
   float* part_acc;                   // [pairs][2][kPartFloats] partial results
   const int32_t* col_idx;
@@ -148,7 +151,8 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   fl_grid_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // problem (query block b, head h) of this CTA, and for the pairs at the end of the grid which half of it
-  int item = blockIdx.x, part = 0, pair = -1;
+  const int share = blockIdx.x % a.n_share, row_step = a.n_share * kM;   // row tiles share, share + n_share, ...
+  int item = blockIdx.x / a.n_share, part = 0, pair = -1;
   const int n_items = a.nb * a.H;
   if (item >= a.n_full) {
     pair = (item - a.n_full) >> 1;
@@ -255,8 +259,8 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   tc::tc_fence_after();
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
-  const int q_lo = ctl.q_lo, q_hi = ctl.q_hi;
-  if (q_hi > q_lo) {   // CTA-uniform: blocks without active rows only release the tensor memory
+  const int q_lo = ctl.q_lo + share * kM, q_hi = ctl.q_hi;
+  if (q_hi > q_lo) {   // CTA-uniform: without active rows the CTA only releases the tensor memory
   {
     // causal prefix, stable partition into plain / patched columns: every warp owns a contiguous span
     const int i_last = ctl.i_last;                                   // last active row of the block
@@ -334,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   int fill = 0; // ring slots filled so far: slot = fill % kSlots, phase = (fill / kSlots) & 1
   uint32_t dirty_par_cta = 0;  // per-slot phase parity of the patched[] barriers (they only see dirty chunks)
 
-  for (int s0 = q_lo, tile = 0; s0 < q_hi && !(pair >= 0 && part == 1 && !split); s0 += kM, ++tile) {
+  for (int s0 = q_lo, tile = 0; s0 < q_hi && !(pair >= 0 && part == 1 && !split); s0 += row_step, ++tile) {
   const int n_rows = min(kM, q_hi - s0);
   const int g0 = g, g0_1 = g1, fill0 = fill;
   const uint32_t dirty_par0 = dirty_par_cta;
@@ -605,10 +609,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
         if (ECON || grp == 1) {
           // running reference of the new term: taken from the first columns that show a finite logit and moved
           // (with a rescale of the accumulator row) only when a maximum beats it by more than the threshold
-          float cm = -INFINITY;
-#pragma unroll
-          for (int u = 0; u < 32; u += 2) cm = fmaxf(cm, fmaxf(__uint_as_float(r[u]), __uint_as_float(r[u + 1])));
-          cm *= c2;                                        // c2 > 0: scaling commutes with the maximum
+          const float cm = max32(r) * c2;                                        // c2 > 0: scaling commutes with the maximum
           const bool first = ref == -INFINITY && cm > -INFINITY;
           const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
           if (first) ref = cm;                             // accumulator row is still zero: nothing to rescale
@@ -650,16 +651,10 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
           }
           sub = ref == -INFINITY ? 0.f : ref;
         }
-        float sum = 0.f;
-#pragma unroll
-        for (int u = 0; u < 32; u += 2) {
-          const float p0 = tc::ex2(fmaf(__uint_as_float(r[u]), c2, -sub));
-          const float p1 = tc::ex2(fmaf(__uint_as_float(r[u + 1]), c2, -sub));
-          sum += p0 + p1;
-          r[u >> 1] = tc::pack_bf16(p0, p1);
-        }
+        uint32_t pk[16];
+        const float sum = exp32(r, c2, sub, pk);
         if (!ECON && grp == 0) mass += sum; else ell += sum;
-        tc::tmem_st16(sp_addr + hf * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
+        tc::tmem_st16(sp_addr + hf * 16, pk);
       }
       if (!ok) break;
       // P is announced at once: its PV MMAs free both the ring slot (for the gathers) and this S buffer (for the
@@ -886,7 +881,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     }
   }
   // every role is done with this tile: accumulators, Q tiles and the ring bookkeeping move on together
-  if (s0 + kM < q_hi) {   // CTA-uniform: another row tile of the block follows
+  if (s0 + row_step < q_hi) {   // CTA-uniform: another row tile of the block follows
     if (ECON) { g += (c_hi - c_lo + 1) >> 1; g1 += (c_hi - c_lo) >> 1; }
     else g += c_hi - c_lo;
     int f = fill;
@@ -1012,12 +1007,13 @@ int fl_launch_loop_attn_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const voi
   const int n_items = a.nb * s->n_heads;
   const int rem = n_items % ctx->sm_count;
   const size_t ws_need = (size_t)kMaxSplit * sizeof(int32_t) + (size_t)rem * 2 * kPartFloats * sizeof(float);
-  const bool pairs = ctx->ws != nullptr && rem > 0 && 2 * rem <= ctx->sm_count &&
+  a.n_share = fl_attn_row_shares(s, n_active, ctx->sm_count);
+  const bool pairs = a.n_share == 1 && ctx->ws != nullptr && rem > 0 && 2 * rem <= ctx->sm_count &&
                      rem <= kMaxSplit && ctx->ws_bytes >= ws_need;
   a.n_full = pairs ? n_items - rem : n_items;
   a.part_cnt = static_cast<int32_t*>(ctx->ws);
   a.part_acc = reinterpret_cast<float*>(static_cast<uint8_t*>(ctx->ws) + kMaxSplit * sizeof(int32_t));
-  const dim3 grid(a.n_full + 2 * (n_items - a.n_full));
+  const dim3 grid(a.n_share * (a.n_full + 2 * (n_items - a.n_full)));
 #define FL_TC2(BITS, IDX, ECON)                                                                                  \
   do {                                                                                                           \
     auto kern = loop_attn_tc_kernel<BITS, IDX, ECON>;                                                            \

@@ -2,7 +2,7 @@
 // active list, bf16 packing, the dequantize-and-add of one 16-byte piece and the chunk layout of the partitioned
 // column list.
 #pragma once
-#include "fl_internal.cuh"
+#include "codec.cuh"
 #include "tc_ptx.cuh"
 
 namespace fl_tc {
@@ -76,6 +76,40 @@ __device__ __forceinline__ void unpack8(const uint4& raw, float (&x)[8]) {
     x[2 * i] = f.x;
     x[2 * i + 1] = f.y;
   }
+}
+
+// Largest of 32 logits, in four chains.
+__device__ __forceinline__ float max32(const uint32_t (&r)[32]) {
+  float m[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) m[i] = __uint_as_float(r[i]);
+#pragma unroll
+  for (int u = 4; u < 32; u += 8)
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      m[i] = u + 4 < 32 ? fmaxf(fmaxf(m[i], __uint_as_float(r[u + i])), __uint_as_float(r[(u + 4 + i) & 31]))
+                        : fmaxf(m[i], __uint_as_float(r[u + i]));
+  return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+}
+
+// P = 2^(s c2 - sub) of 32 logits: 16 packed bf16 pairs into p, returns the sum of the unrounded values. A softmax warp
+// shares its scheduler with one other and is bound by its own latencies: pairs (.f32x2) halve the instructions around the
+// exponentials, and the sum runs in independent chains.
+__device__ __forceinline__ float exp32(const uint32_t (&r)[32], float c2, float sub, uint32_t (&p)[16]) {
+  using namespace fl_codec;
+  const f32x2 cc = pair(c2, c2), ns = pair(-sub, -sub);
+  f32x2 acc[4];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    float x0, x1;
+    split(fma2(pair_u(r[2 * u], r[2 * u + 1]), cc, ns), x0, x1);
+    const float p0 = tc::ex2(x0), p1 = tc::ex2(x1);
+    acc[u & 3] = u < 4 ? pair(p0, p1) : add2(acc[u & 3], pair(p0, p1));
+    p[u] = tc::pack_bf16(p0, p1);
+  }
+  float a, b;
+  split(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), a, b);
+  return a + b;
 }
 
 // Dequantize-and-add for one 16-byte piece of a column that carries residual payloads (Eq. 8 chain in
