@@ -4,14 +4,15 @@
 // Two kernels, because the statistics need each row's final normaliser:
 //   dense_flash_kernel     one CTA per (128-row query tile, head): S = Q K^T per chunk of 64 keys, online softmax with a
 //                          lazily moved reference, acc += P V; writes O = acc / l and lse = ref + log l.
-//   dense_colsum_kernel    one CTA per (chunk of 128 keys, query block, head): S^T = K Q^T with the KEYS as the
-//                          accumulator's rows, so that the thread that owns a key sums exp(s - lse_i) over the block's
+//   dense_colsum_kernel    one CTA per (chunk of 512 or 128 keys, head, group of query blocks): S^T = K Q^T with the KEYS as the
+//                          accumulator's rows, so that the thread that owns a key sums exp(s - lse_i) over a block's
 //                          queries in registers, in a fixed order (no atomics, no cross-thread reduction):
 //                          col_scores[h, b, j] = sum_{i in block b, i >= j} p_ij.
-// Both keep two CTAs per SM (half the shared memory and 256 tensor-memory columns each) so that one CTA's dependent
-// chain MMA -> exponentials -> MMA runs under the other's. Operand tiles come by plain TMA tile loads (the rows are
+// The flash kernel keeps two CTAs per SM (half the shared memory and 256 tensor-memory columns each) so that one CTA's
+// dependent chain MMA -> exponentials -> MMA runs under the other's. Operand tiles come by plain TMA tile loads (the rows are
 // consecutive), 128B-swizzled; rows beyond L read as zero and are masked. Every mbarrier wait is bounded.
 #include "tc_attn_common.cuh"
+#include <algorithm>
 
 namespace {
 
@@ -280,42 +281,118 @@ __global__ void __launch_bounds__(kThreads, 2) dense_flash_kernel(const __grid_c
 }
 
 // ------------------------------------------------------------------------------------------------------------
-// Column sums. Accumulator tile D[key j (128 lanes)][query i (128 columns)] = K_chunk Q_tile^T; the thread of lane j
-// adds exp(scale s_ji - lse_i) over the queries i >= j of the block, tile after tile.
+// Column sums. Accumulator tile D[key j (128 lanes)][query i (128 columns)] = K Q_tile^T; the thread of lane j adds
+// exp(scale s_ji - lse_i) over the queries i >= j of a block, tile after tile, and writes the sum at the block's end. A CTA
+// keeps its keys and streams the query tiles of one block after the other, so that its start-up is paid once and the
+// loads, the MMAs and the exponentials of successive tiles overlap across block borders.
+//   NH = 4: 512 keys, one CTA per SM. A query tile that crosses L2 serves four accumulators (with 128 keys its 32 KB per
+//           128 x 128 exponentials ask for 32 B/clk of each SM, about what it takes), and 16 warps keep the exponential
+//           unit busy (4 per scheduler: 80% of its cycles; 8 warps with 256 keys and two accumulator buffers: 67%).
+//   NH = 1: 128 keys, two CTAs per SM: for prompts too short to give every SM its 512 keys.
+// Bound by the exponential unit (16 per clock and SM). 32768 x 16 heads: 3730 -> 2570 us, 8192 x 16: 225 -> 180 us.
 // ------------------------------------------------------------------------------------------------------------
-struct __align__(16) ColsumCtl {
-  uint64_t k_full, q_full[2], d_full[2], d_free[2];
+template <int NH> struct ColsumShape {
+  static constexpr int kQSlots = 2;
+  static constexpr int kDBufs = NH == 4 ? 1 : 2;         // accumulators per 128 keys: 512 tensor-memory columns in all
+  static constexpr int kGroups = NH == 4 ? 2 : 4;        // 32-query groups of a tile that a thread takes at a time
+  static constexpr int kEpiWarps = 4 * NH;
+  static constexpr int kIssue = kEpiWarps, kTma = kEpiWarps + 1, kThreads = (kEpiWarps + 2) * 32;
+  static constexpr size_t kTiles = (size_t)(NH + kQSlots) * kQTileBytes;
+};
+constexpr int kLseSlots = 8;   // the TMA warp runs at most kQSlots tiles ahead of the MMAs, those two ahead of the sums
+template <int NH> struct __align__(16) ColsumCtl {
+  uint64_t k_full, q_full[ColsumShape<NH>::kQSlots], q_free[ColsumShape<NH>::kQSlots], lse_full[kLseSlots], d_full[NH][ColsumShape<NH>::kDBufs], d_free[NH][ColsumShape<NH>::kDBufs];
   uint32_t tmem_base;
   int abort_flag;
-  float lse2[2][kM];      // log-normalisers of the tile's queries, in log2 units
+  alignas(16) float neg_lse2[kLseSlots][kM];   // minus the log-normalisers of a tile's queries, in log2 units
 };
-constexpr size_t kColsumSmem = 1024 + 3 * kQTileBytes + sizeof(ColsumCtl);
+template <int NH> constexpr size_t kColsumSmem = 1024 + ColsumShape<NH>::kTiles + sizeof(ColsumCtl<NH>);
 
-__global__ void __launch_bounds__(kThreads, 2) dense_colsum_kernel(const __grid_constant__ DnArgs a) {
+// The query tiles of a CTA in order: blocks b .. b_end - 1, in each the tiles from the first that holds a query at or
+// after key j0.
+struct ColsumTiles {
+  int b, b_end, t, n_tiles, blk_lo, blk_hi;
+  int L, q_block, j0;
+  __device__ ColsumTiles(const DnArgs& a, int j0_, int b_lo, int b_hi) : b(b_lo), b_end(b_hi), L(a.L), q_block(a.q_block), j0(j0_) { enter(); }
+  __device__ void enter() {
+    blk_lo = b * q_block;
+    blk_hi = min(L, blk_lo + q_block);
+    n_tiles = (blk_hi - blk_lo + kM - 1) / kM;
+    t = j0 > blk_lo ? (j0 - blk_lo) / kM : 0;
+  }
+  __device__ bool valid() const { return b < b_end; }
+  __device__ int i0() const { return blk_lo + t * kM; }
+  __device__ bool next() {              // true: the tile left was the last one of its block
+    if (++t < n_tiles) return false;
+    ++b;
+    enter();
+    return true;
+  }
+};
+
+// sum + the probabilities 2^(c2 s + neg_lse2) of a key's 32 G logits, each group of 32 in its own order and the groups one
+// after the other: independent chains keep the exponential unit busy. MASKED: queries before
+// `first` do not see the key.
+template <bool MASKED, int G>
+__device__ __forceinline__ float colsum_tile(const uint32_t (&r)[G][32], fl_codec::f32x2 cc, const float* nl, int first, float sum) {
+  using namespace fl_codec;
+  float part[G];
+#pragma unroll
+  for (int q = 0; q < G; ++q) part[q] = 0.f;
+#pragma unroll
+  for (int u = 0; u < 32; u += 4) {
+#pragma unroll
+    for (int q = 0; q < G; ++q) {
+      const ulonglong2 l = *reinterpret_cast<const ulonglong2*>(nl + q * 32 + u);
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        float x0, x1;
+        split(fma2(pair_u(r[q][u + 2 * v], r[q][u + 2 * v + 1]), cc, v ? l.y : l.x), x0, x1);
+        float p0 = tc::ex2(x0), p1 = tc::ex2(x1);
+        if (MASKED) {
+          p0 = q * 32 + u + 2 * v >= first ? p0 : 0.f;
+          p1 = q * 32 + u + 2 * v + 1 >= first ? p1 : 0.f;
+        }
+        part[q] += p0;
+        part[q] += p1;
+      }
+    }
+  }
+#pragma unroll
+  for (int q = 0; q < G; ++q) sum += part[q];
+  return sum;
+}
+
+template <int NH>
+__global__ void __launch_bounds__(ColsumShape<NH>::kThreads, NH == 1 ? 2 : 1) dense_colsum_kernel(const __grid_constant__ DnArgs a, int b_per) {
+  using Sh = ColsumShape<NH>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* k_tile = smem;                       // [128 keys][128] as the M operand
-  uint8_t* q_ring = smem + kQTileBytes;         // two query tiles [128 queries][128] as the N operand
-  ColsumCtl& ctl = *reinterpret_cast<ColsumCtl*>(q_ring + 2 * kQTileBytes);
+  uint8_t* k_tile = smem;                            // NH x [128 keys][128] as the M operand
+  uint8_t* q_ring = smem + NH * kQTileBytes;         // query tiles [128 queries][128] as the N operand
+  ColsumCtl<NH>& ctl = *reinterpret_cast<ColsumCtl<NH>*>(smem + Sh::kTiles);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int kc = blockIdx.x, b = a.nb - 1 - (int)blockIdx.y, h = blockIdx.z;
-  const int blk_lo = b * a.q_block, blk_hi = min(a.L, (b + 1) * a.q_block);
-  const int j0 = kc * kM;
-  if (j0 >= blk_hi) return;                      // the chunk lies beyond the block's last row: no candidates
-  const int n_tiles = (blk_hi - blk_lo + kM - 1) / kM;
-  const int t_first = j0 > blk_lo ? (j0 - blk_lo) / kM : 0;    // earlier tiles hold no query at or after the first key
+  // the first keys see the most queries: they are dispatched first
+  const int h = blockIdx.x, j0 = (int)blockIdx.z * (NH * kM);
+  const int b_lo = max(j0 / a.q_block, (int)blockIdx.y * b_per), b_hi = min(a.nb, ((int)blockIdx.y + 1) * b_per);
+  if (b_lo >= b_hi) return;                          // the keys lie beyond the last block of the group: no candidates
   if (tid == 0) {
     tc::mbar_init(&ctl.k_full, 1);
-    for (int s = 0; s < 2; ++s) {
-      tc::mbar_init(&ctl.q_full[s], 2);          // the tile's bytes (one arrival with the byte count) + its normalisers
-      tc::mbar_init(&ctl.d_full[s], 1);
-      tc::mbar_init(&ctl.d_free[s], 4);
+    for (int s = 0; s < Sh::kQSlots; ++s) {
+      tc::mbar_init(&ctl.q_full[s], 1);
+      tc::mbar_init(&ctl.q_free[s], 1);
     }
+    for (int s = 0; s < kLseSlots; ++s) tc::mbar_init(&ctl.lse_full[s], 1);
+    for (int g = 0; g < NH; ++g)
+      for (int s = 0; s < Sh::kDBufs; ++s) {
+        tc::mbar_init(&ctl.d_full[g][s], 1);
+        tc::mbar_init(&ctl.d_free[g][s], 4);
+      }
     ctl.abort_flag = 0;
     tc::fence_barrier_init();
   }
-  if (warp == kIssueWarp) {
-    tc::tmem_alloc(&ctl.tmem_base, kTmemCols);
+  if (warp == Sh::kIssue) {
+    tc::tmem_alloc(&ctl.tmem_base, NH * Sh::kDBufs * kM);
     tc::tmem_relinquish();
   }
   tc::tc_fence_before();
@@ -324,108 +401,121 @@ __global__ void __launch_bounds__(kThreads, 2) dense_colsum_kernel(const __grid_
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
 
-  if (warp == kTmaWarp) {
+  if (warp == Sh::kTma) {
     if (lane == 0) {
-      tc::mbar_arrive_expect_tx(&ctl.k_full, kQTileBytes);
-      tc::tma_tile2d(k_tile, &a.k_map, &ctl.k_full, h * kDH, j0);
-      tc::tma_tile2d(k_tile + kM * 128, &a.k_map, &ctl.k_full, h * kDH + 64, j0);
+      tc::mbar_arrive_expect_tx(&ctl.k_full, NH * kQTileBytes);
+#pragma unroll
+      for (int g = 0; g < NH; ++g) {
+        tc::tma_tile2d(k_tile + g * kQTileBytes, &a.k_map, &ctl.k_full, h * kDH, j0 + g * kM);
+        tc::tma_tile2d(k_tile + g * kQTileBytes + kM * 128, &a.k_map, &ctl.k_full, h * kDH + 64, j0 + g * kM);
+      }
     }
-    bool ok = true;
-    for (int t = t_first, n = 0; t < n_tiles && ok; ++t, ++n) {
-      const int sl = n & 1, i0 = blk_lo + t * kM;
-      // the slot is free once the MMAs of the tile two back have completed (they also read its normalisers' slot,
-      // which the epilogue has released by then: it runs behind the MMAs)
-      if (n >= 2) ok = warp_wait(&ctl.d_full[sl], ((n >> 1) - 1) & 1, abort_flag) &&
-                       warp_wait(&ctl.d_free[sl], ((n >> 1) - 1) & 1, abort_flag);
-      if (!ok) break;
+    int n = 0;
+    for (ColsumTiles it(a, j0, b_lo, b_hi); it.valid(); it.next(), ++n) {
+      const int sl = n % Sh::kQSlots, i0 = it.i0();
+      float l2[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int i = i0 + q * 32 + lane;
+        l2[q] = i < it.blk_hi ? __ldg(a.lse + (size_t)h * a.L + i) * kLog2e : INFINITY;
+      }
+      // the slot is free once the MMAs of the tile that was in it have completed
+      if (n >= Sh::kQSlots && !warp_wait(&ctl.q_free[sl], (n / Sh::kQSlots - 1) & 1, abort_flag)) break;
       if (lane == 0) {
         tc::mbar_arrive_expect_tx(&ctl.q_full[sl], kQTileBytes);
         tc::tma_tile2d(q_ring + sl * kQTileBytes, &a.q_map, &ctl.q_full[sl], h * kDH, i0);
         tc::tma_tile2d(q_ring + sl * kQTileBytes + kM * 128, &a.q_map, &ctl.q_full[sl], h * kDH + 64, i0);
       }
+      // normalisers of the tile eight back: the MMAs of tile n - kQSlots were issued after the sums of the tile two
+      // before it had left its accumulator, and so after those of the tile before that were complete
+      static_assert(kLseSlots >= Sh::kQSlots + 4, "the slot's earlier values must have been used");
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = i0 + q * 32 + lane;
-        ctl.lse2[sl][q * 32 + lane] = i < blk_hi ? __ldg(a.lse + (size_t)h * a.L + i) * kLog2e : INFINITY;
-      }
+      for (int q = 0; q < 4; ++q) ctl.neg_lse2[n % kLseSlots][q * 32 + lane] = -l2[q];
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&ctl.q_full[sl]);
+      if (lane == 0) tc::mbar_arrive(&ctl.lse_full[n % kLseSlots]);
     }
-  } else if (warp == kIssueWarp) {
+  } else if (warp == Sh::kIssue) {
     if (lane == 0) {
       const uint32_t idesc = tc::make_idesc_bf16(kM, kM, false);
       const uint64_t k_desc = tc::make_desc_sw128(tc::smem_u32(k_tile), 16, 1024);
       const uint64_t q_desc0 = tc::make_desc_sw128(tc::smem_u32(q_ring), 16, 1024);
       const uint32_t hi = (uint32_t)(k_desc >> 32);
-      const uint32_t k_lo_w = (uint32_t)k_desc, q_lo0 = (uint32_t)q_desc0;
-      for (int t = t_first, n = 0; t < n_tiles; ++t, ++n) {
-        const int sl = n & 1;
-        if (n == 0 && !tc::mbar_wait(&ctl.k_full, 0, abort_flag)) break;
-        if (!tc::mbar_wait(&ctl.q_full[sl], (n >> 1) & 1, abort_flag)) break;
-        if (n >= 2 && !tc::mbar_wait(&ctl.d_free[sl], ((n >> 1) - 1) & 1, abort_flag)) break;
-        tc::tc_fence_after();
-        const uint32_t d_dst = tmem + sl * kM;
-        const uint32_t q_lo = q_lo0 + sl * (kQTileBytes >> 4);
+      bool ok = tc::mbar_wait(&ctl.k_full, 0, abort_flag);
+      int n = 0;
+      for (ColsumTiles it(a, j0, b_lo, b_hi); it.valid() && ok; it.next(), ++n) {
+        const int sl = n % Sh::kQSlots;
+        if (!tc::mbar_wait(&ctl.q_full[sl], (n / Sh::kQSlots) & 1, abort_flag)) break;
+        const uint32_t q_lo = (uint32_t)q_desc0 + sl * (kQTileBytes >> 4);
+#pragma unroll
+        for (int g = 0; g < NH; ++g) {
+          if (n >= Sh::kDBufs && !tc::mbar_wait(&ctl.d_free[g][n % Sh::kDBufs], (n / Sh::kDBufs - 1) & 1, abort_flag)) { ok = false; break; }
+          tc::tc_fence_after();
+          const uint32_t d_dst = tmem + (g * Sh::kDBufs + n % Sh::kDBufs) * kM;
+          const uint32_t k_lo_w = (uint32_t)k_desc + g * (kQTileBytes >> 4);
 #define FL_KQ(KK, ACC)                                                                                       \
   tc::mma_ss_lo<ACC>(d_dst, k_lo_w + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), hi,                  \
                      q_lo + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), hi, idesc)
-        FL_KQ(0, false); FL_KQ(1, true); FL_KQ(2, true); FL_KQ(3, true);
-        FL_KQ(4, true);  FL_KQ(5, true); FL_KQ(6, true); FL_KQ(7, true);
+          FL_KQ(0, false); FL_KQ(1, true); FL_KQ(2, true); FL_KQ(3, true);
+          FL_KQ(4, true);  FL_KQ(5, true); FL_KQ(6, true); FL_KQ(7, true);
 #undef FL_KQ
-        tc::mma_commit(&ctl.d_full[sl]);
+          tc::mma_commit(&ctl.d_full[g][n % Sh::kDBufs]);
+        }
+        if (ok) tc::mma_commit(&ctl.q_free[sl]);
       }
     }
     __syncwarp();
   } else {
     // the thread's key: lane of tensor memory = row of the accumulator
-    const int jr = warp * 32 + lane, j = j0 + jr;
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+    using namespace fl_codec;
+    const int g = warp >> 2, j = j0 + warp * 32 + lane;
+    const uint32_t d_src = tmem + ((uint32_t)((warp & 3) * 32) << 16) + g * Sh::kDBufs * kM;
     const float c2 = a.scale * kLog2e;
+    const f32x2 cc = pair(c2, c2);
     float sum = 0.f;
-    bool ok = true;
-    for (int t = t_first, n = 0; t < n_tiles; ++t, ++n) {
-      const int sl = n & 1, i0 = blk_lo + t * kM;
-      if (!warp_wait(&ctl.q_full[sl], (n >> 1) & 1, abort_flag)) { ok = false; break; }   // the normalisers
-      if (!warp_wait(&ctl.d_full[sl], (n >> 1) & 1, abort_flag)) { ok = false; break; }
+    int n = 0;
+    for (ColsumTiles it(a, j0, b_lo, b_hi); it.valid(); ++n) {
+      const int i0 = it.i0();
+      if (!warp_wait(&ctl.lse_full[n % kLseSlots], (n / kLseSlots) & 1, abort_flag)) break;
+      if (!warp_wait(&ctl.d_full[g][n % Sh::kDBufs], (n / Sh::kDBufs) & 1, abort_flag)) break;
       tc::tc_fence_after();
       // queries before the key see nothing of it; queries beyond the block carry lse = +inf (probability 0)
+      const bool any_visible = j0 + (warp & ~3) * 32 < i0 + kM;     // of the accumulator's 128 keys
       const bool all_visible = __all_sync(0xffffffffu, j <= i0);
-#pragma unroll 1
-      for (int q = 0; q < 4; ++q) {
-        uint32_t r[32];
-        tc::tmem_ld32(tmem + lane_base + sl * kM + q * 32, r);
-        tc::tmem_wait_ld();
-        const float* l2 = ctl.lse2[sl] + q * 32;
-        float part = 0.f;
-        if (all_visible) {
+      const float* nl = ctl.neg_lse2[n % kLseSlots];
 #pragma unroll
-          for (int u = 0; u < 32; ++u) part += tc::ex2(fmaf(__uint_as_float(r[u]), c2, -l2[u]));
-        } else {
-          const int first = j - (i0 + q * 32);        // queries u >= first are at or after the key
+      for (int q0 = 0; q0 < 4; q0 += Sh::kGroups) {
+        uint32_t r[Sh::kGroups][32];
+        if (any_visible) {
 #pragma unroll
-          for (int u = 0; u < 32; ++u) {
-            const float p = tc::ex2(fmaf(__uint_as_float(r[u]), c2, -l2[u]));
-            part += u >= first ? p : 0.f;
-          }
+          for (int q = 0; q < Sh::kGroups; ++q) tc::tmem_ld32(d_src + n % Sh::kDBufs * kM + (q0 + q) * 32, r[q]);
+          tc::tmem_wait_ld();
         }
-        sum += part;
+        if (q0 + Sh::kGroups == 4) {                // the accumulator is in registers
+          tc::tc_fence_before();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&ctl.d_free[g][n % Sh::kDBufs]);
+        }
+        if (any_visible)
+          sum = all_visible ? colsum_tile<false, Sh::kGroups>(r, cc, nl + q0 * 32, 0, sum)
+                            : colsum_tile<true, Sh::kGroups>(r, cc, nl + q0 * 32, j - i0 - q0 * 32, sum);
       }
-      tc::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&ctl.d_free[sl]);
+      const int b = it.b, blk_hi = it.blk_hi;
+      if (it.next()) {
+        if (j < blk_hi) a.col_scores[((size_t)h * a.nb + b) * a.L + j] = sum;
+        sum = 0.f;
+      }
     }
-    if (ok && j < blk_hi) a.col_scores[((size_t)h * a.nb + b) * a.L + j] = sum;
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == kIssueWarp) {
+  if (warp == Sh::kIssue) {
     if (ctl.abort_flag) {
-      if (lane == 0) tc::mma_commit(&ctl.d_full[0]);
+      if (lane == 0) tc::mma_commit(&ctl.d_full[0][0]);
       __syncwarp();
       for (int it = 0; it < (1 << 16); ++it) __nanosleep(256);
     }
     tc::tc_fence_after();
-    tc::tmem_dealloc(tmem, kTmemCols);
+    tc::tmem_dealloc(tmem, NH * Sh::kDBufs * kM);
   }
   if (tid == 0 && ctl.abort_flag && a.status != nullptr) atomicExch(a.status, (int)FL_ERR_TIMEOUT);
 }
@@ -656,7 +746,7 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_colsum_kernel(const __grid
 int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void* k, const void* v, void* o, float* lse,
                        float* col_scores, int32_t* status, cudaStream_t st) {
   if (s->dtype != FL_BF16 || s->head_dim != kDH || ctx->force_simt) return FL_ERR_UNSUPPORTED;
-  if ((size_t)ctx->max_smem_optin < kColsumSmem || ctx->encode_tiled == nullptr || ctx->tmaps == nullptr)
+  if ((size_t)ctx->max_smem_optin < kColsumSmem<4> || ctx->encode_tiled == nullptr || ctx->tmaps == nullptr)
     return FL_ERR_UNSUPPORTED;
   DnArgs a{};
   const int64_t d_row = (int64_t)s->n_heads * s->head_dim;
@@ -675,8 +765,21 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
   int rc = fl_launch_status();
   if (rc != FL_OK || col_scores == nullptr) return rc;
   if (!fl_tile_tmap(ctx, k, s->L, d_row, kM, &a.k_map)) return FL_ERR_CUDA;
-  FL_FUNC_ATTR_ONCE(ctx, dense_colsum_kernel, kColsumSmem, true);
-  dense_colsum_kernel<<<dim3(n_tiles, a.nb, s->n_heads), kThreads, kColsumSmem, st>>>(a);
+  // 512 keys per CTA where that still gives (with one job per query block) three jobs to two SMs, else 128; the blocks are
+  // dealt to as many CTAs as make two jobs per SM slot, and never to one (half a head's queries stay in L2 at 32K rows).
+  // Measured, one CTA per (keys, head) / dealt: 2500 x 8 heads 34 / 21 us (128 keys; 512: 26), 2500 x 16 57 / 29 (512 keys;
+  // 128: 34), 8192 x 4 173 / 51, 8192 x 16 177 / 181, 32768 x 16 2760 / 2570.
+  const int wide_jobs = (n_tiles + 3) / 4 * s->n_heads;
+#define FL_CS(NH, JOBS, SLOTS)                                                                                            \
+  do {                                                                                                                    \
+    auto kern = dense_colsum_kernel<NH>;                                                                                  \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kColsumSmem<NH>, true);                                                                  \
+    const int groups = std::max(2, (2 * (SLOTS) + (JOBS)-1) / (JOBS)), b_per = (a.nb + groups - 1) / groups;              \
+    kern<<<dim3(s->n_heads, (a.nb + b_per - 1) / b_per, (n_tiles + NH - 1) / NH), ColsumShape<NH>::kThreads, kColsumSmem<NH>, st>>>(a, b_per); \
+  } while (0)
+  if (2 * (int64_t)wide_jobs * a.nb >= 3 * ctx->sm_count) FL_CS(4, wide_jobs, ctx->sm_count);
+  else FL_CS(1, n_tiles * s->n_heads, 2 * ctx->sm_count);
+#undef FL_CS
   return fl_launch_status();
 }
 
