@@ -225,6 +225,11 @@ FL_API int fl_select_columns(fl_ctx* ctx, const fl_shape* shape, const float* co
  * fl_set_workspace (NULL detaches it). Attention calls of one context that may overlap in time (different
  * streams) must not share a workspace. */
 FL_API int fl_loop_attention_workspace_bytes(fl_ctx* ctx, const fl_shape* shape, int64_t* bytes /* host */);
+/* Bytes of a workspace that also has room for the rebuilt rows of the tokens whose payloads are all from earlier loops
+ * ([L, H, dh] storage type per side; token sets that shrink leave such tokens): a launch that recomputes the old term then
+ * rebuilds each of them once instead of once per problem that selects it. Equal to the size above where that does not
+ * apply (binary32 storage, or more than 256 MB of rows). Either size is accepted by fl_set_workspace. */
+FL_API int fl_loop_attention_full_workspace_bytes(fl_ctx* ctx, const fl_shape* shape, int64_t* bytes /* host */);
 FL_API int fl_set_workspace(fl_ctx* ctx, void* workspace /* device */, int64_t bytes, void* stream);
 
 /* Stages 2 + 4 -- Eq. 7 (equivalently Eq. 3) over the reconstructed K/V (Eq. 4 / Eq. 8): rows of tokens that are

@@ -95,6 +95,7 @@ def _load() -> C.CDLL:
         "fl_kv_store_bytes": [C.POINTER(FlShape), C.POINTER(FlKvStore), C.c_int, C.c_int,
                               C.POINTER(i64), C.POINTER(i64)],
         "fl_loop_attention_workspace_bytes": [p, C.POINTER(FlShape), C.POINTER(i64)],
+        "fl_loop_attention_full_workspace_bytes": [p, C.POINTER(FlShape), C.POINTER(i64)],
         "fl_set_workspace": [p, p, i64, p],
     }
     for name, args in sig.items():
@@ -213,6 +214,13 @@ def fl_loop_attention_workspace_bytes(ctx, shape) -> int:
     out = C.c_int64(0)
     _check("fl_loop_attention_workspace_bytes", lib.fl_loop_attention_workspace_bytes(_h(ctx), C.byref(shape),
                                                                                       C.byref(out)), True)
+    return int(out.value)
+
+
+def fl_loop_attention_full_workspace_bytes(ctx, shape) -> int:
+    out = C.c_int64(0)
+    _check("fl_loop_attention_full_workspace_bytes",
+           lib.fl_loop_attention_full_workspace_bytes(_h(ctx), C.byref(shape), C.byref(out)), True)
     return int(out.value)
 
 

@@ -523,16 +523,18 @@ __global__ void __launch_bounds__(ColsumShape<NH>::kThreads, NH == 1 ? 2 : 1) de
 // ------------------------------------------------------------------------------------------------------------
 // Next-loop column scores of a SPARSE loop (Appendix D.2: a sparse source loop offers its own selected columns as
 // candidates, scored by the block sums of its new probabilities): the same K Q^T tiles, with the 128 keys of a tile
-// gathered by position from the base (four rows per TMA copy) and the columns that carry residual payloads rebuilt
-// in place (Eq. 8 chain up to the loop itself), and the queries taken from the compact rows of the block's active
-// tokens. col_scores_next[h, b, u] = sum over the block's active rows i >= S[u] of exp(s_iu - lse_i), lse the loop's
-// new log-normaliser.
+// gathered by position and the queries taken from the compact rows of the block's active tokens.
+// col_scores_next[h, b, u] = sum over the block's active rows i >= S[u] of exp(s_iu - lse_i), lse the loop's new
+// log-normaliser. A key comes from where its Khat^(r) already stands: the base, the rows that the loop's quantization
+// materialized, or the rows rebuilt for the attention (16 copies of 16 bytes in flight per thread: no four-row gathers, which
+// take one source each); only without those the Eq. 8 chain is run here.
 // ------------------------------------------------------------------------------------------------------------
 struct alignas(64) SpArgs {
-  CUtensorMap k_map;      // K base [L, d], box 64 x 1 (row gathers)
   CUtensorMap q_map;      // compact new Q rows [n_active, d], box 64 x 128
   DevSide k;
   int n_use;              // residual streams contained in Khat^(r): loop_r - 1
+  const __nv_bfloat16* k_rows;    // [n_active, d]: Khat^(r) of the loop's active tokens, or null
+  const __nv_bfloat16* k_stale;   // [L, d]: Khat^(r) of the tokens with payloads of earlier loops only, or null
   const int32_t* active_idx;
   int n_active;
   const int32_t* col_idx;
@@ -546,12 +548,14 @@ struct alignas(64) SpArgs {
 };
 
 struct __align__(16) SpColsumCtl {
-  uint64_t k_full, k_ready, q_full[2], d_full[2], d_free[2];
+  uint64_t k_ready, q_full[2], d_full[2], d_free[2];
   uint32_t tmem_base;
   int abort_flag;
   int q_lo, q_hi;
-  float lse2[2][kM];
+  alignas(16) float neg_lse2[2][kM];
   int pos[2][kM];
+  const __nv_bfloat16* src[kM];   // where the key's row stands, null beyond the count
+  bool chain[kM];                 // base row that still needs the chain
 };
 constexpr size_t kSpColsumSmem = 1024 + 3 * kQTileBytes + sizeof(SpColsumCtl);
 
@@ -569,14 +573,40 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_colsum_kernel(const __grid
   const int u0 = kc * kM;
   if (u0 >= cnt) return;
   const int32_t* cols = a.col_idx + prob * a.c;
-  if (warp < 2) {
-    const int target = warp == 0 ? b * a.q_block : min(a.L, (b + 1) * a.q_block);
+  if (warp >= 4) {
+    const int target = warp == 4 ? b * a.q_block : min(a.L, (b + 1) * a.q_block);
     int below;
     const int r = lower_bound_warp(a.active_idx, a.n_active, target, lane, &below);
-    if (lane == 0) { if (warp == 0) ctl.q_lo = r; else ctl.q_hi = r; }
+    if (lane == 0) { if (warp == 4) ctl.q_lo = r; else ctl.q_hi = r; }
+  } else {
+    // thread u finds out where key u0 + u stands; the slots of four streams are looked up at a time
+    const int j = u0 + tid < cnt ? __ldg(cols + u0 + tid) : -1;
+    const __nv_bfloat16* src = nullptr;
+    bool chain = false;
+    if (j >= 0) {
+      bool earlier = false;
+      int own = -1;
+#pragma unroll 1
+      for (int sg = 0; sg < a.n_use; sg += 4) {
+        int sl[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) sl[q] = sg + q < a.n_use ? __ldg(a.k.s[sg + q].slot + j) : -1;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (sg + q == a.n_use - 1) own = sl[q];
+          else earlier |= sl[q] >= 0;
+        }
+      }
+      src = static_cast<const __nv_bfloat16*>(a.k.base) + (size_t)j * a.d;
+      if (own >= 0 && a.k_rows != nullptr) src = a.k_rows + (size_t)own * a.d;
+      else if (own < 0 && earlier && a.k_stale != nullptr) src = a.k_stale + (size_t)j * a.d;
+      else chain = own >= 0 || earlier;
+      src += h * kDH;
+    }
+    ctl.src[tid] = src;
+    ctl.chain[tid] = chain;
   }
   if (tid == 0) {
-    tc::mbar_init(&ctl.k_full, 1);
     tc::mbar_init(&ctl.k_ready, 4);
     for (int s = 0; s < 2; ++s) {
       tc::mbar_init(&ctl.q_full[s], 2);
@@ -604,19 +634,6 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_colsum_kernel(const __grid
   const int n_tiles = (q_hi - q_lo + kM - 1) / kM;
 
   if (warp == kTmaWarp) {
-    // the tile's 128 selected columns: base rows by position, four per copy; positions past the count read as zero
-    if (lane == 0) tc::mbar_arrive_expect_tx(&ctl.k_full, kQTileBytes);
-    __syncwarp();
-    {
-      int y[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int u = u0 + lane * 4 + i;
-        y[i] = u < cnt ? __ldg(cols + u) : a.L;
-      }
-      tc::tma_gather4(k_tile + lane * 512, &a.k_map, &ctl.k_full, h * kDH, y[0], y[1], y[2], y[3]);
-      tc::tma_gather4(k_tile + kM * 128 + lane * 512, &a.k_map, &ctl.k_full, h * kDH + 64, y[0], y[1], y[2], y[3]);
-    }
     bool ok = true;
     for (int t = 0; t < n_tiles && ok; ++t) {
       const int sl = t & 1, s0 = q_lo + t * kM;
@@ -631,9 +648,9 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_colsum_kernel(const __grid
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const int i = s0 + q * 32 + lane;
-        const int pos = i < q_hi ? __ldg(a.active_idx + i) : -1;
+        const int pos = i < q_hi ? __ldg(a.active_idx + i) : INT32_MAX;      // ascending
         ctl.pos[sl][q * 32 + lane] = pos;
-        ctl.lse2[sl][q * 32 + lane] = pos >= 0 ? __ldg(a.lse + (size_t)h * a.L + pos) * kLog2e : INFINITY;
+        ctl.neg_lse2[sl][q * 32 + lane] = i < q_hi ? -(__ldg(a.lse + (size_t)h * a.L + pos) * kLog2e) : -INFINITY;
       }
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&ctl.q_full[sl]);
@@ -664,61 +681,63 @@ __global__ void __launch_bounds__(kThreads, 2) sparse_colsum_kernel(const __grid
     }
     __syncwarp();
   } else {
-    // ---- the four epilogue warps first rebuild the columns that carry residual payloads (Eq. 8 chain) ----------
-    bool ok = warp_wait(&ctl.k_full, 0, abort_flag);
-    if (ok) {
-      const int ch = tid & 15;                        // 16-byte piece of the row
-      const int elem = h * kDH + ch * 8;
-      const __nv_bfloat16* base_rows = static_cast<const __nv_bfloat16*>(a.k.base) + elem;
-#pragma unroll 1
-      for (int u = tid >> 4; u < kM; u += 8) {
-        if (u0 + u >= cnt) break;
-        const int j = __ldg(cols + u0 + u);
-        float x[8];
-        unpack8(__ldg(reinterpret_cast<const uint4*>(base_rows + (size_t)j * a.d)), x);
-        bool any = false;
-#pragma unroll 1
-        for (int s = 0; s < a.n_use; ++s) any |= apply_stream8<__nv_bfloat16, BITS>(a.k.s[s], j, elem, a.d, a.group, x);
-        if (any) *reinterpret_cast<uint4*>(k_tile + (ch >> 3) * (kM * 128) + tc::sw128_offset(u, ch & 7)) = pack8(x);
-      }
-      tc::fence_proxy_async_smem();
+    // ---- the four epilogue warps bring the keys in: 16 threads per row, all 16 copies of a thread in flight ----
+    const int ch = tid & 15;                        // 16-byte piece of the row
+    uint8_t* dst = k_tile + (ch >> 3) * (kM * 128);
+#pragma unroll
+    for (int u = tid >> 4; u < kM; u += 8) {
+      uint8_t* to = dst + tc::sw128_offset(u, ch & 7);
+      const __nv_bfloat16* src = ctl.src[u];
+      if (src != nullptr) tc::cp_async16(to, src + ch * 8);
+      else *reinterpret_cast<uint4*>(to) = make_uint4(0, 0, 0, 0);
     }
+    tc::cp_async_commit();
+    tc::cp_async_wait<0>();
+    const int elem = h * kDH + ch * 8;
+#pragma unroll 1
+    for (int u = tid >> 4; u < kM; u += 8) {        // Eq. 8 chain of the rows that stand nowhere (a thread's own pieces)
+      if (!ctl.chain[u]) continue;
+      const int j = __ldg(cols + u0 + u);
+      uint4* cell = reinterpret_cast<uint4*>(dst + tc::sw128_offset(u, ch & 7));
+      float x[8];
+      unpack8(*cell, x);
+#pragma unroll 1
+      for (int s = 0; s < a.n_use; ++s) apply_stream8<__nv_bfloat16, BITS>(a.k.s[s], j, elem, a.d, a.group, x);
+      *cell = pack8(x);
+    }
+    tc::fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) tc::mbar_arrive(&ctl.k_ready);
     // ---- then sum the tiles: the thread of lane u owns selected column u0 + u -----------------------------------
     const int ur = warp * 32 + lane;
-    const int jpos = u0 + ur < cnt ? __ldg(cols + u0 + ur) : INT32_MAX;
+    const int jpos = u0 + ur < cnt ? __ldg(cols + u0 + ur) : -1;
     const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
     const float c2 = a.scale * kLog2e;
+    const fl_codec::f32x2 cc = fl_codec::pair(c2, c2);
     float sum = 0.f;
+    bool ok = true;
     for (int t = 0; t < n_tiles && ok; ++t) {
       const int sl = t & 1;
       if (!warp_wait(&ctl.q_full[sl], (t >> 1) & 1, abort_flag)) { ok = false; break; }
       if (!warp_wait(&ctl.d_full[sl], (t >> 1) & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
+      uint32_t r[4][32];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) tc::tmem_ld32(tmem + lane_base + sl * kM + q * 32, r[q]);
       // the active rows ascend: when the tile's first row lies at or after every column of the warp nothing is masked
-      const int pos_first = ctl.pos[sl][0];
-      const bool all_visible = __all_sync(0xffffffffu, jpos == INT32_MAX || jpos <= pos_first);
-#pragma unroll 1
-      for (int q = 0; q < 4; ++q) {
-        uint32_t r[32];
-        tc::tmem_ld32(tmem + lane_base + sl * kM + q * 32, r);
-        tc::tmem_wait_ld();
-        const float* l2 = ctl.lse2[sl] + q * 32;
-        float part = 0.f;
-        if (all_visible) {
-#pragma unroll
-          for (int u = 0; u < 32; ++u) part += tc::ex2(fmaf(__uint_as_float(r[u]), c2, -l2[u]));
-        } else {
-          const int* ps = ctl.pos[sl] + q * 32;
-#pragma unroll
-          for (int u = 0; u < 32; ++u) {
-            const float p = tc::ex2(fmaf(__uint_as_float(r[u]), c2, -l2[u]));
-            part += ps[u] >= jpos ? p : 0.f;
-          }
+      const int* ps = ctl.pos[sl];
+      const bool all_visible = __all_sync(0xffffffffu, jpos <= ps[0]);
+      int first = 0;                                // rows before `first` of the tile do not see the column
+      if (!all_visible) {
+        int hi = kM;
+        while (first < hi) {
+          const int mid = (first + hi) >> 1;
+          if (ps[mid] < jpos) first = mid + 1; else hi = mid;
         }
-        sum += part;
       }
+      tc::tmem_wait_ld();
+      const float* nl = ctl.neg_lse2[sl];
+      sum = all_visible ? colsum_tile<false, 4>(r, cc, nl, 0, sum) : colsum_tile<true, 4>(r, cc, nl, first, sum);
       tc::tc_fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&ctl.d_free[sl]);
@@ -786,17 +805,19 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
 // Next-loop column scores of a sparse loop on the tensor path; FL_ERR_UNSUPPORTED when it does not cover the request.
 int fl_launch_sparse_colsum_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const void* q_new, const int32_t* active_idx,
                                int n_active, const fl_kv_store* store, const int32_t* col_idx, const int32_t* col_cnt,
-                               int c, const float* lse, float* out, int32_t* status, cudaStream_t st) {
+                               int c, const float* lse, float* out, const FlStaleRows& stale, int32_t* status,
+                               cudaStream_t st) {
   if (s->dtype != FL_BF16 || s->head_dim != kDH || ctx->force_simt || n_active < 1) return FL_ERR_UNSUPPORTED;
   if ((size_t)ctx->max_smem_optin < kSpColsumSmem || ctx->encode_tiled == nullptr || ctx->tmaps == nullptr)
     return FL_ERR_UNSUPPORTED;
   SpArgs a{};
   const int64_t d_row = (int64_t)s->n_heads * s->head_dim;
-  if (!fl_tile_tmap(ctx, store->k_base, s->L, d_row, 1, &a.k_map) ||
-      !fl_tile_tmap(ctx, q_new, n_active, d_row, kM, &a.q_map))
-    return FL_ERR_UNSUPPORTED;
+  if (!fl_tile_tmap(ctx, q_new, n_active, d_row, kM, &a.q_map)) return FL_ERR_UNSUPPORTED;
   fl_dev_side(store, true, &a.k);
   a.n_use = loop_r - 1;
+  const fl_kv_stream& own = store->k_res[loop_r - 2];
+  a.k_rows = own.n_rows == n_active ? static_cast<const __nv_bfloat16*>(own.rows_cur) : nullptr;
+  a.k_stale = static_cast<const __nv_bfloat16*>(stale.k);
   a.active_idx = active_idx; a.n_active = n_active;
   a.col_idx = col_idx; a.col_cnt = col_cnt; a.c = c;
   a.lse = lse; a.out = out; a.status = status;

@@ -56,7 +56,14 @@ constexpr int kFlPartFloats = 2 * 128 * 128 + 4 * 128;
 constexpr int kFlMaxSplit = 256;
 
 // Bytes of workspace with which the loop-attention launch can split the problems of its last wave (0: never useful).
-size_t fl_attn_workspace_bytes(const fl_ctx* ctx, const fl_shape* s);
+size_t fl_attn_split_bytes(const fl_ctx* ctx, const fl_shape* s);   // counters and partial results (0: no split)
+// Behind them: rebuilt rows of tokens with payloads of earlier loops only, [L, d] per side.
+struct FlStaleRows {
+  const void* k;
+  const void* v;
+};
+int fl_launch_stale_rows(fl_ctx* ctx, const fl_shape* s, int loop_r, const fl_kv_store* store, int n_active,
+                         FlStaleRows* out, cudaStream_t st);
 
 // Tensor map of a row-major bf16 matrix [rows, row_elems] for TMA: box = 64 elements x box_rows rows,
 // 128-byte swizzle, out-of-range rows read as zero. box_rows = 1 is the map for row gathers (tile::gather4),

@@ -9,18 +9,20 @@ int fl_launch_sparse_colscore(const fl_ctx* ctx, const fl_shape* s, const void* 
 
 int fl_launch_sparse_colsum_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const void* q_new, const int32_t* active_idx,
                                int n_active, const fl_kv_store* store, const int32_t* col_idx, const int32_t* col_cnt,
-                               int c, const float* lse, float* out, int32_t* status, cudaStream_t st);
+                               int c, const float* lse, float* out, const FlStaleRows& stale, int32_t* status,
+                               cudaStream_t st);
 
 // next-loop column scores: tensor path when it covers the request, the binary32 kernel otherwise
 static int fl_next_col_scores(fl_ctx* ctx, const fl_shape* s, int loop_r, const void* q_new, const int32_t* active_idx,
                               int n_active, const fl_kv_store* store, const int32_t* col_idx, const int32_t* col_cnt,
-                              int c, const float* lse, float* out, int32_t* status, cudaStream_t st);
+                              int c, const float* lse, float* out, const FlStaleRows& stale, int32_t* status,
+                              cudaStream_t st);
 
 int fl_launch_loop_attn_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const void* q_new, const void* q_old,
                            const int32_t* active_idx, int n_active, const fl_kv_store* store, const int32_t* col_idx,
                            const int32_t* col_cnt, int c, const float* lse_prev, float* lse_out, const void* o_prev,
-                           void* o_out, int indexed, void* q_store, const fl_attn_carry* carry, int32_t* status,
-                           cudaStream_t st);
+                           void* o_out, int indexed, void* q_store, const fl_attn_carry* carry, const FlStaleRows& stale,
+                           int32_t* status, cudaStream_t st);
 
 // the same call as one or two single-term launches (needs the loop's materialized rows and the carried buffers)
 int fl_launch_loop_attn_stream(fl_ctx* ctx, const fl_shape* s, int loop_r, const void* q_new, const void* q_store_in,
@@ -252,14 +254,19 @@ extern "C" int fl_loop_attention(fl_ctx* ctx, const fl_shape* shape, int loop_r,
 
   DevSide kside;
   fl_dev_side(store, true, &kside);
+  FlStaleRows stale{};
   if (!ctx->force_simt) {
     // tensor path (bf16 storage, head_dim 128); anything else runs on the binary32 SIMT kernel below
+    if (fl_loop_attn_tc_covers(ctx, shape, c)) {
+      rc = fl_launch_stale_rows(ctx, shape, loop_r, store, n_active, &stale, st);
+      if (rc != FL_OK) return rc;
+    }
     rc = fl_launch_loop_attn_tc(ctx, shape, loop_r, q_new, q_old, active_idx, n_active, store, col_idx, col_cnt, c,
-                                lse_prev, lse_out, o_prev, o_out, 0, nullptr, nullptr, status, st);
+                                lse_prev, lse_out, o_prev, o_out, 0, nullptr, nullptr, stale, status, st);
     if (rc == FL_OK) {
       if (col_scores_next == nullptr) return FL_OK;
       return fl_next_col_scores(ctx, shape, loop_r, q_new, active_idx, n_active, store, col_idx, col_cnt, c, lse_out,
-                                col_scores_next, status, st);
+                                col_scores_next, stale, status, st);
     }
     if (rc != FL_ERR_UNSUPPORTED) return rc;
   }
@@ -284,7 +291,7 @@ extern "C" int fl_loop_attention(fl_ctx* ctx, const fl_shape* shape, int loop_r,
   if (rc != FL_OK || col_scores_next == nullptr) return rc;
   // column scores that prepare a pruned selection for loop r+1 (Eq. 6 with a sparse source loop)
   return fl_next_col_scores(ctx, shape, loop_r, q_new, active_idx, n_active, store, col_idx, col_cnt, c, lse_out,
-                            col_scores_next, status, st);
+                            col_scores_next, stale, status, st);
 }
 
 // Host-side checks of the position-indexed form, shared with the entry point that brings its own scratch.
@@ -350,12 +357,16 @@ extern "C" int fl_loop_attention_indexed_carry(fl_ctx* ctx, const fl_shape* shap
   if (carry != nullptr && !ctx->fused_attn && (carry->reuse != 0 || ctx->two_pass))
     rc = fl_launch_loop_attn_stream(ctx, shape, loop_r, q_new, q_store_in, q_store_out, active_idx, n_active, store,
                                     col_idx, col_cnt, c, lse_in, lse_out, o_store_in, o_store_out, carry, status, st);
-  if (rc == FL_ERR_UNSUPPORTED)
+  FlStaleRows stale{};
+  if (rc == FL_ERR_UNSUPPORTED) {
+    rc = fl_launch_stale_rows(ctx, shape, loop_r, store, n_active, &stale, st);
+    if (rc != FL_OK) return rc;
     rc = fl_launch_loop_attn_tc(ctx, shape, loop_r, q_new, q_store_in, active_idx, n_active, store, col_idx, col_cnt,
-                                c, lse_in, lse_out, o_store_in, o_store_out, 1, q_store_out, carry, status, st);
+                                c, lse_in, lse_out, o_store_in, o_store_out, 1, q_store_out, carry, stale, status, st);
+  }
   if (rc != FL_OK || col_scores_next == nullptr) return rc;
   return fl_next_col_scores(ctx, shape, loop_r, q_new, active_idx, n_active, store, col_idx, col_cnt, c, lse_out,
-                            col_scores_next, status, st);
+                            col_scores_next, stale, status, st);
 }
 
 extern "C" int fl_loop_attention_indexed(fl_ctx* ctx, const fl_shape* shape, int loop_r, const void* q_new,
@@ -371,9 +382,10 @@ extern "C" int fl_loop_attention_indexed(fl_ctx* ctx, const fl_shape* shape, int
 
 static int fl_next_col_scores(fl_ctx* ctx, const fl_shape* s, int loop_r, const void* q_new, const int32_t* active_idx,
                               int n_active, const fl_kv_store* store, const int32_t* col_idx, const int32_t* col_cnt,
-                              int c, const float* lse, float* out, int32_t* status, cudaStream_t st) {
+                              int c, const float* lse, float* out, const FlStaleRows& stale, int32_t* status,
+                              cudaStream_t st) {
   const int rc = fl_launch_sparse_colsum_tc(ctx, s, loop_r, q_new, active_idx, n_active, store, col_idx, col_cnt, c, lse,
-                                            out, status, st);
+                                            out, stale, status, st);
   if (rc != FL_ERR_UNSUPPORTED) return rc;
   DevSide kside;
   fl_dev_side(store, true, &kside);

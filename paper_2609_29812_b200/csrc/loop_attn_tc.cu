@@ -20,7 +20,8 @@
 // The second kind are the loop's active tokens: the quantization kernel of the same loop, which holds both
 // Xhat^(r-1) and Xhat^(r) of those rows in registers, leaves them as bf16 rows in a transient workspace, and the
 // old / new tiles are plain gathers from there (indexed by the token's row in the loop's stream). Without that
-// workspace, and for columns whose only payloads are from earlier loops, the patch warps rebuild the rows here.
+// workspace the patch warps rebuild the rows here. Columns whose payloads are all from earlier loops form a third kind:
+// one tile for both terms, gathered from rows rebuilt ahead of the launch (or rebuilt here like the others, as plain ones).
 //
 // Per chunk of 64 columns and per term: S (f32, 64 tensor-memory columns, two buffers: the next chunk's QK^T runs
 // under the current chunk's exponentials); P (bf16, 32 columns) is written over the first half of the S buffer it
@@ -65,7 +66,7 @@ constexpr int kSlotGathers = kSlotBytes / 512;   // 64 four-row gathers of 128-b
 constexpr int kThreads = kWarps * 32;
 constexpr int kColWarps = 14;               // warps that read the column list in the prologue (the other two search rows)
 constexpr int kMaxCols = 3072;              // column budget the shared-memory column list can hold
-constexpr int kMaxChunks = kMaxCols / kNC + 2;
+constexpr int kMaxChunks = kMaxCols / kNC + 3;
 constexpr uint32_t kAccOld = 0, kAccNew = 128, kSOld = 256, kSNew = 384;   // two S buffers of kNC columns each
 // A problem can be split over two CTAs, each taking half of the chunks: a CTA's partial result is both accumulators
 // (column-major, so that the row-owning threads write and read coalesced) and the three per-row statistics.
@@ -79,6 +80,8 @@ struct alignas(64) TcArgs {
   CUtensorMap k_map, v_map;          // row-gather maps of the K / V base ([L, d] bf16, box 64 x 1, 128B swizzle)
   CUtensorMap k_prev_map, k_cur_map;  // use_rows: row-gather maps of the loop's materialized rows ([n_active, d] bf16):
   CUtensorMap v_prev_map, v_cur_map;  // Khat / Vhat of the active tokens before and after the loop's residual
+  CUtensorMap k_stale_map, v_stale_map;   // use_stale: row-gather maps of the rows rebuilt for tokens with payloads of
+                                          // earlier loops only ([L, d] bf16, by position)
   CUtensorMap q_new_map, q_old_map;  // tile maps of the compact Q rows ([n_active, d] bf16, box 64 x 128); in the
                                      // indexed form q_old_map is a row-gather map of the Q store ([L, d], box 64 x 1)
   const __nv_bfloat16* o_prev;       // compact rows; in the indexed form the O stores [L, d] (may be the same)
@@ -93,6 +96,7 @@ struct alignas(64) TcArgs {
   DevSide k, v;
   int n_old;
   int use_rows;                      // columns active in this loop are gathered from the materialized rows
+  int use_stale;                     // columns whose payloads are all from earlier loops are gathered from the rebuilt rows
   int n_full;                        // CTAs 0 .. n_full-1 take one problem each; the rest are pairs sharing one
   int n_share;                       // > 1: that many CTAs take the row tiles of each problem in turn (no pairs then)
   int32_t* part_cnt;                 // [kMaxSplit] arrival counters of the pairs (zero between launches)
@@ -120,10 +124,11 @@ struct __align__(16) TcSmemCtl {
   uint32_t tmem_base;
   int abort_flag;
   int q_lo, q_hi, i_last;    // block's slot range in active_idx, position of its last active row
-  int n_plain, n_patch;      // columns without / with a payload in the current loop
+  int n_plain, n_patch;      // columns without / with a payload in the current loop,
+  int n_stale;               // and those with payloads of earlier loops only that are gathered from the rebuilt rows
   int merge_role;            // split problems: 0 = this CTA finished first (the other one merges), 1 = it merges,
                              // 2 = it should have merged but gave up waiting for the other's partial result
-  int warp_cnt[kWarps][2];
+  int warp_cnt[kWarps][3];
   int chunk_last[kMaxChunks];       // largest column position of the chunk, INT32_MAX if the chunk is padded
   uint32_t chunk_mask[kMaxChunks];  // OR of the stream masks of the chunk's columns (0: plain gather only)
   float mass[kM];            // ECON: row sums of stream 0
@@ -266,29 +271,34 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     const int i_last = ctl.i_last;                                   // last active row of the block
     const int span = ((cnt + kWarps - 1) / kWarps + 31) & ~31;
     const int beg = warp * span, end = min(cnt, beg + span);
-    int n0 = 0, n1 = 0;                                              // plain / patched columns in this warp's span
+    int n0 = 0, n1 = 0, n2 = 0;                                      // plain / patched / stale columns in this warp's span
 #pragma unroll 1
     for (int base = beg; base < end; base += 32) {
       const int u = base + lane;
       const bool live = u < end && raw_col[u] <= i_last;
       const bool patched = live && ((raw_mask[u] >> a.n_old) & 1u);
-      n0 += __popc(__ballot_sync(0xffffffffu, live && !patched));
+      const bool stale = live && !patched && a.use_stale && raw_mask[u] != 0;
+      n0 += __popc(__ballot_sync(0xffffffffu, live && !patched && !stale));
       n1 += __popc(__ballot_sync(0xffffffffu, patched));
+      n2 += __popc(__ballot_sync(0xffffffffu, stale));
     }
-    if (lane == 0) { ctl.warp_cnt[warp][0] = n0; ctl.warp_cnt[warp][1] = n1; }
+    if (lane == 0) { ctl.warp_cnt[warp][0] = n0; ctl.warp_cnt[warp][1] = n1; ctl.warp_cnt[warp][2] = n2; }
     __syncthreads();
-    // exclusive prefix over the warps' counts: lane w of every warp holds warp w's pair
+    // exclusive prefix over the warps' counts: lane w of every warp holds warp w's counts
     static_assert(kWarps <= 32, "one lane per warp");
     int inc0 = lane < kWarps ? ctl.warp_cnt[lane][0] : 0, inc1 = lane < kWarps ? ctl.warp_cnt[lane][1] : 0;
+    int inc2 = lane < kWarps ? ctl.warp_cnt[lane][2] : 0;
 #pragma unroll
     for (int off = 1; off < kWarps; off <<= 1) {
       const int t0 = __shfl_up_sync(0xffffffffu, inc0, off), t1 = __shfl_up_sync(0xffffffffu, inc1, off);
-      if (lane >= off) { inc0 += t0; inc1 += t1; }
+      const int t2 = __shfl_up_sync(0xffffffffu, inc2, off);
+      if (lane >= off) { inc0 += t0; inc1 += t1; inc2 += t2; }
     }
     const int tot0 = __shfl_sync(0xffffffffu, inc0, kWarps - 1), tot1 = __shfl_sync(0xffffffffu, inc1, kWarps - 1);
     const int up0 = __shfl_sync(0xffffffffu, inc0, (warp + 31) & 31), up1 = __shfl_sync(0xffffffffu, inc1, (warp + 31) & 31);
-    int before0 = warp > 0 ? up0 : 0, before1 = warp > 0 ? up1 : 0;
-    if (tid == 0) { ctl.n_plain = tot0; ctl.n_patch = tot1; }
+    const int tot2 = __shfl_sync(0xffffffffu, inc2, kWarps - 1), up2 = __shfl_sync(0xffffffffu, inc2, (warp + 31) & 31);
+    int before0 = warp > 0 ? up0 : 0, before1 = warp > 0 ? up1 : 0, before2 = warp > 0 ? up2 : 0;
+    if (tid == 0) { ctl.n_plain = tot0; ctl.n_patch = tot1; ctl.n_stale = tot2; }
     const uint32_t lt = (1u << lane) - 1;
 #pragma unroll 1
     for (int base = beg; base < end; base += 32) {
@@ -297,21 +307,25 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       const uint32_t mask = u < end ? raw_mask[u] : 0u;
       const bool live = j <= i_last;
       const bool patched = live && ((mask >> a.n_old) & 1u);
-      const uint32_t m0 = __ballot_sync(0xffffffffu, live && !patched);
+      const bool stale = live && !patched && a.use_stale && mask != 0;
+      const uint32_t m0 = __ballot_sync(0xffffffffu, live && !patched && !stale);
       const uint32_t m1 = __ballot_sync(0xffffffffu, patched);
+      const uint32_t m2 = __ballot_sync(0xffffffffu, stale);
       if (live) {
-        const int dst = patched ? tot0 + before1 + __popc(m1 & lt) : before0 + __popc(m0 & lt);
+        const int dst = patched ? tot0 + before1 + __popc(m1 & lt)
+                                : (stale ? tot0 + tot1 + before2 + __popc(m2 & lt) : before0 + __popc(m0 & lt));
         ord_col[dst] = j;
         // a column that is gathered from the materialized rows needs its row there, not its stream mask
-        ord_mask[dst] = (patched && a.use_rows) ? (uint32_t)raw_slot[u] : mask;
+        ord_mask[dst] = (patched && a.use_rows) ? (uint32_t)raw_slot[u] : (stale ? 0u : mask);
       }
       before0 += __popc(m0);
       before1 += __popc(m1);
+      before2 += __popc(m2);
     }
     __syncthreads();
   }
-  const int n_plain = ctl.n_plain, n_patch = ctl.n_patch;
-  const int n_chunks = (n_plain + kNC - 1) / kNC + (n_patch + kNC - 1) / kNC;
+  const int n_plain = ctl.n_plain, n_patch = ctl.n_patch, n_stale = ctl.n_stale;
+  const int n_chunks = (n_plain + kNC - 1) / kNC + (n_patch + kNC - 1) / kNC + (n_stale + kNC - 1) / kNC;
   // A pair splits its problem's chunks in the middle, unless the block has several row tiles or a single chunk: then
   // the first CTA of the pair does everything and the second nothing (both see the same numbers).
   const bool split = pair >= 0 && q_hi - q_lo <= kM && n_chunks >= 2;
@@ -320,7 +334,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   const int c_hi = (pair >= 0 && part == 1 && !split) ? 0 : ((split && part == 0) ? c_mid : n_chunks);
   // per chunk: the OR of its columns' stream masks and its last column (a warp per chunk, two columns per lane)
   for (int ci = warp; ci < n_chunks; ci += kWarps) {
-    const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
+    const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
     uint32_t m = 0;
     if (!(ck.patch && a.use_rows)) {   // chunks gathered from the materialized rows are never rewritten
       if (lane < ck.n_valid) m |= ord_mask[ck.off + lane];
@@ -390,7 +404,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     bool ok = true;
 #pragma unroll 1
     for (int ci = c_lo; ci < c_hi && ok; ++ci) {
-      const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
+      const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
       const int n_slots = (ck.patch && !ECON) ? 2 : 1;    // ECON: only the tiles after the loop's residual are needed
       const bool dirty = ctl.chunk_mask[ci] != 0;
       for (int k = 0; k < n_slots && ok; ++k)
@@ -413,7 +427,8 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
         }
         for (int k = 0; k < n_slots; ++k) {
           const int slot = (f + k) % kSlots;
-          const void* src = !from_rows ? map
+          const void* src = ck.stale ? (is_v ? static_cast<const void*>(&a.v_stale_map) : static_cast<const void*>(&a.k_stale_map))
+                            : !from_rows ? map
                             : ((k == 0 && !ECON) ? (is_v ? static_cast<const void*>(&a.v_prev_map) : static_cast<const void*>(&a.k_prev_map))
                                       : (is_v ? static_cast<const void*>(&a.v_cur_map) : static_cast<const void*>(&a.k_cur_map)));
           tc::tma_gather4(ring + slot * kSlotBytes + is_v * kTileBytes + slab * (kNC * 128) + grp * 512, src,
@@ -498,7 +513,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
         const int gc = gbase + n;
         int qk_slot = 0, qk_slot1 = -1;
         if (n < n_mine) {
-          const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
+          const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
           if (ECON) f = fill0 + (ci - c_lo);    // one slot per chunk, filled in chunk order
           const bool two = ck.patch && !ECON;
           const int slot0 = f % kSlots, slot1 = (f + 1) % kSlots;
@@ -580,7 +595,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       int vis = kNC;
       if (!unmasked) {
         // the chunk's columns ascend: the visible ones are a prefix, found by bisection; the rest read as -inf
-        const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
+        const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
         const int32_t* cp = ord_col + ck.off;
         int lo = 0, hi = row_ok ? ck.n_valid : 0;
         while (lo < hi) {
@@ -886,7 +901,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     else g += c_hi - c_lo;
     int f = fill;
     for (int ci = c_lo; ci < c_hi; ++ci) {   // replay the tile's fills (same for every role)
-      const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
+      const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
       const int n_slots = (ck.patch && !ECON) ? 2 : 1;
       if (ctl.chunk_mask[ci] != 0)
         for (int k = 0; k < n_slots; ++k) dirty_par_cta ^= 1u << ((f + k) % kSlots);
@@ -918,7 +933,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
 
 }  // namespace
 
-size_t fl_attn_workspace_bytes(const fl_ctx* ctx, const fl_shape* s) {
+size_t fl_attn_split_bytes(const fl_ctx* ctx, const fl_shape* s) {
   if (s->dtype != FL_BF16 || s->head_dim != kDH) return 0;
   const int n_items = fl_n_blocks(s) * s->n_heads;
   const int rem = n_items % ctx->sm_count;
@@ -930,7 +945,7 @@ extern "C" int fl_loop_attention_workspace_bytes(fl_ctx* ctx, const fl_shape* sh
   FL_REQUIRE(ctx != nullptr && bytes != nullptr);
   const int rc = fl_check_shape(shape);
   if (rc != FL_OK) return rc;
-  *bytes = (int64_t)fl_attn_workspace_bytes(ctx, shape);
+  *bytes = (int64_t)fl_attn_split_bytes(ctx, shape);
   return FL_OK;
 }
 
@@ -961,8 +976,8 @@ bool fl_loop_attn_tc_covers(const fl_ctx* ctx, const fl_shape* s, int c) {
 int fl_launch_loop_attn_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const void* q_new, const void* q_old,
                            const int32_t* active_idx, int n_active, const fl_kv_store* store, const int32_t* col_idx,
                            const int32_t* col_cnt, int c, const float* lse_prev, float* lse_out, const void* o_prev,
-                           void* o_out, int indexed, void* q_store, const fl_attn_carry* carry, int32_t* status,
-                           cudaStream_t st) {
+                           void* o_out, int indexed, void* q_store, const fl_attn_carry* carry, const FlStaleRows& stale,
+                           int32_t* status, cudaStream_t st) {
   if (!fl_loop_attn_tc_covers(ctx, s, c)) return FL_ERR_UNSUPPORTED;
   TcArgs a{};
   const int64_t d_row = (int64_t)s->n_heads * s->head_dim;
@@ -996,6 +1011,10 @@ int fl_launch_loop_attn_tc(fl_ctx* ctx, const fl_shape* s, int loop_r, const voi
                      !fl_tile_tmap(ctx, ks.rows_cur, n_active, d_row, 1, &a.k_cur_map) ||
                      !fl_tile_tmap(ctx, vs.rows_prev, n_active, d_row, 1, &a.v_prev_map) ||
                      !fl_tile_tmap(ctx, vs.rows_cur, n_active, d_row, 1, &a.v_cur_map)))
+    return FL_ERR_UNSUPPORTED;
+  a.use_stale = stale.k != nullptr;
+  if (a.use_stale && (!fl_tile_tmap(ctx, stale.k, s->L, d_row, 1, &a.k_stale_map) ||
+                      !fl_tile_tmap(ctx, stale.v, s->L, d_row, 1, &a.v_stale_map)))
     return FL_ERR_UNSUPPORTED;
   a.col_idx = col_idx; a.col_cnt = col_cnt; a.c = c;
   a.lse_prev = lse_prev; a.lse_out = lse_out; a.status = status;

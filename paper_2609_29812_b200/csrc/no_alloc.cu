@@ -38,7 +38,7 @@ extern "C" int fl_loop_attention_indexed_static(fl_ctx* ctx, const fl_shape* sha
   if (rc != FL_OK) return rc;
   FL_REQUIRE(ctx->device >= 0 && ctx->device < kMaxDevices);
   // the split this shape would use must fit the fixed array: no silent fall-back to something else
-  const size_t need = fl_attn_workspace_bytes(ctx, shape);
+  const size_t need = fl_attn_split_bytes(ctx, shape);
   if (need > kStaticBytes) return FL_ERR_WORKSPACE;
   fl_ctx with_scratch = *ctx;   // differs from the caller's context only in its workspace (owns nothing)
   with_scratch.ws = nullptr;

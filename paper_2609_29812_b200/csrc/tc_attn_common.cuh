@@ -128,22 +128,30 @@ __device__ __forceinline__ void patch_piece(const DevSide& side, int n_old, uint
   v_new = ((mask >> n_old) & 1u) ? pack8(x) : v_old;
 }
 
-// chunk ci of the partitioned column list: patched chunks first (the first two are built by the whole CTA
-// before the pipeline starts), then plain chunks. In the ordered list the plain columns come first.
+// chunk ci of the partitioned column list: patched chunks first, then stale ones, then plain ones. In the ordered list
+// the plain columns come first, then the patched, then the stale ones.
 struct ChunkInfo {
   int off;      // offset into the ordered column list
   int n_valid;  // valid columns (<= kNC)
   bool patch;   // columns carry a payload in the current loop: separate old / new operand tiles (two slots)
+  bool stale;   // columns with payloads of earlier loops only, in rows rebuilt ahead of the launch
 };
-__device__ __forceinline__ ChunkInfo chunk_info(int ci, int n_plain, int n_patch) {
-  const int n_patch_chunks = (n_patch + kNC - 1) / kNC;
+__device__ __forceinline__ ChunkInfo chunk_info(int ci, int n_plain, int n_patch, int n_stale = 0) {
+  const int n_patch_chunks = (n_patch + kNC - 1) / kNC, n_stale_chunks = (n_stale + kNC - 1) / kNC;
   ChunkInfo c;
+  c.stale = false;
   if (ci < n_patch_chunks) {
     c.off = n_plain + ci * kNC;
     c.n_valid = min(kNC, n_patch - ci * kNC);
     c.patch = true;
-  } else {
+  } else if (ci < n_patch_chunks + n_stale_chunks) {
     const int k = ci - n_patch_chunks;
+    c.off = n_plain + n_patch + k * kNC;
+    c.n_valid = min(kNC, n_stale - k * kNC);
+    c.patch = false;
+    c.stale = true;
+  } else {
+    const int k = ci - n_patch_chunks - n_stale_chunks;
     c.off = k * kNC;
     c.n_valid = min(kNC, n_plain - c.off);
     c.patch = false;

@@ -87,13 +87,15 @@ def status_word(dev):
 
 def lend_workspace(ctx, shape, dev) -> int:
     """Hands the context the workspace with which the attention launch splits the problems of its last, partly empty
-    wave over two CTAs each (a scheduling aid; 0 bytes when the shape cannot profit).  The tensor stays referenced
-    by the Context object.  Returns the bytes lent."""
+    wave over two CTAs each (a scheduling aid; 0 bytes when the shape cannot profit), with room behind it for the rows
+    that a launch with shrunken token sets rebuilds once.  The tensor stays referenced by the Context object.  Returns
+    the bytes of the split's part."""
     need = B.fl_loop_attention_workspace_bytes(ctx, shape)
-    if need > 0:
+    full = B.fl_loop_attention_full_workspace_bytes(ctx, shape)
+    if full > 0:
         ws = getattr(ctx, "_workspace", None)
-        if ws is None or ws.numel() < need:
-            ws = torch.empty(need, dtype=torch.uint8, device=dev)
+        if ws is None or ws.numel() < full:
+            ws = torch.empty(full, dtype=torch.uint8, device=dev)
         # a context that holds this workspace already keeps it: every launch leaves its counters cleared
         if getattr(ctx, "_lent", None) != (ws.data_ptr(), ws.numel()):
             B.fl_set_workspace(ctx, ws, ws.numel())

@@ -1,0 +1,47 @@
+"""Shrinking token sets: rows of tokens whose payloads are all from earlier loops, rebuilt once per launch when the workspace
+has room for them.  Every code width, few and many heads, against the oracle and against the chain
+inside the kernels (a context without a workspace)."""
+import pytest
+
+from paper_2609_29812_b200 import workloads
+from helpers import assert_attn_close, to_dev, to_np
+from test_gpu_economy import run_oracle
+from test_gpu_parity import oracle_selection, small_bf16
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("bits,group,H,L,loops", [(4, 128, 2, 700, 4), (2, 32, 4, 1201, 3), (8, 64, 2, 903, 4), (16, 128, 2, 700, 3),
+                                                  (4, 32, 2, 803, 7)])
+def test_rows_of_dropped_tokens(bits, group, H, L, loops):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_29812_b200 import binding as B, pipeline as P
+    w = workloads.replace(workloads.config2(L=L, n_heads=H), n_loops=loops, q_block=256, col_budget=96, bits=bits, group=group,
+                          changed_fracs=tuple(0.5 * 0.6 ** i for i in range(loops - 1)))
+    x = workloads.make_layer_inputs(w, seed=L)
+    k_tok = [max(8, int(L * 0.4 * 0.6 ** i)) for i in range(loops - 1)]
+    ref = run_oracle(w, x, k_tok=k_tok)
+    scores = {}
+    for lent in (True, False):
+        ctx = B.Context(0)
+        st = P.LayerState(ctx, w, split=lent)
+        assert not lent or B.fl_loop_attention_full_workspace_bytes(ctx, st.shape) >= 4 * L * w.d
+        st.dense_loop(to_dev(x.Q[0], w), to_dev(x.K[0], w), to_dev(x.V[0], w))
+        st.select_columns_dense()
+        for r in range(2, loops + 1):
+            rec, act = ref["loops"][r - 2], ref["active"][r - 2]
+            sel = oracle_selection(P, w, ref, r)
+            st.alloc_stream(sel)
+            st.quantize(r, to_dev(x.K[r - 1][act], w), to_dev(x.V[r - 1][act], w), sel)
+            csn = torch.zeros(H, st.nb, st.c, device="cuda")
+            B.fl_loop_attention_indexed(ctx, st.shape, r, to_dev(x.Q[r - 1][act], w), st.q_store, st.q_store, sel.active_idx, sel.n,
+                                        st.store, st.col_idx, st.col_cnt, st.c, st.lse, st.lse, st.o_store, st.o_store, csn,
+                                        status=st.status)
+            st.check_status()
+            assert_attn_close(to_np(st.o_store)[act], rec["O_rows"], f"loop {r} lent {lent}", carried=r - 1)
+            scores[r, lent] = csn
+        ctx.close()
+    for r in range(2, loops + 1):
+        torch.testing.assert_close(scores[r, True], scores[r, False], rtol=2e-2, atol=1e-4)
