@@ -88,7 +88,8 @@ struct __align__(16) StSmemCtl {
   int q_lo, q_hi, i_last;
   int n_plain, n_patch;
   int warp_cnt[kWarps][2];
-  int chunk_last[kMaxChunks];        // largest column position of the chunk, INT32_MAX if the chunk is padded
+  int chunk_last[kMaxChunks];        // largest entry of the chunk, INT32_MAX if the chunk is padded
+  int pos[kM];                       // positions of the tile's rows
   uint32_t stale[kMaxCols / 32];     // bit u: ordered column u carries a payload from an earlier loop only
 };
 
@@ -104,7 +105,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   uint8_t* k_ring = smem + kQTileBytes;                 // two K tiles
   uint8_t* v_ring = k_ring + 2 * kTileBytes;            // two V tiles
   StSmemCtl& ctl = *reinterpret_cast<StSmemCtl*>(v_ring + 2 * kTileBytes);
-  int32_t* ord_col = reinterpret_cast<int32_t*>(&ctl + 1);   // [kMaxCols] column positions: plain ones, then patched ones
+  // [kMaxCols]: positions of the plain columns, then the patched columns' rows in the loop's own stream (both ascend)
+  int32_t* ord_col = reinterpret_cast<int32_t*>(&ctl + 1);
 
   fl_grid_wait();      // nothing below runs ahead of the previous kernel of the stream
   fl_grid_release();
@@ -138,7 +140,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   for (int i = tid; i < kMaxCols / 32; i += kThreads) ctl.stale[i] = 0u;
   // ---- prologue: the raw column list, a flag per column and the rows of the block ------------------------------
   int32_t* raw_col = reinterpret_cast<int32_t*>(k_ring);                   // [kMaxCols], staged in the idle rings
-  uint32_t* raw_flag = reinterpret_cast<uint32_t*>(raw_col + kMaxCols);    // bit 0: payload in this loop, bit 1: in an earlier one
+  uint32_t* raw_flag = reinterpret_cast<uint32_t*>(raw_col + kMaxCols);
   const int c_cap = min(a.c, kMaxCols);
   if (warp >= kColWarps) {
     const int target = warp == kColWarps ? b * a.q_block : min(a.L, (b + 1) * a.q_block);
@@ -151,11 +153,11 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   } else {
     // the whole row of the column table is read without waiting for its count (entries past the count are -1); the
     // thread that read a column looks it up in the slot map of every residual stream
-    constexpr int kBatch = 3, kStride = kColWarps * 32;
+    constexpr int kBatch = 5, kStride = kColWarps * 32;
 #pragma unroll 1
     for (int u0 = tid; u0 < c_cap; u0 += kBatch * kStride) {
       int j[kBatch];
-      uint32_t flag[kBatch];
+      uint32_t flag[kBatch];               // bit 0: payload in an earlier loop, above: 1 + row in this loop's stream
 #pragma unroll
       for (int k = 0; k < kBatch; ++k) {
         j[k] = u0 + k * kStride < c_cap ? __ldg(cols + u0 + k * kStride) : -1;
@@ -173,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
         for (int k = 0; k < kBatch; ++k)
 #pragma unroll
           for (int q = 0; q < 4; ++q)
-            if (sl[k][q] >= 0) flag[k] |= (sg + q == a.n_old) ? 1u : 2u;
+            if (sl[k][q] >= 0) flag[k] |= (sg + q == a.n_old) ? (uint32_t)(sl[k][q] + 1) << 1 : 1u;
       }
 #pragma unroll
       for (int k = 0; k < kBatch; ++k)
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     for (int base = beg; base < end; base += 32) {
       const int u = base + lane;
       const bool live = u < end && raw_col[u] <= i_last;
-      const bool patched = live && (raw_flag[u] & 1u);
+      const bool patched = live && raw_flag[u] > 1u;
       n0 += __popc(__ballot_sync(0xffffffffu, live && !patched));
       n1 += __popc(__ballot_sync(0xffffffffu, patched));
     }
@@ -219,7 +221,14 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     const int tot0 = __shfl_sync(0xffffffffu, inc0, kWarps - 1), tot1 = __shfl_sync(0xffffffffu, inc1, kWarps - 1);
     const int up0 = __shfl_sync(0xffffffffu, inc0, (warp + 31) & 31), up1 = __shfl_sync(0xffffffffu, inc1, (warp + 31) & 31);
     int before0 = warp > 0 ? up0 : 0, before1 = warp > 0 ? up1 : 0;
-    if (tid == 0) { ctl.n_plain = tot0; ctl.n_patch = tot1; }
+    if (tid == 0) {
+      ctl.n_plain = tot0;
+      ctl.n_patch = tot1;
+      // the last chunk of each kind is padded unless it is full
+      const int n_patch_chunks = (tot1 + kNC - 1) / kNC;
+      if (tot1 % kNC) ctl.chunk_last[n_patch_chunks - 1] = INT32_MAX;
+      if (tot0 % kNC) ctl.chunk_last[n_patch_chunks + tot0 / kNC] = INT32_MAX;
+    }
     const uint32_t lt = (1u << lane) - 1;
 #pragma unroll 1
     for (int base = beg; base < end; base += 32) {
@@ -227,13 +236,15 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       const int j = u < end ? raw_col[u] : INT32_MAX;
       const uint32_t flag = u < end ? raw_flag[u] : 0u;
       const bool live = j <= i_last;
-      const bool patched = live && (flag & 1u);
+      const bool patched = live && flag > 1u;
       const uint32_t m0 = __ballot_sync(0xffffffffu, live && !patched);
       const uint32_t m1 = __ballot_sync(0xffffffffu, patched);
       if (live) {
         const int dst = patched ? tot0 + before1 + __popc(m1 & lt) : before0 + __popc(m0 & lt);
-        ord_col[dst] = j;
-        if (!patched && (flag & 2u)) atomicOr(&ctl.stale[dst >> 5], 1u << (dst & 31));
+        const int entry = patched ? (int)(flag >> 1) - 1 : j, nth = patched ? dst - tot0 : dst;
+        ord_col[dst] = entry;
+        if (nth % kNC == kNC - 1) ctl.chunk_last[nth / kNC + (patched ? 0 : (tot1 + kNC - 1) / kNC)] = entry;
+        if (!patched && (flag & 1u)) atomicOr(&ctl.stale[dst >> 5], 1u << (dst & 31));
       }
       before0 += __popc(m0);
       before1 += __popc(m1);
@@ -242,11 +253,6 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   }
   const int n_plain = ctl.n_plain, n_patch = ctl.n_patch;
   const int n_chunks = (n_plain + kNC - 1) / kNC + (n_patch + kNC - 1) / kNC;
-  for (int ci = tid; ci < n_chunks; ci += kThreads) {
-    const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
-    ctl.chunk_last[ci] = ck.n_valid == kNC ? ord_col[ck.off + kNC - 1] : INT32_MAX;
-  }
-  __syncthreads();
   // plain chunks start at multiples of 64 in the ordered list: two words of the stale bit map per chunk
   auto chunk_dirty = [&](const ChunkInfo& ck) -> bool {
     return !ck.patch && (ctl.stale[ck.off >> 5] | ctl.stale[(ck.off >> 5) + 1]) != 0u;
@@ -311,8 +317,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
           const int u = grp * 4 + i;
           // a row past the end of the tensor reads as zero. Columns that are active in this loop come from the
           // materialized rows, indexed by their row in the loop's stream
-          if (ck.patch) y[i] = u < ck.n_valid ? __ldg(a.k.s[a.n_old].slot + ord_col[ck.off + u]) : a.n_active;
-          else y[i] = u < ck.n_valid ? ord_col[ck.off + u] : a.L;
+          y[i] = u < ck.n_valid ? ord_col[ck.off + u] : (ck.patch ? a.n_active : a.L);
         }
         const void* src = ck.patch ? (is_v ? static_cast<const void*>(&a.v_rows_map) : static_cast<const void*>(&a.k_rows_map))
                                    : (is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map));
@@ -436,11 +441,27 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     const int pos = row_ok ? __ldg(a.active_idx + s0 + row) : -1;
     const float c2 = a.scale * kLog2e;
     const float lse2 = ((row_ok && MODE == kOldPass) ? a.lse_prev[(size_t)h * a.L + pos] : 0.f) * kLog2e;
+    const float mass = (row_ok && MODE == kNewPass) ? a.mass[(size_t)h * a.L + pos] : 0.f;
     // the epilogue reads the row's previous output (NEW pass: its background): have it in L2 by then
     if (row_ok) {
       tc::prefetch_l2(a.rows_in + (size_t)pos * a.d + h * kDH);
       tc::prefetch_l2(a.rows_in + (size_t)pos * a.d + h * kDH + 64);
     }
+    ctl.pos[row] = pos;
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    const size_t col0 = (size_t)h * kDH;
+    uint8_t* stage = q_tile;                     // [128 rows][16 x 16 B], 16-byte cells XOR-swizzled by row
+    // The rows that come in (previous outputs / backgrounds) are staged in the Q tile with coalesced asynchronous copies.
+    // Every QK^T has read it once the last chunk's S is there: the copies run under that chunk's exponentials.
+    auto stage_rows = [&]() {
+#pragma unroll 4
+      for (int k = 0; k < 16; ++k) {
+        const int rr = k * 8 + (tid >> 4), cc = tid & 15;
+        if (rr < n_rows)
+          tc::cp_async16(stage + rr * 256 + ((cc ^ (rr & 7)) << 4), a.rows_in + (size_t)ctl.pos[rr] * a.d + col0 + cc * 8);
+      }
+      tc::cp_async_commit();
+    };
     const uint32_t s_addr = tmem + lane_base + kS;
     float ell = 0.f, ref = -INFINITY;    // OLD pass: ell is the mass, ref stays unused
     bool ok = true;
@@ -448,18 +469,21 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       const int gc = g0 + ci, pb = gc & 1, n_use = gc >> 1;
       if (!warp_wait(&ctl.s_full[pb], n_use & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
+      if (ci == n_chunks - 1) stage_rows();
       // rows of a warp that lie at or after every column of the chunk need no causal mask; rows beyond the
-      // tile's last (their results are never stored) must not force the masked path
-      const bool unmasked = __all_sync(0xffffffffu, !row_ok || ctl.chunk_last[ci] <= pos);
+      // tile's last (their results are never stored) must not force the masked path. Entries that are rows of the loop's
+      // stream compare with the row's own index there (both ascend with the position).
+      const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
+      const int key = ck.patch ? s0 + row : pos;
+      const bool unmasked = __all_sync(0xffffffffu, !row_ok || ctl.chunk_last[ci] <= key);
       int vis = kNC;
       if (!unmasked) {
         // the chunk's columns ascend: the visible ones are a prefix, found by bisection; the rest read as -inf
-        const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
         const int32_t* cp = ord_col + ck.off;
         int lo = 0, hi = row_ok ? ck.n_valid : 0;
         while (lo < hi) {
           const int mid = (lo + hi) >> 1;
-          if (cp[mid] <= pos) lo = mid + 1; else hi = mid;
+          if (cp[mid] <= key) lo = mid + 1; else hi = mid;
         }
         vis = lo;
       }
@@ -532,24 +556,13 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       if (lane == 0) tc::mbar_arrive(&ctl.p_full[pb]);
     }
     // ---- epilogue ------------------------------------------------------------------------------------
-    // The rows that come in (previous outputs / backgrounds) are staged in the Q tile (every QK^T has retired once
-    // the last S arrived) with coalesced asynchronous copies, combined in place by the row-owning threads, and
-    // written out coalesced again.
-    uint8_t* stage = q_tile;                     // [128 rows][16 x 16 B], 16-byte cells XOR-swizzled by row
-    const size_t col0 = (size_t)h * kDH;
+    // The staged rows are combined in place by the row-owning threads and written out coalesced again.
     // a tile without a single chunk: nobody has waited for the Q tile, which is still on its way into this memory
-    if (ok && n_chunks == 0) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
-    asm volatile("bar.sync 1, 128;" ::: "memory");    // every softmax warp is past its last S: no QK^T reads Q any more
-#pragma unroll 1
-    for (int k = 0; k < 16; ++k) {
-      const int idx = k * 128 + tid, rr = idx >> 4, cc = idx & 15;
-      if (rr < n_rows) {
-        const size_t src_row = (size_t)__ldg(a.active_idx + s0 + rr);
-        tc::cp_async16(stage + rr * 256 + ((cc ^ (rr & 7)) << 4), a.rows_in + src_row * a.d + col0 + cc * 8);
-      }
+    if (n_chunks == 0) {
+      if (ok) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
+      if (ok) stage_rows();
     }
-    tc::cp_async_commit();
-    float m_i = MODE == kNewPass ? (row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f) : ell;
+    const float m_i = MODE == kNewPass ? mass : ell;
     if (ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
     tc::tc_fence_after();
     tc::cp_async_wait<0>();
@@ -565,19 +578,24 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       w = -1.f;
     }
 #pragma unroll 1
-    for (int c16 = 0; c16 < 16; ++c16) {   // 8 head-dim columns = one 16-byte cell of the staged row at a time
-      uint32_t av[8];
-      if (valid) {
-        tc::tmem_ld8(tmem + lane_base + kAcc + c16 * 8, av);
-        tc::tmem_wait_ld();
-      }
-      if (has) {
-        uint4* cell = reinterpret_cast<uint4*>(stage + row * 256 + ((c16 ^ (row & 7)) << 4));
-        float pv[8];
-        unpack8(*cell, pv);
+    for (int c0 = 0; c0 < kDH && valid; c0 += 32) {   // four 16-byte cells of the staged row at a time
+      uint32_t av[32];
+      tc::tmem_ld32(tmem + lane_base + kAcc + c0, av);
+      uint4* cell[4];
+      float pv[4][8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) pv[i] = pv[i] + w * __uint_as_float(av[i]);
-        *cell = pack8(pv);
+      for (int q = 0; q < 4; ++q) {
+        cell[q] = reinterpret_cast<uint4*>(stage + row * 256 + (((c0 / 8 + q) ^ (row & 7)) << 4));
+        unpack8(*cell[q], pv[q]);
+      }
+      tc::tmem_wait_ld();
+      if (has) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) pv[q][i] = pv[q][i] + w * __uint_as_float(av[q * 8 + i]);
+          *cell[q] = pack8(pv[q]);
+        }
       }
     }
     if (row_ok) {
@@ -589,14 +607,12 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       }
     }
     asm volatile("bar.sync 1, 128;" ::: "memory");
-#pragma unroll 1
+#pragma unroll 4
     for (int k = 0; k < 16; ++k) {
-      const int idx = k * 128 + tid, rr = idx >> 4, cc = idx & 15;
-      if (rr < n_rows) {
-        const size_t dst_row = (size_t)__ldg(a.active_idx + s0 + rr);
-        *reinterpret_cast<uint4*>(a.rows_out + dst_row * a.d + col0 + cc * 8) =
+      const int rr = k * 8 + (tid >> 4), cc = tid & 15;
+      if (rr < n_rows)
+        *reinterpret_cast<uint4*>(a.rows_out + (size_t)ctl.pos[rr] * a.d + col0 + cc * 8) =
             *reinterpret_cast<const uint4*>(stage + rr * 256 + ((cc ^ (rr & 7)) << 4));
-      }
     }
   }
   // every role is done with this tile: accumulator, Q tile and the ring bookkeeping move on together
