@@ -131,6 +131,7 @@ struct __align__(16) TcSmemCtl {
   int warp_cnt[kWarps][3];
   int chunk_last[kMaxChunks];       // largest column position of the chunk, INT32_MAX if the chunk is padded
   uint32_t chunk_mask[kMaxChunks];  // OR of the stream masks of the chunk's columns (0: plain gather only)
+  int pos[2][kM];            // positions of the tile's rows, one copy per softmax group
   float mass[kM];            // ECON: row sums of stream 0
   float ell[kM];
   float ref[kM];
@@ -188,7 +189,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       tc::mbar_init(&ctl.patched[s], kTmaWarps);
       tc::mbar_init(&ctl.done[s], ECON ? 1 : 2);   // ECON: a slot is read by one stream only
     }
-    tc::mbar_init(&ctl.q_full, 1);
+    tc::mbar_init(&ctl.q_full, (INDEXED && !ECON) ? 1 + kSoftmaxWarps : 1);
     for (int t = 0; t < 2; ++t) {
       for (int pb = 0; pb < 2; ++pb) {
         tc::mbar_init(&ctl.s_full[t][pb], 1);
@@ -217,9 +218,9 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     }
   } else {
     // The whole row of the column table is read without waiting for its count (entries past the count are -1),
-    // and the thread that read a column goes on to look it up in the slot map of every residual stream: three
+    // and the thread that read a column goes on to look it up in the slot map of every residual stream: five
     // columns per thread and up to four streams at a time are in flight, two dependent rounds in all.
-    constexpr int kBatch = 3, kStride = kColWarps * 32;
+    constexpr int kBatch = 5, kStride = kColWarps * 32;
 #pragma unroll 1
     for (int u0 = tid; u0 < c_cap; u0 += kBatch * kStride) {
       int j[kBatch], sl_new[kBatch];
@@ -360,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     // Q tiles of this row tile: two 64-element slabs each; rows past the compact list read as zero, rows of the
     // next block (past n_rows) are computed and dropped
     if (lane == 0) {
-      tc::mbar_arrive_expect_tx(&ctl.q_full, ECON ? kQTileBytes : 2 * kQTileBytes);
+      tc::mbar_arrive_expect_tx(&ctl.q_full, (ECON || INDEXED) ? kQTileBytes : 2 * kQTileBytes);
       tc::tma_tile2d(q_new_tile, &a.q_new_map, &ctl.q_full, h * kDH, s0);
       tc::tma_tile2d(q_new_tile + kM * 128, &a.q_new_map, &ctl.q_full, h * kDH + 64, s0);
       if (!INDEXED && !ECON) {
@@ -368,18 +369,25 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
         tc::tma_tile2d(q_old_tile + kM * 128, &a.q_old_map, &ctl.q_full, h * kDH + 64, s0);
       }
     }
-    if (INDEXED && !ECON) {
-      // the previous loop's Q rows come from the store: four-row gathers by position, one group of rows per lane
-      __syncwarp();
+  }
+  if (INDEXED && !ECON && warp < kSoftmaxWarps) {
+    // the previous loop's Q rows come from the store: four-row gathers by position, eight of the 64 per softmax warp,
+    // which has nothing else to do yet (from one warp they took 9 k of a problem's 66 k cycles at 1024 columns: a warp's
+    // requests are taken one after the other, ~130 cycles each, and its share of the first K and V tiles came after them)
+    if (lane == 0) tc::mbar_arrive_expect_tx(&ctl.q_full, 8 * 512);
+    __syncwarp();
+    if (lane < 8) {
+      const int grp4 = warp * 4 + (lane & 3), slab = lane >> 2;
       int y[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = lane * 4 + i;
+        const int r = grp4 * 4 + i;
         y[i] = r < n_rows ? __ldg(a.active_idx + s0 + r) : a.L;   // row L is outside the tensor: reads as zero
       }
-      tc::tma_gather4(q_old_tile + lane * 512, &a.q_old_map, &ctl.q_full, h * kDH, y[0], y[1], y[2], y[3]);
-      tc::tma_gather4(q_old_tile + kM * 128 + lane * 512, &a.q_old_map, &ctl.q_full, h * kDH + 64, y[0], y[1], y[2], y[3]);
+      tc::tma_gather4(q_old_tile + slab * (kM * 128) + grp4 * 512, &a.q_old_map, &ctl.q_full, h * kDH + slab * 64, y[0],
+                      y[1], y[2], y[3]);
     }
+    __syncwarp();
   }
 
   if (warp >= kTmaWarp) {
@@ -580,6 +588,30 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     const __nv_bfloat16* prev_rows = ECON ? a.bg_in : a.o_prev;
     if (row_ok)
       tc::prefetch_l2(prev_rows + (INDEXED ? (size_t)pos : (size_t)(s0 + row)) * a.d + h * kDH + grp * 64);
+    ctl.pos[grp][row] = pos;
+    asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
+    const int* row_pos = ctl.pos[grp];
+    // Each group finishes 64 of the 128 head-dim columns. Its half of the O_prev tile (ECON: of the background rows) is
+    // staged in shared memory with coalesced asynchronous copies, which run under the group's last chunk: the staging area
+    // is the first half of the group's own Q tile (the QK^T MMAs of the group's term have all retired once its last S
+    // arrived); the second half takes the background rows a recomputing launch leaves for later loops. In ECON both streams
+    // read the new Q tile until the very end and the old one is never loaded: the groups stage in its two halves.
+    uint8_t* stage = ECON ? q_old_tile + grp * (kM * 128)    // [128 rows][8 x 16 B], 16-byte chunks XOR-swizzled by row
+                          : (grp ? q_new_tile : q_old_tile);
+    const size_t o_col0 = (size_t)h * kDH + grp * 64;
+    bool staged = false;
+    auto stage_rows = [&]() {
+      staged = true;
+#pragma unroll 4
+      for (int k = 0; k < 8; ++k) {
+        const int rr = k * 16 + (gt >> 3), cc = gt & 7;
+        if (rr < n_rows) {
+          const size_t src_row = INDEXED ? (size_t)row_pos[rr] : (size_t)(s0 + rr);
+          tc::cp_async16(stage + rr * 128 + ((cc ^ (rr & 7)) << 4), prev_rows + src_row * a.d + o_col0 + cc * 8);
+        }
+      }
+      tc::cp_async_commit();
+    };
     const uint32_t s_addr = tmem + lane_base + (grp ? kSNew : kSOld);
     float mass = 0.f, ell = 0.f, ref = -INFINITY;
     bool ok = true;
@@ -589,6 +621,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       const int gc = gbase + n, pb = gc & 1, n_use = gc >> 1;
       if (!warp_wait(&ctl.s_full[grp][pb], n_use & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
+      if (ci + kStep >= c_hi) stage_rows();
       // rows of a warp that lie at or after every column of the chunk need no causal mask; rows beyond the
       // tile's last (their results are never stored) must not force the masked path
       const bool unmasked = __all_sync(0xffffffffu, !row_ok || ctl.chunk_last[ci] <= pos);
@@ -680,29 +713,13 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       if (lane == 0) tc::mbar_arrive(&ctl.p_full[grp][pb]);
     }
     // ---- epilogue ------------------------------------------------------------------------------------
-    // Each group finishes 64 of the 128 head-dim columns. Its half of the O_prev tile (ECON: of the background rows) is
-    // staged in shared memory with coalesced asynchronous copies, combined in place by the row-owning threads, and
-    // written out coalesced again. The staging area is the first half of the group's own Q tile (the QK^T MMAs of
-    // the group's term have all retired once its last S arrived); the second half takes the background rows a
-    // recomputing launch leaves for later loops. In ECON both streams read the new Q tile until the very end and the
-    // old one is never loaded: the groups stage in its two halves.
-    uint8_t* stage = ECON ? q_old_tile + grp * (kM * 128)    // [128 rows][8 x 16 B], 16-byte chunks XOR-swizzled by row
-                          : (grp ? q_new_tile : q_old_tile);
+    // The staged rows are combined in place by the row-owning threads and written out coalesced again.
     uint8_t* stage_bg = stage + kM * 128;                    // recomputing launch with bg_out only
     const bool write_bg = !ECON && INDEXED && a.bg_out != nullptr;   // CTA-uniform
-    const size_t o_col0 = (size_t)h * kDH + grp * 64;
     // a tile without a single chunk (empty column set): no issuer has waited for the Q tiles, which are still on
     // their way into the very memory the rows are staged in
     if (ok && c_hi == c_lo) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
-#pragma unroll 1
-    for (int k = 0; k < 8; ++k) {
-      const int idx = k * 128 + gt, rr = idx >> 3, cc = idx & 7;
-      if (rr < n_rows) {
-        const size_t src_row = INDEXED ? (size_t)__ldg(a.active_idx + s0 + rr) : (size_t)(s0 + rr);
-        tc::cp_async16(stage + rr * 128 + ((cc ^ (rr & 7)) << 4), prev_rows + src_row * a.d + o_col0 + cc * 8);
-      }
-    }
-    tc::cp_async_commit();
+    if (ok && !staged) stage_rows();
     if (ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
     tc::tc_fence_after();
     if (ECON) {
@@ -815,20 +832,20 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     const bool has = valid_a && ref_i > -INFINITY && (!ECON || m_i > 0.f);   // per row: T_i is not empty
     const float w = has ? m_i / l_i : 0.f;
 #pragma unroll 1
-    for (int c8 = 0; c8 < 8 && writer; ++c8) {   // 8 head-dim columns = one 16-byte cell of the staged row at a time
-      uint32_t ao[8], an[8];
-      const int col = grp * 64 + c8 * 8;
-      if (valid_a) tc::tmem_ld8(tmem + lane_base + kAccOld + col, ao);
-      if (valid_b) tc::tmem_ld8(tmem + lane_base + kAccNew + col, an);
+    for (int c0 = 0; c0 < 64 && writer; c0 += 16) {   // 16 head-dim columns = two 16-byte cells of the staged row at a time
+      uint32_t ao[16], an[16];
+      const int col = grp * 64 + c0;
+      if (valid_a) tc::tmem_ld16(tmem + lane_base + kAccOld + col, ao);
+      if (valid_b) tc::tmem_ld16(tmem + lane_base + kAccNew + col, an);
       tc::tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < 16; ++i) {
         if (!valid_a) ao[i] = 0u;
         if (!valid_b) an[i] = 0u;
       }
       if (ECON) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 16; ++i) {
           float v = __fadd_rn(__fmul_rn(__uint_as_float(ao[i]), f_a), __fmul_rn(__uint_as_float(an[i]), f_b));
           if (other != nullptr)
             v = __fadd_rn(v, __fadd_rn(__fmul_rn(other[(col + i) * kM + row], f_oa),
@@ -837,28 +854,32 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
         }
       } else if (other != nullptr) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 16; ++i) {
           ao[i] = __float_as_uint(__fadd_rn(__uint_as_float(ao[i]), other[(col + i) * kM + row]));
           an[i] = __float_as_uint(__fadd_rn(__fmul_rn(__uint_as_float(an[i]), f_b),
                                             __fmul_rn(other[(kDH + col + i) * kM + row], f_ob)));
         }
       }
-      uint4* cell = reinterpret_cast<uint4*>(stage + row * 128 + ((c8 ^ (row & 7)) << 4));
-      uint4* cell_bg = reinterpret_cast<uint4*>(stage_bg + row * 128 + ((c8 ^ (row & 7)) << 4));
-      if (has) {
-        float pv[8];
-        unpack8(*cell, pv);
-        if (!ECON) {
-          // background of the row: what stays of its previous output once the old term is taken out
 #pragma unroll
-          for (int i = 0; i < 8; ++i) pv[i] = pv[i] - __uint_as_float(ao[i]);
-          if (write_bg) *cell_bg = pack8(pv);
+      for (int q = 0; q < 2; ++q) {
+        const int off = row * 128 + (((c0 / 8 + q) ^ (row & 7)) << 4);
+        uint4* cell = reinterpret_cast<uint4*>(stage + off);
+        uint4* cell_bg = reinterpret_cast<uint4*>(stage_bg + off);
+        if (has) {
+          float pv[8];
+          unpack8(*cell, pv);
+          if (!ECON) {
+            // background of the row: what stays of its previous output once the old term is taken out
+#pragma unroll
+            for (int i = 0; i < 8; ++i) pv[i] = pv[i] - __uint_as_float(ao[q * 8 + i]);
+            if (write_bg) *cell_bg = pack8(pv);
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) pv[i] = pv[i] + w * __uint_as_float(an[q * 8 + i]);
+          *cell = pack8(pv);
+        } else if (write_bg) {
+          *cell_bg = *cell;                                   // empty T_i: the row itself is its background
         }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) pv[i] = pv[i] + w * __uint_as_float(an[i]);
-        *cell = pack8(pv);
-      } else if (write_bg) {
-        *cell_bg = *cell;                                   // empty T_i: the row itself is its background
       }
     }
     if (grp == 1 && row_ok && writer) {
@@ -868,16 +889,16 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     }
     if (write_bg && grp == 0 && row_ok && writer) a.mass[(size_t)h * a.L + pos] = has ? m_i : 0.f;
     asm volatile("bar.sync 1, 256;" ::: "memory");
-#pragma unroll 1
-    for (int k = 0; k < 8 && writer; ++k) {
-      const int idx = k * 128 + gt, rr = idx >> 3, cc = idx & 7;
-      if (rr < n_rows) {
-        const size_t dst_row = INDEXED ? (size_t)__ldg(a.active_idx + s0 + rr) : (size_t)(s0 + rr);
-        *reinterpret_cast<uint4*>(a.o_out + dst_row * a.d + o_col0 + cc * 8) =
-            *reinterpret_cast<const uint4*>(stage + rr * 128 + ((cc ^ (rr & 7)) << 4));
-        if (write_bg)
-          *reinterpret_cast<uint4*>(a.bg_out + dst_row * a.d + o_col0 + cc * 8) =
-              *reinterpret_cast<const uint4*>(stage_bg + rr * 128 + ((cc ^ (rr & 7)) << 4));
+    if (writer) {
+#pragma unroll 4
+      for (int k = 0; k < 8; ++k) {
+        const int rr = k * 16 + (gt >> 3), cc = gt & 7;
+        if (rr < n_rows) {
+          const size_t dst = (INDEXED ? (size_t)row_pos[rr] : (size_t)(s0 + rr)) * a.d + o_col0 + cc * 8;
+          const int off = rr * 128 + ((cc ^ (rr & 7)) << 4);
+          *reinterpret_cast<uint4*>(a.o_out + dst) = *reinterpret_cast<const uint4*>(stage + off);
+          if (write_bg) *reinterpret_cast<uint4*>(a.bg_out + dst) = *reinterpret_cast<const uint4*>(stage_bg + off);
+        }
       }
     }
   }
