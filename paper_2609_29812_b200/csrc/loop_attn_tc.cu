@@ -62,7 +62,7 @@ constexpr int kTmaWarp = 10;       // first of the TMA / patch warps
 constexpr int kTmaWarps = 6;       // a warp's four-row gathers are taken one lane after the other (~100 cycles each):
                                    // the 64 gathers of a ring slot need as many warps as can be had
 constexpr int kWarps = kSoftmaxWarps + kIssueWarps + kTmaWarps;  // 16
-constexpr int kSlotGathers = kSlotBytes / 512;   // 64 four-row gathers of 128-byte rows fill a slot
+constexpr int kTileGathers = kTileBytes / 512;   // 32 four-row gathers of 128-byte rows fill a K or V tile
 constexpr int kThreads = kWarps * 32;
 constexpr int kColWarps = 14;               // warps that read the column list in the prologue (the other two search rows)
 constexpr int kMaxCols = 3072;              // column budget the shared-memory column list can hold
@@ -112,10 +112,11 @@ struct alignas(64) TcArgs {
 };
 
 struct __align__(16) TcSmemCtl {
-  uint64_t landed[kSlots];   // TMA -> everyone: the slot's gathered tiles (32 KB) have arrived
+  uint64_t k_landed[kSlots], v_landed[kSlots];   // TMA -> everyone: the slot's K / V tile (16 KB each) has arrived
   uint64_t patched[kSlots];  // patch -> QK issuers: residual-carrying columns of the slot are rewritten (dirty chunks only)
-  uint64_t done[kSlots];     // the two PV issuers -> TMA: the MMAs that read the slot have finished (a term's PV of a chunk
-                             // is issued after its softmax, hence after its QK^T of the chunk has completed)
+  // the two issuers -> TMA: the QK^T that read the slot's K tile, the PV that read its V tile have finished. Apart, because
+  // a K tile is free a whole softmax before the V tile of its chunk
+  uint64_t k_done[kSlots], v_done[kSlots];
   uint64_t q_full;           // TMA -> QK issuers: the Q tiles of the current row tile have arrived
   uint64_t s_full[2][2];     // QK issuer -> softmax (per term, per S buffer): S of the chunk is in tensor memory
   uint64_t p_full[2][2];     // softmax -> PV issuer (per term, per buffer): P of the chunk is in tensor memory
@@ -185,9 +186,11 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
 
   if (tid == 0) {
     for (int s = 0; s < kSlots; ++s) {
-      tc::mbar_init(&ctl.landed[s], kTmaWarps);
+      tc::mbar_init(&ctl.k_landed[s], kTmaWarps);
+      tc::mbar_init(&ctl.v_landed[s], kTmaWarps);
       tc::mbar_init(&ctl.patched[s], kTmaWarps);
-      tc::mbar_init(&ctl.done[s], ECON ? 1 : 2);   // ECON: a slot is read by one stream only
+      tc::mbar_init(&ctl.v_done[s], ECON ? 1 : 2);
+      tc::mbar_init(&ctl.k_done[s], ECON ? 1 : 2);   // ECON: a slot is read by one stream only
     }
     tc::mbar_init(&ctl.q_full, (INDEXED && !ECON) ? 1 + kSoftmaxWarps : 1);
     for (int t = 0; t < 2; ++t) {
@@ -392,60 +395,79 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
 
   if (warp >= kTmaWarp) {
     // ========================================== TMA + patch ==========================================
-    // In-order fills of the ring; the lookahead is whatever the four slots allow. The 64 four-row gathers
-    // of a slot (K: 2 slabs x 16 groups, V: the same) are dealt round robin to the six warps, one per lane;
-    // every warp announces its own share of the bytes on the slot's barrier. Chunks whose columns carry
-    // residual payloads are then rewritten in place by the same warps (6 columns at a time, lanes 0-15 the K
-    // row, lanes 16-31 the V row).
+    // In-order fills of the ring, the K tiles one chunk ahead of the V tiles; the lookahead is whatever the four slots
+    // allow. A step's four-row gathers (the K tiles of the next chunk, then the V tiles of this one, 32 per tile: 2 slabs x
+    // 16 groups) are dealt round robin to the six warps, one per lane; every warp announces its own share of the bytes on
+    // the tile's barrier (K and V in steps of their own, with half the lanes busy, cost 128K columns-2048 launches 14%; slots
+    // held as a whole until the chunk's PV cost launches of two-slot chunks 17%). Chunks whose columns carry residual payloads are then rewritten in place by the same warps (6
+    // columns at a time, lanes 0-15 the K row, lanes 16-31 the V row).
     const int tw = warp - kTmaWarp;
-    // gather `req` of a slot: tile (K, V), 64-element slab, group of four columns
     const int req = lane * kTmaWarps + tw;
-    const int my_reqs = (kSlotGathers - 1 - tw) / kTmaWarps + 1;      // requests of this warp (lanes 0 .. my_reqs - 1)
-    const int is_v = (req >> 5) & 1, slab = (req >> 4) & 1, grp = req & 15;
-    const void* map = is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map);
+    const int my_tile = req / kTileGathers, slab = (req >> 4) & 1, grp = req & 15;
+    auto share = [&](int t) {     // this warp's requests of the step's tile t
+      return (kTileGathers * (t + 1) - tw + kTmaWarps - 1) / kTmaWarps - (kTileGathers * t - tw + kTmaWarps - 1) / kTmaWarps;
+    };
     const int half = lane >> 4, ch = lane & 15;
     const DevSide& side = half ? a.v : a.k;
     const int elem = h * kDH + ch * 8;
     const __nv_bfloat16* base_rows = static_cast<const __nv_bfloat16*>(side.base) + elem;
     const uint32_t ch_off = (ch >> 3) * (kNC * 128);
-    int f = fill0;
-    bool ok = true;
-#pragma unroll 1
-    for (int ci = c_lo; ci < c_hi && ok; ++ci) {
-      const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
-      const int n_slots = (ck.patch && !ECON) ? 2 : 1;    // ECON: only the tiles after the loop's residual are needed
-      const bool dirty = ctl.chunk_mask[ci] != 0;
-      for (int k = 0; k < n_slots && ok; ++k)
-        if (f + k >= kSlots) ok = warp_wait(&ctl.done[(f + k) % kSlots], (((f + k) / kSlots) - 1) & 1, abort_flag);
-      if (!ok) break;
-      if (lane == 0)
-        for (int k = 0; k < n_slots; ++k) tc::mbar_arrive_expect_tx(&ctl.landed[(f + k) % kSlots], my_reqs * 512);
+    auto slots_of = [&](const ChunkInfo& ck) { return (ck.patch && !ECON) ? 2 : 1; };  // ECON: only the new tiles are needed
+    // one step: the K tiles of chunk ck (k_slots of them, 0: none) at ring position fk, the V tiles of chunk cv at fv
+    auto fill_tiles = [&](const ChunkInfo& ck, int fk, int k_slots, const ChunkInfo& cv, int fv, int v_slots) -> bool {
+      for (int k = 0; k < k_slots; ++k)
+        if (fk + k >= kSlots && !warp_wait(&ctl.k_done[(fk + k) % kSlots], ((fk + k) / kSlots - 1) & 1, abort_flag)) return false;
+      for (int k = 0; k < v_slots; ++k)
+        if (fv + k >= kSlots && !warp_wait(&ctl.v_done[(fv + k) % kSlots], ((fv + k) / kSlots - 1) & 1, abort_flag)) return false;
+      if (lane < k_slots + v_slots) {
+        const bool v = lane >= k_slots;
+        const int slot = (v ? fv + lane - k_slots : fk + lane) % kSlots;
+        tc::mbar_arrive_expect_tx(v ? &ctl.v_landed[slot] : &ctl.k_landed[slot], share(lane) * 512);
+      }
       __syncwarp();
-      // columns that are active in this loop come from the materialized rows (old tile: before the loop's
-      // residual, new tile: after it), indexed by their row in the loop's stream; all others from the base
-      const bool from_rows = ck.patch && a.use_rows;
-      if (req < kSlotGathers) {
+      if (my_tile < k_slots + v_slots) {
+        const bool is_v = my_tile >= k_slots;
+        const ChunkInfo& c = is_v ? cv : ck;
+        const int second = is_v ? my_tile - k_slots : my_tile;
+        // columns that are active in this loop come from the materialized rows (old tile: before the loop's
+        // residual, new tile: after it), indexed by their row in the loop's stream; stale ones from the rebuilt rows, all
+        // others from the base
+        const bool from_rows = c.patch && a.use_rows;
         int y[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const int u = grp * 4 + i;
           // a row past the end of the tensor reads as zero
-          if (from_rows) y[i] = u < ck.n_valid ? (int)ord_mask[ck.off + u] : a.n_active;
-          else y[i] = u < ck.n_valid ? ord_col[ck.off + u] : a.L;
+          if (from_rows) y[i] = u < c.n_valid ? (int)ord_mask[c.off + u] : a.n_active;
+          else y[i] = u < c.n_valid ? ord_col[c.off + u] : a.L;
         }
-        for (int k = 0; k < n_slots; ++k) {
-          const int slot = (f + k) % kSlots;
-          const void* src = ck.stale ? (is_v ? static_cast<const void*>(&a.v_stale_map) : static_cast<const void*>(&a.k_stale_map))
-                            : !from_rows ? map
-                            : ((k == 0 && !ECON) ? (is_v ? static_cast<const void*>(&a.v_prev_map) : static_cast<const void*>(&a.k_prev_map))
-                                      : (is_v ? static_cast<const void*>(&a.v_cur_map) : static_cast<const void*>(&a.k_cur_map)));
-          tc::tma_gather4(ring + slot * kSlotBytes + is_v * kTileBytes + slab * (kNC * 128) + grp * 512, src,
-                          &ctl.landed[slot], h * kDH + slab * 64, y[0], y[1], y[2], y[3]);
-        }
+        const void* src;
+        if (c.stale) src = is_v ? static_cast<const void*>(&a.v_stale_map) : static_cast<const void*>(&a.k_stale_map);
+        else if (!from_rows) src = is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map);
+        else if (second == 0 && !ECON) src = is_v ? static_cast<const void*>(&a.v_prev_map) : static_cast<const void*>(&a.k_prev_map);
+        else src = is_v ? static_cast<const void*>(&a.v_cur_map) : static_cast<const void*>(&a.k_cur_map);
+        const int slot = ((is_v ? fv : fk) + second) % kSlots;
+        tc::tma_gather4(ring + slot * kSlotBytes + (is_v ? kTileBytes : 0) + slab * (kNC * 128) + grp * 512, src,
+                        is_v ? &ctl.v_landed[slot] : &ctl.k_landed[slot], h * kDH + slab * 64, y[0], y[1], y[2], y[3]);
       }
+      __syncwarp();
+      return true;
+    };
+    int f = fill0;
+    bool ok = true;
+    ChunkInfo ck = chunk_info(c_lo, n_plain, n_patch, n_stale);
+    if (c_lo < c_hi) ok = fill_tiles(ck, f, slots_of(ck), ck, f, 0);
+#pragma unroll 1
+    for (int ci = c_lo; ci < c_hi && ok; ++ci) {
+      const int n_slots = slots_of(ck);
+      const bool dirty = ctl.chunk_mask[ci] != 0;
+      const ChunkInfo nx = chunk_info(ci + 1, n_plain, n_patch, n_stale);
+      ok = fill_tiles(nx, f + n_slots, ci + 1 < c_hi ? slots_of(nx) : 0, ck, f, n_slots);
+      if (!ok) break;
       if (dirty) {
         for (int k = 0; k < n_slots && ok; ++k)
-          ok = warp_wait(&ctl.landed[(f + k) % kSlots], ((f + k) / kSlots) & 1, abort_flag);
+          ok = warp_wait(&ctl.k_landed[(f + k) % kSlots], ((f + k) / kSlots) & 1, abort_flag) &&
+               warp_wait(&ctl.v_landed[(f + k) % kSlots], ((f + k) / kSlots) & 1, abort_flag);
         if (!ok) break;
         uint8_t* t_old = ring + (f % kSlots) * kSlotBytes + half * kTileBytes + ch_off;
         uint8_t* t_new = ring + ((f + 1) % kSlots) * kSlotBytes + half * kTileBytes + ch_off;
@@ -471,6 +493,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
           for (int k = 0; k < n_slots; ++k) tc::mbar_arrive(&ctl.patched[(f + k) % kSlots]);
       }
       f += n_slots;
+      ck = nx;
     }
     if (INDEXED && a.q_store != nullptr && ok && !split) {
       // The Q store rows of this (row tile, head) were read by the gathers that completed q_full and belong to
@@ -508,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       const uint32_t acc = tmem + (t ? kAccNew : kAccOld);
       int f = fill0;             // ring position of the chunk whose QK^T is issued next
       int pv_slot = 0;           // slots of the chunk whose PV is issued next (the previous QK^T's)
-      int pv_slot1 = -1;
+      int pv_slot1 = -1, pv_fill = 0;
       uint32_t dirty_par = dirty_par0;
       // the chunks this thread issues: all of them, or (ECON) every other one starting at the stream's number
       constexpr int kStep = ECON ? 2 : 1;
@@ -519,7 +542,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       for (int n = 0; n <= n_mine; ++n) {
         const int ci = first + n * kStep;
         const int gc = gbase + n;
-        int qk_slot = 0, qk_slot1 = -1;
+        int qk_slot = 0, qk_slot1 = -1, qk_fill = 0;
         if (n < n_mine) {
           const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
           if (ECON) f = fill0 + (ci - c_lo);    // one slot per chunk, filled in chunk order
@@ -529,7 +552,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
           // a term reads one slot of the chunk only (the new term of a two-slot chunk the second): it starts on it
           // without waiting for the other
           const int my_slot = (t && two) ? slot1 : slot0, my_fill = (t && two) ? f + 1 : f;
-          if (!tc::mbar_wait(&ctl.landed[my_slot], (my_fill / kSlots) & 1, abort_flag)) break;
+          if (!tc::mbar_wait(&ctl.k_landed[my_slot], (my_fill / kSlots) & 1, abort_flag)) break;
           if (ctl.chunk_mask[ci] != 0) {       // residual-carrying columns are rewritten by the patch warps
             // (ECON: the ring has an even number of slots and the streams alternate, so within a row tile a slot
             // always serves the same stream, which therefore sees every phase of the slot's barrier)
@@ -549,26 +572,31 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
           FL_QK(4, true);  FL_QK(5, true); FL_QK(6, true); FL_QK(7, true);
 #undef FL_QK
           tc::mma_commit(&ctl.s_full[t][gc & 1]);
+          tc::mma_commit(&ctl.k_done[slot0]);
+          if (two) tc::mma_commit(&ctl.k_done[slot1]);
+          qk_fill = my_fill;
           qk_slot = slot0;
           qk_slot1 = two ? slot1 : -1;
           f += two ? 2 : 1;
         }
         if (n > 0) {
           const int gp = gc - 1, pb = gp & 1;
+          if (!tc::mbar_wait(&ctl.v_landed[pv_fill % kSlots], (pv_fill / kSlots) & 1, abort_flag)) break;
           if (!tc::mbar_wait(&ctl.p_full[t][pb], (gp >> 1) & 1, abort_flag)) break;
           tc::tc_fence_after();
-          const uint32_t v_lo = v_lo0 + ((t && pv_slot1 >= 0) ? pv_slot1 : pv_slot) * (kSlotBytes >> 4);
+          const uint32_t v_lo = v_lo0 + (pv_fill % kSlots) * (kSlotBytes >> 4);
           const uint32_t p_src = s_base + pb * kNC;
           const uint32_t acc0 = n > 1 ? 1u : 0u;           // the thread's first chunk of the tile overwrites the accumulator
 #pragma unroll
           for (int kk = 0; kk < kNC / 16; ++kk)
             tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc_pv, kk > 0 ? 1u : acc0);
           tc::mma_commit(&ctl.p_free[t][pb]);
-          tc::mma_commit(&ctl.done[pv_slot]);
-          if (pv_slot1 >= 0) tc::mma_commit(&ctl.done[pv_slot1]);
+          tc::mma_commit(&ctl.v_done[pv_slot]);
+          if (pv_slot1 >= 0) tc::mma_commit(&ctl.v_done[pv_slot1]);
         }
         pv_slot = qk_slot;
         pv_slot1 = qk_slot1;
+        pv_fill = qk_fill;
       }
       tc::mma_commit(&ctl.acc_done);
     }
