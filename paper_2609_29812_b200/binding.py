@@ -171,6 +171,16 @@ def make_store(k_base, v_base, k_streams: Sequence[dict] = (), v_streams: Sequen
     return st
 
 
+def extend_store(store: FlKvStore, k_stream: dict, v_stream: dict) -> FlKvStore:
+    """A copy of `store` with one more stream per side (make_store looks at every stream again)."""
+    st = FlKvStore.from_buffer_copy(store)
+    i = st.n_streams
+    assert i < FL_MAX_LOOPS
+    st.k_res[i], st.v_res[i] = _stream_struct(k_stream), _stream_struct(v_stream)
+    st.n_streams = i + 1
+    return st
+
+
 class Context:
     """Owns an fl_ctx.  Use as a context manager or call close()."""
 

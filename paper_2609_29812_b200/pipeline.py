@@ -204,6 +204,13 @@ class LayerState:
         d = w.d
         ws = rows_workspace(self.dev, n, d) if rows and self.dt == torch.bfloat16 and n > 0 else None
 
+        # K and V in one allocation each for the codes and for scales and offsets (an allocation costs the host about as
+        # much as a view of all of them), where the pieces keep the 16-byte alignment of allocations of their own
+        m, codes, meta = max(n, 1), None, None
+        if self.bits != 16 and (m * d * self.bits // 8) % 16 == 0 and (m * (d // w.group) * 2) % 16 == 0:
+            codes = torch.empty(2, m, d * self.bits // 8, dtype=torch.uint8, device=self.dev).unbind(0)
+            meta = torch.empty(4, m, d // w.group, dtype=torch.float16, device=self.dev).unbind(0)
+
         def one(side):
             st = {"slot_of_pos": sel.slot_of_pos, "n_rows": n}
             if ws is not None:
@@ -212,7 +219,9 @@ class LayerState:
                 st["rows_cur"] = cur if whole else cur[:n]
                 if rows != "cur":    # rows="cur": a loop that reuses the carried old term reads nothing else
                     st["rows_prev"] = prev if whole else prev[:n]
-            if self.bits == 16:
+            if codes is not None:
+                st["codes"], st["scale"], st["zero"] = codes[side], meta[2 * side], meta[2 * side + 1]
+            elif self.bits == 16:
                 st.update(codes=torch.empty(max(n, 1), d, dtype=self.dt, device=self.dev), scale=None, zero=None)
             else:
                 st.update(codes=torch.empty(max(n, 1), d * self.bits // 8, dtype=torch.uint8, device=self.dev),
@@ -223,7 +232,10 @@ class LayerState:
         # quantized last, and only that loop's attention call reads it
         self.k_streams.append(one(0))
         self.v_streams.append(one(1))
-        self._rebuild_store()
+        self.store = B.extend_store(self.store, self.k_streams[-1], self.v_streams[-1]) \
+            if self.store is not None and self.store.n_streams + 1 == len(self.k_streams) else None
+        if self.store is None:
+            self._rebuild_store()
 
     def quantize(self, loop_r, k_new, v_new, sel: TokenSelection):
         B.fl_quant_kv_residual(self.ctx, self.shape, loop_r, k_new, v_new, sel.active_idx, sel.n, self.store)
