@@ -398,9 +398,10 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     // In-order fills of the ring, the K tiles one chunk ahead of the V tiles; the lookahead is whatever the four slots
     // allow. A step's four-row gathers (the K tiles of the next chunk, then the V tiles of this one, 32 per tile: 2 slabs x
     // 16 groups) are dealt round robin to the six warps, one per lane; every warp announces its own share of the bytes on
-    // the tile's barrier (K and V in steps of their own, with half the lanes busy, cost 128K columns-2048 launches 14%; slots
-    // held as a whole until the chunk's PV cost launches of two-slot chunks 17%). Chunks whose columns carry residual payloads are then rewritten in place by the same warps (6
-    // columns at a time, lanes 0-15 the K row, lanes 16-31 the V row).
+    // the tile's barrier. K and V in steps of their own, with half the lanes busy, cost launches of 2048 columns at 128K 14%;
+    // slots held as a whole until the chunk's PV cost launches of two-slot chunks 17%. Chunks whose columns carry residual
+    // payloads are then rewritten in place by the same warps (6 columns at a time, lanes 0-15 the K row, lanes 16-31 the V
+    // row).
     const int tw = warp - kTmaWarp;
     const int req = lane * kTmaWarps + tw;
     const int my_tile = req / kTileGathers, slab = (req >> 4) & 1, grp = req & 15;

@@ -51,7 +51,7 @@ def select_tokens(ctx, shape, loop_r, g_prev, g_cur, cand: Optional[torch.Tensor
     active = torch.empty(max(n, 1), dtype=torch.int32, device=dev)
     slot = torch.empty(L, dtype=torch.int32, device=dev)
     B.fl_select_tokens(ctx, shape, loop_r, g_prev, g_cur, cand, n_cand, k, scores, active, slot)
-    return TokenSelection(active[:n], slot, scores, n)
+    return TokenSelection(active if n > 0 else active[:0], slot, scores, n)
 
 
 _ROWS_WS: dict = {}
@@ -90,8 +90,11 @@ def lend_workspace(ctx, shape, dev) -> int:
     wave over two CTAs each (a scheduling aid; 0 bytes when the shape cannot profit), with room behind it for the rows
     that a launch with shrunken token sets rebuilds once.  The tensor stays referenced by the Context object.  Returns
     the bytes of the split's part."""
-    need = B.fl_loop_attention_workspace_bytes(ctx, shape)
-    full = B.fl_loop_attention_full_workspace_bytes(ctx, shape)
+    sizes = ctx.__dict__.setdefault("_workspace_sizes", {})      # two calls into the library per layer state otherwise
+    key = (shape.L, shape.n_heads, shape.head_dim, shape.dtype, shape.q_block)
+    if key not in sizes:
+        sizes[key] = (B.fl_loop_attention_workspace_bytes(ctx, shape), B.fl_loop_attention_full_workspace_bytes(ctx, shape))
+    need, full = sizes[key]
     if full > 0:
         ws = getattr(ctx, "_workspace", None)
         if ws is None or ws.numel() < full:
