@@ -15,7 +15,7 @@ namespace {
 
 constexpr int kWarps = 8;
 constexpr int kPos = 4;          // positions per CTA; its warps take the stale ones of them, K and V rows apart
-constexpr int kChunk = 32;       // elements a lane takes at a time: one group's scale and offset, 16 bytes of 4-bit codes
+constexpr int kChunk = 32;       // elements a lane takes at a time: 16 bytes of 4-bit codes
 constexpr int kBatch = 4;        // streams whose loads are in flight together
 
 struct StaleArgs {
@@ -24,7 +24,9 @@ struct StaleArgs {
   int n_old, L, d, group;
 };
 
-template <int BITS>
+// META: scales and offsets that a chunk needs per stream. One for groups of 32 and more; groups of 8 and 16 take one for
+// each of the chunk's four pieces of 8 elements (a form of its own, so that the usual groups do not pay for the reads).
+template <int BITS, int META>
 __global__ void __launch_bounds__(kWarps * 32) stale_rows_kernel(const __grid_constant__ StaleArgs a) {
   fl_grid_wait();
   fl_grid_release();
@@ -71,7 +73,7 @@ __global__ void __launch_bounds__(kWarps * 32) stale_rows_kernel(const __grid_co
 #pragma unroll 1
     for (uint32_t m = streams; m != 0;) {
       uint32_t words[kBatch][kWords];
-      __half sc[kBatch], zr[kBatch];
+      __half sc[kBatch][META], zr[kBatch][META];
       bool have[kBatch];
 #pragma unroll
       for (int q = 0; q < (BITS == 16 ? 1 : kBatch); ++q) {
@@ -93,9 +95,12 @@ __global__ void __launch_bounds__(kWarps * 32) stale_rows_kernel(const __grid_co
               }
             }
             if (BITS != 16) {
-              const size_t gi = row * (a.d >> gs) + (e0 >> gs);
-              sc[q] = __ldg(sd.s[s].scale + gi);
-              zr[q] = __ldg(sd.s[s].zero + gi);
+#pragma unroll
+              for (int i = 0; i < META; ++i) {
+                const size_t gi = row * (a.d >> gs) + ((e0 + i * 8) >> gs);
+                sc[q][i] = __ldg(sd.s[s].scale + gi);
+                zr[q][i] = __ldg(sd.s[s].zero + gi);
+              }
             }
           }
         }
@@ -111,7 +116,7 @@ __global__ void __launch_bounds__(kWarps * 32) stale_rows_kernel(const __grid_co
             else if (BITS == 8) { pl.raw.x = words[q][(2 * i) % kWords]; pl.raw.y = words[q][(2 * i + 1) % kWords]; }
             else if (BITS == 4) pl.raw.x = words[q][i % kWords];
             else pl.raw.x = (words[q][(i / 2) % kWords] >> (16 * (i & 1))) & 0xffffu;
-            if (BITS != 16) { pl.sc = sc[q]; pl.zr = zr[q]; }
+            if (BITS != 16) { pl.sc = sc[q][i % META]; pl.zr = zr[q][i % META]; }
             payload_apply<__nv_bfloat16, BITS>(pl, x[i]);
           }
         }
@@ -168,12 +173,14 @@ int fl_launch_stale_rows(fl_ctx* ctx, const fl_shape* s, int loop_r, const fl_kv
   a.out[1] = a.out[0] + bytes / 2 / sizeof(__nv_bfloat16);
   a.n_old = loop_r - 2; a.L = s->L; a.d = s->n_heads * s->head_dim; a.group = s->group;
   const dim3 grid((s->L + kPos - 1) / kPos), block(kWarps * 32);
+  const bool fine = s->group < kChunk;      // groups of 8 and 16: metadata per piece of 8 elements
+  auto kern = stale_rows_kernel<16, 1>;
   switch (s->bits) {
-    case 2: FL_CHECK_CUDA(fl_launch(ctx, stale_rows_kernel<2>, grid, block, 0, st, a)); break;
-    case 4: FL_CHECK_CUDA(fl_launch(ctx, stale_rows_kernel<4>, grid, block, 0, st, a)); break;
-    case 8: FL_CHECK_CUDA(fl_launch(ctx, stale_rows_kernel<8>, grid, block, 0, st, a)); break;
-    default: FL_CHECK_CUDA(fl_launch(ctx, stale_rows_kernel<16>, grid, block, 0, st, a)); break;
+    case 2: kern = fine ? stale_rows_kernel<2, 4> : stale_rows_kernel<2, 1>; break;
+    case 4: kern = fine ? stale_rows_kernel<4, 4> : stale_rows_kernel<4, 1>; break;
+    case 8: kern = fine ? stale_rows_kernel<8, 4> : stale_rows_kernel<8, 1>; break;
   }
+  FL_CHECK_CUDA(fl_launch(ctx, kern, grid, block, 0, st, a));
   out->k = a.out[0];
   out->v = a.out[1];
   return fl_launch_status();

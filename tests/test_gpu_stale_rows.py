@@ -1,8 +1,10 @@
 """Shrinking token sets: rows of tokens whose payloads are all from earlier loops, rebuilt once per launch when the workspace
 has room for them.  Every code width, few and many heads, against the oracle and against the chain
 inside the kernels (a context without a workspace)."""
+import numpy as np
 import pytest
 
+from oracle import flashloop_oracle as fo
 from paper_2609_29812_b200 import workloads
 from helpers import assert_attn_close, to_dev, to_np
 from test_gpu_economy import run_oracle
@@ -45,3 +47,43 @@ def test_rows_of_dropped_tokens(bits, group, H, L, loops):
         ctx.close()
     for r in range(2, loops + 1):
         torch.testing.assert_close(scores[r, True], scores[r, False], rtol=2e-2, atol=1e-4)
+
+
+@pytest.mark.parametrize("bits,group", [(2, 8), (2, 16), (2, 128), (4, 8), (4, 16), (4, 32), (8, 8), (8, 16), (8, 64), (16, 8)])
+def test_rebuilt_rows_bit_exact(bits, group):
+    """The rows behind the split's part of the workspace, on both sides of the 32 elements that a lane rebuilds at a time (one
+    scale and offset, or one per 8 elements): the binary32 chain of the oracle, rounded once to bf16."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_29812_b200 import binding as B, pipeline as P
+    rng = np.random.default_rng(bits * 256 + group)
+    L, H, dh, loops = 421, 2, 128, 4
+    w = workloads.replace(workloads.config2(L=L, n_heads=H), n_loops=loops, q_block=256, col_budget=64, bits=bits, group=group)
+    bf = fo.round_bf16
+    draw = lambda n: bf(rng.standard_normal((n, H, dh)).astype(np.float32))
+    ctx = B.Context(0)
+    st = P.LayerState(ctx, w)
+    hat = {"k": draw(L), "v": draw(L)}
+    st.dense_loop(to_dev(draw(L), w), to_dev(hat["k"], w), to_dev(hat["v"], w))
+    st.select_columns_dense()
+    order, seen = rng.permutation(L), np.zeros(L, dtype=bool)
+    for r in range(2, loops + 1):                       # nested sets: 60%, 30%, 20% of the rows
+        act = np.sort(order[: int(0.6 * L / (r - 1))])
+        new = {s: bf(hat[s][act] + 0.3 * draw(len(act))) for s in "kv"}
+        sel = P.TokenSelection(torch.from_numpy(act.astype(np.int32)).cuda(),
+                               torch.from_numpy(fo.slot_map(act, L).astype(np.int32)).cuda(), None, len(act))
+        st.alloc_stream(sel)
+        st.quantize(r, to_dev(new["k"], w), to_dev(new["v"], w), sel)
+        st.attention_indexed(r, to_dev(draw(len(act)), w), sel)
+        st.check_status()
+        for s in "kv":
+            hat[s], _ = fo.residual_update(new[s], hat[s], act, bits, group)
+        stale = np.setdiff1d(np.flatnonzero(seen), act)
+        seen[act] = True
+        if len(stale) == 0:
+            continue
+        full = B.fl_loop_attention_full_workspace_bytes(ctx, st.shape)
+        rows = to_np(ctx._workspace[full - 4 * L * w.d:full].view(torch.bfloat16).view(2, L, H, dh))
+        for i, s in enumerate("kv"):
+            assert np.array_equal(rows[i, stale], bf(hat[s][stale])), (r, s)
+    ctx.close()
