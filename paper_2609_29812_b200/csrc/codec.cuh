@@ -67,14 +67,24 @@ __device__ __forceinline__ float scale_rcp(float s) {
   return s == 0.f ? 0.f : r;
 }
 
+// The largest of three numbers, or not-a-number if one of them is none.
+__device__ __forceinline__ float max3_nan(float a, float b, float c) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // Codes of P pairs: q = round-half-even of the binary32 quotient t / scale, t = x - zero (already rounded). The quotient
 // is estimated by t * inv (inv = the reciprocal within an ulp): within 2 ulp of the correctly rounded one, 2^(BITS - 23)
 // absolute, so both round to the same integer unless the estimate lies within twice that of a half-integer; only then
 // are the true divisions made (one warp in a hundred at 4 bits). t * inv + 1.5 * 2^23 leaves the rounded integer in the low mantissa bits. No clamp:
 // t >= 0 (the offset was rounded down) and max / scale <= 2^bits - 1 (the scale was rounded up).
 // scale(i) gives the scales of pair i (asked for in the rare branch only: they need not stay in registers).
+// Returns whether the branch was taken. Only then can a quotient be no integer of that range: elements that are not
+// numbers or not finite, and groups whose offset or scale leaves fp16. The maximum keeps a not-a-number, so that these
+// always take the branch; the caller packs such quotients through clean_codes.
 template <int BITS, int P, typename Scale>
-__device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv)[P], const f32x2 (&neg_inv)[P],
+__device__ __forceinline__ bool quotients(const f32x2 (&t)[P], const f32x2 (&inv)[P], const f32x2 (&neg_inv)[P],
                                           Scale scale, f32x2 (&q)[P]) {
   const f32x2 magic = pair(12582912.f, 12582912.f), neg_magic = pair(-12582912.f, -12582912.f);
   float far = 0.f;
@@ -84,10 +94,11 @@ __device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv
     const f32x2 fr = fma2(t[i], neg_inv[i], q[i]);   // integer - estimate
     float a, b;
     split(fr, a, b);
-    far = fmaxf(far, fmaxf(fabsf(a), fabsf(b)));
+    far = max3_nan(far, fabsf(a), fabsf(b));
   }
   constexpr float kNear = 0.5f - (float)(1 << BITS) / 4194304.f;
-  if (far > kNear) {
+  const bool rare = !(far <= kNear);
+  if (rare) {
 #pragma unroll
     for (int i = 0; i < P; ++i) {
       float a, b, sa, sb;
@@ -95,6 +106,20 @@ __device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv
       split(scale(i), sa, sb);
       q[i] = pair(sa == 0.f ? 0.f : rintf(__fdiv_rn(a, sa)), sb == 0.f ? 0.f : rintf(__fdiv_rn(b, sb)));
     }
+  }
+  return rare;
+}
+// Codes that can be packed: a quotient that is not a number becomes code 0, one past the range the nearest end of it.
+// Codes are packed by adding them up, so without this one such element would spoil the codes of its three neighbours
+// (other channels, and other groups where the groups run along the positions).
+template <int BITS, int P>
+__device__ __forceinline__ void clean_codes(f32x2 (&q)[P]) {
+  constexpr float n = (float)((1 << BITS) - 1);
+#pragma unroll
+  for (int i = 0; i < P; ++i) {
+    float a, b;
+    split(q[i], a, b);
+    q[i] = pair(fminf(fmaxf(a, 0.f), n), fminf(fmaxf(b, 0.f), n));
   }
 }
 

@@ -89,3 +89,82 @@ def test_packed_base_and_masked_rebuild(env, Lq, group, bits, dtype):
             if mask is not None:
                 want[:Lq][~mask.T[:Lq]] = 9.0
             assert np.array_equal(to_np(got), want)
+
+
+SPECIALS = (np.nan, np.inf, -np.inf, 3.0e38, -3.0e38)     # the last two overflow the fp16 scale and offset
+
+
+def plant(x, at, groups_of):
+    """`x` [rows, d] with SPECIALS at `at`; the mask of the elements in a group with one that is no finite fp16 number
+    (codes 0, metadata not finite); the not-a-number element counts for nobody but itself."""
+    bad, lost = x.copy(), np.zeros(x.shape, dtype=bool)
+    for value, (i, j) in zip(SPECIALS, at):
+        bad[i, j] = value
+        if not np.isnan(value):
+            lost[groups_of(i, j)] = True
+    return bad, lost
+
+
+@pytest.mark.parametrize("H,bits,group,dtype", [(4, 4, 128, "bf16"), (4, 2, 32, "bf16"), (4, 8, 16, "bf16"), (2, 4, 8, "bf16"),
+                                                (2, 8, 64, "bf16"), (4, 4, 32, "f32"), (4, 8, 64, "f32")])
+def test_not_finite_elements_spoil_nothing_else(env, H, bits, group, dtype):
+    """Residual rows with an element that is no number, or not finite in fp16: codes, metadata and rows of every other
+    element (its neighbours in the same word) and group are those of rows without it; its own code is 0."""
+    B, P, ctx = env
+    rng = np.random.default_rng(bits)
+    L, n, dh = 64, 16, 128 if dtype == "bf16" else 64
+    w = workloads.replace(workloads.config2(L=L, n_heads=H), n_loops=2, head_dim=dh, dtype=dtype, bits=bits, group=group)
+    rnd = fo.round_bf16 if dtype == "bf16" else (lambda a: a)
+    hat = rnd(rng.standard_normal((L, H, dh)).astype(np.float32))
+    act = np.sort(rng.permutation(L)[:n])
+    new = rnd(hat[act] + rng.standard_normal((n, H, dh)).astype(np.float32)).reshape(n, H * dh)
+    at = [(2 * i, 7 + 9 * i) for i in range(len(SPECIALS))]
+    new[0, 7] = hat[act].reshape(n, -1)[0, 7]              # where the not-a-number goes: no extremum of its group
+    bad, lost = plant(new, at, lambda i, j: (i, slice(j // group * group, (j // group + 1) * group)))
+    nxt, pay = fo.residual_update(new.reshape(n, H, dh), hat, act, bits, group)
+    codes = pay["codes"].reshape(n, -1).copy()
+    codes[lost | np.isnan(bad)] = 0
+    st = P.LayerState(ctx, w, split=False)
+    st.k_base = st.v_base = to_dev(hat, w)
+    sel = P.TokenSelection(torch.from_numpy(act.astype(np.int32)).cuda(),
+                           torch.from_numpy(fo.slot_map(act, L).astype(np.int32)).cuda(), None, n)
+    st.alloc_stream(sel)
+    st.quantize(2, to_dev(bad.reshape(n, H, dh), w), to_dev(new.reshape(n, H, dh), w), sel)
+    torch.cuda.synchronize()
+    k, v, ok = st.k_streams[-1], st.v_streams[-1], ~lost.reshape(n, -1, group).any(axis=2)
+    assert np.array_equal(to_np(k["codes"]), fo.pack_codes(codes, bits))
+    assert np.array_equal(to_np(v["codes"]), pay["packed"].reshape(n, -1))
+    for m in ("scale", "zero"):
+        assert np.array_equal(to_np(k[m]).view(np.uint16)[ok], pay[m].reshape(n, -1).view(np.uint16)[ok]), m
+    if dtype == "bf16":
+        keep = ~lost & ~np.isnan(bad)
+        assert np.array_equal(to_np(k["rows_cur"])[keep], fo.round_bf16(nxt[act]).reshape(n, -1)[keep])
+
+
+@pytest.mark.parametrize("bits,group,dtype", [(4, 64, "bf16"), (2, 32, "bf16"), (8, 128, "bf16"), (4, 32, "f32")])
+def test_packed_base_with_elements_that_are_not_finite(env, bits, group, dtype):
+    """The same for the packed base, where four neighbouring key codes belong to four groups."""
+    B, P, ctx = env
+    rng = np.random.default_rng(group)
+    H, dh = (2, 128) if dtype == "bf16" else (4, 64)
+    L, tail = 300, 11
+    Lq = L - tail
+    w = workloads.replace(workloads.config2(L=L, n_heads=H), head_dim=dh, dtype=dtype, bits=bits, group=min(group, dh))
+    rnd = fo.round_bf16 if dtype == "bf16" else (lambda a: a)
+    k, v = (rnd(rng.standard_normal((L, H * dh)).astype(np.float32)) for _ in range(2))
+    at = [(3 + 40 * i, 5 + 9 * i) for i in range(len(SPECIALS))]
+    k[3, 5], v[3, 5] = k[4, 5], v[3, 6]                    # the not-a-number takes no extremum away
+    k_bad, k_lost = plant(k, at, lambda i, j: (slice(i // group * group, min(Lq, (i // group + 1) * group)), j))
+    v_bad, v_lost = plant(v, at, lambda i, j: (i, slice(j // group * group, (j // group + 1) * group)))
+    ref = fo.quantize_base(k, v, bits, group, tail, storage_round=rnd if dtype == "bf16" else None)
+    st = P.LayerState(ctx, w, split=False)
+    st.pack_base(to_dev(k_bad.reshape(L, H, dh), w), to_dev(v_bad.reshape(L, H, dh), w), group, tail)
+    kc, ks, kz, vc, vs, vz = [to_np(t) for t in st.base_tensors[:6]]
+    for got, name, bad, lost in ((kc, "k_codes", k_bad, k_lost), (vc, "v_codes", v_bad, v_lost)):
+        codes = ref[name].copy()
+        codes[lost[:Lq] | np.isnan(bad[:Lq])] = 0
+        assert np.array_equal(got, fo.pack_codes(codes, bits)), name
+    k_ok = ~np.stack([k_lost[g * group:min(Lq, (g + 1) * group)].any(axis=0) for g in range(ks.shape[0])])
+    v_ok = ~v_lost[:Lq].reshape(Lq, -1, group).any(axis=2)
+    for got, name, ok in ((ks, "k_scale", k_ok), (kz, "k_zero", k_ok), (vs, "v_scale", v_ok), (vz, "v_zero", v_ok)):
+        assert np.array_equal(got.view(np.uint16)[ok], ref[name].view(np.uint16)[ok]), name

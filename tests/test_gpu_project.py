@@ -183,3 +183,46 @@ def test_projection_with_codec_epilogue(env, bits, group, H, n_loops):
                 assert torch.equal(a_[key], b_[key]), (r, key)
         assert np.array_equal(to_np(st_ref.k_streams[-1]["rows_cur"]), rows_cur[0])
         assert np.array_equal(to_np(st_ref.v_streams[-1]["rows_prev"]), rows_prev[1])
+
+
+@pytest.mark.parametrize("bits,group", [(4, 128), (8, 64), (2, 32)])
+def test_codec_epilogue_with_a_channel_that_is_not_finite(env, bits, group):
+    """One K channel without a value (a weight that is not a number), one V channel beyond fp16: the epilogue's streams are
+    those of the unfused calls, and the K channel's code is 0 and spoils no neighbour's."""
+    from paper_2609_29812_b200 import pipeline as P
+    B, ctx = env
+    w = small_bf16(L=300, H=2, R=2, bits=bits, group=group)
+    L, d = w.L, w.d
+    rng = np.random.default_rng(bits)
+    draw = lambda *s: round_to_bf16(rng.standard_normal(s).astype(np.float32))
+    hd, wd = dev(draw(L, d), torch.bfloat16), dev(draw(3 * d, d) / 16, torch.bfloat16)
+    act = np.sort(rng.permutation(L)[:70])
+    sel = P.TokenSelection(torch.from_numpy(act.astype(np.int32)).cuda(), torch.from_numpy(fo.slot_map(act, L)).cuda(), None, 70)
+    k1, v1 = (to_dev(draw(L, w.n_heads, w.head_dim), w) for _ in range(2))
+    codes = {}
+    for name in ("finite", "fused", "unfused"):
+        if name != "finite":
+            wd[d + 6, 0], wd[2 * d + 9] = float("nan"), 1e30
+        st = P.LayerState(ctx, w)
+        st.k_base, st.v_base = k1, v1
+        st.alloc_stream(sel)
+        status = torch.zeros(1, dtype=torch.int32, device="cuda:0")
+        if name == "unfused":
+            qkv = torch.empty(70, 3 * d, dtype=torch.bfloat16, device="cuda:0")
+            B.fl_project_rows(ctx, hd, L, sel.active_idx, 70, d, wd, 3 * d, qkv, 70, None, 0, status)
+            st.quantize(2, qkv[:, d:2 * d].contiguous(), qkv[:, 2 * d:].contiguous(), sel)
+        else:
+            q_out, kv_out = (torch.empty(70, m * d, dtype=torch.bfloat16, device="cuda:0") for m in (1, 2))
+            B.fl_project_qkv_quant(ctx, st.shape, 2, hd, L, sel.active_idx, 70, wd, q_out, kv_out, st.store, status)
+        torch.cuda.synchronize()
+        assert int(status.item()) == 0
+        codes[name] = [to_np(s["codes"]) for s in (st.k_streams[0], st.v_streams[0])]
+        meta = [to_np(s[m]) for s in (st.k_streams[0], st.v_streams[0]) for m in ("scale", "zero")]
+        if name == "fused":
+            fused_meta = meta
+    assert all(np.array_equal(a, b) for a, b in zip(codes["fused"], codes["unfused"]))
+    assert all(np.array_equal(a, b, equal_nan=True) for a, b in zip(fused_meta, meta))
+    k = fo.unpack_codes(codes["fused"][0], bits)
+    assert not k[:, 6].any()
+    other = np.arange(d) >= group                          # the channel is missing from its own group's range only
+    assert np.array_equal(k[:, other], fo.unpack_codes(codes["finite"][0], bits)[:, other])
