@@ -54,6 +54,12 @@ def select_tokens(ctx, shape, loop_r, g_prev, g_cur, cand: Optional[torch.Tensor
     return TokenSelection(active if n > 0 else active[:0], slot, scores, n)
 
 
+def _device(dev) -> torch.device:
+    """`dev` with its index ("cuda" is the device that is current now): what the process's pools are keyed by."""
+    dev = torch.device(dev)
+    return dev if dev.type != "cuda" or dev.index is not None else torch.device("cuda", torch.cuda.current_device())
+
+
 _ROWS_WS: dict = {}
 
 
@@ -61,7 +67,8 @@ def rows_workspace(dev, n: int, d: int):
     """Transient bf16 buffers [n, d] for the materialized rows of one loop: ((K before, K after), (V before,
     V after)).  One set per device, grown on demand and reused by every layer and loop: a loop's rows are dead once
     its attention call has been issued on the stream."""
-    key = (str(dev), d)
+    dev = _device(dev)
+    key = (dev, d)
     ws = _ROWS_WS.get(key)
     if ws is None or ws[0][0].shape[0] < n:
         ws = tuple(tuple(torch.empty(n, d, dtype=torch.bfloat16, device=dev) for _ in range(2)) for _ in range(2))
@@ -76,7 +83,9 @@ def status_word(dev):
     """A zeroed int32 device word of its own: one of a block of 1024 that is cleared once, on the stream that will use it
     (a fill kernel per word costs more host time than the call whose errors it collects). A block lives as long as
     any word of it; words are not handed out again."""
-    key = (dev, B._stream(None))
+    dev = _device(dev)
+    here = dev.index == torch.cuda.current_device()
+    key = (dev, B._stream(None) if here else torch.cuda.current_stream(dev).cuda_stream or None)
     while True:
         block = _STATUS.get(key)
         i = next(block[1]) if block is not None else 1024
