@@ -121,20 +121,25 @@ def _ptr(x) -> Optional[int]:
     return x.data_ptr()
 
 
-_current_stream = None   # () -> raw handle of torch's current stream
+_raw_stream = _current_device = None   # index -> raw handle of torch's current stream there; () -> current device
+
+
+def _stream_of(index: Optional[int]) -> Optional[int]:
+    """Raw handle of torch's current stream on a device (None: the current one)."""
+    global _raw_stream, _current_device
+    if _raw_stream is None:
+        import torch
+        torch.cuda.current_stream()       # initialises CUDA
+        raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        # the stream object of the public call costs 3 us, as much as a kernel launch; the handle alone 0.2 us
+        _current_device = dev if dev is not None else torch.cuda.current_device
+        _raw_stream = raw if raw is not None else (lambda i: int(torch.cuda.current_stream(i).cuda_stream))
+    return _raw_stream(_current_device() if index is None else index) or None
 
 
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        global _current_stream
-        if _current_stream is None:
-            import torch
-            torch.cuda.current_stream()       # initialises CUDA
-            raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
-            # the stream object of the public call costs 3 us, as much as a kernel launch; the handle alone 0.2 us
-            _current_stream = ((lambda: raw(dev())) if raw is not None and dev is not None
-                               else (lambda: int(torch.cuda.current_stream().cuda_stream)))
-        return _current_stream() or None
+        return _stream_of(None)
     if isinstance(stream, int):
         return stream or None
     return int(stream.cuda_stream) or None

@@ -84,8 +84,7 @@ def status_word(dev):
     (a fill kernel per word costs more host time than the call whose errors it collects). A block lives as long as
     any word of it; words are not handed out again."""
     dev = _device(dev)
-    here = dev.index == torch.cuda.current_device()
-    key = (dev, B._stream(None) if here else torch.cuda.current_stream(dev).cuda_stream or None)
+    key = (dev, B._stream_of(dev.index))
     while True:
         block = _STATUS.get(key)
         i = next(block[1]) if block is not None else 1024

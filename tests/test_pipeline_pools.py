@@ -18,10 +18,9 @@ def two_gpus(monkeypatch):
         return real(*size, dtype=dtype)
     monkeypatch.setattr(P, "_STATUS", {})
     monkeypatch.setattr(P, "_ROWS_WS", {})
-    monkeypatch.setattr(B, "_stream", lambda s: None)              # the default stream of either device
-    for name, fake in (("current_device", lambda: gpu[0]), ("current_stream", lambda d=None: type("S", (), {"cuda_stream": 0})()),
-                       ("is_current_stream_capturing", lambda: False)):
-        monkeypatch.setattr(torch.cuda, name, fake)
+    monkeypatch.setattr(B, "_stream_of", lambda index: None)       # the default stream of either device
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: gpu[0])
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
     monkeypatch.setattr(torch, "zeros", alloc)
     monkeypatch.setattr(torch, "empty", alloc)
     return P, made, gpu
