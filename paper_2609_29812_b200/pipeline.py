@@ -56,8 +56,9 @@ def select_tokens(ctx, shape, loop_r, g_prev, g_cur, cand: Optional[torch.Tensor
 
 def _device(dev) -> torch.device:
     """`dev` with its index ("cuda" is the device that is current now): what the process's pools are keyed by."""
-    dev = torch.device(dev)
-    return dev if dev.type != "cuda" or dev.index is not None else torch.device("cuda", torch.cuda.current_device())
+    if not isinstance(dev, torch.device):
+        dev = torch.device(dev)
+    return dev if dev.index is not None or dev.type != "cuda" else torch.device("cuda", torch.cuda.current_device())
 
 
 _ROWS_WS: dict = {}
@@ -82,8 +83,11 @@ _STATUS: dict = {}     # (device, stream) -> (zeroed words, counter of the words
 def status_word(dev):
     """A zeroed int32 device word of its own: one of a block of 1024 that is cleared once, on the stream that will use it
     (a fill kernel per word costs more host time than the call whose errors it collects). A block lives as long as
-    any word of it; words are not handed out again."""
+    any word of it; words are not handed out again. Under graph capture a clear is recorded and not executed: there a word
+    is an allocation of its own, which every replay clears."""
     dev = _device(dev)
+    if torch.cuda.is_current_stream_capturing():
+        return torch.zeros(1, dtype=torch.int32, device=dev)
     key = (dev, B._stream_of(dev.index))
     while True:
         block = _STATUS.get(key)
