@@ -114,6 +114,8 @@ def lend_workspace(ctx, shape, dev) -> int:
         # a context that holds this workspace already keeps it: every launch leaves its counters cleared
         if getattr(ctx, "_lent", None) != (ws.data_ptr(), ws.numel()):
             B.fl_set_workspace(ctx, ws, ws.numel())
+            if torch.cuda.is_current_stream_capturing():
+                ctx._lent = None     # the counters' clear is recorded and not executed: the next state sets it again
         ctx._workspace = ws
     return need
 
