@@ -97,26 +97,30 @@ def status_word(dev):
         _STATUS[key] = (torch.zeros(1024, dtype=torch.int32, device=dev), itertools.count())
 
 
-def lend_workspace(ctx, shape, dev) -> int:
+def lend_workspace(ctx, shape, dev, stale_rows: bool = True) -> int:
     """Hands the context the workspace with which the attention launch splits the problems of its last, partly empty
     wave over two CTAs each (a scheduling aid; 0 bytes when the shape cannot profit), with room behind it for the rows
-    that a launch with shrunken token sets rebuilds once.  The tensor stays referenced by the Context object.  Returns
-    the bytes of the split's part."""
+    that a launch with shrunken token sets rebuilds once (up to 256 MB; stale_rows=False: without, for a program whose
+    sets keep their size).  The tensor stays referenced by the Context object.  Returns the bytes of the split's part."""
     sizes = ctx.__dict__.setdefault("_workspace_sizes", {})      # two calls into the library per layer state otherwise
     key = (shape.L, shape.n_heads, shape.head_dim, shape.dtype, shape.q_block)
     if key not in sizes:
         sizes[key] = (B.fl_loop_attention_workspace_bytes(ctx, shape), B.fl_loop_attention_full_workspace_bytes(ctx, shape))
     need, full = sizes[key]
-    if full > 0:
+    want = full if stale_rows else need
+    if want > 0:
         ws = getattr(ctx, "_workspace", None)
-        if ws is None or ws.numel() < full:
-            ws = torch.empty(full, dtype=torch.uint8, device=dev)
+        if ws is None or ws.numel() < want:
+            if stale_rows and not getattr(ctx, "_row_room", False):
+                ctx._workspace_before = ws      # the split's part alone (< 20 MB): a captured graph may still use it
+            ws = torch.empty(want, dtype=torch.uint8, device=dev)
         # a context that holds this workspace already keeps it: every launch leaves its counters cleared
         if getattr(ctx, "_lent", None) != (ws.data_ptr(), ws.numel()):
             B.fl_set_workspace(ctx, ws, ws.numel())
             if torch.cuda.is_current_stream_capturing():
                 ctx._lent = None     # the counters' clear is recorded and not executed: the next state sets it again
         ctx._workspace = ws
+        ctx._row_room = stale_rows or getattr(ctx, "_row_room", False)
     return need
 
 
@@ -131,9 +135,11 @@ class LayerState:
         self.c = c or w.col_budget
         self.nb = (w.L + self.shape.q_block - 1) // self.shape.q_block
         self.dt = torch_dtype(w)
+        self._max_rows = 0              # of the streams so far
+        self._lends = split and self.dt == torch.bfloat16
         if self.dt == torch.bfloat16:
-            if split:
-                lend_workspace(ctx, self.shape, self.dev)
+            if split:                   # the room for rebuilt rows follows with the first set that shrinks
+                lend_workspace(ctx, self.shape, self.dev, stale_rows=False)
             else:   # the context's attention launches go back to one CTA per problem
                 B.fl_set_workspace(ctx, None, 0)
                 ctx._workspace = None
@@ -219,6 +225,13 @@ class LayerState:
         rows after the loop's residual (all a call that reuses the carried old term reads)."""
         w, n = self.w, sel.n
         d = w.d
+        # a set that shrinks leaves tokens whose rows an attention call rebuilds: room for them (256 MB at 32K, so not before;
+        # not under capture, where the memory would be the graph's: the kernels then rebuild them on the fly)
+        if n < self._max_rows and self._lends and not torch.cuda.is_current_stream_capturing():
+            if getattr(self.ctx, "_workspace", self) is not None:      # None: detached by a state without the split
+                lend_workspace(self.ctx, self.shape, self.dev)
+            self._lends = False
+        self._max_rows = max(self._max_rows, n)
         ws = rows_workspace(self.dev, n, d) if rows and self.dt == torch.bfloat16 and n > 0 else None
 
         # K and V in one allocation each for the codes and for scales and offsets (an allocation costs the host about as

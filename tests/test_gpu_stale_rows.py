@@ -87,3 +87,36 @@ def test_rebuilt_rows_bit_exact(bits, group):
         for i, s in enumerate("kv"):
             assert np.array_equal(rows[i, stale], bf(hat[s][stale])), (r, s)
     ctx.close()
+
+
+def test_room_for_rows_comes_with_the_first_set_that_shrinks():
+    """Sets of one size: the split's part of the workspace alone.  The first smaller set: room for the rebuilt rows, and what
+    the context held before stays allocated (a captured graph may use it).  A detached context gets nothing."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_29812_b200 import binding as B, pipeline as P
+    w = workloads.replace(workloads.config2(L=2000, n_heads=2), n_loops=4, q_block=256, col_budget=96)
+    base = torch.zeros(w.L, 2, 128, dtype=torch.bfloat16, device="cuda")
+
+    def sel(n):
+        idx = torch.arange(n, dtype=torch.int32, device="cuda")
+        return P.TokenSelection(idx, torch.full((w.L,), -1, dtype=torch.int32, device="cuda"), None, n)
+    for split in (True, False):
+        ctx = B.Context(0)
+        st = P.LayerState(ctx, w)
+        need, full = B.fl_loop_attention_workspace_bytes(ctx, st.shape), B.fl_loop_attention_full_workspace_bytes(ctx, st.shape)
+        assert 0 < need < full and ctx._workspace.numel() == need
+        st.k_base = st.v_base = base
+        st.alloc_stream(sel(200))
+        st.alloc_stream(sel(200))
+        before = ctx._workspace
+        assert before.numel() == need
+        if not split:
+            P.LayerState(ctx, w, split=False)
+        st.alloc_stream(sel(100))
+        if split:
+            assert ctx._workspace.numel() == full and ctx._workspace_before is before and not ctx._workspace[:1024].any()
+            assert ctx._lent == (ctx._workspace.data_ptr(), full)
+        else:
+            assert ctx._workspace is None and ctx._lent is None
+        ctx.close()
