@@ -1,0 +1,60 @@
+"""Decode calls with little work: their time has to follow the work.  Ratios of times on one GPU, not times: twice the queries
+where the GPU has room for them, and a short list against a longer one."""
+import pytest
+
+from paper_2609_29812_b200 import workloads
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def time_of():
+    """Time of a decode call of one layer (8192 positions, 16 heads, loop 4, a tenth of the rows with payloads), by the number
+    of queries and columns: the best of several replays of a graph of 32 calls, in us."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2609_29812_b200 import binding as B, pipeline as P
+    L, H, loops, calls = 8192, 16, 4, 32
+    w = workloads.replace(workloads.config2(L=L, n_heads=H), n_loops=loops)
+    ctx = B.Context(0)
+    st = P.LayerState(ctx, w)
+    rand = lambda *s: torch.randn(*s, device="cuda").to(torch.bfloat16)
+    st.k_base, st.v_base = rand(L, H, 128), rand(L, H, 128)
+    order = torch.randperm(L, device="cuda")
+    for r in range(2, loops + 1):
+        act = torch.sort(order[:L // 10])[0]
+        slot = torch.full((L,), -1, dtype=torch.int32, device="cuda")
+        slot[act] = torch.arange(len(act), dtype=torch.int32, device="cuda")
+        sel = P.TokenSelection(act.to(torch.int32), slot, None, len(act))
+        st.alloc_stream(sel, rows=False)
+        st.quantize(r, rand(len(act), H, 128), rand(len(act), H, 128), sel)
+
+    def measure(queries, c):
+        idx = torch.sort(torch.topk(torch.rand(queries * H, L, device="cuda"), c, dim=1)[1], dim=1)[0].to(torch.int32)
+        cnt = torch.full((queries, H), c, dtype=torch.int32, device="cuda")
+        q, lse, out = rand(3, queries, H, 128), torch.full((queries, H), 9.5, device="cuda"), rand(queries, H, 128)
+        lse_out = torch.empty_like(lse)
+        call = lambda: B.fl_decode_attention(ctx, st.shape, loops, q[0], q[1], queries, st.store, idx, cnt, c, lse, lse_out, q[2], out)
+        call()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            for _ in range(calls):
+                call()
+        best = float("inf")
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            graph.replay()
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3 / calls)
+        return best
+    yield measure
+    ctx.close()
+
+
+def test_more_queries_do_not_wait_for_a_second_wave(time_of):
+    t2, t4 = time_of(2, 512), time_of(4, 512)
+    assert t4 < 1.6 * t2, f"two queries {t2:.1f} us, four {t4:.1f} us"          # 15.3 and 29.3 when a list was split too far
