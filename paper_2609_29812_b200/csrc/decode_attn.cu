@@ -550,12 +550,12 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
 #pragma unroll
       for (int hf = 0; hf < 2; ++hf) {
         const float c0 = st.acc[m][2 * hf], c1 = st.acc[m][2 * hf + 1];
-        // t = 0: old hi, mid; t = 1: old lo, new hi; t = 2: new mid, lo
+        // t = 0: old hi, mid; t = 1: old lo, new hi; t = 2: new mid, lo. One predicated store for both terms: a branch
+        // each made the warp part and join 32 times, 2700 cycles of a call with few columns.
         const float from1_old = __shfl_sync(0xffffffffu, c0, (lane & ~3) + 1);
         const float from1_new = __shfl_sync(0xffffffffu, c1, (lane & ~3) + 1);
-        const int dim = m * 16 + hf * 8 + g;
-        if (t == 0) ctl.acc[warp][0][dim] = (c0 + c1) + from1_old;
-        if (t == 2) ctl.acc[warp][1][dim] = from1_new + (c0 + c1);
+        const float sum = (c0 + c1) + (t == 0 ? from1_old : from1_new);
+        if ((t & 1) == 0) ctl.acc[warp][t >> 1][m * 16 + hf * 8 + g] = sum;
       }
     float mass = st.mass, l = st.l;
 #pragma unroll
