@@ -453,13 +453,18 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
   // The warp's tiles: plain ones first (dealt round robin from warp 0), then those of columns with a payload (from the
   // last warp down). Base rows come by asynchronous copies, one tile ahead; a payload tile needs the other stage for
   // its second pair of tiles, so the tile after it is asked for when it is done.
-  const int plain_tiles = (n_plain + kMmaTile - 1) / kMmaTile, pay_tiles = (n - n_plain + kMmaTile - 1) / kMmaTile;
+  // Up to four tiles of payload columns are dealt evenly, in whole rounds of the rebuild below (2 E columns, each round a
+  // trip to memory that nothing hides when the list is short), instead of sixteen to the first warp.
+  constexpr int E = 2;
+  const int n_pay = n - n_plain;
+  const int pay_len = min(kMmaTile, (n_pay + 2 * E * kMmaWarps - 1) / (2 * E * kMmaWarps) * (2 * E));   // columns of a payload tile
+  const int plain_tiles = (n_plain + kMmaTile - 1) / kMmaTile, pay_tiles = n_pay > 0 ? (n_pay + pay_len - 1) / pay_len : 0;
   const int my_plain = plain_tiles > warp ? (plain_tiles - warp + kMmaWarps - 1) / kMmaWarps : 0;
   const int pw = kMmaWarps - 1 - warp;
   const int my_tiles_n = my_plain + (pay_tiles > pw ? (pay_tiles - pw + kMmaWarps - 1) / kMmaWarps : 0);
   // first ordered column of the warp's tile i, and the end of its class
   auto tile_first = [&](int i) { return i < my_plain ? (i * kMmaWarps + warp) * kMmaTile
-                                                     : n_plain + ((i - my_plain) * kMmaWarps + pw) * kMmaTile; };
+                                                     : n_plain + ((i - my_plain) * kMmaWarps + pw) * pay_len; };
   auto issue = [&](int i, int stage) {
     const int first = tile_first(i), last = (i < my_plain ? n_plain : n) - 1;
     const uint32_t dst = my_addr + stage * kMmaStageBytes;
@@ -492,7 +497,7 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
     } else {
       // Xhat^(r-1) takes the place of the base rows, Xhat^(r) goes to the other stage; each lane rebuilds the pieces it
       // copied itself. The lanes of a half warp look up one stream row each and hand it on.
-      const int n_valid = min(kMmaTile, n - first);
+      const int n_valid = min(pay_len, n - first);
       const int jl = ord_col[min(first + (lane & 15), n - 1)];
       int slot[NS];
 #pragma unroll
@@ -501,9 +506,8 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
       uint8_t* t_new = my_tiles + (stage ^ 1) * kMmaStageBytes;
       const uint32_t kn = my_addr + (stage ^ 1) * kMmaStageBytes;
       bool landed = false;
-      constexpr int E = (NS == 1 || (NS == 2 && BITS <= 4)) ? 4 : 2;   // columns per half warp whose payloads fit the registers
 #pragma unroll 1
-      for (int q0 = 0; q0 < 8; q0 += E) {
+      for (int q0 = 0; q0 * 2 < n_valid; q0 += E) {
         Payload8<T, BITS> pk[E][NS], pv[E][NS];
         int sl[E][NS];
 #pragma unroll
@@ -535,6 +539,10 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
           }
         }
       }
+      // rows past the last round: their weights are zero, what they hold must be a number
+#pragma unroll 1
+      for (int q = (n_valid + 2 * E - 1) / (2 * E) * E; q < 8; ++q)
+        *reinterpret_cast<uint4*>(t_new + kMmaTileBytes + tile_off(q * 2 + rsub, ch)) = make_uint4(0, 0, 0, 0);
       __syncwarp();
       dec_tile(st, bq, kt, kn, vt, kn + kMmaTileBytes, true, n_valid, a.scale, lse_p, ord_u + first, logit_s, lane);
       __syncwarp();

@@ -14,11 +14,25 @@ torch = pytest.importorskip("torch")
 @pytest.mark.parametrize("c,loops,bits,group", [(1, 2, 4, 128), (16, 3, 8, 64), (17, 2, 2, 32), (127, 4, 4, 32), (513, 5, 4, 128),
                                                 (1100, 3, 16, 128), (257, 6, 4, 64)])
 def test_tile_and_split_edges(c, loops, bits, group):
+    run_case(c, loops, bits, group)
+
+
+# pieces of at most a tile per warp, columns dealt evenly over the warps (few problems) or by whole tiles (many), no payload,
+# some or nearly all columns with one, and the first sizes past them
+@pytest.mark.parametrize("c,loops,bits,group,Bq,frac", [(3, 5, 8, 16, 3, 0.75), (63, 4, 4, 128, 2, 0.75), (64, 5, 2, 8, 2, 0.1),
+                                                        (64, 2, 16, 128, 3, 0.3), (65, 3, 4, 64, 2, 0.75), (200, 5, 16, 128, 3, 0.75),
+                                                        (20, 4, 4, 32, 130, 0.3), (64, 3, 8, 64, 120, 0.75), (50, 2, 4, 8, 240, 0.1),
+                                                        (70, 4, 2, 64, 120, 0.3), (512, 4, 8, 128, 4, 0.1), (130, 5, 4, 16, 40, 0.5)])
+def test_short_pieces(c, loops, bits, group, Bq, frac):
+    run_case(c, loops, bits, group, Bq, frac)
+
+
+def run_case(c, loops, bits, group, Bq=3, frac=0.75):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2609_29812_b200 import binding as B, pipeline as P
     rng = np.random.default_rng(c)
-    L, H, dh, Bq = 1300, 2, 128, 3
+    L, H, dh = 1300, 2, 128
     w = workloads.replace(workloads.config2(L=L, n_heads=H), n_loops=loops, bits=bits, group=group)
     bf = fo.round_bf16
     ctx = B.Context(0)
@@ -27,8 +41,8 @@ def test_tile_and_split_edges(c, loops, bits, group):
     st.k_base, st.v_base = to_dev(k1, w), to_dev(v1, w)
     order = rng.permutation(L)
     khat, vhat, k_prev, v_prev = k1.copy(), v1.copy(), None, None
-    for r in range(2, loops + 1):                       # nested sets, from three quarters of the rows down
-        act = np.sort(order[: int(0.75 * L / (r - 1))])
+    for r in range(2, loops + 1):                       # nested sets, from `frac` of the rows down
+        act = np.sort(order[: int(frac * L / (r - 1))])
         kr, vr = (bf(x[act] + 0.3 * rng.standard_normal((len(act), H, dh)).astype(np.float32)) for x in (khat, vhat))
         sel = P.TokenSelection(torch.from_numpy(act.astype(np.int32)).cuda(),
                                torch.from_numpy(fo.slot_map(act, L).astype(np.int32)).cuda(), None, len(act))
@@ -44,7 +58,7 @@ def test_tile_and_split_edges(c, loops, bits, group):
     lse = np.zeros((Bq, H))
     for t in range(Bq):
         for h in range(H):
-            n = [c, max(0, c - 1), c // 2, min(c, 15), min(c, 16), 0][t * H + h]
+            n = [c, max(0, c - 1), c // 2, min(c, 15), min(c, 16), 0][(t * H + h) % 6]
             S = np.sort(rng.permutation(L)[:n])
             col_idx[t, h, :n], col_cnt[t, h], sets[(t, h)] = S, n, S
             logits = (bf(k_prev[:, h]).astype(np.float64) @ q_old[t, h].astype(np.float64)) * w.sm_scale
