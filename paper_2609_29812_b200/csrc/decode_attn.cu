@@ -362,9 +362,10 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
   const int h = prob % a.H;
   const size_t qh = (size_t)prob;
   const int cnt = min(__ldg(a.col_cnt + qh), a.c);
-  const int u_lo = min(cnt, part * per_cta), n = min(cnt, (part + 1) * per_cta) - u_lo;
+  const int u_lo = min(a.c, part * per_cta), n = max(0, min(cnt, u_lo + per_cta) - u_lo);
   const int32_t* cols = a.col_idx + qh * a.c + u_lo;
   const float lse_p = a.lse_prev[qh];
+  const T prev_in = static_cast<const T*>(a.o_prev)[qh * DH + tid];
 
   // B operand of the logits: column 0 = q_old, column 1 = q_new, the other six zero
   uint32_t bq[8][2];
@@ -381,19 +382,23 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
   int n_plain;
   {
     int32_t* raw = reinterpret_cast<int32_t*>(tiles);    // staged in the idle tiles: position, complemented with a payload
-    const int span = ((n + kMmaWarps - 1) / kMmaWarps + 31) & ~31;
-    const int beg = warp * span, end = min(n, beg + span);
+    // spans by the length that the list may have: the columns are asked for without waiting for their count
+    const int len = min(per_cta, a.c - part * per_cta);
+    const int span = ((len + kMmaWarps - 1) / kMmaWarps + 31) & ~31;
+    const int beg = warp * span, lim = min(len, beg + span), end = min(n, lim);
     int n0 = 0, n1 = 0;
 #pragma unroll 1
-    for (int base = beg; base < end; base += 128) {      // four columns per lane and step in flight
+    for (int base = beg; base < lim; base += 128) {      // four columns per lane and step in flight
       int j[4];
       bool pay[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int u = base + e * 32 + lane;
-        j[e] = u < end ? __ldg(cols + u) : -1;
+        j[e] = u < lim ? __ldg(cols + u) : -1;
         pay[e] = false;
       }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) j[e] = base + e * 32 + lane < end ? j[e] : -1;     // past the count: whatever the list holds
 #pragma unroll
       for (int s = 0; s < NS; ++s) {
         int sl[4];
@@ -618,10 +623,8 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
   const bool has = cnt > 0 && m_tot > -INFINITY && mass_tot > 0.f;
   const float w = has ? mass_tot / l_tot : 0.f;
   if (part == 0) {
-    const T* op = static_cast<const T*>(a.o_prev) + qh * DH;
     T* oo = static_cast<T*>(a.o_out) + qh * DH;
-    const float prev = __bfloat162float(op[tid]);
-    oo[tid] = has ? __float2bfloat16_rn(prev - so + w * sn) : op[tid];
+    oo[tid] = has ? __float2bfloat16_rn(__bfloat162float(prev_in) - so + w * sn) : prev_in;
     if (tid == 0) a.lse_out[qh] = has ? m_tot + logf(l_tot) - logf(mass_tot) : lse_p;
   }
   if (a.p_new_out != nullptr) {
