@@ -167,6 +167,11 @@ __global__ void __launch_bounds__(kDecThreads) decode_attn_kernel(const __grid_c
 // in registers (Eq. 8 chain) as the rows before and after the loop's own residual and go through two tile pairs.
 // A problem is split over a cluster of SPLIT CTAs (distributed shared memory joins their results): few queries would
 // leave most SMs idle otherwise, and a CTA with at most 512 columns has lists short enough for three CTAs per SM.
+// Long lists are bound by their bytes, 3.3 TB/s of rows at 32 queries x 16 heads x 2048 columns. Few queries are a chain of
+// latencies in each CTA (launch, list, slots, payloads, tiles, merge: 6400 cycles at 16 columns), so pieces of up to 64
+// columns have a form of their own (SHORT). One query x 16 heads, 10% of the columns with payloads, rows in L2, per call:
+// 64 / 256 / 512 columns 4.5 / 6.2 / 7.6 us with one stream, 5.5 / 7.8 / 9.0 with three (one CTA per query and head in
+// registers: 6.1 / 13.6 / 23.3 and 7.3 / 17.4 / 30.7).
 // ------------------------------------------------------------------------------------------------------------
 constexpr int kMmaWarps = 4;
 constexpr int kMmaThreads = kMmaWarps * 32;
@@ -184,9 +189,14 @@ struct DecMmaCtl {
   int warp_cnt[kMmaWarps][2];
 };
 
-__host__ __device__ constexpr size_t decode_mma_smem(int per_cta) {
+// Warps with tiles: a short piece takes the shared memory of those that have some of its columns.
+__host__ __device__ constexpr int decode_mma_tile_warps(int per_cta, int per_warp) {
+  return per_cta >= kMmaWarps * per_warp ? kMmaWarps : (per_cta + per_warp - 1) / per_warp;
+}
+__host__ __device__ constexpr size_t decode_mma_smem(int per_cta, int per_warp) {
   // tiles, control block, then per column: position, logit, index in the piece
-  return 128 + (size_t)kMmaWarps * kMmaStages * kMmaStageBytes + sizeof(DecMmaCtl) + (size_t)per_cta * (4 + 4 + 2);
+  return 128 + (size_t)decode_mma_tile_warps(per_cta, per_warp) * kMmaStages * kMmaStageBytes + sizeof(DecMmaCtl) +
+         (size_t)per_cta * (4 + 4 + 2);
 }
 
 __device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4]) {
@@ -242,6 +252,26 @@ __device__ __forceinline__ void dec_payload(const Payload8<__nv_bfloat16, BITS>&
   }
 }
 
+// One 16-byte piece of a K row and of the V row a tile behind it: the base rows in `t_old` become Xhat^(r-1), Xhat^(r) goes
+// to `t_new` (Eq. 8 chain), both rounded to the storage type as attention consumes them.
+template <int BITS, int NS>
+__device__ __forceinline__ void dec_rebuild(uint8_t* t_old, uint8_t* t_new, const int (&sl)[NS],
+                                            const Payload8<__nv_bfloat16, BITS> (&pk)[NS],
+                                            const Payload8<__nv_bfloat16, BITS> (&pv)[NS]) {
+#pragma unroll
+  for (int kv = 0; kv < 2; ++kv) {
+    uint4* old_p = reinterpret_cast<uint4*>(t_old + kv * kMmaTileBytes);
+    fl_codec::f32x2 x[4];
+    fl_codec::unpack_bf16(*old_p, x);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      if (s == NS - 1 && NS > 1) *old_p = fl_codec::pack_bf16(x);
+      if (sl[s] >= 0) dec_payload<BITS>(kv ? pv[s] : pk[s], x);
+    }
+    *reinterpret_cast<uint4*>(t_new + kv * kMmaTileBytes) = fl_codec::pack_bf16(x);
+  }
+}
+
 // Running state of a warp: both terms' weighted sums as D[dim][variant] tiles, the old term's mass, the new term's
 // reference and sum (mass and sum as per-lane partials of the lanes that hold logits).
 struct DecMmaState {
@@ -250,7 +280,9 @@ struct DecMmaState {
 };
 
 // One tile: logits from k_old / k_new (the same address for plain columns), probabilities, weighted sums of v_old /
-// v_new. `n_valid` columns count; `lu` is the local index of the lane's column pair (valid in lanes t == 0).
+// v_new. `n_valid` columns count; logits go to logit_s by the columns' index in the CTA's piece of the list: ord_u, or the
+// order of the tile itself (ORDERED false).
+template <bool ORDERED>
 __device__ __forceinline__ void dec_tile(DecMmaState& st, const uint32_t (&bq)[8][2], uint32_t k_old, uint32_t k_new,
                                          uint32_t v_old, uint32_t v_new, bool two, int n_valid, float scale, float lse_p,
                                          const uint16_t* ord_u, float* logit_s, int lane) {
@@ -282,8 +314,8 @@ __device__ __forceinline__ void dec_tile(DecMmaState& st, const uint32_t (&bq)[8
   // lanes t == 0 hold (old, new) logits of columns g and g + 8
   const bool on0 = t == 0 && g < n_valid, on1 = t == 0 && g + 8 < n_valid;
   const float sn0 = s[1] * scale, sn1 = s[3] * scale;
-  if (on0) logit_s[ord_u[g]] = sn0;
-  if (on1) logit_s[ord_u[g + 8]] = sn1;
+  if (on0) logit_s[ORDERED ? ord_u[g] : g] = sn0;
+  if (on1) logit_s[ORDERED ? ord_u[g + 8] : g + 8] = sn1;
   float mx = fmaxf(on0 ? sn0 : -INFINITY, on1 ? sn1 : -INFINITY);
 #pragma unroll
   for (int o = 16; o >= 4; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -343,14 +375,16 @@ __device__ __forceinline__ void dec_tile(DecMmaState& st, const uint32_t (&bq)[8
   }
 }
 
-template <int BITS, int NS>
+// SHORT: pieces of at most one tile per warp (see below).
+template <int BITS, int NS, bool SHORT>
 __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const __grid_constant__ DecodeArgs a, int split,
-                                                                         int per_cta) {
+                                                                         int per_cta, int per_warp) {
   using T = __nv_bfloat16;
   constexpr int DH = 128;
   extern __shared__ __align__(16) uint8_t dyn[];
   uint8_t* tiles = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dyn) + 127) & ~uintptr_t(127));
-  DecMmaCtl& ctl = *reinterpret_cast<DecMmaCtl*>(tiles + kMmaWarps * kMmaStages * kMmaStageBytes);
+  const int tile_warps = SHORT ? decode_mma_tile_warps(per_cta, per_warp) : kMmaWarps;
+  DecMmaCtl& ctl = *reinterpret_cast<DecMmaCtl*>(tiles + tile_warps * kMmaStages * kMmaStageBytes);
   int32_t* ord_col = reinterpret_cast<int32_t*>(&ctl + 1);      // [per_cta] positions: plain columns, then the others
   float* logit_s = reinterpret_cast<float*>(ord_col + per_cta);   // [per_cta] by index in the CTA's piece of the list
   uint16_t* ord_u = reinterpret_cast<uint16_t*>(logit_s + per_cta);   // [per_cta] index in the piece of an ordered column
@@ -378,69 +412,6 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
       for (int hf = 0; hf < 2; ++hf)
         bq[kk][hf] = g < 2 ? __ldg(reinterpret_cast<const uint32_t*>(q + kk * 16 + hf * 8 + t * 2)) : 0u;
   }
-  // ---- partition: a warp owns a contiguous span of the piece; columns without a payload first --------------------
-  int n_plain;
-  {
-    int32_t* raw = reinterpret_cast<int32_t*>(tiles);    // staged in the idle tiles: position, complemented with a payload
-    // spans by the length that the list may have: the columns are asked for without waiting for their count
-    const int len = min(per_cta, a.c - part * per_cta);
-    const int span = ((len + kMmaWarps - 1) / kMmaWarps + 31) & ~31;
-    const int beg = warp * span, lim = min(len, beg + span), end = min(n, lim);
-    int n0 = 0, n1 = 0;
-#pragma unroll 1
-    for (int base = beg; base < lim; base += 128) {      // four columns per lane and step in flight
-      int j[4];
-      bool pay[4];
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int u = base + e * 32 + lane;
-        j[e] = u < lim ? __ldg(cols + u) : -1;
-        pay[e] = false;
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) j[e] = base + e * 32 + lane < end ? j[e] : -1;     // past the count: whatever the list holds
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        int sl[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) sl[e] = j[e] >= 0 ? __ldg(a.k.s[s].slot + j[e]) : -1;
-#pragma unroll
-        for (int e = 0; e < 4; ++e) pay[e] |= sl[e] >= 0;
-      }
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int u = base + e * 32 + lane;
-        n0 += __popc(__ballot_sync(0xffffffffu, u < end && !pay[e]));
-        n1 += __popc(__ballot_sync(0xffffffffu, u < end && pay[e]));
-        if (u < end) raw[u] = pay[e] ? ~j[e] : j[e];
-      }
-    }
-    if (lane == 0) { ctl.warp_cnt[warp][0] = n0; ctl.warp_cnt[warp][1] = n1; }
-    __syncthreads();
-    int tot0 = 0, before0 = 0, before1 = 0;
-#pragma unroll
-    for (int w = 0; w < kMmaWarps; ++w) {
-      tot0 += ctl.warp_cnt[w][0];
-      if (w < warp) { before0 += ctl.warp_cnt[w][0]; before1 += ctl.warp_cnt[w][1]; }
-    }
-    n_plain = tot0;
-    const uint32_t lt = (1u << lane) - 1;
-#pragma unroll 1
-    for (int base = beg; base < end; base += 32) {
-      const int u = base + lane;
-      const int r = u < end ? raw[u] : 0;
-      const bool pay = u < end && r < 0, plain = u < end && r >= 0;
-      const uint32_t m0 = __ballot_sync(0xffffffffu, plain), m1 = __ballot_sync(0xffffffffu, pay);
-      if (u < end) {
-        const int dst = pay ? tot0 + before1 + __popc(m1 & lt) : before0 + __popc(m0 & lt);
-        ord_col[dst] = pay ? ~r : r;
-        ord_u[dst] = (uint16_t)u;
-      }
-      before0 += __popc(m0);
-      before1 += __popc(m1);
-    }
-    __syncthreads();
-  }
   DecMmaState st;
   st.mass = st.l = 0.f;
   st.ref = -INFINITY;
@@ -455,105 +426,246 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
   const T* kb = static_cast<const T*>(a.k.base) + elem;
   const T* vb = static_cast<const T*>(a.v.base) + elem;
 
-  // The warp's tiles: plain ones first (dealt round robin from warp 0), then those of columns with a payload (from the
-  // last warp down). Base rows come by asynchronous copies, one tile ahead; a payload tile needs the other stage for
-  // its second pair of tiles, so the tile after it is asked for when it is done.
-  // Up to four tiles of payload columns are dealt evenly, in whole rounds of the rebuild below (2 E columns, each round a
-  // trip to memory that nothing hides when the list is short), instead of sixteen to the first warp.
-  constexpr int E = 2;
-  const int n_pay = n - n_plain;
-  const int pay_len = min(kMmaTile, (n_pay + 2 * E * kMmaWarps - 1) / (2 * E * kMmaWarps) * (2 * E));   // columns of a payload tile
-  const int plain_tiles = (n_plain + kMmaTile - 1) / kMmaTile, pay_tiles = n_pay > 0 ? (n_pay + pay_len - 1) / pay_len : 0;
-  const int my_plain = plain_tiles > warp ? (plain_tiles - warp + kMmaWarps - 1) / kMmaWarps : 0;
-  const int pw = kMmaWarps - 1 - warp;
-  const int my_tiles_n = my_plain + (pay_tiles > pw ? (pay_tiles - pw + kMmaWarps - 1) / kMmaWarps : 0);
-  // first ordered column of the warp's tile i, and the end of its class
-  auto tile_first = [&](int i) { return i < my_plain ? (i * kMmaWarps + warp) * kMmaTile
-                                                     : n_plain + ((i - my_plain) * kMmaWarps + pw) * pay_len; };
-  auto issue = [&](int i, int stage) {
-    const int first = tile_first(i), last = (i < my_plain ? n_plain : n) - 1;
-    const uint32_t dst = my_addr + stage * kMmaStageBytes;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const int row = q * 2 + rsub;
-      const size_t off = (size_t)ord_col[min(first + row, last)] * a.d;   // past the end: any row (its weight is zero)
-      const uint32_t o = dst + tile_off(row, ch);
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o), "l"(kb + off) : "memory");
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o + kMmaTileBytes), "l"(vb + off) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  if (my_tiles_n > 0) issue(0, 0);
-  int stage = 0;
-#pragma unroll 1
-  for (int i = 0; i < my_tiles_n; ++i) {
-    const int first = tile_first(i);
-    const uint32_t kt = my_addr + stage * kMmaStageBytes, vt = kt + kMmaTileBytes;
-    if (i < my_plain) {
-      if (i + 1 < my_tiles_n) {
-        issue(i + 1, stage ^ 1);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-      } else {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-      }
-      __syncwarp();
-      dec_tile(st, bq, kt, kt, vt, vt, false, n_plain - first, a.scale, lse_p, ord_u + first, logit_s, lane);
-      __syncwarp();
-    } else {
-      // Xhat^(r-1) takes the place of the base rows, Xhat^(r) goes to the other stage; each lane rebuilds the pieces it
-      // copied itself. The lanes of a half warp look up one stream row each and hand it on.
-      const int n_valid = min(pay_len, n - first);
-      const int jl = ord_col[min(first + (lane & 15), n - 1)];
+  if constexpr (SHORT) {
+    // A list this short is one chain of latencies, so nothing is sorted: a warp takes its columns of the list as they come,
+    // asks for their base rows and their rows in the streams at once, copies the tile, rebuilds the rows with a payload in
+    // both, and makes one pass over the pair. Three dependent trips to memory (list, rows and slots, payloads) and one tile;
+    // the general form (partition, a plain tile, a payload tile) takes 0.6 to 2.4 us longer per call at 16 to 512 columns.
+    const int len = min(per_cta, a.c - part * per_cta), first = warp * per_warp, row0 = lane & (kMmaTile - 1);
+    int j = row0 < per_warp && first + row0 < len ? __ldg(cols + first + row0) : 0;    // asked for ahead of the count
+    const int n_valid = min(per_warp, n - first);
+    if (n_valid > 0) {
+      const int j0 = __shfl_sync(0xffffffffu, j, 0);
+      if (row0 >= n_valid) j = j0;                                 // past the end: any row (its weight is zero)
       int slot[NS];
+      uint32_t pay = 0;
 #pragma unroll
-      for (int s = 0; s < NS; ++s) slot[s] = __ldg(a.k.s[s].slot + jl);
-      uint8_t* t_old = my_tiles + stage * kMmaStageBytes;
-      uint8_t* t_new = my_tiles + (stage ^ 1) * kMmaStageBytes;
-      const uint32_t kn = my_addr + (stage ^ 1) * kMmaStageBytes;
-      bool landed = false;
-#pragma unroll 1
-      for (int q0 = 0; q0 * 2 < n_valid; q0 += E) {
+      for (int s = 0; s < NS; ++s) slot[s] = row0 < n_valid ? __ldg(a.k.s[s].slot + j) : -1;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const size_t off = (size_t)__shfl_sync(0xffffffffu, j, q * 2 + rsub) * a.d;
+        const uint32_t o = my_addr + tile_off(q * 2 + rsub, ch);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o), "l"(kb + off) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o + kMmaTileBytes), "l"(vb + off) : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll
+      for (int s = 0; s < NS; ++s) pay |= __ballot_sync(0xffffffffu, slot[s] >= 0);
+      pay &= 0xffffu;                                              // rows of the tile with a payload in any stream
+      uint8_t* t_new = my_tiles + kMmaStageBytes;
+      const uint32_t kn = my_addr + kMmaStageBytes;
+      const bool two = pay != 0;
+      bool copied = false;
+      while (pay != 0) {
+        // up to four of those rows, two per half warp
+        constexpr int E = 2;
         Payload8<T, BITS> pk[E][NS], pv[E][NS];
-        int sl[E][NS];
+        int row[E], sl[E][NS];
 #pragma unroll
-        for (int e = 0; e < E; ++e)
+        for (int e = 0; e < E; ++e) {
+          const int r0 = __ffs(pay) - 1;
+          pay &= pay - 1;
+          const int r1 = __ffs(pay) - 1;
+          pay &= pay - 1;                                          // 0 stays 0
+          row[e] = rsub ? r1 : r0;                                 // -1: none left
 #pragma unroll
           for (int s = 0; s < NS; ++s) {
-            sl[e][s] = __shfl_sync(0xffffffffu, slot[s], (q0 + e) * 2 + rsub);
+            sl[e][s] = __shfl_sync(0xffffffffu, slot[s], max(row[e], 0));
+            if (row[e] < 0) sl[e][s] = -1;
+          }
+          if constexpr (BITS == 16 && NS > 2) {     // stored rows: a later one takes an earlier one's place
+            bool later = sl[e][NS - 2] >= 0;
+#pragma unroll
+            for (int s = NS - 3; s >= 0; --s) {
+              if (later) sl[e][s] = -1;
+              later |= sl[e][s] >= 0;
+            }
+          }
+#pragma unroll
+          for (int s = 0; s < NS; ++s)
             if (sl[e][s] >= 0) {
               payload_load<T, BITS>(a.k.s[s], sl[e][s], elem, a.d, a.group, pk[e][s]);
               payload_load<T, BITS>(a.v.s[s], sl[e][s], elem, a.d, a.group, pv[e][s]);
             }
-          }
-        if (!landed) { asm volatile("cp.async.wait_group 0;" ::: "memory"); landed = true; }
+        }
+        if (!copied) {          // under the payloads' trip; each lane copies and rebuilds the pieces it fetched itself
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
 #pragma unroll
-        for (int e = 0; e < E; ++e) {
-          const uint32_t o = tile_off((q0 + e) * 2 + rsub, ch);
+          for (int q = 0; q < 8; ++q)
 #pragma unroll
-          for (int kv = 0; kv < 2; ++kv) {
-            uint4* old_p = reinterpret_cast<uint4*>(t_old + o + kv * kMmaTileBytes);
-            fl_codec::f32x2 x[4];
-            fl_codec::unpack_bf16(*old_p, x);
-#pragma unroll
-            for (int s = 0; s < NS; ++s) {
-              // Xhat^(r-1), rounded to the storage type as attention consumes it
-              if (s == NS - 1 && NS > 1) *old_p = fl_codec::pack_bf16(x);
-              if (sl[e][s] >= 0) dec_payload<BITS>(kv ? pv[e][s] : pk[e][s], x);
+            for (int kv = 0; kv < 2; ++kv) {
+              const uint32_t o = tile_off(q * 2 + rsub, ch) + kv * kMmaTileBytes;
+              *reinterpret_cast<uint4*>(t_new + o) = *reinterpret_cast<const uint4*>(my_tiles + o);
             }
-            *reinterpret_cast<uint4*>(t_new + o + kv * kMmaTileBytes) = fl_codec::pack_bf16(x);
+          copied = true;
+          __syncwarp();         // a row with a payload may belong to the other half
+        }
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (row[e] >= 0) {
+            const uint32_t o = tile_off(row[e], ch);
+            dec_rebuild<BITS, NS>(my_tiles + o, t_new + o, sl[e], pk[e], pv[e]);
           }
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      __syncwarp();
+      const uint32_t k_new = two ? kn : my_addr;
+      dec_tile<false>(st, bq, my_addr, k_new, my_addr + kMmaTileBytes, k_new + kMmaTileBytes, two, n_valid, a.scale, lse_p, nullptr,
+               logit_s + first, lane);
+    }
+  } else {
+    // ---- partition: a warp owns a contiguous span of the piece; columns without a payload first --------------------
+    int n_plain;
+    {
+      int32_t* raw = reinterpret_cast<int32_t*>(tiles);    // staged in the idle tiles: position, complemented with a payload
+      // spans by the length that the list may have: the columns are asked for without waiting for their count
+      const int len = max(0, min(per_cta, a.c - part * per_cta));
+      const int span = ((len + kMmaWarps - 1) / kMmaWarps + 31) & ~31;
+      const int beg = warp * span, lim = min(len, beg + span), end = min(n, lim);
+      int n0 = 0, n1 = 0;
+#pragma unroll 1
+      for (int base = beg; base < lim; base += 128) {      // four columns per lane and step in flight
+        int j[4];
+        bool pay[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int u = base + e * 32 + lane;
+          j[e] = u < lim ? __ldg(cols + u) : -1;
+          pay[e] = false;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) j[e] = base + e * 32 + lane < end ? j[e] : -1;     // past the count: whatever the list holds
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+          int sl[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) sl[e] = j[e] >= 0 ? __ldg(a.k.s[s].slot + j[e]) : -1;
+#pragma unroll
+          for (int e = 0; e < 4; ++e) pay[e] |= sl[e] >= 0;
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const int u = base + e * 32 + lane;
+          n0 += __popc(__ballot_sync(0xffffffffu, u < end && !pay[e]));
+          n1 += __popc(__ballot_sync(0xffffffffu, u < end && pay[e]));
+          if (u < end) raw[u] = pay[e] ? ~j[e] : j[e];
         }
       }
-      // rows past the last round: their weights are zero, what they hold must be a number
+      if (lane == 0) { ctl.warp_cnt[warp][0] = n0; ctl.warp_cnt[warp][1] = n1; }
+      __syncthreads();
+      int tot0 = 0, before0 = 0, before1 = 0;
+#pragma unroll
+      for (int w = 0; w < kMmaWarps; ++w) {
+        tot0 += ctl.warp_cnt[w][0];
+        if (w < warp) { before0 += ctl.warp_cnt[w][0]; before1 += ctl.warp_cnt[w][1]; }
+      }
+      n_plain = tot0;
+      const uint32_t lt = (1u << lane) - 1;
 #pragma unroll 1
-      for (int q = (n_valid + 2 * E - 1) / (2 * E) * E; q < 8; ++q)
-        *reinterpret_cast<uint4*>(t_new + kMmaTileBytes + tile_off(q * 2 + rsub, ch)) = make_uint4(0, 0, 0, 0);
-      __syncwarp();
-      dec_tile(st, bq, kt, kn, vt, kn + kMmaTileBytes, true, n_valid, a.scale, lse_p, ord_u + first, logit_s, lane);
-      __syncwarp();
-      if (i + 1 < my_tiles_n) issue(i + 1, stage ^ 1);
+      for (int base = beg; base < end; base += 32) {
+        const int u = base + lane;
+        const int r = u < end ? raw[u] : 0;
+        const bool pay = u < end && r < 0, plain = u < end && r >= 0;
+        const uint32_t m0 = __ballot_sync(0xffffffffu, plain), m1 = __ballot_sync(0xffffffffu, pay);
+        if (u < end) {
+          const int dst = pay ? tot0 + before1 + __popc(m1 & lt) : before0 + __popc(m0 & lt);
+          ord_col[dst] = pay ? ~r : r;
+          ord_u[dst] = (uint16_t)u;
+        }
+        before0 += __popc(m0);
+        before1 += __popc(m1);
+      }
+      __syncthreads();
     }
-    stage ^= 1;
+    // The warp's tiles: plain ones first (dealt round robin from warp 0), then those of columns with a payload (from the
+    // last warp down). Base rows come by asynchronous copies, one tile ahead; a payload tile needs the other stage for
+    // its second pair of tiles, so the tile after it is asked for when it is done.
+    // Up to four tiles of payload columns are dealt evenly, in whole rounds of the rebuild below (2 E columns, each round a
+    // trip to memory that nothing hides when the list is short), instead of sixteen to the first warp. E columns per half
+    // warp: their payloads fit the registers for up to four streams.
+    constexpr int E = 2;
+    const int n_pay = n - n_plain;
+    const int pay_len = min(kMmaTile, (n_pay + 2 * E * kMmaWarps - 1) / (2 * E * kMmaWarps) * (2 * E));   // columns of a payload tile
+    const int plain_tiles = (n_plain + kMmaTile - 1) / kMmaTile, pay_tiles = n_pay > 0 ? (n_pay + pay_len - 1) / pay_len : 0;
+    const int my_plain = plain_tiles > warp ? (plain_tiles - warp + kMmaWarps - 1) / kMmaWarps : 0;
+    const int pw = kMmaWarps - 1 - warp;
+    const int my_tiles_n = my_plain + (pay_tiles > pw ? (pay_tiles - pw + kMmaWarps - 1) / kMmaWarps : 0);
+    // first ordered column of the warp's tile i, and the end of its class
+    auto tile_first = [&](int i) { return i < my_plain ? (i * kMmaWarps + warp) * kMmaTile
+                                                       : n_plain + ((i - my_plain) * kMmaWarps + pw) * pay_len; };
+    auto issue = [&](int i, int stage) {
+      const int first = tile_first(i), last = (i < my_plain ? n_plain : n) - 1;
+      const uint32_t dst = my_addr + stage * kMmaStageBytes;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int row = q * 2 + rsub;
+        const size_t off = (size_t)ord_col[min(first + row, last)] * a.d;   // past the end: any row (its weight is zero)
+        const uint32_t o = dst + tile_off(row, ch);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o), "l"(kb + off) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(o + kMmaTileBytes), "l"(vb + off) : "memory");
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    if (my_tiles_n > 0) issue(0, 0);
+    int stage = 0;
+#pragma unroll 1
+    for (int i = 0; i < my_tiles_n; ++i) {
+      const int first = tile_first(i);
+      const uint32_t kt = my_addr + stage * kMmaStageBytes, vt = kt + kMmaTileBytes;
+      if (i < my_plain) {
+        if (i + 1 < my_tiles_n) {
+          issue(i + 1, stage ^ 1);
+          asm volatile("cp.async.wait_group 1;" ::: "memory");
+        } else {
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+        }
+        __syncwarp();
+        dec_tile<true>(st, bq, kt, kt, vt, vt, false, n_plain - first, a.scale, lse_p, ord_u + first, logit_s, lane);
+        __syncwarp();
+      } else {
+        // Xhat^(r-1) takes the place of the base rows, Xhat^(r) goes to the other stage; each lane rebuilds the pieces it
+        // copied itself. The lanes of a half warp look up one stream row each and hand it on.
+        const int n_valid = min(pay_len, n - first);
+        const int jl = ord_col[min(first + (lane & 15), n - 1)];
+        int slot[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) slot[s] = __ldg(a.k.s[s].slot + jl);
+        uint8_t* t_old = my_tiles + stage * kMmaStageBytes;
+        uint8_t* t_new = my_tiles + (stage ^ 1) * kMmaStageBytes;
+        const uint32_t kn = my_addr + (stage ^ 1) * kMmaStageBytes;
+        bool landed = false;
+#pragma unroll 1
+        for (int q0 = 0; q0 * 2 < n_valid; q0 += E) {
+          Payload8<T, BITS> pk[E][NS], pv[E][NS];
+          int sl[E][NS];
+#pragma unroll
+          for (int e = 0; e < E; ++e)
+#pragma unroll
+            for (int s = 0; s < NS; ++s) {
+              sl[e][s] = __shfl_sync(0xffffffffu, slot[s], (q0 + e) * 2 + rsub);
+              if (sl[e][s] >= 0) {
+                payload_load<T, BITS>(a.k.s[s], sl[e][s], elem, a.d, a.group, pk[e][s]);
+                payload_load<T, BITS>(a.v.s[s], sl[e][s], elem, a.d, a.group, pv[e][s]);
+              }
+            }
+          if (!landed) { asm volatile("cp.async.wait_group 0;" ::: "memory"); landed = true; }
+#pragma unroll
+          for (int e = 0; e < E; ++e) {
+            const uint32_t o = tile_off((q0 + e) * 2 + rsub, ch);
+            dec_rebuild<BITS, NS>(t_old + o, t_new + o, sl[e], pk[e], pv[e]);
+          }
+        }
+        // rows past the last round: their weights are zero, what they hold must be a number
+#pragma unroll 1
+        for (int q = (n_valid + 2 * E - 1) / (2 * E) * E; q < 8; ++q)
+          *reinterpret_cast<uint4*>(t_new + kMmaTileBytes + tile_off(q * 2 + rsub, ch)) = make_uint4(0, 0, 0, 0);
+        __syncwarp();
+        dec_tile<true>(st, bq, kt, kn, vt, kn + kMmaTileBytes, true, n_valid, a.scale, lse_p, ord_u + first, logit_s, lane);
+        __syncwarp();
+        if (i + 1 < my_tiles_n) issue(i + 1, stage ^ 1);
+      }
+      stage ^= 1;
+    }
   }
   // ---- warps, then CTAs of the cluster, in a fixed order -------------------------------------------------------------
   {
@@ -638,15 +750,21 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
 template <int BITS>
 int launch_decode_mma(const fl_ctx* ctx, const DecodeArgs& a, int n_problems, cudaStream_t st) {
   // Split of a problem: until a CTA has at most 512 columns (lists of ~10 KB, three CTAs per SM), and further while the
-  // CTAs all find room at once (three per SM) and a CTA keeps a tile for each of its warps. One more doubling, into a second
-  // wave, took 29.3 us instead of 17.0 for four queries x 16 heads x 512 columns with three streams.
+  // CTAs all find room at once (three per SM) and a CTA has more than a tile for each of its warps. One more doubling, into
+  // a second wave, took 29.3 us instead of 13.5 for four queries x 16 heads x 512 columns with three streams.
   int split = 1;
   while (split < kMmaMaxSplit && ((a.c + split - 1) / split > 512 ||
-                                  ((int64_t)n_problems * split * 2 <= 3 * ctx->sm_count && a.c >= 2 * split * kMmaWarps * kMmaTile)))
+                                  ((int64_t)n_problems * split * 2 <= 3 * ctx->sm_count && a.c > split * kMmaWarps * kMmaTile)))
     split *= 2;
   const int per_cta = ((a.c + split - 1) / split + kMmaTile - 1) / kMmaTile * kMmaTile;
   const int ns = a.n_old + 1;
-  const size_t smem = decode_mma_smem(per_cta);
+  // Columns per warp of a short piece: dealt evenly while there are at most three CTAs for two SMs (fewer payload rows per
+  // warp: 12 queries x 16 columns with three streams 5.8 us against 6.3), else by whole tiles, so that a CTA takes the shared
+  // memory of fewer warps and more of them run at once (64 queries x 16 columns 14.0 us against 14.9).
+  const bool is_short = per_cta <= kMmaWarps * kMmaTile;
+  const bool even = is_short && 2 * (int64_t)n_problems * split <= 3 * ctx->sm_count;
+  const int per_warp = even ? (min(per_cta, a.c) + kMmaWarps - 1) / kMmaWarps : kMmaTile;
+  const size_t smem = decode_mma_smem(per_cta, per_warp);
   // the partition stages the positions in the tiles; indices are 16 bits wide (implied)
   if ((size_t)per_cta * 4 > (size_t)kMmaWarps * kMmaStages * kMmaStageBytes || smem > (size_t)ctx->max_smem_optin)
     return FL_ERR_UNSUPPORTED;
@@ -657,12 +775,13 @@ int launch_decode_mma(const fl_ctx* ctx, const DecodeArgs& a, int n_problems, cu
   cfg.stream = st;
   cudaLaunchAttribute attr[2];
   fl_cluster_attrs(ctx, split, attr, &cfg);
-#define FL_DECM(NS)                                                                                        \
+#define FL_DECM2(NS, SHORT)                                                                                \
   do {                                                                                                     \
-    auto kern = decode_attn_mma_kernel<BITS, NS>;                                                          \
+    auto kern = decode_attn_mma_kernel<BITS, NS, SHORT>;                                                   \
     FL_FUNC_ATTR_ONCE(ctx, kern, ctx->max_smem_optin, true);                                               \
-    FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, a, split, per_cta));                                      \
+    FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, a, split, per_cta, per_warp));                            \
   } while (0)
+#define FL_DECM(NS) do { if (is_short) FL_DECM2(NS, true); else FL_DECM2(NS, false); } while (0)
   switch (ns) {
     case 1: FL_DECM(1); break;
     case 2: FL_DECM(2); break;
@@ -670,6 +789,7 @@ int launch_decode_mma(const fl_ctx* ctx, const DecodeArgs& a, int n_problems, cu
     default: FL_DECM(4); break;
   }
 #undef FL_DECM
+#undef FL_DECM2
   return fl_launch_status();
 }
 

@@ -58,3 +58,8 @@ def time_of():
 def test_more_queries_do_not_wait_for_a_second_wave(time_of):
     t2, t4 = time_of(2, 512), time_of(4, 512)
     assert t4 < 1.6 * t2, f"two queries {t2:.1f} us, four {t4:.1f} us"          # 15.3 and 29.3 when a list was split too far
+
+
+def test_a_short_list_takes_less_than_a_longer_one(time_of):
+    t64, t512 = time_of(1, 64), time_of(1, 512)
+    assert t64 < 0.72 * t512, f"64 columns {t64:.1f} us, 512 columns {t512:.1f} us"     # 12.2 and 14.3 with one form for all
