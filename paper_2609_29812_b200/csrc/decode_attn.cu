@@ -221,22 +221,6 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
 // eight rows of an 8x8 matrix lie in different banks
 __device__ __forceinline__ uint32_t tile_off(int row, int ch) { return (uint32_t)(row * 256 + ((ch ^ (row & 7)) << 4)); }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ float dsmem_ld(const float* p, uint32_t rank) {
-  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
-  float v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(r) : "memory");
-  return v;
-}
-
 // One stream's payload of eight elements added to their pairs (BITS 16: the stored row takes their place).
 template <int BITS>
 __device__ __forceinline__ void dec_payload(const Payload8<__nv_bfloat16, BITS>& p, fl_codec::f32x2 (&x)[4]) {

@@ -160,6 +160,32 @@ inline cudaError_t fl_launch(const fl_ctx* ctx, void (*kernel)(KArgs...), dim3 g
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// ---- thread-block clusters -------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The place of `p`, an address in this CTA's shared memory, in the shared memory of CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_map(const void* p, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ float dsmem_ld(const float* p, uint32_t rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_map(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint2 dsmem_ld2(const uint32_t* p, uint32_t rank) {
+  uint2 v;
+  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(cluster_map(p, rank)) : "memory");
+  return v;
+}
+
 // Cluster dimension and (unless FL_NO_PDL) programmatic serialization of a launch; attr has room for two.
 static inline void fl_cluster_attrs(const fl_ctx* ctx, int n_ctas, cudaLaunchAttribute* attr, cudaLaunchConfig_t* cfg) {
   int n = 0;

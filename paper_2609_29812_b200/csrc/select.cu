@@ -235,22 +235,6 @@ __device__ __forceinline__ void find_bin(uint32_t c0, uint32_t c1, uint32_t rank
   __syncthreads();
 }
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-__device__ __forceinline__ uint2 dsmem_ld2(const uint32_t* p, uint32_t rank) {
-  uint32_t a = (uint32_t)__cvta_generic_to_shared(p), r;
-  uint2 v;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
-  asm volatile("ld.shared::cluster.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(r) : "memory");
-  return v;
-}
-
 // Token selection by a cluster of CTAs. A single CTA that walks the scores in global memory five times is bound by its
 // latency (53 us for 32 k candidates, 254 us for 128 k); here every CTA of a cluster of `n_ctas` keeps the keys of its
 // piece in shared memory, three radix passes at most find the threshold (the leading bits that all keys share are

@@ -51,87 +51,87 @@ __global__ void __launch_bounds__(kWarps * 32) stale_rows_kernel(const __grid_co
   __syncthreads();
 #pragma unroll 1
   for (int n = tid >> 5; n < n_list; n += kWarps) {
-  const int side = list[n] / kPos, p = list[n] % kPos, j = j0 + p;
-  const DevSide& sd = a.side[side];
-  const int* row_of = slots[side][p];
-  static_assert(FL_MAX_LOOPS <= 32, "one lane per stream");
-  uint32_t streams = __ballot_sync(0xffffffffu, lane < a.n_old && row_of[lane] >= 0);
-  if (BITS == 16 && streams != 0) streams = 1u << (31 - __clz(streams));   // exact rows: the last one is the value
-  const __nv_bfloat16* base = static_cast<const __nv_bfloat16*>(sd.base) + (size_t)j * a.d;
-  __nv_bfloat16* out = a.out[side] + (size_t)j * a.d;
-  constexpr int kWords = BITS == 16 ? 16 : BITS;      // 32-bit words of a chunk's codes
-  const int gs = 31 - __clz(a.group);
+    const int side = list[n] / kPos, p = list[n] % kPos, j = j0 + p;
+    const DevSide& sd = a.side[side];
+    const int* row_of = slots[side][p];
+    static_assert(FL_MAX_LOOPS <= 32, "one lane per stream");
+    uint32_t streams = __ballot_sync(0xffffffffu, lane < a.n_old && row_of[lane] >= 0);
+    if (BITS == 16 && streams != 0) streams = 1u << (31 - __clz(streams));   // exact rows: the last one is the value
+    const __nv_bfloat16* base = static_cast<const __nv_bfloat16*>(sd.base) + (size_t)j * a.d;
+    __nv_bfloat16* out = a.out[side] + (size_t)j * a.d;
+    constexpr int kWords = BITS == 16 ? 16 : BITS;      // 32-bit words of a chunk's codes
+    const int gs = 31 - __clz(a.group);
 #pragma unroll 1
-  for (int c0 = 0; c0 < a.d / kChunk; c0 += 32) {
-    const int e0 = (c0 + lane) * kChunk;
-    const bool mine = e0 < a.d;
-    float x[4][8];
-    if (mine) {
+    for (int c0 = 0; c0 < a.d / kChunk; c0 += 32) {
+      const int e0 = (c0 + lane) * kChunk;
+      const bool mine = e0 < a.d;
+      float x[4][8];
+      if (mine) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) load8<__nv_bfloat16>(base + e0 + i * 8, x[i]);
-    }
+        for (int i = 0; i < 4; ++i) load8<__nv_bfloat16>(base + e0 + i * 8, x[i]);
+      }
 #pragma unroll 1
-    for (uint32_t m = streams; m != 0;) {
-      uint32_t words[kBatch][kWords];
-      __half sc[kBatch][META], zr[kBatch][META];
-      bool have[kBatch];
+      for (uint32_t m = streams; m != 0;) {
+        uint32_t words[kBatch][kWords];
+        __half sc[kBatch][META], zr[kBatch][META];
+        bool have[kBatch];
 #pragma unroll
-      for (int q = 0; q < (BITS == 16 ? 1 : kBatch); ++q) {
-        have[q] = m != 0;
-        if (have[q]) {
-          const int s = __ffs(m) - 1;
-          const size_t row = row_of[s];
-          m &= m - 1;
-          if (mine) {
-            const uint8_t* src = sd.s[s].codes + (row * a.d + e0) * BITS / 8;
-            if (BITS == 2) {
-              const uint2 t = __ldg(reinterpret_cast<const uint2*>(src));
-              words[q][0] = t.x; words[q][1] = t.y;
-            } else {
+        for (int q = 0; q < (BITS == 16 ? 1 : kBatch); ++q) {
+          have[q] = m != 0;
+          if (have[q]) {
+            const int s = __ffs(m) - 1;
+            const size_t row = row_of[s];
+            m &= m - 1;
+            if (mine) {
+              const uint8_t* src = sd.s[s].codes + (row * a.d + e0) * BITS / 8;
+              if (BITS == 2) {
+                const uint2 t = __ldg(reinterpret_cast<const uint2*>(src));
+                words[q][0] = t.x; words[q][1] = t.y;
+              } else {
 #pragma unroll
-              for (int i = 0; i < kWords; i += 4) {
-                const uint4 t = __ldg(reinterpret_cast<const uint4*>(src) + i / 4);
-                words[q][i] = t.x; words[q][i + 1] = t.y; words[q][i + 2] = t.z; words[q][i + 3] = t.w;
+                for (int i = 0; i < kWords; i += 4) {
+                  const uint4 t = __ldg(reinterpret_cast<const uint4*>(src) + i / 4);
+                  words[q][i] = t.x; words[q][i + 1] = t.y; words[q][i + 2] = t.z; words[q][i + 3] = t.w;
+                }
               }
-            }
-            if (BITS != 16) {
+              if (BITS != 16) {
 #pragma unroll
-              for (int i = 0; i < META; ++i) {
-                const size_t gi = row * (a.d >> gs) + ((e0 + i * 8) >> gs);
-                sc[q][i] = __ldg(sd.s[s].scale + gi);
-                zr[q][i] = __ldg(sd.s[s].zero + gi);
+                for (int i = 0; i < META; ++i) {
+                  const size_t gi = row * (a.d >> gs) + ((e0 + i * 8) >> gs);
+                  sc[q][i] = __ldg(sd.s[s].scale + gi);
+                  zr[q][i] = __ldg(sd.s[s].zero + gi);
+                }
               }
             }
           }
         }
-      }
 #pragma unroll
-      for (int q = 0; q < (BITS == 16 ? 1 : kBatch); ++q)
-        if (have[q] && mine) {
+        for (int q = 0; q < (BITS == 16 ? 1 : kBatch); ++q)
+          if (have[q] && mine) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            Payload8<__nv_bfloat16, BITS> pl;
-            if (BITS == 16) pl.raw = make_uint4(words[q][(4 * i) % kWords], words[q][(4 * i + 1) % kWords],
-                                                words[q][(4 * i + 2) % kWords], words[q][(4 * i + 3) % kWords]);
-            else if (BITS == 8) { pl.raw.x = words[q][(2 * i) % kWords]; pl.raw.y = words[q][(2 * i + 1) % kWords]; }
-            else if (BITS == 4) pl.raw.x = words[q][i % kWords];
-            else pl.raw.x = (words[q][(i / 2) % kWords] >> (16 * (i & 1))) & 0xffffu;
-            if (BITS != 16) { pl.sc = sc[q][i % META]; pl.zr = zr[q][i % META]; }
-            payload_apply<__nv_bfloat16, BITS>(pl, x[i]);
+            for (int i = 0; i < 4; ++i) {
+              Payload8<__nv_bfloat16, BITS> pl;
+              if (BITS == 16) pl.raw = make_uint4(words[q][(4 * i) % kWords], words[q][(4 * i + 1) % kWords],
+                                                  words[q][(4 * i + 2) % kWords], words[q][(4 * i + 3) % kWords]);
+              else if (BITS == 8) { pl.raw.x = words[q][(2 * i) % kWords]; pl.raw.y = words[q][(2 * i + 1) % kWords]; }
+              else if (BITS == 4) pl.raw.x = words[q][i % kWords];
+              else pl.raw.x = (words[q][(i / 2) % kWords] >> (16 * (i & 1))) & 0xffffu;
+              if (BITS != 16) { pl.sc = sc[q][i % META]; pl.zr = zr[q][i % META]; }
+              payload_apply<__nv_bfloat16, BITS>(pl, x[i]);
+            }
           }
+      }
+      if (mine) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          uint32_t o[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e)
+            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(o[e]) : "f"(x[i][2 * e + 1]), "f"(x[i][2 * e]));
+          *reinterpret_cast<uint4*>(out + e0 + i * 8) = make_uint4(o[0], o[1], o[2], o[3]);
         }
-    }
-    if (mine) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        uint32_t o[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(o[e]) : "f"(x[i][2 * e + 1]), "f"(x[i][2 * e]));
-        *reinterpret_cast<uint4*>(out + e0 + i * 8) = make_uint4(o[0], o[1], o[2], o[3]);
       }
     }
-  }
   }
 }
 
