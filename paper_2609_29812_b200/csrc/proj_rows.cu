@@ -145,7 +145,7 @@ __device__ __forceinline__ void codec_row(const ProjArgs& a, uint32_t tmem_row, 
           h[u] = pair(xh[2 * u], xh[2 * u + 1]);
           t2[u] = add2(sub2(xn[u], h[u]), nz2);
         }
-        const bool rare = quotients<BITS, 4>(t2, inv, ninv, [&](int) { return s2; }, q);
+        quotients<BITS, 4>(t2, inv, ninv, [&](int) { return s2; }, q);
         if (rows_prev != nullptr) *reinterpret_cast<uint4*>(rows_prev + (size_t)t * d + e_p + v * 8) = fl_codec::pack_bf16(h);
         if (rows_cur != nullptr) {
 #pragma unroll
@@ -154,7 +154,6 @@ __device__ __forceinline__ void codec_row(const ProjArgs& a, uint32_t tmem_row, 
         }
         if (a.kv_out != nullptr)
           *reinterpret_cast<uint4*>(a.kv_out + (size_t)t * (2 * d) + (is_v ? d : 0) + e_p + v * 8) = fl_codec::pack_bf16(xn);
-        if (rare) clean_codes<BITS, 4>(q);
         uint32_t w[BITS == 8 ? 2 : 1];
         pack_codes<BITS, 4>(q, w);
         if constexpr (BITS == 8) { packed[2 * v] = w[0]; packed[2 * v + 1] = w[1]; }

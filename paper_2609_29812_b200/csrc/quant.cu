@@ -79,14 +79,13 @@ __device__ __forceinline__ void encode(const QuantArgs& a, bool is_v, int t, int
       inv[i] = pair(r, r);
       ninv[i] = pair(-r, -r);
     }
-    const bool rare = quotients<BITS, P>(dl, inv, ninv, [&](int) { return s2; }, q);
+    quotients<BITS, P>(dl, inv, ninv, [&](int) { return s2; }, q);
     if (rows_cur != nullptr) {
       // the reconstruction every later reader of this stream forms: Xhat + (code * scale + zero), Eq. 8
 #pragma unroll
       for (int i = 0; i < P; ++i) xh[i] = add2(xh[i], fma2(q[i], s2, z2));
       store_pairs<T, P>(rows_cur + row_off, xh);
     }
-    if (rare) clean_codes<BITS, P>(q);
     store_codes<BITS, P>(codes + row_off * BITS / 8, q);
     constexpr int kLog = P == 8 ? 4 : 3;
     if (((elem >> kLog) & (lanes_per_group - 1)) == 0) {
