@@ -166,8 +166,8 @@ base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas) {
       raw[i].pairs(x);
 #pragma unroll
       for (int e = 0; e < 4; ++e) x[e] = add2(x[e], nz[e]);
-      quotients<BITS, 4, true>(x, inv, ninv, [&](int e) { return *reinterpret_cast<const f32x2*>(&meta[1][lane * 8 + 2 * e]); }, q);
-      store_codes<BITS, 4, false>(dst, q);
+      quotients<BITS, 4>(x, inv, ninv, [&](int e) { return *reinterpret_cast<const f32x2*>(&meta[1][lane * 8 + 2 * e]); }, q);
+      store_codes<BITS, 4>(dst, q);
       dst += (size_t)ROWL * a.d * BITS / 8;
     }
   } else {
@@ -230,9 +230,9 @@ __global__ void __launch_bounds__(kBvThreads) base_quant_v_kernel(const __grid_c
       inv[e] = pair(r, r);
       ninv[e] = pair(-r, -r);
     }
-    quotients<BITS, 8, true>(x, inv, ninv, [&](int) { return pair(s, s); }, q);
+    quotients<BITS, 8>(x, inv, ninv, [&](int) { return pair(s, s); }, q);
     if (!on) continue;
-    store_codes<BITS, 8, false>(a.v_codes + i * 2 * BITS, q);
+    store_codes<BITS, 8>(a.v_codes + i * 2 * BITS, q);
     if ((lane & (lanes_per_group - 1)) == 0) {
       const int64_t gi = (i * 16) >> gs;
       a.v_scale[gi] = sh;

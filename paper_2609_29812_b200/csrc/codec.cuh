@@ -81,11 +81,10 @@ __device__ __forceinline__ float max3_nan(float a, float b, float c) {
 // mantissa bits. No clamp: t >= 0 (the offset was rounded down) and max / scale <= 2^bits - 1 (the scale was rounded up).
 // scale(i) gives the scales of pair i (asked for in the rare branch only: they need not stay in registers).
 // Elements that are not numbers or not finite, and groups whose offset or scale leaves fp16, have quotients that are no
-// integers of the range. CLEAN: they become code 0 (not a number) or the nearest end of the range here, in the rare branch;
-// the maximum keeps a not-a-number, so that they always take it. Without, such quotients stay what they are, for callers
-// whose rows shall show them, and pack_codes looks after them (the residual quantizer with the branch here and a second
-// one around its rows: 17.3 us a call at 1902 rows of 2048, int4, loops 2 to 8; with the check in pack_codes 17.05, without any 16.85).
-template <int BITS, int P, bool CLEAN = false, typename Scale>
+// integers of the range; packed by addition (below) they would spoil the codes of their neighbours, which may belong to other
+// channels and groups. They become code 0 (not a number) or the nearest end of the range, in the rare branch: the maximum
+// keeps a not-a-number, so that they always take it.
+template <int BITS, int P, typename Scale>
 __device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv)[P], const f32x2 (&neg_inv)[P],
                                           Scale scale, f32x2 (&q)[P]) {
   const f32x2 magic = pair(12582912.f, 12582912.f), neg_magic = pair(-12582912.f, -12582912.f);
@@ -97,10 +96,10 @@ __device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv
     const f32x2 fr = fma2(t[i], neg_inv[i], q[i]);   // integer - estimate
     float a, b;
     split(fr, a, b);
-    far = CLEAN ? max3_nan(far, fabsf(a), fabsf(b)) : fmaxf(far, fmaxf(fabsf(a), fabsf(b)));
+    far = max3_nan(far, fabsf(a), fabsf(b));
   }
   constexpr float kNear = 0.5f - (float)(1 << BITS) / 4194304.f;
-  if (CLEAN ? !(far <= kNear) : far > kNear) {
+  if (!(far <= kNear)) {
 #pragma unroll
     for (int i = 0; i < P; ++i) {
       float a, b, sa, sb;
@@ -108,69 +107,51 @@ __device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv
       split(scale(i), sa, sb);
       a = sa == 0.f ? 0.f : rintf(__fdiv_rn(a, sa));
       b = sb == 0.f ? 0.f : rintf(__fdiv_rn(b, sb));
-      q[i] = CLEAN ? pair(fminf(fmaxf(a, 0.f), n), fminf(fmaxf(b, 0.f), n)) : pair(a, b);
+      q[i] = pair(fminf(fmaxf(a, 0.f), n), fminf(fmaxf(b, 0.f), n));
     }
   }
 }
 
 // Packs 2 P codes (integers in binary32) little-endian into P * BITS / 16 words; exact: every partial sum is < 2^23.
-// CHECK: quotients that are no integers of the range (see above) would spoil their word, i.e. the codes of their neighbours:
-// other channels, and other groups where the groups run along the positions. Sums of codes have the exponent of 2^23; one
-// that has not sends the thread round again with such quotients at code 0, or at the nearest end of the range.
-template <int BITS, int P, bool CHECK = true>
+template <int BITS, int P>
 __device__ __forceinline__ void pack_codes(const f32x2 (&q)[P], uint32_t* w) {
-  constexpr int N = BITS == 8 ? P : P / 2;
-  uint32_t sum[N], all = 0;
-  constexpr float r1 = (float)(1 << BITS), r2 = r1 * r1;
+  if constexpr (BITS == 8) {
 #pragma unroll
-  for (int i = 0; i < P; i += 2) {
-    if constexpr (BITS == 8) {
+    for (int i = 0; i < P; i += 2) {
       float a, b, c, d;
       split(q[i], a, b);
       split(q[i + 1], c, d);
-      sum[i] = __float_as_uint(__fmaf_rn(b, 256.f, __fadd_rn(a, 8388608.f)));
-      sum[i + 1] = __float_as_uint(__fmaf_rn(d, 256.f, __fadd_rn(c, 8388608.f)));
-    } else {
+      const uint32_t lo = __float_as_uint(__fmaf_rn(b, 256.f, __fadd_rn(a, 8388608.f)));
+      const uint32_t hi = __float_as_uint(__fmaf_rn(d, 256.f, __fadd_rn(c, 8388608.f)));
+      w[i >> 1] = __byte_perm(lo, hi, 0x5410);
+    }
+  } else {
+    constexpr float r1 = (float)(1 << BITS), r2 = r1 * r1;
+    uint32_t quad[P / 2];
+#pragma unroll
+    for (int i = 0; i < P; i += 2) {
       const f32x2 s = fma2(q[i + 1], pair(r2, r2), add2(q[i], pair(8388608.f, 0.f)));
       float lo, hi;
       split(s, lo, hi);
-      sum[i >> 1] = __float_as_uint(__fmaf_rn(hi, r1, lo));
+      quad[i >> 1] = __float_as_uint(__fmaf_rn(hi, r1, lo));
     }
-  }
-  if constexpr (CHECK) {
+    if constexpr (BITS == 4) {
 #pragma unroll
-    for (int i = 0; i < N; ++i) all |= sum[i];
-    if (all >= 0x4C000000u) {
-      f32x2 c[P];
+      for (int i = 0; i < P / 2; i += 2) w[i >> 1] = __byte_perm(quad[i], quad[i + 1], 0x5410);
+    } else if constexpr (P == 4) {
+      w[0] = __byte_perm(quad[0], quad[1], 0x0040);      // low 16 bits
+    } else {
 #pragma unroll
-      for (int i = 0; i < P; ++i) {
-        float a, b;
-        split(q[i], a, b);
-        c[i] = pair(fminf(fmaxf(a, 0.f), r1 - 1.f), fminf(fmaxf(b, 0.f), r1 - 1.f));     // not a number: 0
-      }
-      pack_codes<BITS, P, false>(c, w);
-      return;
+      for (int i = 0; i < P / 2; i += 4)
+        w[i >> 2] = __byte_perm(__byte_perm(quad[i], quad[i + 1], 0x0040), __byte_perm(quad[i + 2], quad[i + 3], 0x0040), 0x5410);
     }
-  }
-  if constexpr (BITS == 8) {
-#pragma unroll
-    for (int i = 0; i < P; i += 2) w[i >> 1] = __byte_perm(sum[i], sum[i + 1], 0x5410);
-  } else if constexpr (BITS == 4) {
-#pragma unroll
-    for (int i = 0; i < P / 2; i += 2) w[i >> 1] = __byte_perm(sum[i], sum[i + 1], 0x5410);
-  } else if constexpr (P == 4) {
-    w[0] = __byte_perm(sum[0], sum[1], 0x0040);      // low 16 bits
-  } else {
-#pragma unroll
-    for (int i = 0; i < P / 2; i += 4)
-      w[i >> 2] = __byte_perm(__byte_perm(sum[i], sum[i + 1], 0x0040), __byte_perm(sum[i + 2], sum[i + 3], 0x0040), 0x5410);
   }
 }
 // The same words stored where the codes of an element offset begin (P = 4: 8 codes, P = 8: 16 codes).
-template <int BITS, int P, bool CHECK = true>
+template <int BITS, int P>
 __device__ __forceinline__ void store_codes(uint8_t* dst, const f32x2 (&q)[P]) {
   uint32_t w[P * BITS >= 16 ? P * BITS / 16 : 1];
-  pack_codes<BITS, P, CHECK>(q, w);
+  pack_codes<BITS, P>(q, w);
   constexpr int kBytes = P * BITS / 4;
   if constexpr (kBytes == 16) *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
   else if constexpr (kBytes == 8) *reinterpret_cast<uint2*>(dst) = make_uint2(w[0], w[1]);
