@@ -167,11 +167,11 @@ __global__ void __launch_bounds__(kDecThreads) decode_attn_kernel(const __grid_c
 // in registers (Eq. 8 chain) as the rows before and after the loop's own residual and go through two tile pairs.
 // A problem is split over a cluster of SPLIT CTAs (distributed shared memory joins their results): few queries would
 // leave most SMs idle otherwise, and a CTA with at most 512 columns has lists short enough for three CTAs per SM.
-// Long lists are bound by their bytes, 3.3 TB/s of rows at 32 queries x 16 heads x 2048 columns. Few queries are a chain of
-// latencies in each CTA (launch, list, slots, payloads, tiles, merge: 6400 cycles at 16 columns), so pieces of up to 64
-// columns have a form of their own (SHORT). One query x 16 heads, 10% of the columns with payloads, rows in L2, per call:
-// 64 / 256 / 512 columns 4.5 / 6.2 / 7.6 us with one stream, 5.5 / 7.8 / 9.0 with three (one CTA per query and head in
-// registers: 6.1 / 13.6 / 23.3 and 7.3 / 17.4 / 30.7).
+// Long lists are bound by their bytes, 3.6 TB/s of rows at 32 queries x 16 heads x 2048 columns. Few queries are a chain of
+// latencies in each CTA (launch, list, slots, payloads, tiles, merge), so pieces of up to 64 columns have a form of their own
+// (SHORT). One query x 16 heads, 10% of the columns with payloads, rows in L2, per call: 64 / 256 / 512 columns 4.5 / 6.2 /
+// 7.4 us with one stream, 5.5 / 7.5 / 8.8 with three (in registers, one CTA per query and head: 6.1 / 13.6 / 23.3 and 7.3 /
+// 17.4 / 30.7; with one form for all lists 8.9 / 10.4 / 11.3 and 12.2 / 13.5 / 14.3).
 // ------------------------------------------------------------------------------------------------------------
 constexpr int kMmaWarps = 4;
 constexpr int kMmaThreads = kMmaWarps * 32;
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(kMmaThreads, 3) decode_attn_mma_kernel(const _
     // A list this short is one chain of latencies, so nothing is sorted: a warp takes its columns of the list as they come,
     // asks for their base rows and their rows in the streams at once, copies the tile, rebuilds the rows with a payload in
     // both, and makes one pass over the pair. Three dependent trips to memory (list, rows and slots, payloads) and one tile;
-    // the general form (partition, a plain tile, a payload tile) takes 0.6 to 2.4 us longer per call at 16 to 512 columns.
+    // the general form (partition, a plain tile, a payload tile) takes 0.7 to 1.8 us longer per call at 16 to 512 columns.
     const int len = min(per_cta, a.c - part * per_cta), first = warp * per_warp, row0 = lane & (kMmaTile - 1);
     int j = row0 < per_warp && first + row0 < len ? __ldg(cols + first + row0) : 0;    // asked for ahead of the count
     const int n_valid = min(per_warp, n - first);
@@ -743,7 +743,7 @@ int launch_decode_mma(const fl_ctx* ctx, const DecodeArgs& a, int n_problems, cu
   const int per_cta = ((a.c + split - 1) / split + kMmaTile - 1) / kMmaTile * kMmaTile;
   const int ns = a.n_old + 1;
   // Columns per warp of a short piece: dealt evenly while there are at most three CTAs for two SMs (fewer payload rows per
-  // warp: 12 queries x 16 columns with three streams 5.8 us against 6.3), else by whole tiles, so that a CTA takes the shared
+  // warp: 12 queries x 16 columns with three streams 5.7 us against 6.3), else by whole tiles, so that a CTA takes the shared
   // memory of fewer warps and more of them run at once (64 queries x 16 columns 14.0 us against 14.9).
   const bool is_short = per_cta <= kMmaWarps * kMmaTile;
   const bool even = is_short && 2 * (int64_t)n_problems * split <= 3 * ctx->sm_count;

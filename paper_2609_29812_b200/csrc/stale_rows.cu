@@ -3,7 +3,8 @@
 // materialized, so the attention would run the Eq. 8 chain for them wherever their column is selected: once per (query
 // block, head, row tile), on the warps that issue the gathers, stream after stream behind its own loads. At 8192 rows, 90 -
 // 20% of the tokens and 2048 - 256 columns that took most of the attention (loops 3 - 8: 810, 866, 868, 785, 549, 270 us; now
-// 551, 400, 282, 188, 114, 70) and of the next-loop scores (237 - 160 us; now 107 - 31). Here every stale row is rebuilt
+// 456, 339, 242, 164, 94, 49, and this kernel 15, 20, 25, 31, 41, 51) and of the next-loop scores (237 - 160 us; now 115 - 34;
+// times of single launches as profiled, caches cold). Here every stale row is rebuilt
 // once, the loads of up to four streams in flight together, into a buffer [L, d] per side that the consumers gather from
 // by position like from the base. Bound by memory latency: a CTA takes four positions, so that the few stale ones spread
 // over the chip (16 per CTA: 5 us more per loop).
