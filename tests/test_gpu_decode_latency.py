@@ -11,7 +11,8 @@ torch = pytest.importorskip("torch")
 @pytest.fixture(scope="module")
 def time_of():
     """Time of a decode call of one layer (8192 positions, 16 heads, loop 4, a tenth of the rows with payloads), by the number
-    of queries and columns: the best of several replays of a graph of 32 calls, in us."""
+    of queries and columns: the best of several replays of a graph of 32 calls, the mean over four draws of the columns (how many
+    payloads meet in one warp moves a short call by 10%), in us."""
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     from paper_2609_29812_b200 import binding as B, pipeline as P
@@ -30,7 +31,7 @@ def time_of():
         st.alloc_stream(sel, rows=False)
         st.quantize(r, rand(len(act), H, 128), rand(len(act), H, 128), sel)
 
-    def measure(queries, c):
+    def one(queries, c):
         idx = torch.sort(torch.topk(torch.rand(queries * H, L, device="cuda"), c, dim=1)[1], dim=1)[0].to(torch.int32)
         cnt = torch.full((queries, H), c, dtype=torch.int32, device="cuda")
         q, lse, out = rand(3, queries, H, 128), torch.full((queries, H), 9.5, device="cuda"), rand(queries, H, 128)
@@ -51,15 +52,19 @@ def time_of():
             torch.cuda.synchronize()
             best = min(best, a.elapsed_time(b) * 1e3 / calls)
         return best
+
+    def measure(queries, c):
+        return sum(one(queries, c) for _ in range(4)) / 4
     yield measure
     ctx.close()
 
 
 def test_more_queries_do_not_wait_for_a_second_wave(time_of):
     t2, t4 = time_of(2, 512), time_of(4, 512)
-    assert t4 < 1.6 * t2, f"two queries {t2:.1f} us, four {t4:.1f} us"          # 15.3 and 29.3 when a list was split too far
+    assert t4 < 1.6 * t2, f"two queries {t2:.1f} us, four {t4:.1f} us"          # 1.32 (ten runs); 1.92 when a list was split too far
 
 
 def test_a_short_list_takes_less_than_a_longer_one(time_of):
     t64, t512 = time_of(1, 64), time_of(1, 512)
-    assert t64 < 0.72 * t512, f"64 columns {t64:.1f} us, 512 columns {t512:.1f} us"     # 12.2 and 14.3 with one form for all
+    # halfway between 0.64 to 0.72 (ten runs) and the 0.84 of one form for all lists (11.9 and 14.1 us)
+    assert t64 < 0.78 * t512, f"64 columns {t64:.1f} us, 512 columns {t512:.1f} us"
