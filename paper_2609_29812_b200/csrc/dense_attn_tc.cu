@@ -2,15 +2,14 @@
 // (Eq. 2) and the block column statistics loop 2 starts from (Eq. 6 with every causal key a candidate and m_C = 1).
 //
 // Two kernels, because the statistics need each row's final normaliser:
-//   dense_flash_kernel     one CTA per (128-row query tile, head): S = Q K^T per chunk of 64 keys, online softmax with a
+//   dense_flash_kernel     one CTA per (256 query rows, head): S = Q K^T per chunk of 128 keys, online softmax with a
 //                          lazily moved reference, acc += P V; writes O = acc / l and lse = ref + log l.
 //   dense_colsum_kernel    one CTA per (chunk of 512 or 128 keys, head, group of query blocks): S^T = K Q^T with the KEYS as the
 //                          accumulator's rows, so that the thread that owns a key sums exp(s - lse_i) over a block's
 //                          queries in registers, in a fixed order (no atomics, no cross-thread reduction):
 //                          col_scores[h, b, j] = sum_{i in block b, i >= j} p_ij.
-// The flash kernel keeps two CTAs per SM (half the shared memory and 256 tensor-memory columns each) so that one CTA's
-// dependent chain MMA -> exponentials -> MMA runs under the other's. Operand tiles come by plain TMA tile loads (the rows are
-// consecutive), 128B-swizzled; rows beyond L read as zero and are masked. Every mbarrier wait is bounded.
+// Operand tiles come by plain TMA tile loads (the rows are consecutive), 128B-swizzled; rows beyond L read as zero and are
+// masked. Every mbarrier wait is bounded.
 #include "tc_attn_common.cuh"
 #include <algorithm>
 
@@ -25,9 +24,7 @@ constexpr uint32_t kAcc = 0, kS = 128;
 constexpr uint32_t kTmemCols = 256;
 
 struct alignas(64) DnArgs {
-  CUtensorMap q_map;      // [L, d] bf16, box 64 elements x 128 rows
-  CUtensorMap k_map;      // box 64 x 64 rows (flash: a chunk of keys) or 64 x 128 rows (column sums: K is the M operand)
-  CUtensorMap v_map;      // box 64 x 64 rows
+  CUtensorMap q_map, k_map, v_map;   // [L, d] bf16, box 64 elements x 128 rows
   __nv_bfloat16* o;       // [L, d]
   float* lse;             // [H, L] (flash: written, may be null; column sums: read)
   float* col_scores;      // [H, nb, L]
@@ -36,41 +33,65 @@ struct alignas(64) DnArgs {
   float scale;
 };
 
+// ------------------------------------------------------------------------------------------------------------
+// Flash. A CTA takes two neighbouring query tiles of a head, which share every key and value tile that comes in. Chunks of
+// 128 keys: an M128 x N128 x K16 MMA reads 8 KB of operands from shared memory in the 64 cycles that it takes, an N64 one
+// 6 KB in 48. Tensor memory (512 columns): two accumulators, ONE S that the tiles use in turn, a P each. S is free again as
+// soon as its 128 columns are in the softmax threads' registers, so QK^T of either tile runs under the exponentials of both;
+// with a P that takes the place of its S, a tile's chain S -> P -> PV -> next S is longer than the work on the tensor pipe.
+// QK^T and PV are issued by a thread each: a wait between two batches of one thread costs the pipe about 200 cycles.
+// Bound by the turns at S: QK^T, its 250 cycles of latency and the hand-over to the other tile take 1.5 k of the 2.9 k cycles
+// that a chunk of both tiles lasts, in which the tensor pipe works for 2048 and the exponential unit for 2048. 32768 x 16
+// heads, one call 3865 -> 3266 us, back to back at the power cap 4377 -> 3720; 8192 x 16: 289 -> 245. Measured before: one
+// query tile and 64 keys, two CTAs per SM (the first figures); P over its own S, one issuing thread: 4139 us (4218 without a
+// maximum in the softmax); part of the exponentials on the FMA pipe: 3620 us and more, their chains are longer.
+// ------------------------------------------------------------------------------------------------------------
+constexpr int kFlWarps = 11;                       // 0-3 softmax of the first tile, 4-7 of the second, then:
+constexpr int kFlQk = 8, kFlPv = 9, kFlTma = 10;
+constexpr int kFlSlots = 4;                        // ring of K and V tiles in the order K0 V0 K1 V1 ...
+constexpr int kFlNC = 128;                         // keys per chunk
+constexpr uint32_t kFlAcc = 0, kFlS = 256, kFlP = 384;     // tensor-memory columns: accumulators, S, P (64 columns each)
 struct __align__(16) FlashCtl {
-  uint64_t q_full, k_landed[2], v_landed[2], s_full[2], p_full[2], p_free[2], acc_done;
+  uint64_t q_full[2];                              // TMA -> QK issuer: the tile's Q
+  uint64_t kv_full[kFlSlots], kv_free[kFlSlots];   // TMA -> issuers, issuers -> TMA
+  uint64_t s_full[2], s_free[2];                   // QK issuer -> softmax: S of the tile's chunk; back: it is in registers
+  uint64_t p_full[2], pv_done[2];                  // softmax -> PV issuer: P of the chunk; back: the MMAs that read it are done
   uint32_t tmem_base;
   int abort_flag;
 };
-constexpr size_t kFlashSmem = 1024 + kQTileBytes + 4 * kTileBytes + sizeof(FlashCtl);
+constexpr size_t kFlashSmem = 1024 + 2 * kQTileBytes + kFlSlots * kQTileBytes + sizeof(FlashCtl);
 
-__global__ void __launch_bounds__(kThreads, 2) dense_flash_kernel(const __grid_constant__ DnArgs a) {
+__global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __grid_constant__ DnArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* q_tile = smem;
-  uint8_t* k_ring = smem + kQTileBytes;
-  uint8_t* v_ring = k_ring + 2 * kTileBytes;
-  FlashCtl& ctl = *reinterpret_cast<FlashCtl*>(v_ring + 2 * kTileBytes);
+  uint8_t* q_tiles = smem;
+  uint8_t* ring = smem + 2 * kQTileBytes;
+  FlashCtl& ctl = *reinterpret_cast<FlashCtl*>(ring + kFlSlots * kQTileBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // later tiles see more keys: they are dispatched first
-  const int n_tiles = (a.L + kM - 1) / kM;
-  const int tile = n_tiles - 1 - (int)(blockIdx.x / a.H), h = blockIdx.x % a.H;
-  const int s0 = tile * kM, n_rows = min(kM, a.L - s0);
-  const int n_chunks = (s0 + n_rows + kNC - 1) / kNC;
+  const int n_pairs = (a.L + 2 * kM - 1) / (2 * kM);
+  const int h = blockIdx.x % a.H, s0 = (n_pairs - 1 - (int)(blockIdx.x / a.H)) * 2 * kM;
+  // chunks of the two tiles (the second may have no rows, else it sees at least as many keys as the first)
+  const int n_first = (min(a.L, s0 + kM) + kFlNC - 1) / kFlNC;
+  const int n_second = s0 + kM < a.L ? (min(a.L, s0 + 2 * kM) + kFlNC - 1) / kFlNC : 0;
+  const int n_chunks = max(n_first, n_second);
   if (tid == 0) {
-    tc::mbar_init(&ctl.q_full, 1);
-    for (int s = 0; s < 2; ++s) {
-      tc::mbar_init(&ctl.k_landed[s], 1);
-      tc::mbar_init(&ctl.v_landed[s], 1);
-      tc::mbar_init(&ctl.s_full[s], 1);
-      tc::mbar_init(&ctl.p_full[s], 4);
-      tc::mbar_init(&ctl.p_free[s], 1);
+    for (int s = 0; s < kFlSlots; ++s) {
+      tc::mbar_init(&ctl.kv_full[s], 1);
+      tc::mbar_init(&ctl.kv_free[s], 1);
     }
-    tc::mbar_init(&ctl.acc_done, 1);
+    for (int t = 0; t < 2; ++t) {
+      tc::mbar_init(&ctl.q_full[t], 1);
+      tc::mbar_init(&ctl.s_full[t], 1);
+      tc::mbar_init(&ctl.s_free[t], 4);
+      tc::mbar_init(&ctl.p_full[t], 4);
+      tc::mbar_init(&ctl.pv_done[t], 1);
+    }
     ctl.abort_flag = 0;
     tc::fence_barrier_init();
   }
-  if (warp == kIssueWarp) {
-    tc::tmem_alloc(&ctl.tmem_base, kTmemCols);
+  if (warp == kFlQk) {
+    tc::tmem_alloc(&ctl.tmem_base, 512);
     tc::tmem_relinquish();
   }
   tc::tc_fence_before();
@@ -79,203 +100,191 @@ __global__ void __launch_bounds__(kThreads, 2) dense_flash_kernel(const __grid_c
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
 
-  if (warp == kTmaWarp) {
+  if (warp == kFlTma) {
     if (lane == 0) {
-      tc::mbar_arrive_expect_tx(&ctl.q_full, kQTileBytes);
-      tc::tma_tile2d(q_tile, &a.q_map, &ctl.q_full, h * kDH, s0);
-      tc::tma_tile2d(q_tile + kM * 128, &a.q_map, &ctl.q_full, h * kDH + 64, s0);
-      auto fill = [&](int ci, bool is_v) {
-        uint64_t* bar = is_v ? &ctl.v_landed[ci & 1] : &ctl.k_landed[ci & 1];
-        uint8_t* dst = (is_v ? v_ring : k_ring) + (ci & 1) * kTileBytes;
-        const void* map = is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map);
-        tc::mbar_arrive_expect_tx(bar, kTileBytes);
-        tc::tma_tile2d(dst, map, bar, h * kDH, ci * kNC);
-        tc::tma_tile2d(dst + kNC * 128, map, bar, h * kDH + 64, ci * kNC);
+      auto load = [&](uint8_t* dst, const void* map, uint64_t* bar, int row) {
+        tc::mbar_arrive_expect_tx(bar, kQTileBytes);
+        tc::tma_tile2d(dst, map, bar, h * kDH, row);
+        tc::tma_tile2d(dst + kM * 128, map, bar, h * kDH + 64, row);
       };
-      bool ok = true;
-      fill(0, false);
-      // K of chunk n + 1 (free once QK^T of chunk n - 1 has completed), then V of chunk n (free once PV of n - 2 has)
-      for (int ci = 0; ci < n_chunks && ok; ++ci) {
-        if (ci + 1 < n_chunks) {
-          if (ci + 1 >= 2) ok = tc::mbar_wait(&ctl.s_full[(ci + 1) & 1], (((ci + 1) >> 1) - 1) & 1, abort_flag);
-          if (!ok) break;
-          fill(ci + 1, false);
-        }
-        if (ci >= 2) ok = tc::mbar_wait(&ctl.p_free[ci & 1], ((ci >> 1) - 1) & 1, abort_flag);
-        if (!ok) break;
-        fill(ci, true);
+      load(q_tiles, &a.q_map, &ctl.q_full[0], s0);
+      for (int i = 0; i < 2 * n_chunks; ++i) {
+        const int sl = i % kFlSlots;
+        if (i >= kFlSlots && !tc::mbar_wait(&ctl.kv_free[sl], (i / kFlSlots - 1) & 1, abort_flag)) break;
+        load(ring + sl * kQTileBytes, (i & 1) ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map),
+             &ctl.kv_full[sl], (i >> 1) * kFlNC);
+        if (i == 0 && n_second > 0) load(q_tiles + kQTileBytes, &a.q_map, &ctl.q_full[1], s0 + kM);
       }
     }
     __syncwarp();
-  } else if (warp == kIssueWarp) {
+  } else if (warp == kFlQk) {
     if (lane == 0) {
-      const uint32_t idesc_qk = tc::make_idesc_bf16(kM, kNC, false);
-      const uint32_t idesc_pv = tc::make_idesc_bf16(kM, kDH, true);
-      const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32(q_tile), 16, 1024);
-      const uint64_t k_desc0 = tc::make_desc_sw128(tc::smem_u32(k_ring), 16, 1024);
-      const uint32_t kq_hi = (uint32_t)(k_desc0 >> 32);
-      const uint32_t q_lo_w = (uint32_t)q_desc, k_lo0 = (uint32_t)k_desc0;
-      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(v_ring), kNC * 128, 1024);
-      const uint32_t v_hi = (uint32_t)(v_desc0 >> 32), v_lo0 = (uint32_t)v_desc0;
-      const uint32_t s_base = tmem + kS, acc = tmem + kAcc;
+      const uint32_t idesc = tc::make_idesc_bf16(kM, kFlNC, false);
+      const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32(q_tiles), 16, 1024);
+      const uint64_t k_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), 16, 1024);
+      const uint32_t hi = (uint32_t)(k_desc0 >> 32);
+      const uint32_t q_lo0 = (uint32_t)q_desc, k_lo0 = (uint32_t)k_desc0, s_dst = tmem + kFlS;
+      bool ok = true;
 #pragma unroll 1
-      for (int n = 0; n <= n_chunks; ++n) {
-        if (n < n_chunks) {
-          const int sl = n & 1;
-          if (n == 0 && !tc::mbar_wait(&ctl.q_full, 0, abort_flag)) break;
-          if (!tc::mbar_wait(&ctl.k_landed[sl], (n >> 1) & 1, abort_flag)) break;
-          if (n >= 2 && !tc::mbar_wait(&ctl.p_free[sl], ((n >> 1) - 1) & 1, abort_flag)) break;
-          const uint32_t s_dst = s_base + sl * kNC;
-          tc::tc_fence_after();
-          const uint32_t k_lo = k_lo0 + sl * (kTileBytes >> 4);
+      for (int i = 0; i < 2 * n_chunks; ++i) {           // tiles in turn
+        const int n = i >> 1, t = i & 1, sl = (2 * n) % kFlSlots;
+        if (n >= (t ? n_second : n_first)) continue;      // (the last tile of a chunk frees its K)
+        if (n == 0) ok = tc::mbar_wait(&ctl.q_full[t], 0, abort_flag);
+        if (!ok || !tc::mbar_wait(&ctl.kv_full[sl], (2 * n / kFlSlots) & 1, abort_flag)) break;
+        // the S before this one: the other tile's, or the same tile's where the other has none
+        if (i > 0) {
+          const bool other = t ? n < n_first : n - 1 < n_second;
+          const int po = other ? t ^ 1 : t, pn = other && t ? n : n - 1;
+          if (!tc::mbar_wait(&ctl.s_free[po], pn & 1, abort_flag)) break;
+        }
+        tc::tc_fence_after();
+        const uint32_t q_lo = q_lo0 + t * (kQTileBytes >> 4), k_lo = k_lo0 + sl * (kQTileBytes >> 4);
 #define FL_QK(KK, ACC)                                                                                       \
-  tc::mma_ss_lo<ACC>(s_dst, q_lo_w + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), kq_hi,               \
-                     k_lo + ((((KK) >> 2) * (kNC * 128) + ((KK)&3) * 32) >> 4), kq_hi, idesc_qk)
-          FL_QK(0, false); FL_QK(1, true); FL_QK(2, true); FL_QK(3, true);
-          FL_QK(4, true);  FL_QK(5, true); FL_QK(6, true); FL_QK(7, true);
+  tc::mma_ss_lo<ACC>(s_dst, q_lo + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), hi,                    \
+                     k_lo + ((((KK) >> 2) * (kFlNC * 128) + ((KK)&3) * 32) >> 4), hi, idesc)
+        FL_QK(0, false); FL_QK(1, true); FL_QK(2, true); FL_QK(3, true);
+        FL_QK(4, true);  FL_QK(5, true); FL_QK(6, true); FL_QK(7, true);
 #undef FL_QK
-          tc::mma_commit(&ctl.s_full[sl]);
-        }
-        if (n > 0) {
-          const int gp = n - 1, pb = gp & 1;
-          if (!tc::mbar_wait(&ctl.v_landed[pb], (gp >> 1) & 1, abort_flag)) break;
-          if (!tc::mbar_wait(&ctl.p_full[pb], (gp >> 1) & 1, abort_flag)) break;
-          tc::tc_fence_after();
-          const uint32_t v_lo = v_lo0 + pb * (kTileBytes >> 4);
-          const uint32_t p_src = s_base + pb * kNC;
-          const uint32_t acc0 = n > 1 ? 1u : 0u;
-#pragma unroll
-          for (int kk = 0; kk < kNC / 16; ++kk)
-            tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc_pv, kk > 0 ? 1u : acc0);
-          tc::mma_commit(&ctl.p_free[pb]);
-        }
+        tc::mma_commit(&ctl.s_full[t]);
+        if (t == 1 || n >= n_second) tc::mma_commit(&ctl.kv_free[sl]);
       }
-      tc::mma_commit(&ctl.acc_done);
+    }
+    __syncwarp();
+  } else if (warp == kFlPv) {
+    if (lane == 0) {
+      const uint32_t idesc = tc::make_idesc_bf16(kM, kDH, true);
+      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), kFlNC * 128, 1024);   // MN-major
+      const uint32_t v_hi = (uint32_t)(v_desc0 >> 32), v_lo0 = (uint32_t)v_desc0;
+#pragma unroll 1
+      for (int i = 0; i < 2 * n_chunks; ++i) {
+        const int n = i >> 1, t = i & 1, vi = 2 * n + 1, sl = vi % kFlSlots;
+        if (n >= (t ? n_second : n_first)) continue;
+        if (!tc::mbar_wait(&ctl.kv_full[sl], (vi / kFlSlots) & 1, abort_flag)) break;
+        if (!tc::mbar_wait(&ctl.p_full[t], n & 1, abort_flag)) break;
+        tc::tc_fence_after();
+        const uint32_t v_lo = v_lo0 + sl * (kQTileBytes >> 4), p_src = tmem + kFlP + t * 64, acc = tmem + kFlAcc + t * kDH;
+#pragma unroll
+        for (int kk = 0; kk < kFlNC / 16; ++kk)            // the first chunk overwrites the accumulator
+          tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc, (n == 0 && kk == 0) ? 0u : 1u);
+        tc::mma_commit(&ctl.pv_done[t]);
+        if (t == 1 || n >= n_second) tc::mma_commit(&ctl.kv_free[sl]);
+      }
     }
     __syncwarp();
   } else {
     // ============================================ softmax ============================================
-    const int row = warp * 32 + lane;
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+    const int t = warp >> 2, gt = tid & 127;           // tile, thread inside its group of four warps
+    const int row = (warp & 3) * 32 + lane;
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    const int lo = s0 + t * kM, n_rows = min(kM, a.L - lo), n_t = t ? n_second : n_first;
     const bool row_ok = row < n_rows;
-    const int pos = s0 + row;
+    const int pos = lo + row;
     const float c2 = a.scale * kLog2e;
-    const uint32_t s_addr = tmem + lane_base + kS;
+    const uint32_t s_addr = tmem + lane_base + kFlS, p_addr = tmem + lane_base + kFlP + t * 64;
+    const uint32_t acc_addr = tmem + lane_base + kFlAcc + t * kDH;
     float ell = 0.f, ref = -INFINITY;
     bool ok = true;
-    for (int ci = 0; ci < n_chunks; ++ci) {
-      const int pb = ci & 1;
-      if (!warp_wait(&ctl.s_full[pb], (ci >> 1) & 1, abort_flag)) { ok = false; break; }
+    for (int n = 0; n < n_t; ++n) {
+      if (!warp_wait(&ctl.s_full[t], n & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
-      // causal mask: the chunk's columns are 64 ci .. 64 ci + 63; the visible ones of a row are a prefix
-      const bool unmasked = __all_sync(0xffffffffu, !row_ok || ci * kNC + kNC - 1 <= pos);
-      const int vis = row_ok ? min(kNC, max(0, pos - ci * kNC + 1)) : 0;
-      const uint32_t sp_addr = s_addr + pb * kNC;
-#pragma unroll 1
-      for (int hf = 0; hf < 2 && ok; ++hf) {
-        uint32_t r[32];
-        tc::tmem_ld32(sp_addr + hf * 32, r);
-        tc::tmem_wait_ld();
-        if (!unmasked) {
-          const int lim = vis - hf * 32;
+      uint32_t r[4][32];
 #pragma unroll
-          for (int u = 0; u < 32; ++u) r[u] = u < lim ? r[u] : 0xff800000u;
-        }
-        float cm = -INFINITY;
+      for (int q = 0; q < 4; ++q) tc::tmem_ld32(s_addr + q * 32, r[q]);
+      tc::tmem_wait_ld();
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&ctl.s_free[t]);
+      // causal mask: the visible keys of a row are a prefix of the chunk
+      if (!__all_sync(0xffffffffu, !row_ok || n * kFlNC + kFlNC - 1 <= pos)) {
+        const int vis = row_ok ? max(0, pos - n * kFlNC + 1) : 0;
 #pragma unroll
-        for (int u = 0; u < 32; u += 2) cm = fmaxf(cm, fmaxf(__uint_as_float(r[u]), __uint_as_float(r[u + 1])));
-        cm *= c2;
-        const bool first = ref == -INFINITY && cm > -INFINITY;
-        const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
-        if (first) ref = cm;
-        if (__any_sync(0xffffffffu, over)) {
-          float factor = 1.f;
-          if (over) { factor = tc::ex2(ref - cm); ref = cm; }
-          if (ci > 0) {
-            if (!warp_wait(&ctl.p_free[(ci - 1) & 1], ((ci - 1) >> 1) & 1, abort_flag)) { ok = false; break; }
-            tc::tc_fence_after();
-#pragma unroll 1
-            for (int q4 = 0; q4 < 8; ++q4) {
-              uint32_t acc[16];
-              tc::tmem_ld16(tmem + lane_base + kAcc + q4 * 16, acc);
-              tc::tmem_wait_ld();
+        for (int q = 0; q < 4; ++q)
 #pragma unroll
-              for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * factor);
-              tc::tmem_st16(tmem + lane_base + kAcc + q4 * 16, acc);
-            }
-            tc::tmem_wait_st();
-          }
-          ell *= factor;
-          if (hf == 1) {
-            uint32_t ph[16];
-            tc::tmem_wait_st();
-            tc::tmem_ld16(sp_addr, ph);
-            tc::tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&ph[i]);
-              const float2 f = __bfloat1622float2(v);
-              ph[i] = tc::pack_bf16(f.x * factor, f.y * factor);
-            }
-            tc::tmem_st16(sp_addr, ph);
-          }
-        }
-        const float sub = ref == -INFINITY ? 0.f : ref;
-        float sum = 0.f;
-#pragma unroll
-        for (int u = 0; u < 32; u += 2) {
-          const float p0 = tc::ex2(fmaf(__uint_as_float(r[u]), c2, -sub));
-          const float p1 = tc::ex2(fmaf(__uint_as_float(r[u + 1]), c2, -sub));
-          sum += p0 + p1;
-          r[u >> 1] = tc::pack_bf16(p0, p1);
-        }
-        ell += sum;
-        tc::tmem_st16(sp_addr + hf * 16, *reinterpret_cast<uint32_t(*)[16]>(&r[0]));
+          for (int u = 0; u < 32; ++u) r[q][u] = q * 32 + u < vis ? r[q][u] : 0xff800000u;
       }
-      if (!ok) break;
+      // running reference: taken from the first keys that show a finite logit (the accumulator row is still zero then) and
+      // moved, with a rescale of the accumulator row, only when a maximum beats it by more than the threshold
+      const float cm0 = max32(r[0]) * c2;
+      const float cm = fmaxf(fmaxf(cm0, max32(r[1]) * c2), fmaxf(max32(r[2]), max32(r[3])) * c2);
+      if (ref == -INFINITY) ref = cm0 > -INFINITY ? cm0 : cm;
+      const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
+      const bool any_over = __any_sync(0xffffffffu, over);
+      const float old_ref = ref;
+      if (over) ref = cm;
+      const float sub = ref == -INFINITY ? 0.f : ref;
+      uint32_t p0[16], p1[16];
+      float sum = exp32(r[0], c2, sub, p0) + exp32(r[1], c2, sub, p1);
+      // the P before this one must have been read, and with it every earlier PV has completed
+      if (n > 0 && !warp_wait(&ctl.pv_done[t], (n - 1) & 1, abort_flag)) { ok = false; break; }
+      tc::tc_fence_after();
+      if (any_over) {
+        const float factor = over ? tc::ex2(old_ref - ref) : 1.f;
+        ell *= factor;
+#pragma unroll 1
+        for (int q4 = 0; q4 < 8 && n > 0; ++q4) {
+          uint32_t acc[16];
+          tc::tmem_ld16(acc_addr + q4 * 16, acc);
+          tc::tmem_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * factor);
+          tc::tmem_st16(acc_addr + q4 * 16, acc);
+        }
+      }
+      tc::tmem_st16(p_addr, p0);
+      tc::tmem_st16(p_addr + 16, p1);
+      sum += exp32(r[2], c2, sub, p0);
+      tc::tmem_st16(p_addr + 32, p0);
+      sum += exp32(r[3], c2, sub, p1);
+      tc::tmem_st16(p_addr + 48, p1);
+      ell += sum;
       tc::tmem_wait_st();
       tc::tc_fence_before();
       __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&ctl.p_full[pb]);
+      if (lane == 0) tc::mbar_arrive(&ctl.p_full[t]);
     }
-    // ---- epilogue: O = acc / l, staged in the Q tile (every QK^T has retired) and written out coalesced ---------
-    if (ok) ok = warp_wait(&ctl.acc_done, 0, abort_flag);
-    tc::tc_fence_after();
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    const float w = (ok && ell > 0.f) ? 1.f / ell : 0.f;
-    uint8_t* stage = q_tile;
+    // ---- epilogue: O = acc / l, staged in the tile's Q (every QK^T has retired) and written out coalesced -------
+    if (n_t > 0) {
+      if (ok) ok = warp_wait(&ctl.pv_done[t], (n_t - 1) & 1, abort_flag);
+      tc::tc_fence_after();
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
+      const float w = (ok && ell > 0.f) ? 1.f / ell : 0.f;
+      uint8_t* stage = q_tiles + t * kQTileBytes;
 #pragma unroll 1
-    for (int c16 = 0; c16 < 16; ++c16) {
-      uint32_t av[8];
-      tc::tmem_ld8(tmem + lane_base + kAcc + c16 * 8, av);
-      tc::tmem_wait_ld();
-      float pv[8];
+      for (int c0 = 0; c0 < kDH; c0 += 32) {
+        uint32_t av[32];
+        tc::tmem_ld32(acc_addr + c0, av);
+        tc::tmem_wait_ld();
 #pragma unroll
-      for (int i = 0; i < 8; ++i) pv[i] = w * __uint_as_float(av[i]);
-      *reinterpret_cast<uint4*>(stage + row * 256 + ((c16 ^ (row & 7)) << 4)) = pack8(pv);
-    }
-    if (row_ok && a.lse != nullptr && ok) a.lse[(size_t)h * a.L + pos] = (ref + log2f(ell)) * kLn2;
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    if (ok) {
-#pragma unroll 1
-      for (int k = 0; k < 16; ++k) {
-        const int idx = k * 128 + tid, rr = idx >> 4, cc = idx & 15;
-        if (rr < n_rows)
-          *reinterpret_cast<uint4*>(a.o + (size_t)(s0 + rr) * a.d + (size_t)h * kDH + cc * 8) =
-              *reinterpret_cast<const uint4*>(stage + rr * 256 + ((cc ^ (rr & 7)) << 4));
+        for (int q = 0; q < 4; ++q) {
+          float pv[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) pv[i] = w * __uint_as_float(av[q * 8 + i]);
+          *reinterpret_cast<uint4*>(stage + row * 256 + (((c0 / 8 + q) ^ (row & 7)) << 4)) = pack8(pv);
+        }
+      }
+      if (row_ok && a.lse != nullptr && ok) a.lse[(size_t)h * a.L + pos] = (ref + log2f(ell)) * kLn2;
+      asm volatile("bar.sync %0, 128;" ::"r"(1 + t) : "memory");
+      if (ok) {
+#pragma unroll 4
+        for (int k = 0; k < 16; ++k) {
+          const int idx = k * 128 + gt, rr = idx >> 4, cc = idx & 15;
+          if (rr < n_rows)
+            *reinterpret_cast<uint4*>(a.o + (size_t)(lo + rr) * a.d + (size_t)h * kDH + cc * 8) =
+                *reinterpret_cast<const uint4*>(stage + rr * 256 + ((cc ^ (rr & 7)) << 4));
+        }
       }
     }
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == kIssueWarp) {
+  if (warp == kFlQk) {
     if (ctl.abort_flag) {
-      if (lane == 0) tc::mma_commit(&ctl.acc_done);
+      if (lane == 0) tc::mma_commit(&ctl.pv_done[0]);
       __syncwarp();
       for (int it = 0; it < (1 << 16); ++it) __nanosleep(256);
     }
     tc::tc_fence_after();
-    tc::tmem_dealloc(tmem, kTmemCols);
+    tc::tmem_dealloc(tmem, 512);
   }
   if (tid == 0 && ctl.abort_flag && a.status != nullptr) atomicExch(a.status, (int)FL_ERR_TIMEOUT);
 }
@@ -769,8 +778,8 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
     return FL_ERR_UNSUPPORTED;
   DnArgs a{};
   const int64_t d_row = (int64_t)s->n_heads * s->head_dim;
-  if (!fl_tile_tmap(ctx, q, s->L, d_row, kM, &a.q_map) || !fl_tile_tmap(ctx, k, s->L, d_row, kNC, &a.k_map) ||
-      !fl_tile_tmap(ctx, v, s->L, d_row, kNC, &a.v_map))
+  if (!fl_tile_tmap(ctx, q, s->L, d_row, kM, &a.q_map) || !fl_tile_tmap(ctx, k, s->L, d_row, kM, &a.k_map) ||
+      !fl_tile_tmap(ctx, v, s->L, d_row, kM, &a.v_map))
     return FL_ERR_UNSUPPORTED;
   a.o = static_cast<__nv_bfloat16*>(o);
   a.lse = lse;
@@ -780,10 +789,9 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
   a.scale = s->sm_scale;
   const int n_tiles = (s->L + kM - 1) / kM;
   FL_FUNC_ATTR_ONCE(ctx, dense_flash_kernel, kFlashSmem, true);
-  dense_flash_kernel<<<dim3(n_tiles * s->n_heads), kThreads, kFlashSmem, st>>>(a);
+  dense_flash_kernel<<<dim3((n_tiles + 1) / 2 * s->n_heads), kFlWarps * 32, kFlashSmem, st>>>(a);
   int rc = fl_launch_status();
   if (rc != FL_OK || col_scores == nullptr) return rc;
-  if (!fl_tile_tmap(ctx, k, s->L, d_row, kM, &a.k_map)) return FL_ERR_CUDA;
   // 512 keys per CTA where that still gives (with one job per query block) three jobs to two SMs, else 128; the blocks are
   // dealt to as many CTAs as make two jobs per SM slot, and never to one (half a head's queries stay in L2 at 32K rows).
   // Measured, one CTA per (keys, head) / dealt: 2500 x 8 heads 34 / 21 us (128 keys; 512: 26), 2500 x 16 57 / 29 (512 keys;

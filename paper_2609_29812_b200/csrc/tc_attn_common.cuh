@@ -78,18 +78,25 @@ __device__ __forceinline__ void unpack8(const uint4& raw, float (&x)[8]) {
   }
 }
 
+// The largest of three numbers in one instruction (numbers win over not-a-number, as with fmaxf).
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float r;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+}
+
 // Largest of 32 logits, in four chains.
 __device__ __forceinline__ float max32(const uint32_t (&r)[32]) {
   float m[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) m[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 4; ++i) m[i] = max3(__uint_as_float(r[i]), __uint_as_float(r[i + 4]), __uint_as_float(r[i + 8]));
 #pragma unroll
-  for (int u = 4; u < 32; u += 8)
+  for (int u = 12; u < 28; u += 8)
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      m[i] = u + 4 < 32 ? fmaxf(fmaxf(m[i], __uint_as_float(r[u + i])), __uint_as_float(r[(u + 4 + i) & 31]))
-                        : fmaxf(m[i], __uint_as_float(r[u + i]));
-  return fmaxf(fmaxf(m[0], m[1]), fmaxf(m[2], m[3]));
+    for (int i = 0; i < 4; ++i) m[i] = max3(m[i], __uint_as_float(r[u + i]), __uint_as_float(r[u + 4 + i]));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) m[i] = fmaxf(m[i], __uint_as_float(r[28 + i]));
+  return fmaxf(max3(m[0], m[1], m[2]), m[3]);
 }
 
 // P = 2^(s c2 - sub) of 32 logits: 16 packed bf16 pairs into p, returns the sum of the unrounded values. A softmax warp
