@@ -61,6 +61,23 @@ struct __align__(16) FlashCtl {
 };
 constexpr size_t kFlashSmem = 1024 + 2 * kQTileBytes + kFlSlots * kQTileBytes + sizeof(FlashCtl);
 
+// P = 2^(s c2 - sub) of 32 logits, as exp32, with the sum taken in ONE order (pair by pair): the row sums, and with them O to
+// the last bit, do not depend on how the keys are cut into chunks. The chain of additions runs beside the exponentials.
+__device__ __forceinline__ float exp32_in_order(const uint32_t (&r)[32], float c2, float sub, uint32_t (&p)[16]) {
+  using namespace fl_codec;
+  const f32x2 cc = pair(c2, c2), ns = pair(-sub, -sub);
+  float sum = 0.f;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    float x0, x1;
+    split(fma2(pair_u(r[2 * u], r[2 * u + 1]), cc, ns), x0, x1);
+    const float p0 = tc::ex2(x0), p1 = tc::ex2(x1);
+    sum += p0 + p1;
+    p[u] = tc::pack_bf16(p0, p1);
+  }
+  return sum;
+}
+
 __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __grid_constant__ DnArgs a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -213,7 +230,7 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
       if (over) ref = cm;
       const float sub = ref == -INFINITY ? 0.f : ref;
       uint32_t p0[16], p1[16];
-      float sum = exp32(r[0], c2, sub, p0) + exp32(r[1], c2, sub, p1);
+      const float sum0 = exp32_in_order(r[0], c2, sub, p0), sum1 = exp32_in_order(r[1], c2, sub, p1);
       // the P before this one must have been read, and with it every earlier PV has completed
       if (n > 0 && !warp_wait(&ctl.pv_done[t], (n - 1) & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
@@ -232,11 +249,12 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
       }
       tc::tmem_st16(p_addr, p0);
       tc::tmem_st16(p_addr + 16, p1);
-      sum += exp32(r[2], c2, sub, p0);
+      ell += sum0;
+      ell += sum1;
+      ell += exp32_in_order(r[2], c2, sub, p0);
       tc::tmem_st16(p_addr + 32, p0);
-      sum += exp32(r[3], c2, sub, p1);
+      ell += exp32_in_order(r[3], c2, sub, p1);
       tc::tmem_st16(p_addr + 48, p1);
-      ell += sum;
       tc::tmem_wait_st();
       tc::tc_fence_before();
       __syncwarp();
