@@ -4,7 +4,8 @@
 // is made first) and whose epilogue writes, or adds into, rows of a position-indexed matrix (the output projection with
 // its residual add scattered back).
 //
-// Persistent kernel, one CTA per SM, 128 x 256 (or 128 x 128) output tiles in a static round-robin order (tiles that share their
+// Two persistent kernels: pairs of CTAs that share a tile (further down) where a cost rule says that they are faster, and
+// one CTA per SM, 128 x 256 (or 128 x 128) output tiles in a static round-robin order (tiles that share their
 // rows of X run side by side on neighbouring SMs). K advances in slabs of 64 elements through a ring of four
 // (16 KB of A + 32 KB of W) stages; tcgen05.mma M128 x N256 x K16 accumulates in one of two accumulators
 // in tensor memory, so that the epilogue of a tile (tensor memory -> registers -> bf16 -> global) runs under the
@@ -15,6 +16,7 @@
 //   warp  5    W slabs (one tile copy per stage); the A slabs too when the rows are not gathered
 //   warps 6-13 A row gathers: four lanes per warp, one four-row copy each per stage
 #include "tc_attn_common.cuh"
+#include <algorithm>
 
 namespace {
 
@@ -43,7 +45,7 @@ struct ProjArgs {
   const int32_t* src_idx;   // [n] rows of X, or null
   const int32_t* dst_idx;   // [n] rows of Y, or null
   __nv_bfloat16* y;
-  int n, d_in, d_out;
+  int n, d_in, d_out, x_rows;
   int y_stride, y_cols;     // row stride of y and the number of output columns that go to it
   int m_tiles, n_tiles;
   int accumulate;
@@ -190,6 +192,60 @@ __device__ __forceinline__ void mma_ss_acc(uint32_t d_tmem, uint32_t a_lo, uint3
       : "memory");
 }
 
+// A tile's plain epilogue by the thread that owns row m: y (+)= the accumulator's `width` columns. `release` is called by the
+// whole warp once the accumulator is in registers (the issuer may then start the tile after next). False: the accumulator
+// never came.
+template <class Release>
+__device__ __forceinline__ bool store_tile(const ProjArgs& a, uint32_t acc, bool row_ok, int m, int n0, int width, uint64_t* full,
+                                           uint32_t parity, volatile int* abort_flag, Release release) {
+  const int64_t dst_row = row_ok ? (a.dst_idx != nullptr ? (int64_t)__ldg(a.dst_idx + m) : (int64_t)m) : 0;
+  __nv_bfloat16* y_row = a.y + dst_row * a.y_stride + n0;
+  // the rows this tile adds into are read one piece ahead of the accumulator (the first piece before the
+  // accumulator is even complete): nothing else writes them during the launch
+  const bool rmw = a.accumulate != 0 && row_ok;
+  const int pieces = width / 32;
+  uint4 old_cur[4], old_nxt[4];
+#pragma unroll
+  for (int v = 0; v < 4; ++v) {
+    old_cur[v] = make_uint4(0u, 0u, 0u, 0u);
+    if (rmw && n0 + v * 8 < a.y_cols) old_cur[v] = *reinterpret_cast<const uint4*>(y_row + v * 8);
+  }
+  if (!warp_wait(full, parity, abort_flag)) return false;
+  tc::tc_fence_after();
+#pragma unroll 1
+  for (int p = 0; p < pieces; ++p) {
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+      old_nxt[v] = make_uint4(0u, 0u, 0u, 0u);
+      if (rmw && p + 1 < pieces && n0 + (p + 1) * 32 + v * 8 < a.y_cols)
+        old_nxt[v] = *reinterpret_cast<const uint4*>(y_row + (p + 1) * 32 + v * 8);
+    }
+    uint32_t r[32];
+    tc::tmem_ld32(acc + p * 32, r);
+    tc::tmem_wait_ld();
+    if (p == pieces - 1) {
+      tc::tc_fence_before();
+      __syncwarp();
+      release();
+    }
+    if (row_ok) {
+#pragma unroll
+      for (int v = 0; v < 4; ++v) {
+        if (n0 + p * 32 + v * 8 < a.y_cols) {
+          float x[8], old[8];
+          fl_tc::unpack8(old_cur[v], old);      // zeros unless the call accumulates
+#pragma unroll
+          for (int u = 0; u < 8; ++u) x[u] = __uint_as_float(r[v * 8 + u]) + old[u];
+          *reinterpret_cast<uint4*>(y_row + p * 32 + v * 8) = fl_tc::pack8(x);
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < 4; ++v) old_cur[v] = old_nxt[v];
+  }
+  return true;
+}
+
 template <bool GATHER, int kBN, int CODEC>   // CODEC: 0, or the bit width of the fused residual codec (wide tiles only)
 __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_constant__ ProjArgs a) {
   constexpr int kBBytes = kBN * kBK * 2;
@@ -234,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
         const int m0 = (w / a.n_tiles) * kBM + g4 * 4;
         int r[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] = __ldg(a.src_idx + min(m0 + q, a.n - 1));   // rows past n repeat the last row
+        for (int q = 0; q < 4; ++q) r[q] = m0 + q < a.n ? __ldg(a.src_idx + m0 + q) : a.x_rows;   // a row outside X reads as zero
         for (int ks = 0; ks < n_slabs; ++ks, ++g) {
           const int st = g % kStages;
           if (g >= kStages) ok = warp_wait(&ctl.empty[st], ((g / kStages) - 1) & 1, abort_flag);
@@ -310,51 +366,10 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
                                           n0 - (is_v ? 2 : 1) * a.d_model, &ctl.acc_free[buf], lane);
         continue;
       }
-      const int64_t dst_row = row_ok ? (a.dst_idx != nullptr ? (int64_t)__ldg(a.dst_idx + m) : (int64_t)m) : 0;
-      __nv_bfloat16* y_row = a.y + dst_row * a.y_stride + n0;
-      // the rows this tile adds into are read one piece ahead of the accumulator (the first piece before the
-      // accumulator is even complete): nothing else writes them during the launch
-      const bool rmw = a.accumulate != 0 && row_ok;
-      uint4 old_cur[4], old_nxt[4];
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        old_cur[v] = make_uint4(0u, 0u, 0u, 0u);
-        if (rmw && n0 + v * 8 < a.y_cols) old_cur[v] = *reinterpret_cast<const uint4*>(y_row + v * 8);
-      }
-      if (!warp_wait(&ctl.acc_full[buf], (i >> 1) & 1, abort_flag)) break;
-      tc::tc_fence_after();
-#pragma unroll 1
-      for (int p = 0; p < kBN / 32; ++p) {
-#pragma unroll
-        for (int v = 0; v < 4; ++v) {
-          old_nxt[v] = make_uint4(0u, 0u, 0u, 0u);
-          if (rmw && p + 1 < kBN / 32 && n0 + (p + 1) * 32 + v * 8 < a.y_cols)
-            old_nxt[v] = *reinterpret_cast<const uint4*>(y_row + (p + 1) * 32 + v * 8);
-        }
-        uint32_t r[32];
-        tc::tmem_ld32(tmem + lane_base + buf * kBN + p * 32, r);
-        tc::tmem_wait_ld();
-        if (p == kBN / 32 - 1) {
-          // the accumulator is in registers: the issuer may start the tile after next
-          tc::tc_fence_before();
-          __syncwarp();
-          if (lane == 0) tc::mbar_arrive(&ctl.acc_free[buf]);
-        }
-        if (row_ok) {
-#pragma unroll
-          for (int v = 0; v < 4; ++v) {
-            if (n0 + p * 32 + v * 8 < a.y_cols) {
-              float x[8], old[8];
-              fl_tc::unpack8(old_cur[v], old);      // zeros unless the call accumulates
-#pragma unroll
-              for (int u = 0; u < 8; ++u) x[u] = __uint_as_float(r[v * 8 + u]) + old[u];
-              *reinterpret_cast<uint4*>(y_row + p * 32 + v * 8) = fl_tc::pack8(x);
-            }
-          }
-        }
-#pragma unroll
-        for (int v = 0; v < 4; ++v) old_cur[v] = old_nxt[v];
-      }
+      if (!store_tile(a, tmem + lane_base + buf * kBN, row_ok, m, n0, kBN, &ctl.acc_full[buf], (i >> 1) & 1, abort_flag, [&]() {
+            if (lane == 0) tc::mbar_arrive(&ctl.acc_free[buf]);
+          }))
+        break;
     }
   }
   tc::tc_fence_before();
@@ -372,7 +387,217 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
   if (tid == 0 && ctl.abort_flag && a.status != nullptr) atomicExch(a.status, (int)FL_ERR_TIMEOUT);
 }
 
+// ---- two CTAs per tile ---------------------------------------------------------------------------------------
+// The plain projection by pairs of neighbouring SMs (tcgen05 with cta_group::2): a pair computes 256 x bn output tiles, each CTA
+// brings in its own 128 rows of X and HALF of the tile's rows of W, which the MMAs of both read: a 256-column tile costs a CTA
+// 32 KB per slab where the kernel above takes 48 KB, and the slabs are what that kernel waits for (950 cycles for 512 of MMA).
+// The CTA of rank 0 issues the MMAs; the copies of both CTAs complete on ITS barriers (with a thread of the other CTA passing its
+// own barriers on, slab by slab, a slab took 2000 cycles). Accumulators, epilogue and tile order as above, per CTA. The tile's width is chosen per call so that the last round over the pairs is full.
+constexpr int kPairStages = 6;
+constexpr int kPairStageBytes = kABytes + 128 * kBK * 2;    // 16 KB of A + up to 16 KB of W
+
+struct __align__(16) PairCtl {
+  uint64_t full[kPairStages];          // rank 0: both CTAs' parts of the stage have arrived
+  uint64_t empty[kPairStages];
+  uint64_t acc_full[2], acc_free[2];   // acc_free of rank 0 counts the epilogue warps of both
+  uint32_t tmem_base;
+  int abort_flag;
+};
+constexpr int pair_threads(bool gather) { return (kFirstGatherWarp + (gather ? kGatherWarps : 0)) * 32; }
+constexpr size_t kPairSmem = 1024 + (size_t)kPairStages * kPairStageBytes + sizeof(PairCtl);
+
+__device__ __forceinline__ void arrive_at(uint64_t* bar, uint32_t rank) {      // on the barrier of the pair's CTA `rank`
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_map(bar, rank)) : "memory");
+}
+// Copies into this CTA's shared memory that complete on a barrier of either CTA of the pair (`bar`: its address in the cluster).
+// No multicast.
+__device__ __forceinline__ void pair_gather4(void* dst, const void* tmap, uint32_t bar, int x, int y0, int y1, int y2, int y3) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes.cta_group::2 "
+      "[%0], [%1, {%3, %4, %5, %6, %7}], [%2];"
+      ::"r"(tc::smem_u32(dst)), "l"(tmap), "r"(bar), "r"(x), "r"(y0), "r"(y1), "r"(y2), "r"(y3)
+      : "memory");
+}
+__device__ __forceinline__ void pair_tile2d(void* dst, const void* tmap, uint32_t bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(tc::smem_u32(dst)), "l"(tmap), "r"(bar), "r"(x), "r"(y)
+      : "memory");
+}
+__device__ __forceinline__ void pair_commit(uint64_t* bar) {                    // arrives on the barrier of both CTAs
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(tc::smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void mma_pair(uint32_t d_tmem, uint32_t a_lo, uint32_t b_lo, uint32_t hi, uint32_t idesc, uint32_t accum) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+      "setp.ne.b32 p, %5, 0;\n\t"
+      "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %4, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_lo), "r"(b_lo), "r"(hi), "r"(idesc), "r"(accum)
+      : "memory");
+}
+
+template <bool GATHER>
+__global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(const __grid_constant__ ProjArgs a, int bn) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  PairCtl& ctl = *reinterpret_cast<PairCtl*>(smem + (size_t)kPairStages * kPairStageBytes);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cluster_rank();
+  const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
+  const int n_slabs = a.d_in / kBK;
+  const int n_work = a.m_tiles * a.n_tiles;          // tiles of 256 rows
+
+  if (tid == 0) {
+    for (int s = 0; s < kPairStages; ++s) {
+      tc::mbar_init(&ctl.full[s], GATHER ? 1 + kGatherWarps : 1);
+      tc::mbar_init(&ctl.empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      tc::mbar_init(&ctl.acc_full[b], 1);
+      tc::mbar_init(&ctl.acc_free[b], 8);
+    }
+    ctl.abort_flag = 0;
+    tc::fence_barrier_init();
+  }
+  if (warp == kIssueWarp) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(tc::smem_u32(&ctl.tmem_base)), "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  cluster_sync();                                    // the other CTA's barriers are there
+  tc::tc_fence_after();
+  const uint32_t tmem = ctl.tmem_base;
+  volatile int* abort_flag = &ctl.abort_flag;
+  fl_grid_wait();
+  fl_grid_release();
+
+  if (warp >= kFirstGatherWarp) {
+    if (GATHER) {
+      const int g4 = (warp - kFirstGatherWarp) * 4 + (lane & 3);     // the lane's group of four rows inside the CTA's 128
+      bool ok = true;
+      int g = 0;
+      for (int w = pair; w < n_work && ok; w += n_pairs) {
+        const int m0 = (w / a.n_tiles) * (2 * kBM) + (int)rank * kBM + g4 * 4;
+        int r[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) r[q] = m0 + q < a.n ? __ldg(a.src_idx + m0 + q) : a.x_rows;   // a row outside X reads as zero
+        for (int ks = 0; ks < n_slabs; ++ks, ++g) {
+          const int st = g % kPairStages;
+          if (g >= kPairStages) ok = warp_wait(&ctl.empty[st], ((g / kPairStages) - 1) & 1, abort_flag);
+          if (!ok) break;
+          // rank 0 announces the bytes of both (the other's may come first: the phase stays open for the announcement)
+          if (rank == 0 && lane == 0) tc::mbar_arrive_expect_tx(&ctl.full[st], 2 * 4 * 512);
+          __syncwarp();
+          if (lane < 4)
+            pair_gather4(smem + (size_t)st * kPairStageBytes + g4 * 512, &a.x_map, cluster_map(&ctl.full[st], 0), ks * kBK, r[0], r[1],
+                         r[2], r[3]);
+        }
+      }
+    }
+  } else if (warp == kLoadWarp) {
+    bool ok = true;
+    int g = 0;
+    for (int w = pair; w < n_work && ok; w += n_pairs) {
+      const int m0 = (w / a.n_tiles) * (2 * kBM) + (int)rank * kBM, n0 = (w % a.n_tiles) * bn + (int)rank * (bn / 2);
+      for (int ks = 0; ks < n_slabs; ++ks, ++g) {
+        const int st = g % kPairStages;
+        if (g >= kPairStages) ok = warp_wait(&ctl.empty[st], ((g / kPairStages) - 1) & 1, abort_flag);
+        if (!ok) break;
+        if (lane == 0) {
+          uint8_t* stage = smem + (size_t)st * kPairStageBytes;
+          if (rank == 0) tc::mbar_arrive_expect_tx(&ctl.full[st], (GATHER ? 0 : 2 * kABytes) + bn * kBK * 2);
+          const uint32_t bar = cluster_map(&ctl.full[st], 0);
+          pair_tile2d(stage + kABytes, &a.w_map, bar, ks * kBK, n0);
+          if (!GATHER) pair_tile2d(stage, &a.x_map, bar, ks * kBK, m0);
+        }
+        __syncwarp();
+      }
+    }
+    // the MMAs' last arrivals on this CTA's barriers have come: it may leave
+    for (int k = max(0, g - kPairStages); k < g && ok; ++k) ok = warp_wait(&ctl.empty[k % kPairStages], (k / kPairStages) & 1, abort_flag);
+  } else if (warp == kIssueWarp) {
+    if (lane == 0 && rank == 0) {
+      const uint32_t idesc = tc::make_idesc_bf16(2 * kBM, bn, false);
+      const uint64_t desc0 = tc::make_desc_sw128(tc::smem_u32(smem), 16, 1024);
+      const uint32_t hi = (uint32_t)(desc0 >> 32), lo0 = (uint32_t)desc0;
+      int g = 0, i = 0;
+      bool ok = true;
+      for (int w = pair; w < n_work && ok; w += n_pairs, ++i) {
+        const int buf = i & 1;
+        if (i >= 2) ok = tc::mbar_wait(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
+        if (!ok) break;
+        tc::tc_fence_after();
+        const uint32_t d_dst = tmem + buf * 256;
+        for (int ks = 0; ks < n_slabs; ++ks, ++g) {
+          const int st = g % kPairStages;
+          if (!tc::mbar_wait(&ctl.full[st], (g / kPairStages) & 1, abort_flag)) { ok = false; break; }
+          tc::tc_fence_after();
+          const uint32_t a_lo = lo0 + ((st * kPairStageBytes) >> 4), b_lo = a_lo + (kABytes >> 4);
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk) mma_pair(d_dst, a_lo + kk * 2, b_lo + kk * 2, hi, idesc, (ks | kk) != 0 ? 1u : 0u);
+          pair_commit(&ctl.empty[st]);
+        }
+        if (ok) pair_commit(&ctl.acc_full[buf]);
+      }
+    }
+    __syncwarp();
+  } else {
+    // epilogue: the thread's row of the CTA's half of the tile is its lane of tensor memory
+    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
+    int i = 0;
+    for (int w = pair; w < n_work; w += n_pairs, ++i) {
+      const int buf = i & 1;
+      const int m = (w / a.n_tiles) * (2 * kBM) + (int)rank * kBM + warp * 32 + lane, n0 = (w % a.n_tiles) * bn;
+      if (!store_tile(a, tmem + lane_base + buf * 256, m < a.n, m, n0, bn, &ctl.acc_full[buf], (i >> 1) & 1, abort_flag, [&]() {
+            if (lane == 0) arrive_at(&ctl.acc_free[buf], 0);
+          }))
+        break;
+    }
+  }
+  tc::tc_fence_before();
+  __syncthreads();
+  if (ctl.abort_flag) {
+    // give copies and MMAs still in flight time to land before the memory is returned
+    if (warp == kIssueWarp)
+      for (int it = 0; it < (1 << 16); ++it) __nanosleep(256);
+    __syncthreads();
+  }
+  cluster_sync();                                    // nothing of this pair is on its way to the other CTA any more
+  if (warp == kIssueWarp) {
+    tc::tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+  if (tid == 0 && ctl.abort_flag && a.status != nullptr) atomicExch(a.status, (int)FL_ERR_TIMEOUT);
+}
+
 }  // namespace
+
+constexpr double kNarrowCost = 0.73;     // of a tile of 128 columns, one of 256 being 1
+
+// Width of the pairs' tiles, or 0 where the one-CTA kernel (tiles of `bn` columns, `rounds` rounds over the SMs) is the faster one.
+// Cycles as measured (d_in 2048, 60 to 12000 rows): a slab of the one-CTA kernel 762, gathered 846 (128 columns: 0.73 of that);
+// of a pair 100 + 2.52 bn, gathered 280 + 2.1 bn; a launch of pairs takes 3300 more (clusters, the pairs' barriers). Pairs are
+// taken where they gain 3% by that. 3277 rows of 32768, d = 2048: Q/K/V 73.7 -> 67.8 us (rows in order 67.3 -> 60.5), output
+// projection added into the store 35.3 -> 28.7; 12000 rows: 260 -> 245 (235 -> 205), 101 -> 97.
+static int fl_proj_pair_width(const fl_ctx* ctx, int n, int d_in, int d_out, bool gather, int bn, double rounds) {
+  if ((size_t)ctx->max_smem_optin < kPairSmem) return 0;
+  const int64_t m_tiles = (n + 2 * kBM - 1) / (2 * kBM), pairs = ctx->sm_count / 2;
+  const double slabs = d_in / kBK;
+  double best = rounds * slabs * (gather ? 846.0 : 762.0) * (bn == 256 ? 0.97 : 0.97 * kNarrowCost);
+  int width = 0;
+  for (int w = 256; w >= 128; w -= 32) {
+    const int64_t tiles = m_tiles * ((d_out + w - 1) / w);
+    const double cost = (double)((tiles + pairs - 1) / pairs) * slabs * (gather ? 280.0 + 2.1 * w : 100.0 + 2.52 * w) + 3300.0;
+    if (cost < best) { best = cost; width = w; }
+  }
+  return width;
+}
 
 extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const int32_t* src_idx, int32_t n,
                                int32_t d_in, const void* w, int32_t d_out, void* y, int64_t y_rows,
@@ -399,14 +624,16 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
   ProjArgs a = {};
   const bool gather = src_idx != nullptr;
   a.m_tiles = (n + kBM - 1) / kBM;
-  // Tile width: 256 columns keep the tensor pipe busiest per byte loaded; 128 columns when that leaves the last of the
-  // rounds over the SMs mostly empty (a narrow tile costs about 0.58 of a wide one, 0.8 when its rows are gathered).
+  // Tile width: 256 columns keep the tensor pipe busiest per byte loaded; 128 columns when that leaves the last of the rounds
+  // over the SMs mostly empty (a narrow tile costs 0.73 of a wide one: 558 cycles a slab for 762, with the SMs full).
   const auto rounds = [&](int bn) {
     const int64_t tiles = (int64_t)a.m_tiles * ((d_out + bn - 1) / bn);
     return (double)((tiles + ctx->sm_count - 1) / ctx->sm_count);
   };
-  const int bn = rounds(128) * (gather ? 0.8 : 0.58) < rounds(256) ? 128 : 256;
-  if (!fl_tile_tmap(ctx, x, x_rows, d_in, gather ? 1 : kBM, &a.x_map) || !fl_tile_tmap(ctx, w, d_out, d_in, bn, &a.w_map))
+  const int bn = rounds(128) * kNarrowCost < rounds(256) ? 128 : 256;
+  const int pair_bn = fl_proj_pair_width(ctx, n, d_in, d_out, gather, bn, rounds(bn));
+  if (!fl_tile_tmap(ctx, x, x_rows, d_in, gather ? 1 : kBM, &a.x_map) ||
+      !fl_tile_tmap(ctx, w, d_out, d_in, pair_bn > 0 ? pair_bn / 2 : bn, &a.w_map))
     return FL_ERR_CUDA;
   a.src_idx = src_idx;
   a.dst_idx = dst_idx;
@@ -416,13 +643,34 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
   a.d_out = d_out;
   a.y_stride = d_out;
   a.y_cols = d_out;
+  a.x_rows = (int)x_rows;
   a.d_model = 0;
   a.n_tiles = (d_out + bn - 1) / bn;
   a.accumulate = accumulate;
   a.status = status;
+  cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (pair_bn > 0) {
+    a.m_tiles = (n + 2 * kBM - 1) / (2 * kBM);
+    a.n_tiles = (d_out + pair_bn - 1) / pair_bn;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * std::min(a.m_tiles * a.n_tiles, ctx->sm_count / 2));
+    cfg.blockDim = dim3(pair_threads(gather));
+    cfg.dynamicSmemBytes = kPairSmem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    fl_cluster_attrs(ctx, 2, attr, &cfg);
+#define FL_PAIR(G)                                                        \
+  do {                                                                    \
+    auto kern = proj_pair_kernel<G>;                                      \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kPairSmem, false);                       \
+    FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, a, pair_bn));            \
+  } while (0)
+    if (gather) FL_PAIR(true); else FL_PAIR(false);
+#undef FL_PAIR
+    return fl_launch_status();
+  }
   const int64_t n_work = (int64_t)a.m_tiles * a.n_tiles;
   const int grid = (int)(n_work < ctx->sm_count ? n_work : ctx->sm_count);
-  cudaStream_t st = static_cast<cudaStream_t>(stream);
 #define FL_PROJ(G, BN)                                                                                              \
   do {                                                                                                              \
     auto kern = proj_rows_kernel<G, BN, 0>;                                                                          \
@@ -482,6 +730,7 @@ extern "C" int fl_project_qkv_quant(fl_ctx* ctx, const fl_shape* shape, int loop
   a.d_out = 3 * d;
   a.y_stride = d;
   a.y_cols = d;
+  a.x_rows = (int)x_rows;
   a.m_tiles = (n_active + kBM - 1) / kBM;
   a.n_tiles = 3 * d / 256;
   a.accumulate = 0;

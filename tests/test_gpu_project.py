@@ -86,6 +86,20 @@ def test_project_rows_several_tiles_per_cta(env):
     check(B, ctx, x, w, y, src, dst, n, 1, rows=rows)
 
 
+@pytest.mark.parametrize("n,d_out,gather,scatter,accumulate", [
+    (1229, 2056, False, True, 1),    # one round; the last tile's second half starts beyond the last column
+    (2500, 3000, True, True, 0),     # two tiles per pair, gathered; 88 columns in a last tile of 224
+    (2561, 2048, False, True, 1),    # the last 256 rows hold one: nothing for the second CTA
+    (3277, 6144, True, False, 0),
+])
+def test_project_rows_pairs_of_ctas(env, n, d_out, gather, scatter, accumulate):
+    """Sizes for which pairs of CTAs share a tile: ragged rows and columns, accumulators used in turn."""
+    B, ctx = env
+    args = make(29, 2 * n if gather else n, 2 * n if scatter else n, n, 2048, d_out, gather, scatter)
+    rows = np.unique(np.r_[0, 127, 128, 255, 256, n - 2, n - 1, np.arange(5, n, 97)])
+    check(B, ctx, *args, n, accumulate, rows=rows)
+
+
 def test_project_rows_single_row_and_empty(env):
     B, ctx = env
     x, w, y, src, dst = make(9, 50, 50, 1, 64, 8, True, True)
