@@ -6,6 +6,8 @@
 // type), so that the cache at rest is the packed form and the bf16 rows are a transient working copy of one layer.
 // HBM-bound kernels, 16-byte accesses, bit-exact arithmetic (binary32, directed fp16 roundings of the metadata).
 #include "codec.cuh"
+#include "tc_ptx.cuh"
+#include <algorithm>
 
 namespace {
 
@@ -30,6 +32,7 @@ template <>
 struct Raw8<__nv_bfloat16> {
   uint4 r;
   __device__ __forceinline__ void load(const __nv_bfloat16* p) { r = __ldg(reinterpret_cast<const uint4*>(p)); }
+  __device__ __forceinline__ void load_smem(const uint4* p) { r = *p; }
   __device__ __forceinline__ void pairs(f32x2 (&x)[4]) const { unpack_bf16(r, x); }
   __device__ __forceinline__ void store(__nv_bfloat16* p) const { *reinterpret_cast<uint4*>(p) = r; }
   static __device__ __forceinline__ uint32_t lo2(uint32_t a, uint32_t b) {
@@ -96,80 +99,111 @@ struct Pair2<float> {
 // dependent walk over the group's rows, and more than ~8 instructions an element (two passes of 64 dependent rows per
 // thread and a division per element took 129 us for the keys and 76 us for the values of 20 k rows of 2048, 0.8 TB/s).
 //
-// Keys: a CTA owns 256 channels of one token group, 32 pieces of 8 channels by ROWL row lanes; a thread loads its rows
-// at once, keeps them in registers, and after the group's minimum and maximum per channel have been joined in shared
-// memory encodes them from there. The CTAs past k_ctas copy the tail rows.
+// Keys: a tile is 256 channels of one token group, 32 pieces of 8 channels by ROWL row lanes; a thread has the tile's rows of its
+// piece at once, and after the group's minimum and maximum per channel have been joined in shared memory encodes them. A CTA
+// (1024 threads per SM in all) walks its tiles: with 16-bit storage a thread asks for its pieces of the tiles NST - 1 ahead
+// by asynchronous copies into slots of its own, so that HBM is read under the joins and the encoding (a CTA per tile, which
+// asked, joined and encoded one after the other, two at a time on an SM: 40 us for the 20 k rows of 2048, now 34.6). With 32-bit storage (NST = 0) a
+// tile takes twice the space and a CTA takes one. The CTAs past k_ctas copy the tail rows.
 template <typename T>
 constexpr int kBqRows = sizeof(T) == 2 ? 4 : 8;        // rows of a token group per thread
-constexpr int kBqCh = 256;                             // channels of a key CTA
+constexpr int kBqCh = 256;                             // channels of a key tile
+template <typename T>
+constexpr int kBqStages = sizeof(T) == 2 ? 2 : 0;
 
 template <typename T, int BITS, int ROWL>
 __global__ void __launch_bounds__(32 * ROWL, (sizeof(T) == 2 ? 1024 : 512) / (32 * ROWL))
-base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas) {
-  constexpr int kThreads = 32 * ROWL;
+base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas, int n_tiles) {
+  constexpr int kThreads = 32 * ROWL, NST = kBqStages<T>, R = kBqRows<T>;
+  extern __shared__ __align__(16) uint4 slots[];       // [NST][R][kThreads]
   __shared__ __align__(16) T red[2][ROWL][kBqCh];
   __shared__ __align__(16) float meta[3][kBqCh];       // offset (negated), scale, reciprocal
   fl_grid_wait();
   fl_grid_release();
   const int tid = threadIdx.x, lane = tid & 31;
   if (blockIdx.x < (unsigned)k_ctas) {
-    const int slabs = a.d / kBqCh;
-    const int g = blockIdx.x / slabs, c0 = (blockIdx.x - g * slabs) * kBqCh;
-    const int elem = c0 + lane * 8, rl = tid >> 5;
-    const int t0 = g * a.group + rl, t1 = min(a.Lq, (g + 1) * a.group);
-    const T* k = static_cast<const T*>(a.k) + elem;
-    Raw8<T> raw[kBqRows<T>];
+    const int slabs = a.d / kBqCh, rl = tid >> 5;
+    const T* k = static_cast<const T*>(a.k) + lane * 8;
+    auto row_of = [&](int tile, int i) {               // a short last group repeats its first row (changes no extremum)
+      const int g = tile / slabs, c0 = (tile - g * slabs) * kBqCh;
+      const int t = g * a.group + rl + i * ROWL;
+      return k + (size_t)(t < min(a.Lq, (g + 1) * a.group) ? t : g * a.group) * a.d + c0;
+    };
+    auto ask = [&](int tile, int st) {
+      if (tile < n_tiles)
 #pragma unroll
-    for (int i = 0; i < kBqRows<T>; ++i) {             // a short last group repeats its first row (changes no extremum)
-      const int t = t0 + i * ROWL < t1 ? t0 + i * ROWL : g * a.group;
-      raw[i].load(k + (size_t)t * a.d);
-    }
-    Raw8<T> mn = raw[0], mx = raw[0];
+        for (int i = 0; i < R; ++i) tc::cp_async16(&slots[(st * R + i) * kThreads + tid], row_of(tile, i));
+      tc::cp_async_commit();
+    };
+    int st = 0;
+    if constexpr (NST > 0)
 #pragma unroll
-    for (int i = 1; i < kBqRows<T>; ++i) { mn.take_min(raw[i]); mx.take_max(raw[i]); }
-    mn.store(&red[0][rl][lane * 8]);
-    mx.store(&red[1][rl][lane * 8]);
-    __syncthreads();
-    for (int ch = tid * 2; ch < kBqCh; ch += kThreads * 2) {     // two channels per thread
-      Pair2<T> lo, hi;
-      lo.load(&red[0][0][ch]);
-      hi.load(&red[1][0][ch]);
+      for (int s = 0; s < NST; ++s) ask(blockIdx.x + s * k_ctas, s);
+    for (int tile = blockIdx.x; tile < n_tiles; tile += k_ctas) {
+      const int g = tile / slabs, c0 = (tile - g * slabs) * kBqCh;
+      const int elem = c0 + lane * 8;
+      const int t0 = g * a.group + rl, t1 = min(a.Lq, (g + 1) * a.group);
+      Raw8<T> raw[R];
+      if constexpr (NST > 0) {
+        tc::cp_async_wait<NST - 1>();
 #pragma unroll
-      for (int r = 1; r < ROWL; ++r) { lo.take_min(&red[0][r][ch]); hi.take_max(&red[1][r][ch]); }
-      const float2 l2 = lo.floats(), h2 = hi.floats();
-      __half zh[2], sh[2];
-      group_meta<BITS>(l2.x, h2.x, zh[0], sh[0]);
-      group_meta<BITS>(l2.y, h2.y, zh[1], sh[1]);
-      *reinterpret_cast<__half2*>(a.k_zero + (size_t)g * a.d + c0 + ch) = __halves2half2(zh[0], zh[1]);
-      *reinterpret_cast<__half2*>(a.k_scale + (size_t)g * a.d + c0 + ch) = __halves2half2(sh[0], sh[1]);
+        for (int i = 0; i < R; ++i) raw[i].load_smem(&slots[(st * R + i) * kThreads + tid]);
+      } else {
 #pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const float s = __half2float(sh[e]);
-        meta[0][ch + e] = -__half2float(zh[e]);
-        meta[1][ch + e] = s;
-        meta[2][ch + e] = scale_rcp(s);
+        for (int i = 0; i < R; ++i) raw[i].load(row_of(tile, i));
+      }
+      Raw8<T> mn = raw[0], mx = raw[0];
+#pragma unroll
+      for (int i = 1; i < R; ++i) { mn.take_min(raw[i]); mx.take_max(raw[i]); }
+      mn.store(&red[0][rl][lane * 8]);
+      mx.store(&red[1][rl][lane * 8]);
+      __syncthreads();
+      if constexpr (NST > 0) {                         // the slots have been read (by their only thread)
+        ask(tile + NST * k_ctas, st);
+        st = st + 1 == NST ? 0 : st + 1;
+      }
+      for (int ch = tid * 2; ch < kBqCh; ch += kThreads * 2) {     // two channels per thread
+        Pair2<T> lo, hi;
+        lo.load(&red[0][0][ch]);
+        hi.load(&red[1][0][ch]);
+#pragma unroll
+        for (int r = 1; r < ROWL; ++r) { lo.take_min(&red[0][r][ch]); hi.take_max(&red[1][r][ch]); }
+        const float2 l2 = lo.floats(), h2 = hi.floats();
+        __half zh[2], sh[2];
+        group_meta<BITS>(l2.x, h2.x, zh[0], sh[0]);
+        group_meta<BITS>(l2.y, h2.y, zh[1], sh[1]);
+        *reinterpret_cast<__half2*>(a.k_zero + (size_t)g * a.d + c0 + ch) = __halves2half2(zh[0], zh[1]);
+        *reinterpret_cast<__half2*>(a.k_scale + (size_t)g * a.d + c0 + ch) = __halves2half2(sh[0], sh[1]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float s = __half2float(sh[e]);
+          meta[0][ch + e] = -__half2float(zh[e]);
+          meta[1][ch + e] = s;
+          meta[2][ch + e] = scale_rcp(s);
+        }
+      }
+      __syncthreads();
+      f32x2 nz[4], inv[4], ninv[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        nz[e] = *reinterpret_cast<const f32x2*>(&meta[0][lane * 8 + 2 * e]);
+        inv[e] = *reinterpret_cast<const f32x2*>(&meta[2][lane * 8 + 2 * e]);
+        ninv[e] = inv[e] ^ 0x8000000080000000ull;
+      }
+      uint8_t* dst = a.k_codes + ((size_t)t0 * a.d + elem) * BITS / 8;
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        if (t0 + i * ROWL >= t1) break;
+        f32x2 x[4], q[4];
+        raw[i].pairs(x);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[e] = add2(x[e], nz[e]);
+        quotients<BITS, 4>(x, inv, ninv, [&](int e) { return *reinterpret_cast<const f32x2*>(&meta[1][lane * 8 + 2 * e]); }, q);
+        store_codes<BITS, 4>(dst, q);
+        dst += (size_t)ROWL * a.d * BITS / 8;
       }
     }
-    __syncthreads();
-    f32x2 nz[4], inv[4], ninv[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      nz[e] = *reinterpret_cast<const f32x2*>(&meta[0][lane * 8 + 2 * e]);
-      inv[e] = *reinterpret_cast<const f32x2*>(&meta[2][lane * 8 + 2 * e]);
-      ninv[e] = inv[e] ^ 0x8000000080000000ull;
-    }
-    uint8_t* dst = a.k_codes + ((size_t)t0 * a.d + elem) * BITS / 8;
-#pragma unroll
-    for (int i = 0; i < kBqRows<T>; ++i) {
-      if (t0 + i * ROWL >= t1) break;
-      f32x2 x[4], q[4];
-      raw[i].pairs(x);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) x[e] = add2(x[e], nz[e]);
-      quotients<BITS, 4>(x, inv, ninv, [&](int e) { return *reinterpret_cast<const f32x2*>(&meta[1][lane * 8 + 2 * e]); }, q);
-      store_codes<BITS, 4>(dst, q);
-      dst += (size_t)ROWL * a.d * BITS / 8;
-    }
+    if constexpr (NST > 0) tc::cp_async_wait<0>();
   } else {
     // tail rows, as they are
     const int64_t n_vec = (int64_t)(a.L - a.Lq) * a.d * sizeof(T) / 16;
@@ -184,37 +218,42 @@ base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas) {
 }
 
 // Values: pieces of 16 elements, their index running over the whole matrix (no row arithmetic: code and metadata offsets
-// follow from it); two pieces per thread are in flight, minima and maxima by shuffles over the lanes of a group.
+// follow from it); two pieces per thread are in flight, minima and maxima by shuffles over the LPG lanes of a group. Bound by
+// its instructions (70% of the issue slots): offsets in 32 bits from the CTA's own place, the group's width a constant (20 k rows
+// of 2048: 32.7 -> 30.5 us).
 constexpr int kBvThreads = 256;
 
-template <typename T, int BITS>
+template <typename T, int BITS, int LPG>
 __global__ void __launch_bounds__(kBvThreads) base_quant_v_kernel(const __grid_constant__ BaseArgs a) {
   constexpr int U = 2;
   const int tid = threadIdx.x, lane = tid & 31;
-  const int lanes_per_group = a.group >> 4, gs = 31 - __clz(a.group);
-  const int64_t total = ((int64_t)a.Lq * a.d) >> 4;
-  const int64_t i0 = (int64_t)blockIdx.x * (kBvThreads * U) + tid;
-  const T* v = static_cast<const T*>(a.v);
+  const int64_t first = (int64_t)blockIdx.x * (kBvThreads * U);        // the CTA's first piece
+  const int left = (int)min((int64_t)(kBvThreads * U), (((int64_t)a.Lq * a.d) >> 4) - first);
+  const T* v = static_cast<const T*>(a.v) + first * 16;
+  uint8_t* codes = a.v_codes + first * (2 * BITS);
+  __half* scale = a.v_scale + first / LPG;
+  __half* zero = a.v_zero + first / LPG;
   fl_grid_wait();
   fl_grid_release();
   Raw8<T> raw[U][2];
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const int64_t i = i0 + u * kBvThreads;
-    if (i < total) { raw[u][0].load(v + i * 16); raw[u][1].load(v + i * 16 + 8); }
+    const int i = tid + u * kBvThreads;
+    if (i < left) { raw[u][0].load(v + i * 16); raw[u][1].load(v + i * 16 + 8); }
   }
 #pragma unroll
   for (int u = 0; u < U; ++u) {
-    const int64_t i = i0 + u * kBvThreads;
-    if (i - lane >= total) break;                      // warp-uniform; total is a multiple of 16, whole half warps
-    const bool on = i < total;
+    const int i = tid + u * kBvThreads;
+    if (i - lane >= left) break;                       // warp-uniform; the pieces are a multiple of 16, whole half warps
+    const bool on = i < left;
     Raw8<T> mnr = raw[u][0], mxr = raw[u][0];
     mnr.take_min(raw[u][1]);
     mxr.take_max(raw[u][1]);
     float mn, mx, skip;
     mnr.range(mn, skip);
     mxr.range(skip, mx);
-    for (int o = 1; o < lanes_per_group; o <<= 1) {
+#pragma unroll
+    for (int o = 1; o < LPG; o <<= 1) {
       mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
       mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     }
@@ -232,11 +271,10 @@ __global__ void __launch_bounds__(kBvThreads) base_quant_v_kernel(const __grid_c
     }
     quotients<BITS, 8>(x, inv, ninv, [&](int) { return pair(s, s); }, q);
     if (!on) continue;
-    store_codes<BITS, 8>(a.v_codes + i * 2 * BITS, q);
-    if ((lane & (lanes_per_group - 1)) == 0) {
-      const int64_t gi = (i * 16) >> gs;
-      a.v_scale[gi] = sh;
-      a.v_zero[gi] = zh;
+    store_codes<BITS, 8>(codes + i * (2 * BITS), q);
+    if ((lane & (LPG - 1)) == 0) {
+      scale[i / LPG] = sh;
+      zero[i / LPG] = zh;
     }
   }
 }
@@ -419,22 +457,35 @@ template <typename T>
 int launch_quant_base(fl_ctx* ctx, const fl_shape* s, const BaseArgs& a, cudaStream_t st) {
   const int threads = 32 * (a.group / kBqRows<T>);
   const int n_tg = (a.Lq + a.group - 1) / a.group;
-  const int64_t k_ctas = (int64_t)n_tg * (a.d / kBqCh);   // d is a multiple of 256; all grids are below 2^31 (L d <= 2^40)
+  const int64_t k_tiles = (int64_t)n_tg * (a.d / kBqCh);   // d is a multiple of 256; all grids are below 2^31 (L d <= 2^40)
+  const size_t k_smem = (size_t)kBqStages<T> * kBqRows<T> * threads * 16;
+  // with tiles asked for ahead: as many CTAs as run at once (1024 threads and up to 180 KB per SM); else one per tile
+  const int64_t k_ctas = kBqStages<T> > 0 ? std::min<int64_t>(k_tiles, (int64_t)ctx->sm_count * (1024 / threads)) : k_tiles;
   const int64_t v_ctas = ((int64_t)a.Lq * a.d / 16 + kBvThreads * 2 - 1) / (kBvThreads * 2);
   int64_t t_ctas = ((int64_t)(a.L - a.Lq) * a.d * (int64_t)sizeof(T) / 16 + threads - 1) / threads;
   if (t_ctas > ctx->sm_count * 4) t_ctas = ctx->sm_count * 4;
   const dim3 kgrid((unsigned)(k_ctas + t_ctas)), vgrid((unsigned)v_ctas);
-#define FL_BASEK(BITS, ROWL) \
-  FL_CHECK_CUDA(fl_launch(ctx, base_quant_k_kernel<T, BITS, ROWL>, kgrid, dim3(threads), 0, st, a, (int)k_ctas))
+#define FL_BASEK(BITS, ROWL)                                                                                        \
+  do {                                                                                                            \
+    auto kern = base_quant_k_kernel<T, BITS, ROWL>;                                                               \
+    FL_FUNC_ATTR_ONCE(ctx, kern, k_smem, true);                                                                   \
+    FL_CHECK_CUDA(fl_launch(ctx, kern, kgrid, dim3(threads), k_smem, st, a, (int)k_ctas, (int)k_tiles));          \
+  } while (0)
+#define FL_BASEG(BITS, GROUP)                                                                                      \
+  do {                                                                                                            \
+    FL_BASEK(BITS, GROUP / kBqRows<T>);                                                                           \
+    if (v_ctas > 0)                                                                                               \
+      FL_CHECK_CUDA(fl_launch(ctx, base_quant_v_kernel<T, BITS, GROUP / 16>, vgrid, dim3(kBvThreads), 0, st, a)); \
+  } while (0)
 #define FL_BASEQ(BITS)                                                                                            \
   do {                                                                                                            \
-    if (a.group == 32) FL_BASEK(BITS, 32 / kBqRows<T>);                                                           \
-    else if (a.group == 64) FL_BASEK(BITS, 64 / kBqRows<T>);                                                      \
-    else FL_BASEK(BITS, 128 / kBqRows<T>);                                                                        \
-    if (v_ctas > 0) FL_CHECK_CUDA(fl_launch(ctx, base_quant_v_kernel<T, BITS>, vgrid, dim3(kBvThreads), 0, st, a)); \
+    if (a.group == 32) FL_BASEG(BITS, 32);                                                                        \
+    else if (a.group == 64) FL_BASEG(BITS, 64);                                                                   \
+    else FL_BASEG(BITS, 128);                                                                                     \
   } while (0)
   if (s->bits == 8) FL_BASEQ(8); else if (s->bits == 4) FL_BASEQ(4); else FL_BASEQ(2);
 #undef FL_BASEQ
+#undef FL_BASEG
 #undef FL_BASEK
   return fl_launch_status();
 }
