@@ -29,6 +29,11 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
   asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) { return fma2(b, pair(-1.f, -1.f), a); }   // a - b, one rounding
 
 // eight bf16 of a 16-byte piece as four pairs, and back (round to nearest even)
@@ -60,53 +65,46 @@ __device__ __forceinline__ void group_meta(float mn, float mx, __half& zh, __hal
   const float q = __fmul_rn(range, y);
   sh = __float2half_ru(__fmaf_rn(__fmaf_rn(-q, n, range), y, q));      // range 0: 0
 }
-// Reciprocal of a scale for the estimate below (within an ulp); 0 for a constant group, whose codes are 0.
+// Reciprocal of a scale for the quotients below (within an ulp); 0 for a constant group, whose codes are 0.
 __device__ __forceinline__ float scale_rcp(float s) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
   return s == 0.f ? 0.f : r;
 }
 
-// The largest of three numbers, or not-a-number if one of them is none.
-__device__ __forceinline__ float max3_nan(float a, float b, float c) {
-  float r;
-  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
-  return r;
-}
-
-// Codes of P pairs: q = round-half-even of the binary32 quotient t / scale, t = x - zero (already rounded). The quotient
-// is estimated by t * inv (inv = the reciprocal within an ulp): within 2 ulp of the correctly rounded one, 2^(BITS - 23)
-// absolute, so both round to the same integer unless the estimate lies within twice that of a half-integer; only then
-// are the true divisions made (one warp in a hundred at 4 bits). t * inv + 1.5 * 2^23 leaves the rounded integer in the low
-// mantissa bits. No clamp: t >= 0 (the offset was rounded down) and max / scale <= 2^bits - 1 (the scale was rounded up).
-// scale(i) gives the scales of pair i (asked for in the rare branch only: they need not stay in registers).
+// Codes of P pairs: q = round-half-even of the binary32 quotient t / scale, t = x - zero (already rounded). The quotient is
+// correctly rounded without a division: e = t * inv (inv = the reciprocal within an ulp) is within 3 ulp, the remainder
+// r = t - e * scale is exact (a scale has 11 bits), and e + r * inv differs from t / scale by less than 2^-20 ulp, while t / scale
+// keeps at least 2^-12 ulp from every midpoint of two numbers (a midpoint has 25 bits: times an 11-bit scale it is no number t
+// of 24 bits, and it misses t by at least a unit of that product). Adding 1.5 * 2^23 rounds to the integer, halves to even.
+// (With an estimate alone and divisions where it came close to a half-integer, 26 warps in 100 divided: values, offsets and
+// scales have few bits, so exact halves are common.) No clamp: t >= 0 (the offset was rounded down) and max / scale <=
+// 2^bits - 1 (the scale was rounded up). neg_scale = -scale.
 // Elements that are not numbers or not finite, and groups whose offset or scale leaves fp16, have quotients that are no
 // integers of the range; packed by addition (below) they would spoil the codes of their neighbours, which may belong to other
-// channels and groups. They become code 0 (not a number) or the nearest end of the range, in the rare branch: the maximum
-// keeps a not-a-number, so that they always take it.
-template <int BITS, int P, typename Scale>
-__device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv)[P], const f32x2 (&neg_inv)[P],
-                                          Scale scale, f32x2 (&q)[P]) {
-  const f32x2 magic = pair(12582912.f, 12582912.f), neg_magic = pair(-12582912.f, -12582912.f);
+// channels and groups. They become code 0 (not a number) or the nearest end of the range, in a branch of their own.
+template <int BITS, int P>
+__device__ __forceinline__ void quotients(const f32x2 (&t)[P], const f32x2 (&inv)[P], const f32x2 (&neg_scale)[P], f32x2 (&q)[P]) {
+  const f32x2 magic = pair(12582912.f, 12582912.f), neg_magic = pair(-12582912.f, -12582912.f), zero = pair(0.f, 0.f);
   constexpr float n = (float)((1 << BITS) - 1);
-  float far = 0.f;
+  f32x2 odd = zero;                                    // becomes not-a-number with the first quotient that is not finite
 #pragma unroll
   for (int i = 0; i < P; ++i) {
-    q[i] = add2(fma2(t[i], inv[i], magic), neg_magic);
-    const f32x2 fr = fma2(t[i], neg_inv[i], q[i]);   // integer - estimate
-    float a, b;
-    split(fr, a, b);
-    far = max3_nan(far, fabsf(a), fabsf(b));
+    const f32x2 e = mul2(t[i], inv[i]);
+    const f32x2 r = fma2(e, neg_scale[i], t[i]);
+    q[i] = add2(add2(fma2(r, inv[i], e), magic), neg_magic);
+    odd = fma2(q[i], zero, odd);
   }
-  constexpr float kNear = 0.5f - (float)(1 << BITS) / 4194304.f;
-  if (!(far <= kNear)) {
+  float a, b;
+  split(odd, a, b);
+  if (!(a + b == 0.f)) {
 #pragma unroll
     for (int i = 0; i < P; ++i) {
-      float a, b, sa, sb;
+      float sa, sb;
       split(t[i], a, b);
-      split(scale(i), sa, sb);
-      a = sa == 0.f ? 0.f : rintf(__fdiv_rn(a, sa));
-      b = sb == 0.f ? 0.f : rintf(__fdiv_rn(b, sb));
+      split(neg_scale[i], sa, sb);
+      a = sa == 0.f ? 0.f : rintf(__fdiv_rn(a, -sa));
+      b = sb == 0.f ? 0.f : rintf(__fdiv_rn(b, -sb));
       q[i] = pair(fminf(fmaxf(a, 0.f), n), fminf(fmaxf(b, 0.f), n));
     }
   }

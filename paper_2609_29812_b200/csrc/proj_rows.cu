@@ -121,7 +121,7 @@ __device__ __forceinline__ void codec_row(const ProjArgs& a, uint32_t tmem_row, 
     const float zf = __half2float(zh), sf = __half2float(sh), rcp = scale_rcp(sf);
     const f32x2 z2 = pair(zf, zf), nz2 = pair(-zf, -zf), s2 = pair(sf, sf);
     const f32x2 inv[4] = {pair(rcp, rcp), pair(rcp, rcp), pair(rcp, rcp), pair(rcp, rcp)};
-    const f32x2 ninv[4] = {pair(-rcp, -rcp), pair(-rcp, -rcp), pair(-rcp, -rcp), pair(-rcp, -rcp)};
+    const f32x2 ns[4] = {pair(-sf, -sf), pair(-sf, -sf), pair(-sf, -sf), pair(-sf, -sf)};
 #pragma unroll 1
     for (int pc = 0; pc < pieces; ++pc) {
       uint32_t r[32];
@@ -147,7 +147,7 @@ __device__ __forceinline__ void codec_row(const ProjArgs& a, uint32_t tmem_row, 
           h[u] = pair(xh[2 * u], xh[2 * u + 1]);
           t2[u] = add2(sub2(xn[u], h[u]), nz2);
         }
-        quotients<BITS, 4>(t2, inv, ninv, [&](int) { return s2; }, q);
+        quotients<BITS, 4>(t2, inv, ns, q);
         if (rows_prev != nullptr) *reinterpret_cast<uint4*>(rows_prev + (size_t)t * d + e_p + v * 8) = fl_codec::pack_bf16(h);
         if (rows_cur != nullptr) {
 #pragma unroll

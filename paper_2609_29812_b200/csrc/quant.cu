@@ -55,7 +55,7 @@ __device__ __forceinline__ void encode(const QuantArgs& a, bool is_v, int t, int
     store_pairs<T, P>(reinterpret_cast<T*>(codes) + row_off, xn);
     if (rows_cur != nullptr) store_pairs<T, P>(rows_cur + row_off, xn);
   } else {
-    f32x2 dl[P], q[P], inv[P], ninv[P];
+    f32x2 dl[P], q[P], inv[P], ns[P];
     float mn = INFINITY, mx = -INFINITY;
 #pragma unroll
     for (int i = 0; i < P; ++i) {
@@ -77,9 +77,9 @@ __device__ __forceinline__ void encode(const QuantArgs& a, bool is_v, int t, int
     for (int i = 0; i < P; ++i) {
       dl[i] = add2(dl[i], nz2);
       inv[i] = pair(r, r);
-      ninv[i] = pair(-r, -r);
+      ns[i] = pair(-sf, -sf);
     }
-    quotients<BITS, P>(dl, inv, ninv, [&](int) { return s2; }, q);
+    quotients<BITS, P>(dl, inv, ns, q);
     if (rows_cur != nullptr) {
       // the reconstruction every later reader of this stream forms: Xhat + (code * scale + zero), Eq. 8
 #pragma unroll

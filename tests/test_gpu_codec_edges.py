@@ -168,3 +168,42 @@ def test_packed_base_with_elements_that_are_not_finite(env, bits, group, dtype):
     v_ok = ~v_lost[:Lq].reshape(Lq, -1, group).any(axis=2)
     for got, name, ok in ((ks, "k_scale", k_ok), (kz, "k_zero", k_ok), (vs, "v_scale", v_ok), (vz, "v_zero", v_ok)):
         assert np.array_equal(got.view(np.uint16)[ok], ref[name].view(np.uint16)[ok]), name
+
+
+def _pack(B, P, ctx, w, k, v, group):
+    st = P.LayerState(ctx, w, split=False)
+    shape = (w.L, w.n_heads, w.head_dim)
+    st.pack_base(to_dev(k.reshape(shape), w), to_dev(v.reshape(shape), w), group, 0)
+    return [to_np(t) for t in st.base_tensors[:6]]
+
+
+@pytest.mark.parametrize("bits", [2, 4, 8])
+def test_quotients_at_and_beside_half_integers(env, bits):
+    """binary32 values whose quotients are exact halves, and the numbers next to those on either side: the code is the rounded
+    quotient, halves to even, as a division gives it."""
+    B, P, ctx = env
+    rng = np.random.default_rng(bits)
+    n, L, d = 2 ** bits - 1, 512, 256
+    s = np.exp2(rng.integers(-9, 4, L)) * (1 + rng.integers(0, 1024, L) / 1024.0)      # scales that fp16 holds
+    half = (rng.integers(0, n, (L, d)) + 0.5) * s[:, None]
+    v = half.astype(np.float32)
+    v = np.choose(rng.integers(0, 3, (L, d)), [v, np.nextafter(v, np.float32(0)), np.nextafter(v, np.float32(np.inf))])
+    v[:, ::32], v[:, 1::32] = 0.0, (n * s[:, None]).astype(np.float32)                 # every group spans 0 .. n s: its scale is s
+    w = workloads.replace(workloads.config2(L=L, n_heads=4), head_dim=64, dtype="f32", bits=bits, group=32)
+    ref = fo.quantize_base(v, v, bits, 32, 0)
+    got = _pack(B, P, ctx, w, v, v, 32)
+    assert np.array_equal(got[3], fo.pack_codes(ref["v_codes"], bits)) and np.array_equal(got[0], fo.pack_codes(ref["k_codes"], bits))
+    assert np.array_equal(got[4].view(np.uint16), ref["v_scale"].view(np.uint16))
+
+
+@pytest.mark.parametrize("L,group", [(40037, 32), (20003, 64)])
+def test_packed_base_with_several_key_tiles_per_cta(env, L, group):
+    B, P, ctx = env
+    rng = np.random.default_rng(L)
+    k, v = (fo.round_bf16(rng.standard_normal((L, 256)).astype(np.float32)) for _ in range(2))
+    w = workloads.replace(workloads.config2(L=L, n_heads=2), bits=4, group=group)
+    ref = fo.quantize_base(k, v, 4, group, 0, storage_round=fo.round_bf16)
+    got = _pack(B, P, ctx, w, k, v, group)
+    for g, name in zip(got, ("k_codes", "k_scale", "k_zero", "v_codes", "v_scale", "v_zero")):
+        want = fo.pack_codes(ref[name], 4) if "codes" in name else ref[name]
+        assert np.array_equal(np.ascontiguousarray(g).view(np.uint8), np.ascontiguousarray(want).view(np.uint8)), name
