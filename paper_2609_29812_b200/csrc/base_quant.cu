@@ -202,6 +202,7 @@ base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas, int n_tiles)
         store_codes<BITS, 4>(dst, q);
         dst += (size_t)ROWL * a.d * BITS / 8;
       }
+      if constexpr (NST == 0) break;                   // one tile per CTA
     }
     if constexpr (NST > 0) tc::cp_async_wait<0>();
   } else {

@@ -653,7 +653,7 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
     a.m_tiles = (n + 2 * kBM - 1) / (2 * kBM);
     a.n_tiles = (d_out + pair_bn - 1) / pair_bn;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * std::min(a.m_tiles * a.n_tiles, ctx->sm_count / 2));
+    cfg.gridDim = dim3(2 * (unsigned)std::min<int64_t>((int64_t)a.m_tiles * a.n_tiles, ctx->sm_count / 2));
     cfg.blockDim = dim3(pair_threads(gather));
     cfg.dynamicSmemBytes = kPairSmem;
     cfg.stream = st;
