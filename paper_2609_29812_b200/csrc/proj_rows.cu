@@ -530,7 +530,8 @@ __global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(cons
       bool ok = true;
       for (int w = pair; w < n_work && ok; w += n_pairs, ++i) {
         const int buf = i & 1;
-        if (i >= 2) ok = tc::mbar_wait(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
+        // the epilogue warps of both CTAs have read the accumulator: an acquire at cluster scope, once per tile
+        if (i >= 2) ok = tc::mbar_wait_cluster(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
         if (!ok) break;
         tc::tc_fence_after();
         const uint32_t d_dst = tmem + buf * 256;

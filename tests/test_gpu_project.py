@@ -100,6 +100,35 @@ def test_project_rows_pairs_of_ctas(env, n, d_out, gather, scatter, accumulate):
     check(B, ctx, *args, n, accumulate, rows=rows)
 
 
+def check_every_row(B, ctx, n, d_in, d_out, gather, scatter, accumulate, launches=1):
+    """All outputs of rows drawn from twice as many against the product in binary64; every launch gives the same bits."""
+    g = torch.Generator(device="cuda").manual_seed(5)
+    x, w = (torch.randn(r, d_in, generator=g, device="cuda").bfloat16() for r in (2 * n, d_out))
+    y0 = torch.randn(2 * n, d_out, generator=g, device="cuda").bfloat16()
+    src, dst = (torch.sort(torch.randperm(2 * n, generator=g, device="cuda")[:n])[0].int() for _ in range(2))
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    outs = []
+    for _ in range(launches):
+        y = y0.clone()
+        B.fl_project_rows(ctx, x, 2 * n, src if gather else None, n, d_in, w, d_out, y, 2 * n, dst if scatter else None, accumulate, status)
+        outs.append(y)
+    assert int(status.item()) == 0 and all(torch.equal(outs[0], o) for o in outs[1:])
+    at = dst.long() if scatter else torch.arange(n, device="cuda")
+    xs, ws, old = (x[src.long()] if gather else x[:n]).double(), w.double(), y0[at].double() * accumulate
+    ref, mag = xs @ ws.T + old, xs.abs() @ ws.abs().T + old.abs()
+    assert ((outs[0][at].double() - ref).abs() <= 2.0 ** -8 * ref.abs() + d_in * 2.0 ** -23 * mag).all()
+    rest = torch.ones(2 * n, dtype=torch.bool, device="cuda")
+    rest[at] = False
+    assert torch.equal(outs[0][rest], y0[rest])
+
+
+def test_project_rows_pairs_reuse_their_accumulators(env):
+    """Five tiles per pair of CTAs, every row of every tile: an accumulator is overwritten only when the epilogues of BOTH CTAs have
+    read it."""
+    B, ctx = env
+    check_every_row(B, ctx, 3277, 2048, 6144, True, True, 1, launches=4)
+
+
 def test_project_rows_single_row_and_empty(env):
     B, ctx = env
     x, w, y, src, dst = make(9, 50, 50, 1, 64, 8, True, True)
