@@ -199,7 +199,7 @@ base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas, int n_tiles)
         raw[i].pairs(x);
 #pragma unroll
         for (int e = 0; e < 4; ++e) x[e] = add2(x[e], nz[e]);
-        quotients<BITS, 4>(x, inv, ns, q);
+        quotients<BITS, 4, kRareHalves<T, BITS>>(x, inv, ns, q);
         store_codes<BITS, 4>(dst, q);
         dst += (size_t)ROWL * a.d * BITS / 8;
       }
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kBvThreads) base_quant_v_kernel(const __grid_c
       inv[e] = pair(r, r);
       ns[e] = pair(-s, -s);
     }
-    quotients<BITS, 8>(x, inv, ns, q);
+    quotients<BITS, 8, false>(x, inv, ns, q);
     if (!on) continue;
     store_codes<BITS, 8>(codes + i * (2 * BITS), q);
     if ((lane & (LPG - 1)) == 0) {
@@ -462,6 +462,8 @@ int launch_quant_base(fl_ctx* ctx, const fl_shape* s, const BaseArgs& a, cudaStr
   const int64_t k_tiles = (int64_t)n_tg * (a.d / kBqCh);   // d is a multiple of 256; all grids are below 2^31 (L d <= 2^40)
   const size_t k_smem = (size_t)kBqStages<T> * kBqRows<T> * threads * 16;
   // with tiles asked for ahead: as many CTAs as run at once (1024 threads and up to 180 KB per SM); else one per tile
+  // No largest carve-out asked for: the room that the slots need is found without, and with 32-bit storage, which has none, an L1 cut
+  // to 28 KB loses the second half of every 32-byte piece before it is read (20 k rows of 2048, groups of 64: 84 us, now 61).
   const int64_t k_ctas = kBqStages<T> > 0 ? std::min<int64_t>(k_tiles, (int64_t)ctx->sm_count * (1024 / threads)) : k_tiles;
   const int64_t v_ctas = ((int64_t)a.Lq * a.d / 16 + kBvThreads * 2 - 1) / (kBvThreads * 2);
   int64_t t_ctas = ((int64_t)(a.L - a.Lq) * a.d * (int64_t)sizeof(T) / 16 + threads - 1) / threads;
@@ -470,7 +472,7 @@ int launch_quant_base(fl_ctx* ctx, const fl_shape* s, const BaseArgs& a, cudaStr
 #define FL_BASEK(BITS, ROWL)                                                                                        \
   do {                                                                                                            \
     auto kern = base_quant_k_kernel<T, BITS, ROWL>;                                                               \
-    FL_FUNC_ATTR_ONCE(ctx, kern, k_smem, true);                                                                   \
+    FL_FUNC_ATTR_ONCE(ctx, kern, k_smem, false);                                                                   \
     FL_CHECK_CUDA(fl_launch(ctx, kern, kgrid, dim3(threads), k_smem, st, a, (int)k_ctas, (int)k_tiles));          \
   } while (0)
 #define FL_BASEG(BITS, GROUP)                                                                                      \

@@ -147,7 +147,7 @@ __device__ __forceinline__ void codec_row(const ProjArgs& a, uint32_t tmem_row, 
           h[u] = pair(xh[2 * u], xh[2 * u + 1]);
           t2[u] = add2(sub2(xn[u], h[u]), nz2);
         }
-        quotients<BITS, 4>(t2, inv, ns, q);
+        quotients<BITS, 4, false>(t2, inv, ns, q);
         if (rows_prev != nullptr) *reinterpret_cast<uint4*>(rows_prev + (size_t)t * d + e_p + v * 8) = fl_codec::pack_bf16(h);
         if (rows_cur != nullptr) {
 #pragma unroll

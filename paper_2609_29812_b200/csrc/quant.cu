@@ -79,7 +79,7 @@ __device__ __forceinline__ void encode(const QuantArgs& a, bool is_v, int t, int
       inv[i] = pair(r, r);
       ns[i] = pair(-sf, -sf);
     }
-    quotients<BITS, P>(dl, inv, ns, q);
+    quotients<BITS, P, kRareHalves<T, BITS>>(dl, inv, ns, q);
     if (rows_cur != nullptr) {
       // the reconstruction every later reader of this stream forms: Xhat + (code * scale + zero), Eq. 8
 #pragma unroll

@@ -155,3 +155,31 @@ def test_dense_and_sparse_loop_on_the_rebuilt_base(env):
     assert np.array_equal(st.k_streams[0]["codes"].cpu().numpy().reshape(len(act), -1),
                           rec["k_payload"]["packed"].reshape(len(act), -1))
     assert_attn_close(to_np(o_rows), rec["O_rows"], "loop 2 on the rebuilt int4 base", carried=1)
+
+
+@pytest.mark.parametrize("d,group,bits", [(2048, 64, 4), (2048, 128, 2), (1024, 32, 4)])
+def test_packing_binary32_takes_less_than_copying(env, d, group, bits):
+    """Packing a base of binary32 rows reads them once and writes a sixth of them, a copy writes as much as it reads: a ratio of
+    times on one GPU. 0.57 to 0.63 of the copy; 0.77 to 0.90 when the L1 was given away to shared memory that the kernel does not
+    use."""
+    B, P, ctx = env
+    L = 20011
+    w = workloads.replace(workloads.config2(L=L, n_heads=d // 128), dtype="f32", bits=bits)
+    st = P.LayerState(ctx, w, split=False)
+    k, v = (torch.randn(L, d // 128, 128, device="cuda") for _ in range(2))
+    k2, v2 = torch.empty_like(k), torch.empty_like(v)
+    st.pack_base(k, v, group, 64)
+
+    def best(call):
+        t = float("inf")
+        for _ in range(12):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(8):
+                call()
+            b.record()
+            torch.cuda.synchronize()
+            t = min(t, a.elapsed_time(b))
+        return t
+    ratio = best(lambda: B.fl_quant_kv_base(ctx, st.shape, k, v, st.base_q)) / best(lambda: (k2.copy_(k), v2.copy_(v)))
+    assert ratio < 0.70, ratio
