@@ -101,11 +101,12 @@ struct Pair2<float> {
 //
 // Keys: a tile is 256 channels of one token group, 32 pieces of 8 channels by ROWL row lanes; a thread has the tile's rows of its
 // piece at once, and after the group's minimum and maximum per channel have been joined in shared memory encodes them. A CTA
-// (1024 threads per SM in all) walks its tiles: with 16-bit storage a thread asks for its pieces of the tiles NST - 1 ahead
-// by asynchronous copies into slots of its own, so that HBM is read under the joins and the encoding (a CTA per tile, which
-// asked, joined and encoded one after the other, two at a time on an SM: 40 us for the 20 k rows of 2048, then 34.6; 33 with
-// codes without divisions). A warp per tile without any barrier is no faster (33.7; groups of 128: 40 for 38). With 32-bit
-// storage (NST = 0) a tile takes twice the space and a CTA takes one. The CTAs past k_ctas copy the tail rows.
+// (1024 threads per SM in all) walks its tiles: the first comes straight to registers, and with 16-bit storage a thread asks for its
+// pieces of the NST tiles after it by asynchronous copies into slots of its own, so that HBM is read under the joins and the
+// encoding (a CTA per tile, which asked, joined and encoded one after the other, two at a time on an SM: 40 us for the 20 k rows of
+// 2048, then 34.6; 33 with codes without divisions). A warp per tile without any barrier is no faster (33.7; groups of 128: 40 for
+// 38). With 32-bit storage (NST = 0) a tile takes twice the space and a CTA takes one; a launch of one tile per CTA gets no slots.
+// The CTAs past k_ctas copy the tail rows.
 template <typename T>
 constexpr int kBqRows = sizeof(T) == 2 ? 4 : 8;        // rows of a token group per thread
 constexpr int kBqCh = 256;                             // channels of a key tile
@@ -136,33 +137,34 @@ base_quant_k_kernel(const __grid_constant__ BaseArgs a, int k_ctas, int n_tiles)
         for (int i = 0; i < R; ++i) tc::cp_async16(&slots[(st * R + i) * kThreads + tid], row_of(tile, i));
       tc::cp_async_commit();
     };
-    int st = 0;
+    Raw8<T> raw[R];                                    // the first tile comes straight to registers
+#pragma unroll
+    for (int i = 0; i < R; ++i) raw[i].load(row_of(blockIdx.x, i));
     if constexpr (NST > 0)
 #pragma unroll
-      for (int s = 0; s < NST; ++s) ask(blockIdx.x + s * k_ctas, s);
+      for (int s = 0; s < NST; ++s) ask(blockIdx.x + (s + 1) * k_ctas, s);
+    int st = 0;
     for (int tile = blockIdx.x; tile < n_tiles; tile += k_ctas) {
       const int g = tile / slabs, c0 = (tile - g * slabs) * kBqCh;
       const int elem = c0 + lane * 8;
       const int t0 = g * a.group + rl, t1 = min(a.Lq, (g + 1) * a.group);
-      Raw8<T> raw[R];
-      if constexpr (NST > 0) {
-        tc::cp_async_wait<NST - 1>();
+      if constexpr (NST > 0)
+        if (tile != (int)blockIdx.x) {
+          tc::cp_async_wait<NST - 1>();
 #pragma unroll
-        for (int i = 0; i < R; ++i) raw[i].load_smem(&slots[(st * R + i) * kThreads + tid]);
-      } else {
-#pragma unroll
-        for (int i = 0; i < R; ++i) raw[i].load(row_of(tile, i));
-      }
+          for (int i = 0; i < R; ++i) raw[i].load_smem(&slots[(st * R + i) * kThreads + tid]);
+        }
       Raw8<T> mn = raw[0], mx = raw[0];
 #pragma unroll
       for (int i = 1; i < R; ++i) { mn.take_min(raw[i]); mx.take_max(raw[i]); }
       mn.store(&red[0][rl][lane * 8]);
       mx.store(&red[1][rl][lane * 8]);
       __syncthreads();
-      if constexpr (NST > 0) {                         // the slots have been read (by their only thread)
-        ask(tile + NST * k_ctas, st);
-        st = st + 1 == NST ? 0 : st + 1;
-      }
+      if constexpr (NST > 0)                           // the slots have been read (by their only thread)
+        if (tile != (int)blockIdx.x) {
+          ask(tile + NST * k_ctas, st);
+          st = st + 1 == NST ? 0 : st + 1;
+        }
       for (int ch = tid * 2; ch < kBqCh; ch += kThreads * 2) {     // two channels per thread
         Pair2<T> lo, hi;
         lo.load(&red[0][0][ch]);
@@ -473,7 +475,7 @@ int launch_quant_base(fl_ctx* ctx, const fl_shape* s, const BaseArgs& a, cudaStr
   do {                                                                                                            \
     auto kern = base_quant_k_kernel<T, BITS, ROWL>;                                                               \
     FL_FUNC_ATTR_ONCE(ctx, kern, k_smem, false);                                                                   \
-    FL_CHECK_CUDA(fl_launch(ctx, kern, kgrid, dim3(threads), k_smem, st, a, (int)k_ctas, (int)k_tiles));          \
+    FL_CHECK_CUDA(fl_launch(ctx, kern, kgrid, dim3(threads), k_tiles > k_ctas ? k_smem : 0, st, a, (int)k_ctas, (int)k_tiles)); \
   } while (0)
 #define FL_BASEG(BITS, GROUP)                                                                                      \
   do {                                                                                                            \

@@ -207,3 +207,21 @@ def test_packed_base_with_several_key_tiles_per_cta(env, L, group):
     for g, name in zip(got, ("k_codes", "k_scale", "k_zero", "v_codes", "v_scale", "v_zero")):
         want = fo.pack_codes(ref[name], 4) if "codes" in name else ref[name]
         assert np.array_equal(np.ascontiguousarray(g).view(np.uint8), np.ascontiguousarray(want).view(np.uint8)), name
+
+
+@pytest.mark.parametrize("L,H,group", [(15001, 16, 128), (64, 4, 128), (20003, 8, 64)])
+def test_packed_base_with_and_without_tiles_asked_for_ahead(env, L, H, group):
+    """CTAs of 1024 and 512 threads: up to seven tiles of 256 channels per CTA (the first from registers, the others from the slots),
+    and a base of one tile per CTA, which has no slots. Channels of every tile against the oracle (keys are grouped per channel)."""
+    B, P, ctx = env
+    g = torch.Generator(device="cuda").manual_seed(L)
+    d = H * 128
+    k, v = (torch.randn(L, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    w = workloads.replace(workloads.config2(L=L, n_heads=H), bits=4, group=group)
+    got = _pack(B, P, ctx, w, to_np(k), to_np(v), group)
+    cols = np.linspace(0, d - 1, group).astype(int)
+    part = to_np(k)[:, cols]
+    ref = fo.quantize_base(part, part, 4, group, 0, storage_round=fo.round_bf16)
+    assert np.array_equal(fo.unpack_codes(got[0], 4)[:, cols], ref["k_codes"])
+    assert np.array_equal(got[1][:, cols].view(np.uint16), ref["k_scale"].view(np.uint16))
+    assert np.array_equal(got[2][:, cols].view(np.uint16), ref["k_zero"].view(np.uint16))
