@@ -20,7 +20,6 @@ using namespace fl_tc;
 constexpr int kIssueWarp = 4;
 constexpr int kTmaWarp = 5;
 constexpr int kThreads = 6 * 32;
-constexpr uint32_t kAcc = 0, kS = 128;
 constexpr uint32_t kTmemCols = 256;
 
 struct alignas(64) DnArgs {
@@ -46,8 +45,11 @@ struct alignas(64) DnArgs {
 // query tile and 64 keys, two CTAs per SM (the first figures); P over its own S, one issuing thread: 4139 us (4218 without a
 // maximum in the softmax); part of the exponentials on the FMA pipe: 3620 us and more, their chains are longer.
 // ------------------------------------------------------------------------------------------------------------
-constexpr int kFlWarps = 11;                       // 0-3 softmax of the first tile, 4-7 of the second, then:
-constexpr int kFlQk = 8, kFlPv = 9, kFlTma = 10;
+// TILES = 1: one query tile per CTA, for prompts that leave SMs idle (the rule stands at the launch). There a warp also skips the half
+// of a chunk that none of its rows sees: a short prompt's time is the chain of its chunks.
+template <int TILES> struct FlashShape {
+  static constexpr int kQk = 4 * TILES, kPv = kQk + 1, kTma = kQk + 2, kThreads = (kQk + 3) * 32;   // warps 0-3, 4-7: softmax of a tile
+};
 constexpr int kFlSlots = 4;                        // ring of K and V tiles in the order K0 V0 K1 V1 ...
 constexpr int kFlNC = 128;                         // keys per chunk
 constexpr uint32_t kFlAcc = 0, kFlS = 256, kFlP = 384;     // tensor-memory columns: accumulators, S, P (64 columns each)
@@ -59,7 +61,7 @@ struct __align__(16) FlashCtl {
   uint32_t tmem_base;
   int abort_flag;
 };
-constexpr size_t kFlashSmem = 1024 + 2 * kQTileBytes + kFlSlots * kQTileBytes + sizeof(FlashCtl);
+template <int TILES> constexpr size_t kFlashSmem = 1024 + (TILES + kFlSlots) * kQTileBytes + sizeof(FlashCtl);
 
 // P = 2^(s c2 - sub) of 32 logits, as exp32, with the sum taken in ONE order (pair by pair): the row sums, and with them O to
 // the last bit, do not depend on how the keys are cut into chunks. The chain of additions runs beside the exponentials.
@@ -78,19 +80,21 @@ __device__ __forceinline__ float exp32_in_order(const uint32_t (&r)[32], float c
   return sum;
 }
 
-__global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __grid_constant__ DnArgs a) {
+template <int TILES>
+__global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_kernel(const __grid_constant__ DnArgs a) {
+  using Sh = FlashShape<TILES>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* q_tiles = smem;
-  uint8_t* ring = smem + 2 * kQTileBytes;
+  uint8_t* ring = smem + TILES * kQTileBytes;
   FlashCtl& ctl = *reinterpret_cast<FlashCtl*>(ring + kFlSlots * kQTileBytes);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // later tiles see more keys: they are dispatched first
-  const int n_pairs = (a.L + 2 * kM - 1) / (2 * kM);
-  const int h = blockIdx.x % a.H, s0 = (n_pairs - 1 - (int)(blockIdx.x / a.H)) * 2 * kM;
+  const int n_groups = (a.L + TILES * kM - 1) / (TILES * kM);
+  const int h = blockIdx.x % a.H, s0 = (n_groups - 1 - (int)(blockIdx.x / a.H)) * TILES * kM;
   // chunks of the two tiles (the second may have no rows, else it sees at least as many keys as the first)
   const int n_first = (min(a.L, s0 + kM) + kFlNC - 1) / kFlNC;
-  const int n_second = s0 + kM < a.L ? (min(a.L, s0 + 2 * kM) + kFlNC - 1) / kFlNC : 0;
+  const int n_second = TILES > 1 && s0 + kM < a.L ? (min(a.L, s0 + 2 * kM) + kFlNC - 1) / kFlNC : 0;
   const int n_chunks = max(n_first, n_second);
   if (tid == 0) {
     for (int s = 0; s < kFlSlots; ++s) {
@@ -107,7 +111,7 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
     ctl.abort_flag = 0;
     tc::fence_barrier_init();
   }
-  if (warp == kFlQk) {
+  if (warp == Sh::kQk) {
     tc::tmem_alloc(&ctl.tmem_base, 512);
     tc::tmem_relinquish();
   }
@@ -117,7 +121,7 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
 
-  if (warp == kFlTma) {
+  if (warp == Sh::kTma) {
     if (lane == 0) {
       auto load = [&](uint8_t* dst, const void* map, uint64_t* bar, int row) {
         tc::mbar_arrive_expect_tx(bar, kQTileBytes);
@@ -134,7 +138,7 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
       }
     }
     __syncwarp();
-  } else if (warp == kFlQk) {
+  } else if (warp == Sh::kQk) {
     if (lane == 0) {
       const uint32_t idesc = tc::make_idesc_bf16(kM, kFlNC, false);
       const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32(q_tiles), 16, 1024);
@@ -167,7 +171,7 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
       }
     }
     __syncwarp();
-  } else if (warp == kFlPv) {
+  } else if (warp == Sh::kPv) {
     if (lane == 0) {
       const uint32_t idesc = tc::make_idesc_bf16(kM, kDH, true);
       const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), kFlNC * 128, 1024);   // MN-major
@@ -190,7 +194,7 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
     __syncwarp();
   } else {
     // ============================================ softmax ============================================
-    const int t = warp >> 2, gt = tid & 127;           // tile, thread inside its group of four warps
+    const int t = TILES > 1 ? warp >> 2 : 0, gt = tid & 127;    // tile, thread inside its group of four warps
     const int row = (warp & 3) * 32 + lane;
     const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
     const int lo = s0 + t * kM, n_rows = min(kM, a.L - lo), n_t = t ? n_second : n_first;
@@ -204,9 +208,13 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
     for (int n = 0; n < n_t; ++n) {
       if (!warp_wait(&ctl.s_full[t], n & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
+      // the last rows of the warp see `seen` keys of the chunk: where that is half of it at most, the other half is not looked at
+      const int seen = min(lo + (warp & 3) * 32 + 31, lo + n_rows - 1) - n * kFlNC + 1;
+      const bool whole = TILES > 1 || seen > 64;
       uint32_t r[4][32];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) tc::tmem_ld32(s_addr + q * 32, r[q]);
+      for (int q = 0; q < 4; ++q)
+        if (q < 2 || whole) tc::tmem_ld32(s_addr + q * 32, r[q]);
       tc::tmem_wait_ld();
       tc::tc_fence_before();
       __syncwarp();
@@ -216,13 +224,15 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
         const int vis = row_ok ? max(0, pos - n * kFlNC + 1) : 0;
 #pragma unroll
         for (int q = 0; q < 4; ++q)
+          if (q < 2 || whole)
 #pragma unroll
-          for (int u = 0; u < 32; ++u) r[q][u] = q * 32 + u < vis ? r[q][u] : 0xff800000u;
+            for (int u = 0; u < 32; ++u) r[q][u] = q * 32 + u < vis ? r[q][u] : 0xff800000u;
       }
       // running reference: taken from the first keys that show a finite logit (the accumulator row is still zero then) and
       // moved, with a rescale of the accumulator row, only when a maximum beats it by more than the threshold
       const float cm0 = max32(r[0]) * c2;
-      const float cm = fmaxf(fmaxf(cm0, max32(r[1]) * c2), fmaxf(max32(r[2]), max32(r[3])) * c2);
+      float cm = fmaxf(cm0, max32(r[1]) * c2);
+      if (whole) cm = fmaxf(cm, fmaxf(max32(r[2]), max32(r[3])) * c2);
       if (ref == -INFINITY) ref = cm0 > -INFINITY ? cm0 : cm;
       const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
       const bool any_over = __any_sync(0xffffffffu, over);
@@ -251,9 +261,14 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
       tc::tmem_st16(p_addr + 16, p1);
       ell += sum0;
       ell += sum1;
-      ell += exp32_in_order(r[2], c2, sub, p0);
+      if (whole) {
+        ell += exp32_in_order(r[2], c2, sub, p0);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 16; ++u) p0[u] = p1[u] = 0u;
+      }
       tc::tmem_st16(p_addr + 32, p0);
-      ell += exp32_in_order(r[3], c2, sub, p1);
+      if (whole) ell += exp32_in_order(r[3], c2, sub, p1);
       tc::tmem_st16(p_addr + 48, p1);
       tc::tmem_wait_st();
       tc::tc_fence_before();
@@ -295,7 +310,7 @@ __global__ void __launch_bounds__(kFlWarps * 32, 1) dense_flash_kernel(const __g
   }
   tc::tc_fence_before();
   __syncthreads();
-  if (warp == kFlQk) {
+  if (warp == Sh::kQk) {
     if (ctl.abort_flag) {
       if (lane == 0) tc::mma_commit(&ctl.pv_done[0]);
       __syncwarp();
@@ -806,8 +821,18 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
   a.L = s->L; a.H = s->n_heads; a.d = (int)d_row; a.q_block = s->q_block; a.nb = fl_n_blocks(s);
   a.scale = s->sm_scale;
   const int n_tiles = (s->L + kM - 1) / kM;
-  FL_FUNC_ATTR_ONCE(ctx, dense_flash_kernel, kFlashSmem, true);
-  dense_flash_kernel<<<dim3((n_tiles + 1) / 2 * s->n_heads), kFlWarps * 32, kFlashSmem, st>>>(a);
+#define FL_FLASH(TILES)                                                                                                    \
+  do {                                                                                                                    \
+    auto kern = dense_flash_kernel<TILES>;                                                                                \
+    FL_FUNC_ATTR_ONCE(ctx, kern, kFlashSmem<TILES>, true);                                                                \
+    kern<<<dim3((n_tiles + TILES - 1) / TILES * s->n_heads), FlashShape<TILES>::kThreads, kFlashSmem<TILES>, st>>>(a);    \
+  } while (0)
+  // One tile per CTA while that leaves no SM with more chunks than the longest tile has (tiles x heads in triangles of chunks, a little
+  // above one wave): the tiles of a pair wait for one another at S and for SMs that stand idle. Measured, replaced kernel / pairs /
+  // single tiles, us: 129 x 16 heads 7.5 / 9.2 / 7.3, 400 x 16 10.9 / 12.0 / 9.6, 1024 x 4 18.6 / 18.0 / 14.7, 2048 x 16 (272) 33.9 /
+  // 31.8 / 28.4, 4096 x 8 (264) 61.5 / 56.4 / 44.7; beyond: 1000 x 32 (288) 20.3 / 19.5 / 19.9, 4096 x 16 71 / 61 / 88.
+  if ((int64_t)(n_tiles + 1) * s->n_heads <= ctx->sm_count * 19 / 10) FL_FLASH(1); else FL_FLASH(2);
+#undef FL_FLASH
   int rc = fl_launch_status();
   if (rc != FL_OK || col_scores == nullptr) return rc;
   // 512 keys per CTA where that still gives (with one job per query block) three jobs to two SMs, else 128; the blocks are
