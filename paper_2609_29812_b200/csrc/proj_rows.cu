@@ -17,6 +17,7 @@
 //   warps 6-13 A row gathers: four lanes per warp, one four-row copy each per stage
 #include "tc_attn_common.cuh"
 #include <algorithm>
+#include <cmath>
 
 namespace {
 
@@ -579,25 +580,48 @@ __global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(cons
 
 }  // namespace
 
-constexpr double kNarrowCost = 0.73;     // of a tile of 128 columns, one of 256 being 1
-
-// Width of the pairs' tiles, or 0 where the one-CTA kernel (tiles of `bn` columns, `rounds` rounds over the SMs) is the faster one.
-// Cycles as measured (d_in 2048, 60 to 12000 rows): a slab of the one-CTA kernel 762, gathered 846 (128 columns: 0.73 of that);
-// of a pair 100 + 2.52 bn, gathered 280 + 2.1 bn; a launch of pairs takes 3300 more (clusters, the pairs' barriers). Pairs are
-// taken where they gain 3% by that. 3277 rows of 32768, d = 2048: Q/K/V 73.7 -> 67.8 us (rows in order 67.3 -> 60.5), output
-// projection added into the store 35.3 -> 28.7; 12000 rows: 260 -> 245 (235 -> 205), 101 -> 97.
-static int fl_proj_pair_width(const fl_ctx* ctx, int n, int d_in, int d_out, bool gather, int bn, double rounds) {
-  if ((size_t)ctx->max_smem_optin < kPairSmem) return 0;
-  const int64_t m_tiles = (n + 2 * kBM - 1) / (2 * kBM), pairs = ctx->sm_count / 2;
-  const double slabs = d_in / kBK;
-  double best = rounds * slabs * (gather ? 846.0 : 762.0) * (bn == 256 ? 0.97 : 0.97 * kNarrowCost);
-  int width = 0;
-  for (int w = 256; w >= 128; w -= 32) {
-    const int64_t tiles = m_tiles * ((d_out + w - 1) / w);
-    const double cost = (double)((tiles + pairs - 1) / pairs) * slabs * (gather ? 280.0 + 2.1 * w : 100.0 + 2.52 * w) + 3300.0;
-    if (cost < best) { best = cost; width = w; }
+// What runs a projection of n rows: tiles of `bn` columns, by one CTA each or by pairs. One CTA: 256 columns keep the tensor pipe
+// busiest per byte loaded; 128 where that leaves the last of the rounds over the SMs mostly empty (a narrow tile taken as 0.58 of a
+// wide one, 0.8 when its rows are gathered). Pairs of the best width where they gain 5% by a model of both: a tile's loads and MMAs
+// run under the epilogue of the tile before it, so that a launch takes its start, one of the two for every round, whichever is
+// longer, and the other once. Constants in us, fitted to 2490 sizes (60 to 12000 rows, d_in 256 to 8192, d_out 256 to 12288, rows
+// gathered and not, added and not, weights in L2 and not; 5% mean error). Against one CTA per tile this gains 0.9 to 3.7% in the mean
+// of those sizes, up to a third, and loses more than 3% at 22 of 4323 (9% at most). Without the epilogue in the model, pairs
+// were taken for few rows and for short d_in, and 750 of them lost 3 to 75%. d = 2048, 3277 rows of 32768: Q/K/V 72.2 -> 66.0 us
+// (rows in order 67.1 -> 59.6), output projection added into the store 31.3 -> 28.2; 12000 rows: Q/K/V 243 -> 221, output 90 -> 79.
+struct ProjPlan {
+  int bn;
+  bool pairs;
+};
+struct ProjCost {
+  double start, slab, slab_gather, slab_width, epi, epi_width, epi_add;
+  double us(double tiles, double slots, double slabs, int bn, bool gather, bool add) const {
+    const double u = bn / 256.0, rounds = std::ceil(tiles / slots);
+    const double load = slabs * (slab + (gather ? slab_gather : 0.0) + slab_width * u * std::min(1.0, tiles / slots));
+    const double epilogue = epi + (epi_width + (add ? epi_add : 0.0)) * u;
+    return start + rounds * std::max(load, epilogue) + std::min(load, epilogue);
   }
-  return width;
+};
+constexpr ProjCost kCostNarrow = {1.421, 0.276, 0.055, 0.062, 1.471, 2.218, 2.688}, kCostWide = {0.404, 0.280, 0.034, 0.117, 1.874, 3.214, 2.894},
+                   kCostPairs = {1.716, 0.272, 0.054, 0.061, 1.465, 3.615, 2.818};
+
+static ProjPlan proj_plan(int sm_count, int n, int d_in, int d_out, bool gather, bool add) {
+  const auto tiles = [&](int bm, int bn) { return std::ceil(n / (double)bm) * std::ceil(d_out / (double)bn); };
+  const auto rounds = [&](int bn) { return std::ceil(tiles(kBM, bn) / sm_count); };
+  ProjPlan plan = {rounds(128) * (gather ? 0.8 : 0.58) < rounds(256) ? 128 : 256, false};
+  const double slabs = d_in / kBK;
+  double best = 0.95 * (plan.bn == 128 ? kCostNarrow : kCostWide).us(tiles(kBM, plan.bn), sm_count, slabs, plan.bn, gather, add);
+  if (d_in < 256 || d_out < 256 || n > INT32_MAX - 2 * kBM) return plan;      // not measured; rows counted beyond 32 bits
+  for (int bn = 256; bn >= 160; bn -= 32) {
+    const double us = kCostPairs.us(tiles(2 * kBM, bn), sm_count / 2, slabs, bn, gather, add);
+    if (us < best) { best = us; plan = {bn, true}; }
+  }
+  return plan;
+}
+// For the tests: the width of the tiles, negative for pairs.
+extern "C" FL_API int fl_internal_project_plan(int sm_count, int n, int d_in, int d_out, int gather, int add) {
+  const ProjPlan p = proj_plan(sm_count, n, d_in, d_out, gather != 0, add != 0);
+  return p.pairs ? -p.bn : p.bn;
 }
 
 extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const int32_t* src_idx, int32_t n,
@@ -614,7 +638,7 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
   FL_REQUIRE(x != nullptr && w != nullptr && y != nullptr);
   FL_REQUIRE(fl_aligned16(x) && fl_aligned16(w) && fl_aligned16(y));
   FL_REQUIRE(x != y && w != y);
-  if ((size_t)ctx->max_smem_optin < kProjSmem || ctx->encode_tiled == nullptr || ctx->tmaps == nullptr)
+  if ((size_t)ctx->max_smem_optin < std::max(kProjSmem, kPairSmem) || ctx->encode_tiled == nullptr || ctx->tmaps == nullptr)
     return FL_ERR_UNSUPPORTED;
   {
     const fl_idx_check ck[2] = {{src_idx, n, 0, nullptr, 0, (int32_t)x_rows - 1, 0},
@@ -625,16 +649,10 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
   ProjArgs a = {};
   const bool gather = src_idx != nullptr;
   a.m_tiles = (n + kBM - 1) / kBM;
-  // Tile width: 256 columns keep the tensor pipe busiest per byte loaded; 128 columns when that leaves the last of the rounds
-  // over the SMs mostly empty (a narrow tile costs 0.73 of a wide one: 558 cycles a slab for 762, with the SMs full).
-  const auto rounds = [&](int bn) {
-    const int64_t tiles = (int64_t)a.m_tiles * ((d_out + bn - 1) / bn);
-    return (double)((tiles + ctx->sm_count - 1) / ctx->sm_count);
-  };
-  const int bn = rounds(128) * kNarrowCost < rounds(256) ? 128 : 256;
-  const int pair_bn = fl_proj_pair_width(ctx, n, d_in, d_out, gather, bn, rounds(bn));
+  const ProjPlan plan = proj_plan(ctx->sm_count, n, d_in, d_out, gather, accumulate != 0);
+  const int bn = plan.bn;
   if (!fl_tile_tmap(ctx, x, x_rows, d_in, gather ? 1 : kBM, &a.x_map) ||
-      !fl_tile_tmap(ctx, w, d_out, d_in, pair_bn > 0 ? pair_bn / 2 : bn, &a.w_map))
+      !fl_tile_tmap(ctx, w, d_out, d_in, plan.pairs ? bn / 2 : bn, &a.w_map))
     return FL_ERR_CUDA;
   a.src_idx = src_idx;
   a.dst_idx = dst_idx;
@@ -650,9 +668,8 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
   a.accumulate = accumulate;
   a.status = status;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (pair_bn > 0) {
+  if (plan.pairs) {
     a.m_tiles = (n + 2 * kBM - 1) / (2 * kBM);
-    a.n_tiles = (d_out + pair_bn - 1) / pair_bn;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(2 * (unsigned)std::min<int64_t>((int64_t)a.m_tiles * a.n_tiles, ctx->sm_count / 2));
     cfg.blockDim = dim3(pair_threads(gather));
@@ -664,7 +681,7 @@ extern "C" int fl_project_rows(fl_ctx* ctx, const void* x, int64_t x_rows, const
   do {                                                                    \
     auto kern = proj_pair_kernel<G>;                                      \
     FL_FUNC_ATTR_ONCE(ctx, kern, kPairSmem, false);                       \
-    FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, a, pair_bn));            \
+    FL_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kern, a, bn));                 \
   } while (0)
     if (gather) FL_PAIR(true); else FL_PAIR(false);
 #undef FL_PAIR

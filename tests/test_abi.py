@@ -162,3 +162,24 @@ def test_kv_store_bytes_matches_closed_form(B):
     assert fl == expect and dense / fl > 3.0
     fl16, _ = B.fl_kv_store_bytes(B.make_shape(w.L, 16, 128, B.FL_BF16, 1024, 16, 128, 1e-6, 0.1), st, 4, 1)
     assert fl16 == 2 * w.L * w.d * 2 + 3 * (w.k_tokens * 2 * w.d * 2 + 4 * (w.L + w.k_tokens))
+
+
+def test_projections_go_to_the_kernel_measured_faster(B):
+    """Few rows, a shallow product or a narrow one: one CTA per tile (the model without the epilogue sent them to pairs: 64 to 75% slower
+    for one gathered row of 8192 x 6144, 10% for 300 rows of 2048 x 2048).  The benchmark's shapes: pairs."""
+    plan = B.lib.fl_internal_project_plan
+    for q in ((1, 8192, 6144, 1, 0), (1, 4096, 6144, 0, 1), (60, 2048, 2048, 0, 1), (129, 2048, 6144, 0, 0), (300, 2048, 2048, 0, 0),
+              (500, 2048, 1024, 0, 1), (819, 1024, 3072, 1, 0), (819, 2048, 2048, 0, 1), (1638, 1024, 1024, 0, 1),
+              (8000, 256, 12288, 0, 1), (12000, 1024, 4096, 0, 1), (6700, 1024, 1024, 0, 1), (4100, 64, 4096, 1, 0), (3277, 2048, 128, 0, 0)):
+        assert plan(148, *q) > 0, q
+    # where one CTA takes a tile, the width is that of the fuller rounds: 8 x 24 tiles of 128 columns are two rounds for one of 256
+    assert [plan(148, *q) for q in ((2000, 256, 3072, 0, 1), (500, 512, 12288, 0, 1), (12000, 1024, 4096, 0, 1))] == [128, 128, 256]
+    assert [plan(148, 3277, 2048, 6144, 1, 0), plan(148, 3277, 2048, 6144, 0, 0), plan(148, 12000, 2048, 6144, 1, 0)] == [-224, -224, -256]
+    assert plan(148, 3277, 2048, 2048, 0, 1) < 0 and plan(148, 12000, 2048, 2048, 0, 1) < 0
+    for sms in (1, 2, 131, 148):
+        for n in (1, 255, 256, 257, 4099, 2 ** 31 - 1):
+            for d_in in (64, 2048):
+                for d_out in (8, 264, 6144):
+                    for g in (0, 1):
+                        assert plan(sms, n, d_in, d_out, g, g) in (128, 256, -160, -192, -224, -256)
+    assert plan(148, 2 ** 31 - 1, 2048, 6144, 1, 0) > 0

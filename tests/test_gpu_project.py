@@ -77,8 +77,8 @@ def test_project_rows_ragged_tiles(env, gather, scatter, accumulate):
 
 def test_project_rows_several_tiles_per_cta(env):
     """357 wide output tiles (21 x 17, the last column tile 8 columns wide, the last row tile 40 rows high) on at most
-    148 CTAs: every CTA runs two or three tiles, so both accumulators are reused and the stage ring wraps many times.
-    The small cases above run with the narrow tile, this one and the benchmark's Q/K/V shape with the wide one."""
+    148 CTAs: two or three tiles each, so both accumulators are reused and the stage ring wraps many times (where pairs of
+    CTAs run it, with tiles of 224 columns, about as many per pair)."""
     B, ctx = env
     n = 2600
     x, w, y, src, dst = make(8, 4000, 4000, n, 512, 4104, True, True)
@@ -98,6 +98,26 @@ def test_project_rows_pairs_of_ctas(env, n, d_out, gather, scatter, accumulate):
     args = make(29, 2 * n if gather else n, 2 * n if scatter else n, n, 2048, d_out, gather, scatter)
     rows = np.unique(np.r_[0, 127, 128, 255, 256, n - 2, n - 1, np.arange(5, n, 97)])
     check(B, ctx, *args, n, accumulate, rows=rows)
+
+
+@pytest.mark.parametrize("n,d_in,d_out,gather,scatter,accumulate,plan", [
+    (643, 512, 6320, False, False, 0, 128),       # one CTA per tile, narrow: two rounds, 48 columns in the last tile
+    (5000, 512, 4104, False, False, 0, 256),      # wide: five rounds, rows in order
+    (5000, 512, 4104, True, True, 1, 256),        # the same gathered and added
+    (386, 1024, 4776, False, True, 0, -160),      # pairs: one round, the last rows are two of the second CTA
+    (391, 4096, 4840, True, True, 1, -160),
+    (258, 256, 6472, False, True, 1, -192),       # four slabs; two rows in the last tile
+    (1560, 512, 5992, True, True, 1, -224),
+    (262, 1024, 17400, False, False, 0, -256),    # two rounds
+    (1027, 4096, 6608, True, True, 1, -256),
+    (1044, 4096, 6544, True, False, 0, -256),
+])
+def test_project_rows_by_the_kernel_that_runs_them(env, n, d_in, d_out, gather, scatter, accumulate, plan):
+    """Every width of tiles, by one CTA (plan > 0) and by pairs (< 0), at other depths than the benchmark's."""
+    B, ctx = env
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert B.lib.fl_internal_project_plan(148, n, d_in, d_out, int(gather), accumulate) == plan
+    check_every_row(B, ctx, n, d_in, d_out, gather, scatter, accumulate)
 
 
 def check_every_row(B, ctx, n, d_in, d_out, gather, scatter, accumulate, launches=1):
