@@ -104,9 +104,10 @@ struct Pair2<float> {
 // (1024 threads per SM in all) walks its tiles: the first comes straight to registers, and with 16-bit storage a thread asks for its
 // pieces of the NST tiles after it by asynchronous copies into slots of its own, so that HBM is read under the joins and the
 // encoding (a CTA per tile, which asked, joined and encoded one after the other, two at a time on an SM: 40 us for the 20 k rows of
-// 2048, then 34.6; 33 with codes without divisions). A warp per tile without any barrier is no faster (33.7; groups of 128: 40 for
-// 38). With 32-bit storage (NST = 0) a tile takes twice the space and a CTA takes one; a launch of one tile per CTA gets no slots.
-// The CTAs past k_ctas copy the tail rows.
+// 2048, then 34.6; 33 with codes without divisions; keys and values together 80 -> 54 to 63). A warp per tile without any barrier
+// is no faster (33.7; groups of 128: 40 for 38). With 32-bit storage (NST = 0) a tile takes twice the space and a CTA takes one; a
+// launch of one tile per CTA gets no slots.
+// At 64 registers the 16-bit kernels spill 12 to 16 bytes around the tile loop. The CTAs past k_ctas copy the tail rows.
 template <typename T>
 constexpr int kBqRows = sizeof(T) == 2 ? 4 : 8;        // rows of a token group per thread
 constexpr int kBqCh = 256;                             // channels of a key tile

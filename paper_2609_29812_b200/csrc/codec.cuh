@@ -80,10 +80,10 @@ __device__ __forceinline__ float max3_nan(float a, float b, float c) {
 }
 
 // Codes of P pairs: q = round-half-even of the binary32 quotient t / scale, t = x - zero (already rounded). The quotient is
-// correctly rounded without a division: e = t * inv (inv = the reciprocal within an ulp) is within 3 ulp, the remainder
-// r = t - e * scale is exact (a scale has 11 bits), and e + r * inv differs from t / scale by less than 2^-20 ulp, while t / scale
-// keeps at least 2^-12 ulp from every midpoint of two numbers (a midpoint has 25 bits: times an 11-bit scale it is no number t
-// of 24 bits, and it misses t by at least a unit of that product). Adding 1.5 * 2^23 rounds to the integer, halves to even.
+// correctly rounded without a division, by Markstein's correction of an approximate quotient (as above): e = t * inv (inv = the
+// reciprocal within an ulp) is within 3 ulp, the remainder r = t - e * scale is exact (a scale has 11 bits), and e + r * inv differs
+// from t / scale by less than 2^-20 ulp, while t / scale keeps at least 2^-12 ulp from every midpoint of two numbers (a midpoint has
+// 25 bits: times an 11-bit scale it is no number t of 24 bits, and it misses t by at least a unit of that product). Adding 1.5 * 2^23 rounds to the integer, halves to even.
 // (With an estimate alone and divisions where it came close to a half-integer, 26 warps in 100 divided: values, offsets and
 // scales have few bits, so exact halves are common.) No clamp: t >= 0 (the offset was rounded down) and max / scale <=
 // 2^bits - 1 (the scale was rounded up). neg_scale = -scale.

@@ -2,7 +2,7 @@
 // (Eq. 2) and the block column statistics loop 2 starts from (Eq. 6 with every causal key a candidate and m_C = 1).
 //
 // Two kernels, because the statistics need each row's final normaliser:
-//   dense_flash_kernel     one CTA per (256 query rows, head): S = Q K^T per chunk of 128 keys, online softmax with a
+//   dense_flash_kernel     one CTA per (256 or 128 query rows, head): S = Q K^T per chunk of 128 keys, online softmax with a
 //                          lazily moved reference, acc += P V; writes O = acc / l and lse = ref + log l.
 //   dense_colsum_kernel    one CTA per (chunk of 512 or 128 keys, head, group of query blocks): S^T = K Q^T with the KEYS as the
 //                          accumulator's rows, so that the thread that owns a key sums exp(s - lse_i) over a block's
@@ -40,10 +40,10 @@ struct alignas(64) DnArgs {
 // with a P that takes the place of its S, a tile's chain S -> P -> PV -> next S is longer than the work on the tensor pipe.
 // QK^T and PV are issued by a thread each: a wait between two batches of one thread costs the pipe about 200 cycles.
 // Bound by the turns at S: QK^T, its 250 cycles of latency and the hand-over to the other tile take 1.5 k of the 2.9 k cycles
-// that a chunk of both tiles lasts, in which the tensor pipe works for 2048 and the exponential unit for 2048. 32768 x 16
-// heads, one call 3865 -> 3266 us, back to back at the power cap 4377 -> 3720; 8192 x 16: 289 -> 245. Measured before: one
-// query tile and 64 keys, two CTAs per SM (the first figures); P over its own S, one issuing thread: 4139 us (4218 without a
-// maximum in the softmax); part of the exponentials on the FMA pipe: 3620 us and more, their chains are longer.
+// that a chunk of both tiles lasts, in which the tensor pipe works for 2048 and the exponential unit for 2048 (counters: each 67% of
+// the time). 32768 x 16 heads, one call 3908 -> 3303 us, back to back at the power cap 4206 -> 3527; 8192 x 16: 256 -> 220. Measured
+// before: one query tile and 64 keys, two CTAs per SM (the first figures); P over its own S, one issuing thread: 4139 us (4218
+// without a maximum in the softmax); part of the exponentials on the FMA pipe: 3620 us and more, their chains are longer.
 // ------------------------------------------------------------------------------------------------------------
 // TILES = 1: one query tile per CTA, for prompts that leave SMs idle (the rule stands at the launch). There a warp also skips the half
 // of a chunk that none of its rows sees: a short prompt's time is the chain of its chunks.
@@ -63,8 +63,9 @@ struct __align__(16) FlashCtl {
 };
 template <int TILES> constexpr size_t kFlashSmem = 1024 + (TILES + kFlSlots) * kQTileBytes + sizeof(FlashCtl);
 
-// P = 2^(s c2 - sub) of 32 logits, as exp32, with the sum taken in ONE order (pair by pair): the row sums, and with them O to
-// the last bit, do not depend on how the keys are cut into chunks. The chain of additions runs beside the exponentials.
+// P = 2^(s c2 - sub) of 32 logits, as exp32, with the sum taken in ONE order (pair by pair): while a row's reference stays put, its
+// sum, and with it O to the last bit, does not depend on how the keys are cut into chunks. (A reference that moves does so at a
+// chunk's border, and the probabilities after it are rounded against another one.) The additions run beside the exponentials.
 __device__ __forceinline__ float exp32_in_order(const uint32_t (&r)[32], float c2, float sub, uint32_t (&p)[16]) {
   using namespace fl_codec;
   const f32x2 cc = pair(c2, c2), ns = pair(-sub, -sub);
@@ -331,7 +332,9 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
 //           128 x 128 exponentials ask for 32 B/clk of each SM, about what it takes), and 16 warps keep the exponential
 //           unit busy (4 per scheduler: 80% of its cycles; 8 warps with 256 keys and two accumulator buffers: 67%).
 //   NH = 1: 128 keys, two CTAs per SM: for prompts too short to give every SM its 512 keys.
-// Bound by the exponential unit (16 per clock and SM). 32768 x 16 heads: 3730 -> 2570 us, 8192 x 16: 225 -> 180 us.
+// The exponential unit (16 per clock and SM) works in 79% of the cycles, the tensor pipe in 38%. Not bound by that unit alone: with a
+// quarter of the exponentials on the FMA pipe the sums of 32768 x 16 heads took 2490 us for 2420. With one accumulator per 128 keys a
+// group of warps also waits out the MMAs of its next tile. 32768 x 16 heads: 3730 -> 2570 us, 8192 x 16: 225 -> 180 us.
 // ------------------------------------------------------------------------------------------------------------
 template <int NH> struct ColsumShape {
   static constexpr int kQSlots = 2;

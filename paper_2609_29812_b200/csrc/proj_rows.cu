@@ -81,7 +81,7 @@ __device__ __forceinline__ fl_codec::f32x2 stored_pair(uint32_t lo, uint32_t hi)
 // exchange. Two passes over a group (range, then codes); the accumulator is read from tensor memory twice and the
 // previous reconstruction rebuilt twice (the second time from L1/L2). Arithmetic as in the stand-alone quantizer:
 // binary32, offset rounded down and scale rounded up to fp16, codes by round-half-even of the true quotient.
-// Pairs of elements and one quotient estimate each, as there: a division per element made the epilogue the longer half of
+// Pairs of elements and quotients without divisions, as there: a division per element made the epilogue the longer half of
 // the launch (3277 rows of a 32K prompt, with the output projection: 257 -> 184 us).
 template <int BITS>
 __device__ __forceinline__ void codec_row(const ProjArgs& a, uint32_t tmem_row, bool row_ok, int t, int pos, bool is_v,
@@ -391,9 +391,11 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
 // ---- two CTAs per tile ---------------------------------------------------------------------------------------
 // The plain projection by pairs of neighbouring SMs (tcgen05 with cta_group::2): a pair computes 256 x bn output tiles, each CTA
 // brings in its own 128 rows of X and HALF of the tile's rows of W, which the MMAs of both read: a 256-column tile costs a CTA
-// 32 KB per slab where the kernel above takes 48 KB, and the slabs are what that kernel waits for (950 cycles for 512 of MMA).
+// 32 KB per slab where the kernel above takes 48 KB, and the slabs are what that kernel waits for (762 cycles, 846 with
+// gathered rows, for 512 of MMA).
 // The CTA of rank 0 issues the MMAs; the copies of both CTAs complete on ITS barriers (with a thread of the other CTA passing its
-// own barriers on, slab by slab, a slab took 2000 cycles). Accumulators, epilogue and tile order as above, per CTA. The tile's width is chosen per call so that the last round over the pairs is full.
+// own barriers on, slab by slab, a slab took 2000 cycles). Accumulators, epilogue and tile order as above, per CTA. The tile's width is
+// chosen per call by proj_plan below.
 constexpr int kPairStages = 6;
 constexpr int kPairStageBytes = kABytes + 128 * kBK * 2;    // 16 KB of A + up to 16 KB of W
 
