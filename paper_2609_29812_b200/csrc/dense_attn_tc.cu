@@ -46,7 +46,8 @@ struct alignas(64) DnArgs {
 // without a maximum in the softmax); part of the exponentials on the FMA pipe: 3620 us and more, their chains are longer.
 // ------------------------------------------------------------------------------------------------------------
 // TILES = 1: one query tile per CTA, for prompts that leave SMs idle (the rule stands at the launch). There a warp also skips the half
-// of a chunk that none of its rows sees: a short prompt's time is the chain of its chunks.
+// of a chunk that none of its rows sees, and the MMAs the second half of a last chunk that has no keys there: a short prompt's time is
+// the chain of its chunks (with whole last chunks 16 x 16 heads took 5.63 us for 5.50, 64 x 16 5.81 for 5.68).
 template <int TILES> struct FlashShape {
   static constexpr int kQk = 4 * TILES, kPv = kQk + 1, kTma = kQk + 2, kThreads = (kQk + 3) * 32;   // warps 0-3, 4-7: softmax of a tile
 };
@@ -97,6 +98,8 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
   const int n_first = (min(a.L, s0 + kM) + kFlNC - 1) / kFlNC;
   const int n_second = TILES > 1 && s0 + kM < a.L ? (min(a.L, s0 + 2 * kM) + kFlNC - 1) / kFlNC : 0;
   const int n_chunks = max(n_first, n_second);
+  // the last chunk of a tile has keys in its first half only
+  const bool half_last = TILES == 1 && min(a.L, s0 + kM) - (n_first - 1) * kFlNC <= kFlNC / 2;
   if (tid == 0) {
     for (int s = 0; s < kFlSlots; ++s) {
       tc::mbar_init(&ctl.kv_full[s], 1);
@@ -141,7 +144,7 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
     __syncwarp();
   } else if (warp == Sh::kQk) {
     if (lane == 0) {
-      const uint32_t idesc = tc::make_idesc_bf16(kM, kFlNC, false);
+      const uint32_t idesc_whole = tc::make_idesc_bf16(kM, kFlNC, false), idesc_half = tc::make_idesc_bf16(kM, kFlNC / 2, false);
       const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32(q_tiles), 16, 1024);
       const uint64_t k_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), 16, 1024);
       const uint32_t hi = (uint32_t)(k_desc0 >> 32);
@@ -161,6 +164,7 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
         }
         tc::tc_fence_after();
         const uint32_t q_lo = q_lo0 + t * (kQTileBytes >> 4), k_lo = k_lo0 + sl * (kQTileBytes >> 4);
+        const uint32_t idesc = half_last && n == n_first - 1 ? idesc_half : idesc_whole;
 #define FL_QK(KK, ACC)                                                                                       \
   tc::mma_ss_lo<ACC>(s_dst, q_lo + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), hi,                    \
                      k_lo + ((((KK) >> 2) * (kFlNC * 128) + ((KK)&3) * 32) >> 4), hi, idesc)
@@ -187,7 +191,8 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
         const uint32_t v_lo = v_lo0 + sl * (kQTileBytes >> 4), p_src = tmem + kFlP + t * 64, acc = tmem + kFlAcc + t * kDH;
 #pragma unroll
         for (int kk = 0; kk < kFlNC / 16; ++kk)            // the first chunk overwrites the accumulator
-          tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc, (n == 0 && kk == 0) ? 0u : 1u);
+          if (kk < kFlNC / 32 || !(half_last && n == n_first - 1))
+            tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc, (n == 0 && kk == 0) ? 0u : 1u);
         tc::mma_commit(&ctl.pv_done[t]);
         if (t == 1 || n >= n_second) tc::mma_commit(&ctl.kv_free[sl]);
       }
@@ -264,13 +269,15 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
       ell += sum1;
       if (whole) {
         ell += exp32_in_order(r[2], c2, sub, p0);
-      } else {
+        tc::tmem_st16(p_addr + 32, p0);
+        ell += exp32_in_order(r[3], c2, sub, p1);
+        tc::tmem_st16(p_addr + 48, p1);
+      } else if (!(half_last && n == n_t - 1)) {           // (else no MMA reads it)
 #pragma unroll
-        for (int u = 0; u < 16; ++u) p0[u] = p1[u] = 0u;
+        for (int u = 0; u < 16; ++u) p0[u] = 0u;
+        tc::tmem_st16(p_addr + 32, p0);
+        tc::tmem_st16(p_addr + 48, p0);
       }
-      tc::tmem_st16(p_addr + 32, p0);
-      if (whole) ell += exp32_in_order(r[3], c2, sub, p1);
-      tc::tmem_st16(p_addr + 48, p1);
       tc::tmem_wait_st();
       tc::tc_fence_before();
       __syncwarp();
@@ -832,7 +839,7 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
   } while (0)
   // One tile per CTA while that leaves no SM with more chunks than the longest tile has (tiles x heads in triangles of chunks, a little
   // above one wave): the tiles of a pair wait for one another at S and for SMs that stand idle. Measured, replaced kernel / pairs /
-  // single tiles, us: 129 x 16 heads 7.5 / 9.2 / 7.3, 400 x 16 10.9 / 12.0 / 9.6, 1024 x 4 18.6 / 18.0 / 14.7, 2048 x 16 (272) 33.9 /
+  // single tiles, us: 16 x 16 heads 5.5 / 6.4 / 5.5, 129 x 16 7.5 / 9.2 / 7.3, 400 x 16 10.9 / 12.0 / 9.6, 1024 x 4 18.6 / 18.0 / 14.7, 2048 x 16 (272) 33.9 /
   // 31.8 / 28.4, 4096 x 8 (264) 61.5 / 56.4 / 44.7; beyond: 1000 x 32 (288) 20.3 / 19.5 / 19.9, 4096 x 16 71 / 61 / 88.
   if ((int64_t)(n_tiles + 1) * s->n_heads <= ctx->sm_count * 19 / 10) FL_FLASH(1); else FL_FLASH(2);
 #undef FL_FLASH
