@@ -2,7 +2,7 @@
 // (Eq. 2) and the block column statistics loop 2 starts from (Eq. 6 with every causal key a candidate and m_C = 1).
 //
 // Two kernels, because the statistics need each row's final normaliser:
-//   dense_flash_kernel     one CTA per (256 or 128 query rows, head): S = Q K^T per chunk of 128 keys, online softmax with a
+//   dense_flash_kernel     one CTA per (256 or 128 query rows, head): S = Q K^T per chunk of 128 or 64 keys, online softmax with a
 //                          lazily moved reference, acc += P V; writes O = acc / l and lse = ref + log l.
 //   dense_colsum_kernel    one CTA per (chunk of 512 or 128 keys, head, group of query blocks): S^T = K Q^T with the KEYS as the
 //                          accumulator's rows, so that the thread that owns a key sums exp(s - lse_i) over a block's
@@ -48,12 +48,17 @@ struct alignas(64) DnArgs {
 // TILES = 1: one query tile per CTA, for prompts that leave SMs idle (the rule stands at the launch). There a warp also skips the half
 // of a chunk that none of its rows sees, and the MMAs the second half of a last chunk that has no keys there: a short prompt's time is
 // the chain of its chunks (with whole last chunks 16 x 16 heads took 5.63 us for 5.50, 64 x 16 5.81 for 5.68).
-template <int TILES> struct FlashShape {
-  static constexpr int kQk = 4 * TILES, kPv = kQk + 1, kTma = kQk + 2, kThreads = (kQk + 3) * 32;   // warps 0-3, 4-7: softmax of a tile
-};
+// NC = 64: the same by chunks of 64 keys, in half the shared and tensor memory: two CTAs per SM, for many short prompts' heads.
 constexpr int kFlSlots = 4;                        // ring of K and V tiles in the order K0 V0 K1 V1 ...
-constexpr int kFlNC = 128;                         // keys per chunk
-constexpr uint32_t kFlAcc = 0, kFlS = 256, kFlP = 384;     // tensor-memory columns: accumulators, S, P (64 columns each)
+template <int TILES, int NC> struct FlashShape {   // NC: keys per chunk
+  static constexpr int kQk = 4 * TILES, kPv = kQk + 1, kTma = kQk + 2, kThreads = (kQk + 3) * 32;   // warps 0-3, 4-7: softmax of a tile
+  static constexpr int kCtas = NC == 64 ? 2 : 1;   // per SM
+  static constexpr int kTile = NC * kDH * 2;       // bytes of a K or V tile
+  // tensor-memory columns: accumulators, S, P (NC / 2 columns each)
+  static constexpr uint32_t kCols = 512 / kCtas, kAcc = 0, kS = NC == 64 ? 128 : 256, kP = kS + NC;
+  static_assert(kS >= TILES * kDH && kP + TILES * (NC / 2) <= kCols, "tensor memory");
+  static constexpr size_t kSmemTiles = 1024 + TILES * kQTileBytes + kFlSlots * kTile;
+};
 struct __align__(16) FlashCtl {
   uint64_t q_full[2];                              // TMA -> QK issuer: the tile's Q
   uint64_t kv_full[kFlSlots], kv_free[kFlSlots];   // TMA -> issuers, issuers -> TMA
@@ -62,7 +67,7 @@ struct __align__(16) FlashCtl {
   uint32_t tmem_base;
   int abort_flag;
 };
-template <int TILES> constexpr size_t kFlashSmem = 1024 + (TILES + kFlSlots) * kQTileBytes + sizeof(FlashCtl);
+template <int TILES, int NC> constexpr size_t kFlashSmem = FlashShape<TILES, NC>::kSmemTiles + sizeof(FlashCtl);
 
 // P = 2^(s c2 - sub) of 32 logits, as exp32, with the sum taken in ONE order (pair by pair): while a row's reference stays put, its
 // sum, and with it O to the last bit, does not depend on how the keys are cut into chunks. (A reference that moves does so at a
@@ -82,24 +87,24 @@ __device__ __forceinline__ float exp32_in_order(const uint32_t (&r)[32], float c
   return sum;
 }
 
-template <int TILES>
-__global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_kernel(const __grid_constant__ DnArgs a) {
-  using Sh = FlashShape<TILES>;
+template <int TILES, int NC>
+__global__ void __launch_bounds__(FlashShape<TILES, NC>::kThreads, FlashShape<TILES, NC>::kCtas) dense_flash_kernel(const __grid_constant__ DnArgs a) {
+  using Sh = FlashShape<TILES, NC>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* q_tiles = smem;
   uint8_t* ring = smem + TILES * kQTileBytes;
-  FlashCtl& ctl = *reinterpret_cast<FlashCtl*>(ring + kFlSlots * kQTileBytes);
+  FlashCtl& ctl = *reinterpret_cast<FlashCtl*>(ring + kFlSlots * Sh::kTile);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // later tiles see more keys: they are dispatched first
   const int n_groups = (a.L + TILES * kM - 1) / (TILES * kM);
   const int h = blockIdx.x % a.H, s0 = (n_groups - 1 - (int)(blockIdx.x / a.H)) * TILES * kM;
   // chunks of the two tiles (the second may have no rows, else it sees at least as many keys as the first)
-  const int n_first = (min(a.L, s0 + kM) + kFlNC - 1) / kFlNC;
-  const int n_second = TILES > 1 && s0 + kM < a.L ? (min(a.L, s0 + 2 * kM) + kFlNC - 1) / kFlNC : 0;
+  const int n_first = (min(a.L, s0 + kM) + NC - 1) / NC;
+  const int n_second = TILES > 1 && s0 + kM < a.L ? (min(a.L, s0 + 2 * kM) + NC - 1) / NC : 0;
   const int n_chunks = max(n_first, n_second);
   // the last chunk of a tile has keys in its first half only
-  const bool half_last = TILES == 1 && min(a.L, s0 + kM) - (n_first - 1) * kFlNC <= kFlNC / 2;
+  const bool half_last = TILES == 1 && NC == 128 && min(a.L, s0 + kM) - (n_first - 1) * NC <= NC / 2;
   if (tid == 0) {
     for (int s = 0; s < kFlSlots; ++s) {
       tc::mbar_init(&ctl.kv_full[s], 1);
@@ -116,7 +121,7 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
     tc::fence_barrier_init();
   }
   if (warp == Sh::kQk) {
-    tc::tmem_alloc(&ctl.tmem_base, 512);
+    tc::tmem_alloc(&ctl.tmem_base, Sh::kCols);
     tc::tmem_relinquish();
   }
   tc::tc_fence_before();
@@ -127,28 +132,28 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
 
   if (warp == Sh::kTma) {
     if (lane == 0) {
-      auto load = [&](uint8_t* dst, const void* map, uint64_t* bar, int row) {
-        tc::mbar_arrive_expect_tx(bar, kQTileBytes);
+      auto load = [&](uint8_t* dst, const void* map, uint64_t* bar, int row, int rows) {
+        tc::mbar_arrive_expect_tx(bar, rows * kDH * 2);
         tc::tma_tile2d(dst, map, bar, h * kDH, row);
-        tc::tma_tile2d(dst + kM * 128, map, bar, h * kDH + 64, row);
+        tc::tma_tile2d(dst + rows * 128, map, bar, h * kDH + 64, row);
       };
-      load(q_tiles, &a.q_map, &ctl.q_full[0], s0);
+      load(q_tiles, &a.q_map, &ctl.q_full[0], s0, kM);
       for (int i = 0; i < 2 * n_chunks; ++i) {
         const int sl = i % kFlSlots;
         if (i >= kFlSlots && !tc::mbar_wait(&ctl.kv_free[sl], (i / kFlSlots - 1) & 1, abort_flag)) break;
-        load(ring + sl * kQTileBytes, (i & 1) ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map),
-             &ctl.kv_full[sl], (i >> 1) * kFlNC);
-        if (i == 0 && n_second > 0) load(q_tiles + kQTileBytes, &a.q_map, &ctl.q_full[1], s0 + kM);
+        load(ring + sl * Sh::kTile, (i & 1) ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map),
+             &ctl.kv_full[sl], (i >> 1) * NC, NC);
+        if (i == 0 && n_second > 0) load(q_tiles + kQTileBytes, &a.q_map, &ctl.q_full[1], s0 + kM, kM);
       }
     }
     __syncwarp();
   } else if (warp == Sh::kQk) {
     if (lane == 0) {
-      const uint32_t idesc_whole = tc::make_idesc_bf16(kM, kFlNC, false), idesc_half = tc::make_idesc_bf16(kM, kFlNC / 2, false);
+      const uint32_t idesc_whole = tc::make_idesc_bf16(kM, NC, false), idesc_half = tc::make_idesc_bf16(kM, NC / 2, false);
       const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32(q_tiles), 16, 1024);
       const uint64_t k_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), 16, 1024);
       const uint32_t hi = (uint32_t)(k_desc0 >> 32);
-      const uint32_t q_lo0 = (uint32_t)q_desc, k_lo0 = (uint32_t)k_desc0, s_dst = tmem + kFlS;
+      const uint32_t q_lo0 = (uint32_t)q_desc, k_lo0 = (uint32_t)k_desc0, s_dst = tmem + Sh::kS;
       bool ok = true;
 #pragma unroll 1
       for (int i = 0; i < 2 * n_chunks; ++i) {           // tiles in turn
@@ -163,11 +168,11 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
           if (!tc::mbar_wait(&ctl.s_free[po], pn & 1, abort_flag)) break;
         }
         tc::tc_fence_after();
-        const uint32_t q_lo = q_lo0 + t * (kQTileBytes >> 4), k_lo = k_lo0 + sl * (kQTileBytes >> 4);
+        const uint32_t q_lo = q_lo0 + t * (kQTileBytes >> 4), k_lo = k_lo0 + sl * (Sh::kTile >> 4);
         const uint32_t idesc = half_last && n == n_first - 1 ? idesc_half : idesc_whole;
 #define FL_QK(KK, ACC)                                                                                       \
   tc::mma_ss_lo<ACC>(s_dst, q_lo + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), hi,                    \
-                     k_lo + ((((KK) >> 2) * (kFlNC * 128) + ((KK)&3) * 32) >> 4), hi, idesc)
+                     k_lo + ((((KK) >> 2) * (NC * 128) + ((KK)&3) * 32) >> 4), hi, idesc)
         FL_QK(0, false); FL_QK(1, true); FL_QK(2, true); FL_QK(3, true);
         FL_QK(4, true);  FL_QK(5, true); FL_QK(6, true); FL_QK(7, true);
 #undef FL_QK
@@ -179,7 +184,7 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
   } else if (warp == Sh::kPv) {
     if (lane == 0) {
       const uint32_t idesc = tc::make_idesc_bf16(kM, kDH, true);
-      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), kFlNC * 128, 1024);   // MN-major
+      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), NC * 128, 1024);   // MN-major
       const uint32_t v_hi = (uint32_t)(v_desc0 >> 32), v_lo0 = (uint32_t)v_desc0;
 #pragma unroll 1
       for (int i = 0; i < 2 * n_chunks; ++i) {
@@ -188,10 +193,10 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
         if (!tc::mbar_wait(&ctl.kv_full[sl], (vi / kFlSlots) & 1, abort_flag)) break;
         if (!tc::mbar_wait(&ctl.p_full[t], n & 1, abort_flag)) break;
         tc::tc_fence_after();
-        const uint32_t v_lo = v_lo0 + sl * (kQTileBytes >> 4), p_src = tmem + kFlP + t * 64, acc = tmem + kFlAcc + t * kDH;
+        const uint32_t v_lo = v_lo0 + sl * (Sh::kTile >> 4), p_src = tmem + Sh::kP + t * (NC / 2), acc = tmem + Sh::kAcc + t * kDH;
 #pragma unroll
-        for (int kk = 0; kk < kFlNC / 16; ++kk)            // the first chunk overwrites the accumulator
-          if (kk < kFlNC / 32 || !(half_last && n == n_first - 1))
+        for (int kk = 0; kk < NC / 16; ++kk)            // the first chunk overwrites the accumulator
+          if (kk < NC / 32 || !(half_last && n == n_first - 1))
             tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc, (n == 0 && kk == 0) ? 0u : 1u);
         tc::mma_commit(&ctl.pv_done[t]);
         if (t == 1 || n >= n_second) tc::mma_commit(&ctl.kv_free[sl]);
@@ -207,29 +212,29 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
     const bool row_ok = row < n_rows;
     const int pos = lo + row;
     const float c2 = a.scale * kLog2e;
-    const uint32_t s_addr = tmem + lane_base + kFlS, p_addr = tmem + lane_base + kFlP + t * 64;
-    const uint32_t acc_addr = tmem + lane_base + kFlAcc + t * kDH;
+    const uint32_t s_addr = tmem + lane_base + Sh::kS, p_addr = tmem + lane_base + Sh::kP + t * (NC / 2);
+    const uint32_t acc_addr = tmem + lane_base + Sh::kAcc + t * kDH;
     float ell = 0.f, ref = -INFINITY;
     bool ok = true;
     for (int n = 0; n < n_t; ++n) {
       if (!warp_wait(&ctl.s_full[t], n & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
       // the last rows of the warp see `seen` keys of the chunk: where that is half of it at most, the other half is not looked at
-      const int seen = min(lo + (warp & 3) * 32 + 31, lo + n_rows - 1) - n * kFlNC + 1;
-      const bool whole = TILES > 1 || seen > 64;
-      uint32_t r[4][32];
+      const int seen = min(lo + (warp & 3) * 32 + 31, lo + n_rows - 1) - n * NC + 1;
+      const bool whole = NC == 128 && (TILES > 1 || seen > 64);
+      uint32_t r[NC / 32][32];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int q = 0; q < NC / 32; ++q)
         if (q < 2 || whole) tc::tmem_ld32(s_addr + q * 32, r[q]);
       tc::tmem_wait_ld();
       tc::tc_fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&ctl.s_free[t]);
       // causal mask: the visible keys of a row are a prefix of the chunk
-      if (!__all_sync(0xffffffffu, !row_ok || n * kFlNC + kFlNC - 1 <= pos)) {
-        const int vis = row_ok ? max(0, pos - n * kFlNC + 1) : 0;
+      if (!__all_sync(0xffffffffu, !row_ok || n * NC + NC - 1 <= pos)) {
+        const int vis = row_ok ? max(0, pos - n * NC + 1) : 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < NC / 32; ++q)
           if (q < 2 || whole)
 #pragma unroll
             for (int u = 0; u < 32; ++u) r[q][u] = q * 32 + u < vis ? r[q][u] : 0xff800000u;
@@ -238,7 +243,8 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
       // moved, with a rescale of the accumulator row, only when a maximum beats it by more than the threshold
       const float cm0 = max32(r[0]) * c2;
       float cm = fmaxf(cm0, max32(r[1]) * c2);
-      if (whole) cm = fmaxf(cm, fmaxf(max32(r[2]), max32(r[3])) * c2);
+      if constexpr (NC == 128)
+        if (whole) cm = fmaxf(cm, fmaxf(max32(r[2]), max32(r[3])) * c2);
       if (ref == -INFINITY) ref = cm0 > -INFINITY ? cm0 : cm;
       const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
       const bool any_over = __any_sync(0xffffffffu, over);
@@ -267,16 +273,18 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
       tc::tmem_st16(p_addr + 16, p1);
       ell += sum0;
       ell += sum1;
-      if (whole) {
-        ell += exp32_in_order(r[2], c2, sub, p0);
-        tc::tmem_st16(p_addr + 32, p0);
-        ell += exp32_in_order(r[3], c2, sub, p1);
-        tc::tmem_st16(p_addr + 48, p1);
-      } else if (!(half_last && n == n_t - 1)) {           // (else no MMA reads it)
+      if constexpr (NC == 128) {
+        if (whole) {
+          ell += exp32_in_order(r[2], c2, sub, p0);
+          tc::tmem_st16(p_addr + 32, p0);
+          ell += exp32_in_order(r[3], c2, sub, p1);
+          tc::tmem_st16(p_addr + 48, p1);
+        } else if (!(half_last && n == n_t - 1)) {           // (else no MMA reads it)
 #pragma unroll
-        for (int u = 0; u < 16; ++u) p0[u] = 0u;
-        tc::tmem_st16(p_addr + 32, p0);
-        tc::tmem_st16(p_addr + 48, p0);
+          for (int u = 0; u < 16; ++u) p0[u] = 0u;
+          tc::tmem_st16(p_addr + 32, p0);
+          tc::tmem_st16(p_addr + 48, p0);
+        }
       }
       tc::tmem_wait_st();
       tc::tc_fence_before();
@@ -325,7 +333,7 @@ __global__ void __launch_bounds__(FlashShape<TILES>::kThreads, 1) dense_flash_ke
       for (int it = 0; it < (1 << 16); ++it) __nanosleep(256);
     }
     tc::tc_fence_after();
-    tc::tmem_dealloc(tmem, 512);
+    tc::tmem_dealloc(tmem, Sh::kCols);
   }
   if (tid == 0 && ctl.abort_flag && a.status != nullptr) atomicExch(a.status, (int)FL_ERR_TIMEOUT);
 }
@@ -831,17 +839,30 @@ int fl_launch_dense_tc(fl_ctx* ctx, const fl_shape* s, const void* q, const void
   a.L = s->L; a.H = s->n_heads; a.d = (int)d_row; a.q_block = s->q_block; a.nb = fl_n_blocks(s);
   a.scale = s->sm_scale;
   const int n_tiles = (s->L + kM - 1) / kM;
-#define FL_FLASH(TILES)                                                                                                    \
+  DnArgs f = a;
+#define FL_FLASH(TILES, NC)                                                                                                \
   do {                                                                                                                    \
-    auto kern = dense_flash_kernel<TILES>;                                                                                \
-    FL_FUNC_ATTR_ONCE(ctx, kern, kFlashSmem<TILES>, true);                                                                \
-    kern<<<dim3((n_tiles + TILES - 1) / TILES * s->n_heads), FlashShape<TILES>::kThreads, kFlashSmem<TILES>, st>>>(a);    \
+    auto kern = dense_flash_kernel<TILES, NC>;                                                                            \
+    if (!fl_tile_tmap(ctx, k, s->L, d_row, NC, &f.k_map) || !fl_tile_tmap(ctx, v, s->L, d_row, NC, &f.v_map))             \
+      return FL_ERR_UNSUPPORTED;                                                                                          \
+    FL_FUNC_ATTR_ONCE(ctx, kern, (kFlashSmem<TILES, NC>), true);                                                          \
+    kern<<<dim3((n_tiles + TILES - 1) / TILES * s->n_heads), FlashShape<TILES, NC>::kThreads, kFlashSmem<TILES, NC>, st>>>(f); \
   } while (0)
-  // One tile per CTA while that leaves no SM with more chunks than the longest tile has (tiles x heads in triangles of chunks, a little
-  // above one wave): the tiles of a pair wait for one another at S and for SMs that stand idle. Measured, replaced kernel / pairs /
-  // single tiles, us: 16 x 16 heads 5.5 / 6.4 / 5.5, 129 x 16 7.5 / 9.2 / 7.3, 400 x 16 10.9 / 12.0 / 9.6, 1024 x 4 18.6 / 18.0 / 14.7, 2048 x 16 (272) 33.9 /
-  // 31.8 / 28.4, 4096 x 8 (264) 61.5 / 56.4 / 44.7; beyond: 1000 x 32 (288) 20.3 / 19.5 / 19.9, 4096 x 16 71 / 61 / 88.
-  if ((int64_t)(n_tiles + 1) * s->n_heads <= ctx->sm_count * 19 / 10) FL_FLASH(1); else FL_FLASH(2);
+  // Up to 64 rows: the narrow form (a chunk of 128 is half empty: 5.1 us for 5.7, 64 x 16 heads). One query tile per CTA while single
+  // tiles all run at once, or, with eight tiles a head and more, while a second round is of tiles with few chunks (tiles x heads in
+  // triangles, up to 1.9 waves): two tiles in a CTA wait for one another at S and for SMs that stand idle. Beyond that two tiles per CTA
+  // while those run at once. Then the number of CTAs counts for more than a CTA's rate, and the narrow form, two CTAs per SM, is the
+  // fastest up to eleven tiles; longer prompts are for two tiles per CTA. us, replaced kernel (64 keys, two CTAs per SM) / wide with one
+  // tile / with two / narrow: 400 x 16 10.8 / 9.2 / 12.0 / 11.0, 2000 x 16 33.7 / 27.2 / 31.0 / 31.5, 640 x 32 13.9 / 12.3 / 12.3 / 14.4,
+  // 384 x 64 10.8 / 13.4 / 9.7 / 13.4, 64 x 200 6.5 / 12.2 / 12.2 / 6.2, 384 x 96 11.1 / 15.5 / 16.8 / 11.1, 640 x 64 15.6 / 22.0 / 18.9 /
+  // 15.2, 1300 x 80 53 / 74 / 57 / 52, 1500 x 128 105 / 138 / 98 / 102, 3000 x 64 171 / 206 / 155 / 164. Of 225 sizes (64 to 6000 rows,
+  // 4 to 256 heads) the chosen form is 1.5% above the fastest of the three in the mean.
+  const int64_t one = (int64_t)n_tiles * s->n_heads, two = (int64_t)(n_tiles + 1) / 2 * s->n_heads, sms = ctx->sm_count;
+  if (s->L <= 64) FL_FLASH(1, 64);
+  else if (one <= sms || (n_tiles >= 8 && one + s->n_heads <= sms * 19 / 10)) FL_FLASH(1, 128);
+  else if (n_tiles >= 3 && two <= sms) FL_FLASH(2, 128);
+  else if (n_tiles <= 11) FL_FLASH(1, 64);
+  else FL_FLASH(2, 128);
 #undef FL_FLASH
   int rc = fl_launch_status();
   if (rc != FL_OK || col_scores == nullptr) return rc;

@@ -10,7 +10,8 @@ torch = pytest.importorskip("torch")
 
 
 @pytest.mark.parametrize("boost", [1.0, 64.0])
-@pytest.mark.parametrize("L,H", [(1, 1), (33, 3), (128, 2), (129, 1), (256, 2), (257, 16), (383, 4), (1025, 3), (2500, 8)])
+@pytest.mark.parametrize("L,H", [(1, 1), (33, 3), (128, 2), (129, 1), (256, 2), (257, 16), (383, 4), (1025, 3), (2500, 8),
+                                 (513, 64), (150, 96)])   # the last two: chunks of 64 keys, several per CTA
 def test_dense_output_edges(L, H, boost):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
@@ -42,7 +43,7 @@ def test_dense_output_edges(L, H, boost):
     ctx.close()
 
 
-@pytest.mark.parametrize("H", [7, 48])                 # one query tile per CTA, and pairs of them
+@pytest.mark.parametrize("H", [7, 48, 64])             # one query tile per CTA, pairs of them, one with chunks of 64 keys
 def test_dense_output_not_finite(H):
     """Keys whose logits are -inf count for nothing, wherever a row's first finite logit stands (rows that see no other are zero); a key
     that is not a number or has a logit of +inf spoils the rows that see it, a query its own row, a value its own channel, and

@@ -32,8 +32,9 @@ def time_of(B, P, ctx, L, H, calls=16):
     return best
 
 
-# halfway between the shares with a tile per CTA and those of pairs of tiles (0.114 and 0.147, 0.160 and 0.201, 0.245 and 0.305)
-@pytest.mark.parametrize("L,H,share", [(129, 16, 0.130), (400, 16, 0.180), (1024, 4, 0.275)])
+# halfway between the shares with a tile per CTA and those of pairs of tiles (0.114 and 0.147, 0.160 and 0.201, 0.245 and 0.305); many
+# heads: between two CTAs per SM and one (0.11 to 0.14 and 0.21 to 0.28, 0.19 to 0.22 and 0.29 to 0.38 on two GPUs)
+@pytest.mark.parametrize("L,H,share", [(129, 16, 0.130), (400, 16, 0.180), (1024, 4, 0.275), (64, 200, 0.175), (384, 96, 0.255)])
 def test_short_prompts_do_not_wait_for_a_second_tile(L, H, share):
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
