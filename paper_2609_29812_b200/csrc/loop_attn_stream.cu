@@ -12,21 +12,29 @@
 // term of loop r-1, so B_i and m_i carry over).
 //
 // A CTA computes one (query block, head) problem with ONE pipeline, which leaves room for two CTAs per SM (half the
-// shared memory, half the tensor memory, 256 threads each): the second CTA's gathers, MMAs and exponentials fill the
+// shared memory, half the tensor memory, 448 threads each): the second CTA's gathers, MMAs and exponentials fill the
 // gaps that the dependent chain  QK^T -> exponentials -> PV  leaves in the first one's, and one CTA's prologue and
 // epilogue run under the other's main loop. (cudaOccupancyMaxActiveBlocksPerMultiprocessor answers 1 for any kernel
-// that allocates tensor memory; two CTAs of 256 columns each do run side by side.) What bounds the pair is the rate
-// at which an SM's TMA unit takes four-row gathers: a 32 KB chunk per ~1.3 k cycles with eight issuing warps.
+// that allocates tensor memory; two CTAs of 256 columns each do run side by side.)
 //
-// Warp roles (9 warps): 0-3 softmax (one row of the 128-row tile per thread), 4 the MMA issuer (one thread), 5-8 TMA:
-// the Q tile, then per chunk of 64 columns the K tile and the V tile, each gathered four rows per copy
-// (cp.async.bulk.tensor tile::gather4) into 128B-swizzled operand tiles. K and V have rings of their own (two tiles
-// each): a K tile is free again as soon as its QK^T has completed, long before the chunk's PV.
+// Warp roles (14 warps): 0-7 softmax (a row of the 128-row tile per thread; warps 0-3 take the first 32 columns of every chunk,
+// 4-7 the others), 8 and 9 the issuers of QK^T and of PV, 10-13 TMA: the Q tile, then per chunk of 64 columns the K tile and the
+// V tile, each gathered four rows per copy (cp.async.bulk.tensor tile::gather4) into 128B-swizzled operand tiles. K and V have
+// rings of their own (two tiles each): a K tile is free again as soon as its QK^T has completed, long before the chunk's PV.
 // Columns that are active in this loop are gathered from the rows fl_quant_kv_residual materialized (before the
 // loop's residual for the OLD pass, after it for the NEW pass); this kernel requires them. Columns that carry a
 // payload from an earlier loop only (token sets that shrink) are rebuilt in place by the TMA warps (Eq. 8 chain).
-// Tensor memory (256 columns): accumulator 0-127, two S / P buffers of 64 columns (P, bf16, is written over the first
-// half of the S buffer it was computed from).
+// Tensor memory (256 columns): accumulator 0-127, two S buffers of 64 columns (P, bf16, is written over the first
+// half of each 32 logits that it was computed from).
+//
+// What bounds it (time stamps of the roles, 32768 rows, c = 1024): with a gather request per lane and MMAs issued inside
+// `if (lane == 0)` the TMA warps took 1400 cycles for a tile's requests and a chunk 2.95 k cycles of a CTA, whatever the softmax
+// did (halving a softmax step from 1.9 to 0.95 k cycles changed nothing). Requests and MMAs by one elected thread from uniform
+// operands, two issuers and two softmax warps per 32 rows: 1.9 k, of which 2 are under way per SM. Then K and V arrive 2 k cycles
+// after they are asked for, 33 B/clk per SM: rows out of DRAM and L2. 88 -> 83 us a launch, 131072 rows, c = 2048: 477 -> 416 us.
+//
+// Probabilities are taken against an estimate of the row's largest logit (NEW pass: lse_prev + log m; see start_ref), not against a
+// running maximum: the two halves of a chunk need not agree on anything, and no accumulator is rescaled.
 // Every mbarrier wait is bounded; on a timeout the CTA raises a flag, drains and reports FL_ERR_TIMEOUT.
 #include "tc_attn_common.cuh"
 
@@ -34,16 +42,16 @@ namespace {
 
 using namespace fl_tc;
 
-constexpr int kSmWarps = 4;
-constexpr int kIssueWarp = 4;
-constexpr int kTmaWarp = 5;
-constexpr int kTmaWarps = 4;
-constexpr int kWarps = 9;
+constexpr int kSmWarps = 8;                    // two halves of a chunk's columns, four warps (128 rows) each
+constexpr int kSmThreads = kSmWarps * 32;
+constexpr int kIssueWarp = 8;                  // QK^T, and PV by the warp after it
+constexpr int kTmaWarp = 10;
+constexpr int kTmaWarps = 4;                   // sixteen rows of a K or V tile each
+constexpr int kWarps = 14;
 constexpr int kThreads = kWarps * 32;
-constexpr int kColWarps = 7;                   // warps that read the column list in the prologue (the other two search rows)
+constexpr int kColWarps = 12;                   // warps that read the column list in the prologue (the other two search rows)
 constexpr int kMaxCols = 3072;
 constexpr int kMaxChunks = kMaxCols / kNC + 2;
-constexpr int kTileGathers = kTileBytes / 512; // 32 four-row gathers of 128-byte rows fill a K or V tile
 constexpr uint32_t kAcc = 0, kS = 128;         // tensor-memory columns
 constexpr uint32_t kTmemCols = 256;
 static_assert(3 * kMaxCols * 4 <= 4 * kTileBytes, "prologue staging must fit in the K and V rings");
@@ -57,7 +65,7 @@ struct alignas(64) StArgs {
   const __nv_bfloat16* rows_in;        // [L, d] by position. OLD: previous outputs; NEW: backgrounds
   __nv_bfloat16* rows_out;             // [L, d] by position. OLD: backgrounds; NEW: outputs
   float* mass;                         // [H, L]: written by the OLD pass, read by the NEW pass
-  const float* lse_prev;               // [H, L]: OLD pass (required); NEW pass: copied to lse_out for rows with empty T_i, or null
+  const float* lse_prev;               // [H, L]: OLD pass (required); NEW pass: a hint, copied to lse_out for rows with empty T_i, or null
   float* lse_out;                      // NEW pass
   const __nv_bfloat16* q_new;          // NEW pass: compact new Q rows, copied into q_store at the end
   __nv_bfloat16* q_store;              // NEW pass: Q store [L, d] that receives them, or null
@@ -90,6 +98,8 @@ struct __align__(16) StSmemCtl {
   int warp_cnt[kWarps][2];
   int chunk_last[kMaxChunks];        // largest entry of the chunk, INT32_MAX if the chunk is padded
   int pos[kM];                       // positions of the tile's rows
+  float sum[2][kM];                  // row sums of the two halves: of the probabilities,
+  float rsum[2][kM];                 // and of what is left of them in bf16 (second pass of a tile: the largest logits)
   uint32_t stale[kMaxCols / 32];     // bit u: ordered column u carries a payload from an earlier loop only
 };
 
@@ -195,7 +205,31 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
   const int q_lo = ctl.q_lo + share * kM, q_hi = ctl.q_hi;
+  auto load_q = [&](int s) {   // one warp
+    if (MODE == kNewPass) {
+      // Q tile of this row tile: two 64-element slabs; rows past the compact list read as zero, rows of the next
+      // block (past n_rows) are computed and dropped
+      if (lane == 0) {
+        tc::mbar_arrive_expect_tx(&ctl.q_full, kQTileBytes);
+        tc::tma_tile2d(q_tile, &a.q_map, &ctl.q_full, h * kDH, s);
+        tc::tma_tile2d(q_tile + kM * 128, &a.q_map, &ctl.q_full, h * kDH + 64, s);
+      }
+    } else {
+      // the previous loop's Q rows come from the store: four-row gathers by position, one group of rows per lane
+      if (lane == 0) tc::mbar_arrive_expect_tx(&ctl.q_full, kQTileBytes);
+      __syncwarp();
+      int y[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const int r = lane * 4 + i;
+        y[i] = s + r < q_hi ? __ldg(a.active_idx + s + r) : a.L;   // row L is outside the tensor: reads as zero
+      }
+      tc::tma_gather4(q_tile + lane * 512, &a.q_map, &ctl.q_full, h * kDH, y[0], y[1], y[2], y[3]);
+      tc::tma_gather4(q_tile + kM * 128 + lane * 512, &a.q_map, &ctl.q_full, h * kDH + 64, y[0], y[1], y[2], y[3]);
+    }
+  };
   if (q_hi > q_lo) {   // CTA-uniform: without active rows the CTA only releases the tensor memory
+  if (warp == kTmaWarp) load_q(q_lo);      // the first tile's rows arrive while the column list is partitioned
   {
     // causal prefix, stable partition into plain / patched columns: every warp owns a contiguous span
     const int i_last = ctl.i_last;
@@ -260,33 +294,32 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   int g = 0;                    // chunks issued so far (all tiles): buffers = g & 1, one phase of their barriers per use
   uint32_t dirty_par_cta = 0;   // per-slot phase parity of the patched[] barriers (they only see dirty chunks)
 
-  for (int s0 = q_lo, tile = 0; s0 < q_hi; s0 += row_step, ++tile) {
+  int pass = 0;
+  for (int s0 = q_lo, tile = 0; s0 < q_hi; ++tile) {
   const int n_rows = min(kM, q_hi - s0);
   const int g0 = g;
   const uint32_t dirty_par0 = dirty_par_cta;
-  if (warp == kTmaWarp) {
-    if (MODE == kNewPass) {
-      // Q tile of this row tile: two 64-element slabs; rows past the compact list read as zero, rows of the next
-      // block (past n_rows) are computed and dropped
-      if (lane == 0) {
-        tc::mbar_arrive_expect_tx(&ctl.q_full, kQTileBytes);
-        tc::tma_tile2d(q_tile, &a.q_map, &ctl.q_full, h * kDH, s0);
-        tc::tma_tile2d(q_tile + kM * 128, &a.q_map, &ctl.q_full, h * kDH + 64, s0);
-      }
-    } else {
-      // the previous loop's Q rows come from the store: four-row gathers by position, one group of rows per lane
-      if (lane == 0) tc::mbar_arrive_expect_tx(&ctl.q_full, kQTileBytes);
-      __syncwarp();
-      int y[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = lane * 4 + i;
-        y[i] = r < n_rows ? __ldg(a.active_idx + s0 + r) : a.L;   // row L is outside the tensor: reads as zero
-      }
-      tc::tma_gather4(q_tile + lane * 512, &a.q_map, &ctl.q_full, h * kDH, y[0], y[1], y[2], y[3]);
-      tc::tma_gather4(q_tile + kM * 128 + lane * 512, &a.q_map, &ctl.q_full, h * kDH + 64, y[0], y[1], y[2], y[3]);
+  if (tile > 0 && warp == kTmaWarp) load_q(s0);
+
+  // softmax threads: a row each, half of a chunk's columns
+  const int half_sm = (warp >> 2) & 1, row = (warp & 3) * 32 + lane;
+  const bool row_ok = warp < kSmWarps && row < n_rows;
+  int pos = -1;
+  float mass = 0.f, ell = 0.f, ref = 0.f;
+  bool ok = true, bad = false, seen = false;
+  uint8_t* stage = q_tile;                     // [128 rows][16 x 16 B], 16-byte cells XOR-swizzled by row
+  const size_t col0 = (size_t)h * kDH;
+  // The rows that come in (previous outputs / backgrounds) are staged in the Q tile with coalesced asynchronous copies.
+  // Every QK^T has read it once the last chunk's S is there: the copies run under that chunk's exponentials.
+  auto stage_rows = [&]() {
+#pragma unroll 4
+    for (int k = 0; k < 8; ++k) {
+      const int rr = k * 16 + (tid >> 4), cc = tid & 15;
+      if (rr < n_rows)
+        tc::cp_async16(stage + rr * 256 + ((cc ^ (rr & 7)) << 4), a.rows_in + (size_t)ctl.pos[rr] * a.d + col0 + cc * 8);
     }
-  }
+    tc::cp_async_commit();
+  };
 
   if (warp >= kTmaWarp) {
     // ========================================== TMA + patch ==========================================
@@ -295,35 +328,22 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     // later than K). The 32 four-row gathers of a tile (2 slabs x 16 groups) are dealt round robin to the warps, one
     // per lane; every warp announces its own share of the bytes on the tile's barrier.
     const int tw = warp - kTmaWarp;
-    const int req = lane * kTmaWarps + tw;
-    const int my_reqs = (kTileGathers - 1 - tw) / kTmaWarps + 1;     // requests of this warp per tile (lanes 0 .. my_reqs - 1)
-    const int slab = (req >> 4) & 1, grp = req & 15;
     const int half = lane >> 4, ch = lane & 15;
     const DevSide& side = half ? a.v : a.k;
     const int elem = h * kDH + ch * 8;
     const __nv_bfloat16* base_rows = static_cast<const __nv_bfloat16*>(side.base) + elem;
     const uint32_t ch_off = (ch >> 3) * (kNC * 128);
-    bool ok = true;
     // gather one tile (is_v: V, else K) of chunk ci into ring slot (gc & 1)
     auto fill = [&](int ci, int gc, bool is_v) {
       const ChunkInfo ck = chunk_info(ci, n_plain, n_patch);
       uint64_t* bar = is_v ? &ctl.v_landed[gc & 1] : &ctl.k_landed[gc & 1];
-      if (lane == 0) tc::mbar_arrive_expect_tx(bar, my_reqs * 512);
-      __syncwarp();
-      if (req < kTileGathers) {
-        int y[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int u = grp * 4 + i;
-          // a row past the end of the tensor reads as zero. Columns that are active in this loop come from the
-          // materialized rows, indexed by their row in the loop's stream
-          y[i] = u < ck.n_valid ? ord_col[ck.off + u] : (ck.patch ? a.n_active : a.L);
-        }
-        const void* src = ck.patch ? (is_v ? static_cast<const void*>(&a.v_rows_map) : static_cast<const void*>(&a.k_rows_map))
-                                   : (is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map));
-        uint8_t* dst = (is_v ? v_ring : k_ring) + (gc & 1) * kTileBytes + slab * (kNC * 128) + grp * 512;
-        tc::tma_gather4(dst, src, bar, h * kDH + slab * 64, y[0], y[1], y[2], y[3]);
-      }
+      // a row past the end of the tensor reads as zero. Columns that are active in this loop come from the
+      // materialized rows, indexed by their row in the loop's stream
+      const int u = tw * 16 + (lane & 15);
+      const int y = u < ck.n_valid ? ord_col[ck.off + u] : (ck.patch ? a.n_active : a.L);
+      const void* src = ck.patch ? (is_v ? static_cast<const void*>(&a.v_rows_map) : static_cast<const void*>(&a.k_rows_map))
+                                 : (is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map));
+      gather_rows<4>((is_v ? v_ring : k_ring) + (gc & 1) * kTileBytes + tw * 2048, kNC * 128, src, bar, h * kDH, y);
     };
     const int n_mine = n_chunks;
     if (n_mine > 0) {
@@ -365,111 +385,105 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
         if (lane == 0) tc::mbar_arrive(&ctl.patched[gc & 1]);
       }
     }
-    if (MODE == kNewPass && a.q_store != nullptr && ok) {
-      // the new Q rows take their place in the Q store for the next loop (this pass reads no Q row from it)
-      const int pt = tid - kTmaWarp * 32;
-#pragma unroll 1
-      for (int it = pt; it < n_rows * 16; it += kTmaWarps * 32) {
-        const int r = it >> 4, c16 = it & 15;
-        const int pos_r = __ldg(a.active_idx + s0 + r);
-        *reinterpret_cast<uint4*>(a.q_store + (size_t)pos_r * a.d + h * kDH + c16 * 8) =
-            __ldg(reinterpret_cast<const uint4*>(a.q_new + (size_t)(s0 + r) * a.d + h * kDH + c16 * 8));
-      }
-    }
-  } else if (warp == kIssueWarp) {
-    // ========================================== MMA issuer ===========================================
-    // QK^T of chunk n (its S buffer is free once PV of chunk n - 2 has retired), then PV of chunk n - 1 (its P is
-    // written while QK^T of chunk n executes).
-    if (lane == 0) {
-      const uint32_t idesc_qk = tc::make_idesc_bf16(kM, kNC, false);
-      const uint32_t idesc_pv = tc::make_idesc_bf16(kM, kDH, true);
+  } else if (warp >= kIssueWarp) {
+    // ========================================== MMA issuers ==========================================
+    // One warp issues S = Q Khat^T of chunk after chunk (its S buffer is free once PV of the chunk before the previous one has
+    // retired), the next one acc += P Vhat. The whole warp walks the chunks and waits, one elected thread issues: with the
+    // loop inside `if (lane == 0)` every operand went through per-lane code, ~90 cycles an MMA and ~300 a wait.
+    const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t s_base = tmem_u + kS;
+    uint32_t dirty_par = dirty_par0;
+    if (warp == kIssueWarp) {
+      const uint32_t idesc = tc::make_idesc_bf16(kM, kNC, false);
       const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32(q_tile), 16, 1024);
       const uint64_t k_desc0 = tc::make_desc_sw128(tc::smem_u32(k_ring), 16, 1024);
       const uint32_t kq_hi = (uint32_t)(k_desc0 >> 32);
       const uint32_t q_lo_w = (uint32_t)q_desc, k_lo0 = (uint32_t)k_desc0;
-      // MN-major Vhat: 16 key rows = two 1024-byte row groups per K step
-      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(v_ring), kNC * 128, 1024);
-      const uint32_t v_hi = (uint32_t)(v_desc0 >> 32), v_lo0 = (uint32_t)v_desc0;
-      const uint32_t s_base = tmem + kS, acc = tmem + kAcc;
-      uint32_t dirty_par = dirty_par0;
+      if (n_chunks > 0) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
 #pragma unroll 1
-      for (int n = 0; n <= n_chunks; ++n) {
-        const int gc = g0 + n;
-        if (n < n_chunks) {
-          const int sl = gc & 1;
-          if (n == 0 && !tc::mbar_wait(&ctl.q_full, tile & 1, abort_flag)) break;
-          if (!tc::mbar_wait(&ctl.k_landed[sl], (gc >> 1) & 1, abort_flag)) break;
-          if (chunk_dirty(chunk_info(n, n_plain, n_patch))) {
-            if (!tc::mbar_wait(&ctl.patched[sl], (dirty_par >> sl) & 1, abort_flag)) break;
-            dirty_par ^= 1u << sl;
-          }
-          // the S buffer holds P of the chunk before the previous one until its PV MMAs have read it
-          if (gc >= 2 && !tc::mbar_wait(&ctl.p_free[sl], ((gc >> 1) - 1) & 1, abort_flag)) break;
+      for (int n = 0; n < n_chunks && ok; ++n) {
+        const int gc = g0 + n, sl = gc & 1;
+        const bool dirty = chunk_dirty(chunk_info(n, n_plain, n_patch));
+        // the S buffer holds P of the chunk before the previous one until its PV MMAs have read it
+        if (gc >= 2 && !warp_wait(&ctl.p_free[sl], ((gc >> 1) - 1) & 1, abort_flag)) break;
+        if (!warp_wait(&ctl.k_landed[sl], (gc >> 1) & 1, abort_flag)) break;
+        if (dirty) {
+          if (!warp_wait(&ctl.patched[sl], (dirty_par >> sl) & 1, abort_flag)) break;
+          dirty_par ^= 1u << sl;
+        }
+        tc::tc_fence_after();
+        if (tc::elect_one()) {
           const uint32_t s_dst = s_base + sl * kNC;
-          tc::tc_fence_after();
           const uint32_t k_lo = k_lo0 + sl * (kTileBytes >> 4);
 #define FL_QK(KK, ACC)                                                                                       \
   tc::mma_ss_lo<ACC>(s_dst, q_lo_w + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), kq_hi,               \
-                     k_lo + ((((KK) >> 2) * (kNC * 128) + ((KK)&3) * 32) >> 4), kq_hi, idesc_qk)
+                     k_lo + ((((KK) >> 2) * (kNC * 128) + ((KK)&3) * 32) >> 4), kq_hi, idesc)
           FL_QK(0, false); FL_QK(1, true); FL_QK(2, true); FL_QK(3, true);
           FL_QK(4, true);  FL_QK(5, true); FL_QK(6, true); FL_QK(7, true);
 #undef FL_QK
           tc::mma_commit(&ctl.s_full[sl]);
         }
-        if (n > 0) {
-          const int gp = gc - 1, pb = gp & 1;
-          if (!tc::mbar_wait(&ctl.v_landed[pb], (gp >> 1) & 1, abort_flag)) break;
-          if (!tc::mbar_wait(&ctl.p_full[pb], (gp >> 1) & 1, abort_flag)) break;
-          tc::tc_fence_after();
+        __syncwarp();
+      }
+    } else {
+      const uint32_t idesc = tc::make_idesc_bf16(kM, kDH, true);
+      // MN-major Vhat: 16 key rows = two 1024-byte row groups per K step
+      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(v_ring), kNC * 128, 1024);
+      const uint32_t v_hi = (uint32_t)(v_desc0 >> 32), v_lo0 = (uint32_t)v_desc0;
+      const uint32_t acc = tmem_u + kAcc;
+#pragma unroll 1
+      for (int n = 0; n < n_chunks; ++n) {
+        const int gc = g0 + n, pb = gc & 1;
+        if (chunk_dirty(chunk_info(n, n_plain, n_patch))) {
+          if (!warp_wait(&ctl.patched[pb], (dirty_par >> pb) & 1, abort_flag)) break;
+          dirty_par ^= 1u << pb;
+        }
+        if (!warp_wait(&ctl.v_landed[pb], (gc >> 1) & 1, abort_flag)) break;
+        if (!warp_wait(&ctl.p_full[pb], (gc >> 1) & 1, abort_flag)) break;
+        tc::tc_fence_after();
+        if (tc::elect_one()) {
           const uint32_t v_lo = v_lo0 + pb * (kTileBytes >> 4);
           const uint32_t p_src = s_base + pb * kNC;
-          const uint32_t acc0 = n > 1 ? 1u : 0u;           // the tile's first chunk overwrites the accumulator
+          const uint32_t acc0 = n > 0 ? 1u : 0u;           // the tile's first chunk overwrites the accumulator
 #pragma unroll
           for (int kk = 0; kk < kNC / 16; ++kk)
-            tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc_pv, kk > 0 ? 1u : acc0);
+            tc::mma_ts_lo(acc, p_src + (kk >> 1) * (kNC / 2) + (kk & 1) * 8, v_lo + kk * (2048 >> 4), v_hi, idesc,
+                          kk > 0 ? 1u : acc0);
           tc::mma_commit(&ctl.p_free[pb]);
         }
+        __syncwarp();
       }
-      tc::mma_commit(&ctl.acc_done);
+      if (tc::elect_one()) tc::mma_commit(&ctl.acc_done);
+      __syncwarp();
     }
-    __syncwarp();
   } else {
     // ============================================ softmax ============================================
-    const int row = warp * 32 + lane;
-    const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-    const bool row_ok = row < n_rows;
-    const int pos = row_ok ? __ldg(a.active_idx + s0 + row) : -1;
+    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+    pos = row_ok ? __ldg(a.active_idx + s0 + row) : -1;
     const float c2 = a.scale * kLog2e;
-    const float lse2 = ((row_ok && MODE == kOldPass) ? a.lse_prev[(size_t)h * a.L + pos] : 0.f) * kLog2e;
-    const float mass = (row_ok && MODE == kNewPass) ? a.mass[(size_t)h * a.L + pos] : 0.f;
-    // the epilogue reads the row's previous output (NEW pass: its background): have it in L2 by then
-    if (row_ok) {
-      tc::prefetch_l2(a.rows_in + (size_t)pos * a.d + h * kDH);
-      tc::prefetch_l2(a.rows_in + (size_t)pos * a.d + h * kDH + 64);
-    }
-    ctl.pos[row] = pos;
-    asm volatile("bar.sync 1, 128;" ::: "memory");
-    const size_t col0 = (size_t)h * kDH;
-    uint8_t* stage = q_tile;                     // [128 rows][16 x 16 B], 16-byte cells XOR-swizzled by row
-    // The rows that come in (previous outputs / backgrounds) are staged in the Q tile with coalesced asynchronous copies.
-    // Every QK^T has read it once the last chunk's S is there: the copies run under that chunk's exponentials.
-    auto stage_rows = [&]() {
-#pragma unroll 4
-      for (int k = 0; k < 16; ++k) {
-        const int rr = k * 8 + (tid >> 4), cc = tid & 15;
-        if (rr < n_rows)
-          tc::cp_async16(stage + rr * 256 + ((cc ^ (rr & 7)) << 4), a.rows_in + (size_t)ctl.pos[rr] * a.d + col0 + cc * 8);
+    // what the row's probabilities are taken against, as a power of two: any number near the row's largest logit does
+    float lse2 = 0.f;
+    if (row_ok && a.lse_prev != nullptr) lse2 = a.lse_prev[(size_t)h * a.L + pos] * kLog2e;
+    if (MODE == kOldPass) {
+      ref = lse2;
+    } else {
+      mass = row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f;
+      if (pass < 2) {
+        ref = start_ref(a.lse_prev != nullptr ? lse2 + log2f(mass) : 0.f);
+      } else {
+        ref = fmaxf(ctl.rsum[0][row], ctl.rsum[1][row]);      // -inf: no column is seen with a finite logit
       }
-      tc::cp_async_commit();
-    };
-    const uint32_t s_addr = tmem + lane_base + kS;
-    float ell = 0.f, ref = -INFINITY;    // OLD pass: ell is the mass, ref stays unused
-    bool ok = true;
+    }
+    // the epilogue reads the row's previous output (NEW pass: its background): have it in L2 by then
+    if (row_ok) tc::prefetch_l2(a.rows_in + (size_t)pos * a.d + h * kDH + half_sm * 64);
+    if (half_sm == 0) ctl.pos[row] = pos;
+    asm volatile("bar.sync 1, %0;" ::"n"(kSmThreads) : "memory");
+    const float sub = ref > -INFINITY ? ref : 0.f;
+    const uint32_t s_addr = tmem + lane_base + kS + half_sm * (kNC / 2);
+    float top = -INFINITY;
+    float2 sums = make_float2(0.f, 0.f);
     for (int ci = 0; ci < n_chunks; ++ci) {
-      const int gc = g0 + ci, pb = gc & 1, n_use = gc >> 1;
-      if (!warp_wait(&ctl.s_full[pb], n_use & 1, abort_flag)) { ok = false; break; }
-      tc::tc_fence_after();
-      if (ci == n_chunks - 1) stage_rows();
+      const int gc = g0 + ci, pb = gc & 1;
       // rows of a warp that lie at or after every column of the chunk need no causal mask; rows beyond the
       // tile's last (their results are never stored) must not force the masked path. Entries that are rows of the loop's
       // stream compare with the row's own index there (both ascend with the position).
@@ -487,118 +501,97 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
         }
         vis = lo;
       }
-      // P goes over the first half of this S buffer: the first 32 logits are in registers before columns 0-15 are
-      // stored, the second 32 (columns 32-63) before columns 16-31 are
+      seen |= vis > 0;
+      if (!warp_wait(&ctl.s_full[pb], (gc >> 1) & 1, abort_flag)) { ok = false; break; }
+      tc::tc_fence_after();
+      if (ci == n_chunks - 1 && pass != 1) stage_rows();
+      // P goes over the first half of the logits it comes from
       const uint32_t sp_addr = s_addr + pb * kNC;
-#pragma unroll 1
-      for (int hf = 0; hf < 2 && ok; ++hf) {
-        uint32_t r[32];
-        tc::tmem_ld32(sp_addr + hf * 32, r);
-        tc::tmem_wait_ld();
-        if (!unmasked) {
-          const int lim = vis - hf * 32;
+      uint32_t r[32], pk[16];
+      tc::tmem_ld32(sp_addr, r);
+      tc::tmem_wait_ld();
+      if (!unmasked) {
+        const int lim = vis - half_sm * (kNC / 2);
 #pragma unroll
-          for (int u = 0; u < 32; ++u) r[u] = u < lim ? r[u] : 0xff800000u;
-        }
-        float sub = lse2;
-        if (MODE == kNewPass) {
-          // running reference: taken from the first columns that show a finite logit and moved (with a rescale of
-          // the accumulator row) only when a maximum beats it by more than the threshold
-          const float cm = max32(r) * c2;                                        // c2 > 0: scaling commutes with the maximum
-          const bool first = ref == -INFINITY && cm > -INFINITY;
-          const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
-          if (first) ref = cm;                             // accumulator row is still zero: nothing to rescale
-          if (__any_sync(0xffffffffu, over)) {
-            float factor = 1.f;
-            if (over) { factor = tc::ex2(ref - cm); ref = cm; }
-            // every earlier PV must have completed before the accumulator rows are rewritten
-            if (ci > 0) {
-              if (!warp_wait(&ctl.p_free[(gc - 1) & 1], ((gc - 1) >> 1) & 1, abort_flag)) { ok = false; break; }
-              tc::tc_fence_after();
-#pragma unroll 1
-              for (int q4 = 0; q4 < 8; ++q4) {
-                uint32_t acc[16];
-                tc::tmem_ld16(tmem + lane_base + kAcc + q4 * 16, acc);
-                tc::tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * factor);
-                tc::tmem_st16(tmem + lane_base + kAcc + q4 * 16, acc);
-              }
-              tc::tmem_wait_st();
-            }
-            ell *= factor;
-            if (hf == 1) {
-              // the first half of this chunk's P was formed against the old reference: bring it along
-              uint32_t ph[16];
-              tc::tmem_wait_st();
-              tc::tmem_ld16(sp_addr, ph);
-              tc::tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&ph[i]);
-                const float2 f = __bfloat1622float2(v);
-                ph[i] = tc::pack_bf16(f.x * factor, f.y * factor);
-              }
-              tc::tmem_st16(sp_addr, ph);
-            }
-          }
-          sub = ref == -INFINITY ? 0.f : ref;
-        }
-        uint32_t pk[16];
-        const float sum = exp32(r, c2, sub, pk);
-        ell += sum;
-        tc::tmem_st16(sp_addr + hf * 16, pk);
+        for (int u = 0; u < 32; ++u) r[u] = u < lim ? r[u] : 0xff800000u;
       }
-      if (!ok) break;
+      if (MODE == kNewPass && pass == 1) top = fmaxf(top, max32(r) * c2);      // c2 > 0: scaling commutes with the maximum
+      exp32(r, c2, sub, pk, sums);
+      tc::tmem_st16(sp_addr, pk);
       tc::tmem_wait_st();
       tc::tc_fence_before();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&ctl.p_full[pb]);
     }
-    // ---- epilogue ------------------------------------------------------------------------------------
-    // The staged rows are combined in place by the row-owning threads and written out coalesced again.
     // a tile without a single chunk: nobody has waited for the Q tile, which is still on its way into this memory
     if (n_chunks == 0) {
       if (ok) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
       if (ok) stage_rows();
     }
-    const float m_i = MODE == kNewPass ? mass : ell;
+    ctl.sum[half_sm][row] = sums.x;
+    ctl.rsum[half_sm][row] = MODE == kNewPass && pass == 1 ? top : sums.y;
     if (ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
     tc::tc_fence_after();
     tc::cp_async_wait<0>();
-    asm volatile("bar.sync 1, 128;" ::: "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(kSmThreads) : "memory");
+    ell = ctl.sum[0][row] + ctl.sum[1][row];
+    bad = MODE == kNewPass && ok && (pass == 1 || (pass == 0 && row_ok && seen && mass > 0.f && !sum_in_range(ell)));
+  }
+  // A row whose sum left the range in which its probabilities are exact (the reference was no estimate of its logits) sends the
+  // tile through two more passes: one finds the largest logits, one takes the probabilities against them.
+  const bool redo = MODE == kNewPass && __syncthreads_or(bad) && !ctl.abort_flag;
+  if (!redo) {
+    if (warp >= kTmaWarp) {
+      if (MODE == kNewPass && a.q_store != nullptr && ok) {
+      // the new Q rows take their place in the Q store for the next loop (this pass reads no Q row from it)
+      const int pt = tid - kTmaWarp * 32;
+#pragma unroll 1
+      for (int it = pt; it < n_rows * 16; it += kTmaWarps * 32) {
+        const int r = it >> 4, c16 = it & 15;
+        const int pos_r = __ldg(a.active_idx + s0 + r);
+        *reinterpret_cast<uint4*>(a.q_store + (size_t)pos_r * a.d + h * kDH + c16 * 8) =
+            __ldg(reinterpret_cast<const uint4*>(a.q_new + (size_t)(s0 + r) * a.d + h * kDH + c16 * 8));
+      }
+    }
+    } else if (warp < kSmWarps) {
+    // ---- epilogue ------------------------------------------------------------------------------------
+    // The staged rows are combined in place by the row-owning threads (each half takes half of the head dimension) and
+    // written out coalesced again.
+    const uint32_t acc_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kAcc;
+    const float m_i = MODE == kNewPass ? mass : ell;
+    const float rsum = ctl.rsum[0][row] + ctl.rsum[1][row];
     const bool valid = ok && n_chunks > 0;                 // warp-uniform: the tensor-memory reads below are collective
     bool has;                                              // per row: T_i is not empty
     float w;
     if (MODE == kNewPass) {
-      has = valid && ref > -INFINITY && m_i > 0.f;
-      w = has ? m_i / ell : 0.f;
+      has = valid && seen && ref > -INFINITY && m_i > 0.f;
+      w = has ? m_i / rsum : 0.f;
     } else {
       has = valid && m_i > 0.f;
       w = -1.f;
     }
 #pragma unroll 1
-    for (int c0 = 0; c0 < kDH && valid; c0 += 32) {   // four 16-byte cells of the staged row at a time
-      uint32_t av[32];
-      tc::tmem_ld32(tmem + lane_base + kAcc + c0, av);
-      uint4* cell[4];
-      float pv[4][8];
+    for (int c0 = half_sm * 64; c0 < half_sm * 64 + 64 && valid; c0 += 16) {   // two 16-byte cells of the staged row at a time
+      uint32_t av[16];
+      tc::tmem_ld16(acc_addr + c0, av);
+      uint4* cell[2];
+      float pv[2][8];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < 2; ++q) {
         cell[q] = reinterpret_cast<uint4*>(stage + row * 256 + (((c0 / 8 + q) ^ (row & 7)) << 4));
         unpack8(*cell[q], pv[q]);
       }
       tc::tmem_wait_ld();
       if (has) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < 2; ++q) {
 #pragma unroll
           for (int i = 0; i < 8; ++i) pv[q][i] = pv[q][i] + w * __uint_as_float(av[q * 8 + i]);
           *cell[q] = pack8(pv[q]);
         }
       }
     }
-    if (row_ok) {
+    if (row_ok && half_sm == 0) {
       if (MODE == kNewPass) {
         if (has) a.lse_out[(size_t)h * a.L + pos] = (ref + log2f(ell)) * kLn2 - logf(m_i);
         else if (a.lse_prev != nullptr) a.lse_out[(size_t)h * a.L + pos] = a.lse_prev[(size_t)h * a.L + pos];
@@ -606,24 +599,32 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
         a.mass[(size_t)h * a.L + pos] = has ? m_i : 0.f;
       }
     }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(kSmThreads) : "memory");
 #pragma unroll 4
-    for (int k = 0; k < 16; ++k) {
-      const int rr = k * 8 + (tid >> 4), cc = tid & 15;
+    for (int k = 0; k < 8; ++k) {
+      const int rr = k * 16 + (tid >> 4), cc = tid & 15;
       if (rr < n_rows)
         *reinterpret_cast<uint4*>(a.rows_out + (size_t)ctl.pos[rr] * a.d + col0 + cc * 8) =
             *reinterpret_cast<const uint4*>(stage + rr * 256 + ((cc ^ (rr & 7)) << 4));
     }
+    }
   }
   // every role is done with this tile: accumulator, Q tile and the ring bookkeeping move on together
-  if (s0 + row_step < q_hi) {   // CTA-uniform: another row tile of the block follows
+  if (redo || s0 + row_step < q_hi) {   // CTA-uniform: this row tile again, or another one of the block
     for (int ci = 0; ci < n_chunks; ++ci)
       if (chunk_dirty(chunk_info(ci, n_plain, n_patch))) dirty_par_cta ^= 1u << ((g + ci) & 1);
     g += n_chunks;
+    tc::fence_proxy_async_smem();     // the staged rows, before the next Q tile comes into their place
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     if (ctl.abort_flag) break;
+  }
+  if (redo) {
+    ++pass;
+  } else {
+    pass = 0;
+    s0 += row_step;
   }
   }  // tiles of the block
   }  // block has active rows

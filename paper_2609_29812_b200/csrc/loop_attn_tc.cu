@@ -4,14 +4,19 @@
 //
 // Warp roles (16 warps, 512 threads):
 //   warps 0-3   softmax of the OLD term  (fixed normaliser lse_prev: p_old = exp(s_old - lse_prev), mass m_i)
-//   warps 4-7   softmax of the NEW term  (running reference, lazy rescale of the accumulator)
-//   warps 8-9   MMA issuers, one thread per term: S = Q Khat^T of chunk n, then acc += P Vhat of chunk n - 1. A single
-//               thread issues a 128x64x16 MMA every ~60-90 cycles while the tensor pipe retires one in 48; two threads
-//               on two schedulers keep up with a chunk period that the exponentials set
-//   warps 10-15 TMA + patch: the Q tiles (two 2-D tile loads each), row gathers (cp.async.bulk.tensor
-//               tile::gather4, 4 selected columns per copy) of bf16 K/V rows straight into 128B-swizzled
-//               operand tiles, and for columns that carry residual payloads which nobody has materialized the
-//               overwrite of the gathered base rows with the dequantize-and-add result (Eq. 8)
+//   warps 4-7   softmax of the NEW term  (against an estimate of the row's largest logit, see start_ref)
+//   warps 8-11  MMA issuers, two warps per term: S = Q Khat^T, and acc += P Vhat. The warps wait as a whole and one elected thread
+//               issues from uniform operands. One thread per term for both kinds, inside `if (lane == 0)`, took 3 k cycles a
+//               chunk whatever the gathers and the exponentials did (~90 cycles an MMA, ~300 a wait)
+//   warps 12-15 TMA + patch: the Q tiles, row gathers (cp.async.bulk.tensor tile::gather4, 4 selected columns per copy) of bf16
+//               K/V rows straight into 128B-swizzled operand tiles, and for columns that carry residual payloads which nobody has
+//               materialized the overwrite of the gathered base rows with the dequantize-and-add result (Eq. 8), shared with the
+//               QK^T issuers
+// A chunk now takes 2.2 k cycles, of which a softmax step (64 logits a thread) is 1.85 k: 1.0 k of the exponential unit for the two
+// warps of a scheduler, both terms in step. 157 -> 136 us a launch (32768 rows, c = 1024), 131072 rows, c = 2048: 873 -> 732 us.
+// Measured and dropped: sixteen softmax warps with half of a chunk's columns each (a step of 1.5 k cycles, but 80 registers: what
+// spilled went through an L1 of 28 KB, and with it the gathers arrived three times as late: 295 us; with registers moved between
+// warpgroups 155); logits in four pieces, each asked for ahead (142 us).
 //
 // Prologue (whole CTA): the block's causal column list is copied to shared memory together with a bit mask
 // of the residual streams that carry each column, and stably partitioned into columns WITHOUT a payload in
@@ -45,8 +50,8 @@
 // and the cached mass m_i is the one of loop w (Eq. 6: it does not change while the set does not). A recomputing
 // launch can leave B (storage type, by position) and m_i (binary32, [H, L]) in buffers of the caller; an ECON launch
 // reads them and computes the new term only. Its two pipelines then are two STREAMS of the new term (even and odd
-// chunks of the column list, an accumulator, a running reference and a row sum each), merged in the epilogue like the
-// two halves of a split problem; the previous loop's Q rows, O rows and log-normalisers are not read.
+// chunks of the column list, an accumulator and row sums each, taken against one reference), added up in the epilogue; the
+// previous loop's Q and O rows are not read, its log-normalisers are a hint.
 #include "tc_attn_common.cuh"
 
 namespace {
@@ -56,15 +61,18 @@ using namespace fl_tc;
 constexpr int kSlots = 4;
 constexpr int kSlotBytes = 2 * kTileBytes;  // K tile | V tile
 constexpr int kSoftmaxWarps = 8;
-constexpr int kIssueWarp = 8;      // warps 8, 9: the MMA issuers of the old and of the new term (QK^T and PV each)
-constexpr int kIssueWarps = 2;
-constexpr int kTmaWarp = 10;       // first of the TMA / patch warps
-constexpr int kTmaWarps = 6;       // a warp's four-row gathers are taken one lane after the other (~100 cycles each):
-                                   // the 64 gathers of a ring slot need as many warps as can be had
+constexpr int kSoftmaxThreads = kSoftmaxWarps * 32;
+constexpr int kTermThreads = kSoftmaxThreads / 2;
+constexpr int kIssueWarp = 8;      // warps 8-11: QK^T and PV issuers of the old term, then of the new term
+constexpr int kIssueWarps = 4;
+constexpr int kTmaWarp = 12;       // first of the TMA / patch warps
+constexpr int kTmaWarps = 4;       // sixteen rows of a K or V tile each
+constexpr int kPatch = 2;          // columns that a warp rebuilds at a time
 constexpr int kWarps = kSoftmaxWarps + kIssueWarps + kTmaWarps;  // 16
-constexpr int kTileGathers = kTileBytes / 512;   // 32 four-row gathers of 128-byte rows fill a K or V tile
 constexpr int kThreads = kWarps * 32;
 constexpr int kColWarps = 14;               // warps that read the column list in the prologue (the other two search rows)
+constexpr int kQWarps = kWarps - kSoftmaxWarps;   // they gather the previous loop's Q rows, sixteen each
+static_assert(kQWarps * 16 == kM, "one tile of Q rows");
 constexpr int kMaxCols = 3072;              // column budget the shared-memory column list can hold
 constexpr int kMaxChunks = kMaxCols / kNC + 3;
 constexpr uint32_t kAccOld = 0, kAccNew = 128, kSOld = 256, kSNew = 384;   // two S buffers of kNC columns each
@@ -127,16 +135,16 @@ struct __align__(16) TcSmemCtl {
   int q_lo, q_hi, i_last;    // block's slot range in active_idx, position of its last active row
   int n_plain, n_patch;      // columns without / with a payload in the current loop,
   int n_stale;               // and those with payloads of earlier loops only that are gathered from the rebuilt rows
+  int split;                 // 2 * pair + half of a problem that is split over two CTAs, else -1
   int merge_role;            // split problems: 0 = this CTA finished first (the other one merges), 1 = it merges,
                              // 2 = it should have merged but gave up waiting for the other's partial result
   int warp_cnt[kWarps][3];
   int chunk_last[kMaxChunks];       // largest column position of the chunk, INT32_MAX if the chunk is padded
   uint32_t chunk_mask[kMaxChunks];  // OR of the stream masks of the chunk's columns (0: plain gather only)
-  int pos[2][kM];            // positions of the tile's rows, one copy per softmax group
-  float mass[kM];            // ECON: row sums of stream 0
-  float ell[kM];
-  float ref[kM];
-  float ref0[kM];            // ECON: running references of stream 0
+  int pos[2][kM];            // positions of the tile's rows, one copy per term
+  float sum[2][kM], rsum[2][kM];   // row sums per term: of the probabilities (old term: the mass), and of what is left of them in bf16
+  float top[2][kM];          // largest logits, second pass of a tile only
+  float ref[2][kM];          // references of the two terms' sums, -inf: no column was seen
 };
 
 constexpr size_t kTcSmemBytes = 1024 /* alignment slack */ + 2 * kQTileBytes + kSlots * kSlotBytes + sizeof(TcSmemCtl) +
@@ -158,7 +166,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   fl_grid_release();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // problem (query block b, head h) of this CTA, and for the pairs at the end of the grid which half of it
-  const int share = blockIdx.x % a.n_share, row_step = a.n_share * kM;   // row tiles share, share + n_share, ...
+  const int share = blockIdx.x % a.n_share;   // row tiles share, share + n_share, ...
   int item = blockIdx.x / a.n_share, part = 0, pair = -1;
   const int n_items = a.nb * a.H;
   if (item >= a.n_full) {
@@ -188,15 +196,15 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     for (int s = 0; s < kSlots; ++s) {
       tc::mbar_init(&ctl.k_landed[s], kTmaWarps);
       tc::mbar_init(&ctl.v_landed[s], kTmaWarps);
-      tc::mbar_init(&ctl.patched[s], kTmaWarps);
+      tc::mbar_init(&ctl.patched[s], kTmaWarps + (ECON ? 1 : 2));
       tc::mbar_init(&ctl.v_done[s], ECON ? 1 : 2);
       tc::mbar_init(&ctl.k_done[s], ECON ? 1 : 2);   // ECON: a slot is read by one stream only
     }
-    tc::mbar_init(&ctl.q_full, (INDEXED && !ECON) ? 1 + kSoftmaxWarps : 1);
+    tc::mbar_init(&ctl.q_full, (INDEXED && !ECON) ? 1 + kQWarps : 1);
     for (int t = 0; t < 2; ++t) {
       for (int pb = 0; pb < 2; ++pb) {
         tc::mbar_init(&ctl.s_full[t][pb], 1);
-        tc::mbar_init(&ctl.p_full[t][pb], 4);
+        tc::mbar_init(&ctl.p_full[t][pb], kSoftmaxWarps / 2);
         tc::mbar_init(&ctl.p_free[t][pb], 1);
       }
     }
@@ -211,7 +219,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   int32_t* raw_slot = reinterpret_cast<int32_t*>(raw_mask + kMaxCols);     // [kMaxCols]: row in the loop's own stream
   const int c_cap = min(a.c, kMaxCols);
   if (warp >= kColWarps) {
-    // warps 14 and 15 search the block's rows in the ascending active list meanwhile
+    // the last two warps search the block's rows in the ascending active list meanwhile
     const int target = warp == kColWarps ? b * a.q_block : min(a.L, (b + 1) * a.q_block);
     int below;
     const int r = lower_bound_warp(a.active_idx, a.n_active, target, lane, &below);
@@ -268,8 +276,32 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   tc::tc_fence_after();
   const uint32_t tmem = ctl.tmem_base;
   volatile int* abort_flag = &ctl.abort_flag;
-  const int q_lo = ctl.q_lo + share * kM, q_hi = ctl.q_hi;
+  const int q_lo = ctl.q_lo + share * kM;
+  int q_hi = ctl.q_hi;
+  // Q tiles of a row tile, by the warps that are not softmax warps: two 64-element slabs each; rows past the compact list read
+  // as zero, rows of the next block are computed and dropped. In the indexed form the previous loop's Q rows come from the
+  // store, four-row gathers by position.
+  auto load_q = [&](int s) {
+    if (warp == kTmaWarp && lane == 0) {
+      tc::mbar_arrive_expect_tx(&ctl.q_full, (ECON || INDEXED) ? kQTileBytes : 2 * kQTileBytes);
+      tc::tma_tile2d(q_new_tile, &a.q_new_map, &ctl.q_full, h * kDH, s);
+      tc::tma_tile2d(q_new_tile + kM * 128, &a.q_new_map, &ctl.q_full, h * kDH + 64, s);
+      if (!INDEXED && !ECON) {
+        tc::tma_tile2d(q_old_tile, &a.q_old_map, &ctl.q_full, h * kDH, s);
+        tc::tma_tile2d(q_old_tile + kM * 128, &a.q_old_map, &ctl.q_full, h * kDH + 64, s);
+      }
+    }
+    __syncwarp();
+    if (INDEXED && !ECON) {
+      const int qw = warp - kSoftmaxWarps, r = s + qw * 16 + lane;
+      const int y = lane < 16 && r < min(q_hi, s + kM) ? __ldg(a.active_idx + r) : a.L;   // row L is outside the tensor: reads as zero
+      gather_rows<4>(q_old_tile + qw * 2048, kM * 128, &a.q_old_map, &ctl.q_full, h * kDH, y);
+    }
+  };
+  // those of the first tile are asked for while the column list is partitioned, but not by a CTA that may find nothing to do
+  const bool q_early = pair < 0 || part == 0;
   if (q_hi > q_lo) {   // CTA-uniform: without active rows the CTA only releases the tensor memory
+  if (q_early && warp >= kSoftmaxWarps) load_q(q_lo);
   {
     // causal prefix, stable partition into plain / patched columns: every warp owns a contiguous span
     const int i_last = ctl.i_last;                                   // last active row of the block
@@ -328,17 +360,25 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     }
     __syncthreads();
   }
-  const int n_plain = ctl.n_plain, n_patch = ctl.n_patch, n_stale = ctl.n_stale;
-  const int n_chunks = (n_plain + kNC - 1) / kNC + (n_patch + kNC - 1) / kNC + (n_stale + kNC - 1) / kNC;
+  // What a tile's loops need of the problem stays in shared memory: registers are what the roles are short of
+  auto chunk = [&](int ci) { return chunk_info(ci, ctl.n_plain, ctl.n_patch, ctl.n_stale); };
+  const int n_chunks = (ctl.n_plain + kNC - 1) / kNC + (ctl.n_patch + kNC - 1) / kNC + (ctl.n_stale + kNC - 1) / kNC;
   // A pair splits its problem's chunks in the middle, unless the block has several row tiles or a single chunk: then
   // the first CTA of the pair does everything and the second nothing (both see the same numbers).
-  const bool split = pair >= 0 && q_hi - q_lo <= kM && n_chunks >= 2;
-  const int c_mid = (n_chunks + 1) >> 1;
-  const int c_lo = (split && part == 1) ? c_mid : 0;
-  const int c_hi = (pair >= 0 && part == 1 && !split) ? 0 : ((split && part == 0) ? c_mid : n_chunks);
+  int c_lo = 0, c_hi = n_chunks;
+  {
+    const bool split = pair >= 0 && q_hi - q_lo <= kM && n_chunks >= 2;
+    if (split) {
+      if (part == 0) c_hi = (n_chunks + 1) >> 1;
+      else c_lo = (n_chunks + 1) >> 1;
+    } else if (pair >= 0 && part == 1) {
+      q_hi = q_lo;
+    }
+    if (tid == 0) ctl.split = split ? 2 * pair + part : -1;
+  }
   // per chunk: the OR of its columns' stream masks and its last column (a warp per chunk, two columns per lane)
   for (int ci = warp; ci < n_chunks; ci += kWarps) {
-    const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
+    const ChunkInfo ck = chunk(ci);
     uint32_t m = 0;
     if (!(ck.patch && a.use_rows)) {   // chunks gathered from the materialized rows are never rewritten
       if (lane < ck.n_valid) m |= ord_mask[ck.off + lane];
@@ -356,582 +396,82 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   int fill = 0; // ring slots filled so far: slot = fill % kSlots, phase = (fill / kSlots) & 1
   uint32_t dirty_par_cta = 0;  // per-slot phase parity of the patched[] barriers (they only see dirty chunks)
 
-  for (int s0 = q_lo, tile = 0; s0 < q_hi && !(pair >= 0 && part == 1 && !split); s0 += row_step, ++tile) {
-  const int n_rows = min(kM, q_hi - s0);
-  const int g0 = g, g0_1 = g1, fill0 = fill;
-  const uint32_t dirty_par0 = dirty_par_cta;
-  if (warp == kTmaWarp) {
-    // Q tiles of this row tile: two 64-element slabs each; rows past the compact list read as zero, rows of the
-    // next block (past n_rows) are computed and dropped
-    if (lane == 0) {
-      tc::mbar_arrive_expect_tx(&ctl.q_full, (ECON || INDEXED) ? kQTileBytes : 2 * kQTileBytes);
-      tc::tma_tile2d(q_new_tile, &a.q_new_map, &ctl.q_full, h * kDH, s0);
-      tc::tma_tile2d(q_new_tile + kM * 128, &a.q_new_map, &ctl.q_full, h * kDH + 64, s0);
-      if (!INDEXED && !ECON) {
-        tc::tma_tile2d(q_old_tile, &a.q_old_map, &ctl.q_full, h * kDH, s0);
-        tc::tma_tile2d(q_old_tile + kM * 128, &a.q_old_map, &ctl.q_full, h * kDH + 64, s0);
-      }
-    }
-  }
-  if (INDEXED && !ECON && warp < kSoftmaxWarps) {
-    // the previous loop's Q rows come from the store: four-row gathers by position, eight of the 64 per softmax warp,
-    // which has nothing else to do yet (from one warp they took 9 k of a problem's 66 k cycles at 1024 columns: a warp's
-    // requests are taken one after the other, ~130 cycles each, and its share of the first K and V tiles came after them)
-    if (lane == 0) tc::mbar_arrive_expect_tx(&ctl.q_full, 8 * 512);
-    __syncwarp();
-    if (lane < 8) {
-      const int grp4 = warp * 4 + (lane & 3), slab = lane >> 2;
-      int y[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = grp4 * 4 + i;
-        y[i] = r < n_rows ? __ldg(a.active_idx + s0 + r) : a.L;   // row L is outside the tensor: reads as zero
-      }
-      tc::tma_gather4(q_old_tile + slab * (kM * 128) + grp4 * 512, &a.q_old_map, &ctl.q_full, h * kDH + slab * 64, y[0],
-                      y[1], y[2], y[3]);
-    }
-    __syncwarp();
-  }
+  // the row tile that is being worked on (or done again: see redo) and where the rings and buffers stand at its start
+  int s0 = q_lo, tile = 0, pass = 0, n_rows = 0, g0 = 0, g0_1 = 0, fill0 = 0;
+  uint32_t dirty_par0 = 0;
+  bool redo = false;
+  auto stage_of = [&](int grp) {      // [128 rows][8 x 16 B], 16-byte chunks XOR-swizzled by row
+    return ECON ? q_old_tile + grp * (kM * 128) : (grp ? q_new_tile : q_old_tile);
+  };
+  const __nv_bfloat16* prev_rows = ECON ? a.bg_in : a.o_prev;
+  int pos = -1;
+  float lse2 = 0.f;
+  bool ok = true, bad = false;
 
-  if (warp >= kTmaWarp) {
-    // ========================================== TMA + patch ==========================================
-    // In-order fills of the ring, the K tiles one chunk ahead of the V tiles; the lookahead is whatever the four slots
-    // allow. A step's four-row gathers (the K tiles of the next chunk, then the V tiles of this one, 32 per tile: 2 slabs x
-    // 16 groups) are dealt round robin to the six warps, one per lane; every warp announces its own share of the bytes on
-    // the tile's barrier. K and V in steps of their own, with half the lanes busy, cost launches of 2048 columns at 128K 14%;
-    // slots held as a whole until the chunk's PV cost launches of two-slot chunks 17%. Chunks whose columns carry residual
-    // payloads are then rewritten in place by the same warps (6 columns at a time, lanes 0-15 the K row, lanes 16-31 the V
-    // row).
-    const int tw = warp - kTmaWarp;
-    const int req = lane * kTmaWarps + tw;
-    const int my_tile = req / kTileGathers, slab = (req >> 4) & 1, grp = req & 15;
-    auto share = [&](int t) {     // this warp's requests of the step's tile t
-      return (kTileGathers * (t + 1) - tw + kTmaWarps - 1) / kTmaWarps - (kTileGathers * t - tw + kTmaWarps - 1) / kTmaWarps;
-    };
-    const int half = lane >> 4, ch = lane & 15;
+  // Columns of a chunk that carry residual payloads which nobody has materialized: their rows are rewritten in the chunk's tiles
+  // (one or two ring slots from position f on), a share by each of the TMA warps and of the QK^T issuers that wait for it
+  // (lanes 0-15 the K rows, lanes 16-31 the V rows)
+  constexpr int kPatchWarps = kTmaWarps + (ECON ? 1 : 2);
+  auto rebuild = [&](const ChunkInfo& ck, int f, int who) -> bool {
+    const int n_slots = (ck.patch && !ECON) ? 2 : 1;
+    for (int k = 0; k < n_slots; ++k)
+      if (!warp_wait(&ctl.k_landed[(f + k) % kSlots], ((f + k) / kSlots) & 1, abort_flag) ||
+          !warp_wait(&ctl.v_landed[(f + k) % kSlots], ((f + k) / kSlots) & 1, abort_flag))
+        return false;
+    const int l = opaque(lane), half = l >> 4, ch = l & 15;
     const DevSide& side = half ? a.v : a.k;
     const int elem = h * kDH + ch * 8;
     const __nv_bfloat16* base_rows = static_cast<const __nv_bfloat16*>(side.base) + elem;
     const uint32_t ch_off = (ch >> 3) * (kNC * 128);
-    auto slots_of = [&](const ChunkInfo& ck) { return (ck.patch && !ECON) ? 2 : 1; };  // ECON: only the new tiles are needed
-    // one step: the K tiles of chunk ck (k_slots of them, 0: none) at ring position fk, the V tiles of chunk cv at fv
-    auto fill_tiles = [&](const ChunkInfo& ck, int fk, int k_slots, const ChunkInfo& cv, int fv, int v_slots) -> bool {
-      for (int k = 0; k < k_slots; ++k)
-        if (fk + k >= kSlots && !warp_wait(&ctl.k_done[(fk + k) % kSlots], ((fk + k) / kSlots - 1) & 1, abort_flag)) return false;
-      for (int k = 0; k < v_slots; ++k)
-        if (fv + k >= kSlots && !warp_wait(&ctl.v_done[(fv + k) % kSlots], ((fv + k) / kSlots - 1) & 1, abort_flag)) return false;
-      if (lane < k_slots + v_slots) {
-        const bool v = lane >= k_slots;
-        const int slot = (v ? fv + lane - k_slots : fk + lane) % kSlots;
-        tc::mbar_arrive_expect_tx(v ? &ctl.v_landed[slot] : &ctl.k_landed[slot], share(lane) * 512);
-      }
-      __syncwarp();
-      if (my_tile < k_slots + v_slots) {
-        const bool is_v = my_tile >= k_slots;
-        const ChunkInfo& c = is_v ? cv : ck;
-        const int second = is_v ? my_tile - k_slots : my_tile;
-        // columns that are active in this loop come from the materialized rows (old tile: before the loop's
-        // residual, new tile: after it), indexed by their row in the loop's stream; stale ones from the rebuilt rows, all
-        // others from the base
-        const bool from_rows = c.patch && a.use_rows;
-        int y[4];
+    uint8_t* t_old = ring + (f % kSlots) * kSlotBytes + half * kTileBytes + ch_off;
+    uint8_t* t_new = ring + ((f + 1) % kSlots) * kSlotBytes + half * kTileBytes + ch_off;
+#pragma unroll 1
+    for (int u = who; u < ck.n_valid; u += kPatch * kPatchWarps) {
+      uint32_t mask[kPatch];
+      int j[kPatch];
+      uint4 base16[kPatch], v_old[kPatch], v_new[kPatch];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int u = grp * 4 + i;
-          // a row past the end of the tensor reads as zero
-          if (from_rows) y[i] = u < c.n_valid ? (int)ord_mask[c.off + u] : a.n_active;
-          else y[i] = u < c.n_valid ? ord_col[c.off + u] : a.L;
-        }
-        const void* src;
-        if (c.stale) src = is_v ? static_cast<const void*>(&a.v_stale_map) : static_cast<const void*>(&a.k_stale_map);
-        else if (!from_rows) src = is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map);
-        else if (second == 0 && !ECON) src = is_v ? static_cast<const void*>(&a.v_prev_map) : static_cast<const void*>(&a.k_prev_map);
-        else src = is_v ? static_cast<const void*>(&a.v_cur_map) : static_cast<const void*>(&a.k_cur_map);
-        const int slot = ((is_v ? fv : fk) + second) % kSlots;
-        tc::tma_gather4(ring + slot * kSlotBytes + (is_v ? kTileBytes : 0) + slab * (kNC * 128) + grp * 512, src,
-                        is_v ? &ctl.v_landed[slot] : &ctl.k_landed[slot], h * kDH + slab * 64, y[0], y[1], y[2], y[3]);
+      for (int n = 0; n < kPatch; ++n) {
+        const int un = u + n * kPatchWarps;
+        mask[n] = un < ck.n_valid ? ord_mask[ck.off + un] : 0u;
+        j[n] = un < ck.n_valid ? ord_col[ck.off + un] : 0;
+        base16[n] = mask[n] ? __ldg(reinterpret_cast<const uint4*>(base_rows + (size_t)j[n] * a.d)) : make_uint4(0u, 0u, 0u, 0u);
       }
-      __syncwarp();
-      return true;
-    };
-    int f = fill0;
-    bool ok = true;
-    ChunkInfo ck = chunk_info(c_lo, n_plain, n_patch, n_stale);
-    if (c_lo < c_hi) ok = fill_tiles(ck, f, slots_of(ck), ck, f, 0);
-#pragma unroll 1
-    for (int ci = c_lo; ci < c_hi && ok; ++ci) {
-      const int n_slots = slots_of(ck);
-      const bool dirty = ctl.chunk_mask[ci] != 0;
-      const ChunkInfo nx = chunk_info(ci + 1, n_plain, n_patch, n_stale);
-      ok = fill_tiles(nx, f + n_slots, ci + 1 < c_hi ? slots_of(nx) : 0, ck, f, n_slots);
-      if (!ok) break;
-      if (dirty) {
-        for (int k = 0; k < n_slots && ok; ++k)
-          ok = warp_wait(&ctl.k_landed[(f + k) % kSlots], ((f + k) / kSlots) & 1, abort_flag) &&
-               warp_wait(&ctl.v_landed[(f + k) % kSlots], ((f + k) / kSlots) & 1, abort_flag);
-        if (!ok) break;
-        uint8_t* t_old = ring + (f % kSlots) * kSlotBytes + half * kTileBytes + ch_off;
-        uint8_t* t_new = ring + ((f + 1) % kSlots) * kSlotBytes + half * kTileBytes + ch_off;
-#pragma unroll 1
-        for (int u = tw; u < ck.n_valid; u += kTmaWarps) {
-          const uint32_t mask = ord_mask[ck.off + u];
-          if (mask == 0) continue;
-          const int j = ord_col[ck.off + u];
-          const uint4 base16 = __ldg(reinterpret_cast<const uint4*>(base_rows + (size_t)j * a.d));
-          uint4 v_old, v_new;
-          patch_piece<BITS>(side, a.n_old, mask, j, elem, a.d, a.group, base16, v_old, v_new);
-          const uint32_t off = tc::sw128_offset(u, ch & 7);
-          if (ECON) {
-            *reinterpret_cast<uint4*>(t_old + off) = v_new;     // the chunk's only slot holds Xhat^(r)
-          } else {
-            if (mask & ((1u << a.n_old) - 1u)) *reinterpret_cast<uint4*>(t_old + off) = v_old;
-            if (ck.patch) *reinterpret_cast<uint4*>(t_new + off) = v_new;
-          }
-        }
-        tc::fence_proxy_async_smem();
-        __syncwarp();
-        if (lane == 0)
-          for (int k = 0; k < n_slots; ++k) tc::mbar_arrive(&ctl.patched[(f + k) % kSlots]);
-      }
-      f += n_slots;
-      ck = nx;
-    }
-    if (INDEXED && a.q_store != nullptr && ok && !split) {
-      // The Q store rows of this (row tile, head) were read by the gathers that completed q_full and belong to
-      // no other CTA: the new rows take their place for the next loop.
-      ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
-      const int pt = tid - kTmaWarp * 32;
-#pragma unroll 1
-      for (int it = pt; ok && it < n_rows * 16; it += kTmaWarps * 32) {
-        const int r = it >> 4, ch = it & 15;
-        const int pos_r = __ldg(a.active_idx + s0 + r);
-        *reinterpret_cast<uint4*>(a.q_store + (size_t)pos_r * a.d + h * kDH + ch * 8) =
-            __ldg(reinterpret_cast<const uint4*>(a.q_new + (size_t)(s0 + r) * a.d + h * kDH + ch * 8));
-      }
-    }
-  } else if (warp >= kIssueWarp) {
-    // ========================================== MMA issuers ==========================================
-    // One thread per term issues both kinds of MMA, in the order their operands become ready: QK^T of chunk n (its S
-    // buffer is free once PV of chunk n - 2 has retired), then PV of chunk n - 1 (its P is written while QK^T of
-    // chunk n executes).
-    const int t = warp - kIssueWarp;      // 0: old term, 1: new term (ECON: streams 0 and 1 of the new term)
-    if (lane == 0) {
-      const uint32_t idesc_qk = tc::make_idesc_bf16(kM, kNC, false);
-      const uint32_t idesc_pv = tc::make_idesc_bf16(kM, kDH, true);
-      // Descriptors differ only in their start-address field (bits 0-13, units of 16 bytes): the low word
-      // moves (no carry into the other fields: shared memory is < 256 KB), the high word stays.
-      // K-major operands (Q, Khat): 32 bytes per 16-element K step inside a 64-element slab, then the next slab.
-      const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32((t || ECON) ? q_new_tile : q_old_tile), 16, 1024);
-      const uint64_t k_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), 16, 1024);
-      const uint32_t kq_hi = (uint32_t)(k_desc0 >> 32);
-      const uint32_t q_lo_w = (uint32_t)q_desc, k_lo0 = (uint32_t)k_desc0;
-      // MN-major Vhat: 16 key rows = two 1024-byte row groups per K step
-      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(ring) + kTileBytes, kNC * 128, 1024);
-      const uint32_t v_hi = (uint32_t)(v_desc0 >> 32), v_lo0 = (uint32_t)v_desc0;
-      const uint32_t s_base = tmem + (t ? kSNew : kSOld);
-      const uint32_t acc = tmem + (t ? kAccNew : kAccOld);
-      int f = fill0;             // ring position of the chunk whose QK^T is issued next
-      int pv_slot = 0;           // slots of the chunk whose PV is issued next (the previous QK^T's)
-      int pv_slot1 = -1, pv_fill = 0;
-      uint32_t dirty_par = dirty_par0;
-      // the chunks this thread issues: all of them, or (ECON) every other one starting at the stream's number
-      constexpr int kStep = ECON ? 2 : 1;
-      const int first = c_lo + (ECON ? t : 0);
-      const int n_mine = first < c_hi ? (c_hi - first + kStep - 1) / kStep : 0;
-      const int gbase = (ECON && t) ? g0_1 : g0;
-#pragma unroll 1
-      for (int n = 0; n <= n_mine; ++n) {
-        const int ci = first + n * kStep;
-        const int gc = gbase + n;
-        int qk_slot = 0, qk_slot1 = -1, qk_fill = 0;
-        if (n < n_mine) {
-          const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
-          if (ECON) f = fill0 + (ci - c_lo);    // one slot per chunk, filled in chunk order
-          const bool two = ck.patch && !ECON;
-          const int slot0 = f % kSlots, slot1 = (f + 1) % kSlots;
-          if (n == 0 && !tc::mbar_wait(&ctl.q_full, tile & 1, abort_flag)) break;
-          // a term reads one slot of the chunk only (the new term of a two-slot chunk the second): it starts on it
-          // without waiting for the other
-          const int my_slot = (t && two) ? slot1 : slot0, my_fill = (t && two) ? f + 1 : f;
-          if (!tc::mbar_wait(&ctl.k_landed[my_slot], (my_fill / kSlots) & 1, abort_flag)) break;
-          if (ctl.chunk_mask[ci] != 0) {       // residual-carrying columns are rewritten by the patch warps
-            // (ECON: the ring has an even number of slots and the streams alternate, so within a row tile a slot
-            // always serves the same stream, which therefore sees every phase of the slot's barrier)
-            if (!tc::mbar_wait(&ctl.patched[my_slot], (dirty_par >> my_slot) & 1, abort_flag)) break;
-            dirty_par ^= 1u << slot0;
-            if (two) dirty_par ^= 1u << slot1;
-          }
-          // the S buffer holds P of the chunk before the previous one until its PV MMAs have read it
-          if (gc >= 2 && !tc::mbar_wait(&ctl.p_free[t][gc & 1], ((gc >> 1) - 1) & 1, abort_flag)) break;
-          const uint32_t s_dst = s_base + (gc & 1) * kNC;
-          tc::tc_fence_after();
-          const uint32_t k_lo = k_lo0 + my_slot * (kSlotBytes >> 4);
-#define FL_QK(KK, ACC)                                                                                       \
-  tc::mma_ss_lo<ACC>(s_dst, q_lo_w + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), kq_hi,               \
-                     k_lo + ((((KK) >> 2) * (kNC * 128) + ((KK)&3) * 32) >> 4), kq_hi, idesc_qk)
-          FL_QK(0, false); FL_QK(1, true); FL_QK(2, true); FL_QK(3, true);
-          FL_QK(4, true);  FL_QK(5, true); FL_QK(6, true); FL_QK(7, true);
-#undef FL_QK
-          tc::mma_commit(&ctl.s_full[t][gc & 1]);
-          tc::mma_commit(&ctl.k_done[slot0]);
-          if (two) tc::mma_commit(&ctl.k_done[slot1]);
-          qk_fill = my_fill;
-          qk_slot = slot0;
-          qk_slot1 = two ? slot1 : -1;
-          f += two ? 2 : 1;
-        }
-        if (n > 0) {
-          const int gp = gc - 1, pb = gp & 1;
-          if (!tc::mbar_wait(&ctl.v_landed[pv_fill % kSlots], (pv_fill / kSlots) & 1, abort_flag)) break;
-          if (!tc::mbar_wait(&ctl.p_full[t][pb], (gp >> 1) & 1, abort_flag)) break;
-          tc::tc_fence_after();
-          const uint32_t v_lo = v_lo0 + (pv_fill % kSlots) * (kSlotBytes >> 4);
-          const uint32_t p_src = s_base + pb * kNC;
-          const uint32_t acc0 = n > 1 ? 1u : 0u;           // the thread's first chunk of the tile overwrites the accumulator
+      patch_pieces<BITS, kPatch>(side, a.n_old, mask, j, elem, a.d, a.group, base16, v_old, v_new);
 #pragma unroll
-          for (int kk = 0; kk < kNC / 16; ++kk)
-            tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc_pv, kk > 0 ? 1u : acc0);
-          tc::mma_commit(&ctl.p_free[t][pb]);
-          tc::mma_commit(&ctl.v_done[pv_slot]);
-          if (pv_slot1 >= 0) tc::mma_commit(&ctl.v_done[pv_slot1]);
-        }
-        pv_slot = qk_slot;
-        pv_slot1 = qk_slot1;
-        pv_fill = qk_fill;
-      }
-      tc::mma_commit(&ctl.acc_done);
-    }
-    __syncwarp();
-  } else {
-    // ============================================ softmax ============================================
-    const int grp = warp >> 2;                    // 0: old term, 1: new term (ECON: streams 0 and 1 of the new term)
-    const int gt = tid & 127;                     // thread inside the term's group of four warps
-    const int row = (warp & 3) * 32 + lane;
-    const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-    const bool row_ok = row < n_rows;
-    const int pos = row_ok ? __ldg(a.active_idx + s0 + row) : -1;
-    const float c2 = a.scale * kLog2e;
-    const float lse2 = ((row_ok && !ECON) ? a.lse_prev[(size_t)h * a.L + pos] : 0.f) * kLog2e;
-    // the epilogue reads the row's previous output (ECON: its background): have it in L2 by then (each group asks
-    // for its 128-byte half)
-    const __nv_bfloat16* prev_rows = ECON ? a.bg_in : a.o_prev;
-    if (row_ok)
-      tc::prefetch_l2(prev_rows + (INDEXED ? (size_t)pos : (size_t)(s0 + row)) * a.d + h * kDH + grp * 64);
-    ctl.pos[grp][row] = pos;
-    asm volatile("bar.sync %0, 128;" ::"r"(2 + grp) : "memory");
-    const int* row_pos = ctl.pos[grp];
-    // Each group finishes 64 of the 128 head-dim columns. Its half of the O_prev tile (ECON: of the background rows) is
-    // staged in shared memory with coalesced asynchronous copies, which run under the group's last chunk: the staging area
-    // is the first half of the group's own Q tile (the QK^T MMAs of the group's term have all retired once its last S
-    // arrived); the second half takes the background rows a recomputing launch leaves for later loops. In ECON both streams
-    // read the new Q tile until the very end and the old one is never loaded: the groups stage in its two halves.
-    uint8_t* stage = ECON ? q_old_tile + grp * (kM * 128)    // [128 rows][8 x 16 B], 16-byte chunks XOR-swizzled by row
-                          : (grp ? q_new_tile : q_old_tile);
-    const size_t o_col0 = (size_t)h * kDH + grp * 64;
-    bool staged = false;
-    auto stage_rows = [&]() {
-      staged = true;
-#pragma unroll 4
-      for (int k = 0; k < 8; ++k) {
-        const int rr = k * 16 + (gt >> 3), cc = gt & 7;
-        if (rr < n_rows) {
-          const size_t src_row = INDEXED ? (size_t)row_pos[rr] : (size_t)(s0 + rr);
-          tc::cp_async16(stage + rr * 128 + ((cc ^ (rr & 7)) << 4), prev_rows + src_row * a.d + o_col0 + cc * 8);
-        }
-      }
-      tc::cp_async_commit();
-    };
-    const uint32_t s_addr = tmem + lane_base + (grp ? kSNew : kSOld);
-    float mass = 0.f, ell = 0.f, ref = -INFINITY;
-    bool ok = true;
-    constexpr int kStep = ECON ? 2 : 1;           // ECON: a group's stream takes every other chunk
-    const int gbase = (ECON && grp) ? g0_1 : g0;
-    for (int ci = c_lo + (ECON ? grp : 0), n = 0; ci < c_hi; ci += kStep, ++n) {
-      const int gc = gbase + n, pb = gc & 1, n_use = gc >> 1;
-      if (!warp_wait(&ctl.s_full[grp][pb], n_use & 1, abort_flag)) { ok = false; break; }
-      tc::tc_fence_after();
-      if (ci + kStep >= c_hi) stage_rows();
-      // rows of a warp that lie at or after every column of the chunk need no causal mask; rows beyond the
-      // tile's last (their results are never stored) must not force the masked path
-      const bool unmasked = __all_sync(0xffffffffu, !row_ok || ctl.chunk_last[ci] <= pos);
-      int vis = kNC;
-      if (!unmasked) {
-        // the chunk's columns ascend: the visible ones are a prefix, found by bisection; the rest read as -inf
-        const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
-        const int32_t* cp = ord_col + ck.off;
-        int lo = 0, hi = row_ok ? ck.n_valid : 0;
-        while (lo < hi) {
-          const int mid = (lo + hi) >> 1;
-          if (cp[mid] <= pos) lo = mid + 1; else hi = mid;
-        }
-        vis = lo;
-      }
-      // P goes over the first half of this S buffer (the QK^T issuer waited for the PV MMAs of chunk gc - 2 before it
-      // overwrote the buffer): the first 32 logits are in registers before columns 0-15 are stored, the second 32
-      // (columns 32-63) before columns 16-31 are
-      const uint32_t sp_addr = s_addr + pb * kNC;
-      // The 64 logits of the row are taken in two halves of 32 (each its own little softmax step): 64 live logits
-      // plus the pipeline's state do not fit 128 registers, and what spills lands in an L1 of ~30 KB.
-#pragma unroll 1
-      for (int hf = 0; hf < 2 && ok; ++hf) {
-        uint32_t r[32];
-        tc::tmem_ld32(sp_addr + hf * 32, r);
-        tc::tmem_wait_ld();
-        if (!unmasked) {
-          const int lim = vis - hf * 32;
-#pragma unroll
-          for (int u = 0; u < 32; ++u) r[u] = u < lim ? r[u] : 0xff800000u;
-        }
-        float sub = lse2;
-        if (ECON || grp == 1) {
-          // running reference of the new term: taken from the first columns that show a finite logit and moved
-          // (with a rescale of the accumulator row) only when a maximum beats it by more than the threshold
-          const float cm = max32(r) * c2;                                        // c2 > 0: scaling commutes with the maximum
-          const bool first = ref == -INFINITY && cm > -INFINITY;
-          const bool over = ref > -INFINITY && cm - ref > kRescaleThreshold;
-          if (first) ref = cm;                             // accumulator row is still zero: nothing to rescale
-          if (__any_sync(0xffffffffu, over)) {
-            float factor = 1.f;
-            if (over) { factor = tc::ex2(ref - cm); ref = cm; }
-            // every earlier PV must have completed before the accumulator rows are rewritten (n >= 1 here: the
-            // reference was set in an earlier chunk, or in this chunk's first half, whose P is not announced yet)
-            if (n > 0) {
-              if (!warp_wait(&ctl.p_free[grp][(gc - 1) & 1], ((gc - 1) >> 1) & 1, abort_flag)) { ok = false; break; }
-              tc::tc_fence_after();
-              const uint32_t acc_col = grp ? kAccNew : kAccOld;    // the group's own accumulator
-#pragma unroll 1
-              for (int q4 = 0; q4 < 8; ++q4) {
-                uint32_t acc[16];
-                tc::tmem_ld16(tmem + lane_base + acc_col + q4 * 16, acc);
-                tc::tmem_wait_ld();
-#pragma unroll
-                for (int i = 0; i < 16; ++i) acc[i] = __float_as_uint(__uint_as_float(acc[i]) * factor);
-                tc::tmem_st16(tmem + lane_base + acc_col + q4 * 16, acc);
-              }
-              tc::tmem_wait_st();
-            }
-            ell *= factor;
-            if (hf == 1) {
-              // the first half of this chunk's P was formed against the old reference: bring it along
-              uint32_t ph[16];
-              tc::tmem_wait_st();
-              tc::tmem_ld16(sp_addr, ph);
-              tc::tmem_wait_ld();
-#pragma unroll
-              for (int i = 0; i < 16; ++i) {
-                const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&ph[i]);
-                const float2 f = __bfloat1622float2(v);
-                ph[i] = tc::pack_bf16(f.x * factor, f.y * factor);
-              }
-              tc::tmem_st16(sp_addr, ph);
-            }
-          }
-          sub = ref == -INFINITY ? 0.f : ref;
-        }
-        uint32_t pk[16];
-        const float sum = exp32(r, c2, sub, pk);
-        if (!ECON && grp == 0) mass += sum; else ell += sum;
-        tc::tmem_st16(sp_addr + hf * 16, pk);
-      }
-      if (!ok) break;
-      // P is announced at once: its PV MMAs free both the ring slot (for the gathers) and this S buffer (for the
-      // QK^T of the chunk after the next), and both are on the critical path
-      tc::tmem_wait_st();
-      tc::tc_fence_before();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(&ctl.p_full[grp][pb]);
-    }
-    // ---- epilogue ------------------------------------------------------------------------------------
-    // The staged rows are combined in place by the row-owning threads and written out coalesced again.
-    uint8_t* stage_bg = stage + kM * 128;                    // recomputing launch with bg_out only
-    const bool write_bg = !ECON && INDEXED && a.bg_out != nullptr;   // CTA-uniform
-    // a tile without a single chunk (empty column set): no issuer has waited for the Q tiles, which are still on
-    // their way into the very memory the rows are staged in
-    if (ok && c_hi == c_lo) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
-    if (ok && !staged) stage_rows();
-    if (ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
-    tc::tc_fence_after();
-    if (ECON) {
-      if (grp == 0) { ctl.mass[row] = ell; ctl.ref0[row] = ref; }
-      else { ctl.ell[row] = ell; ctl.ref[row] = ref; }
-    } else {
-      if (grp == 0) ctl.mass[row] = mass;
-      else { ctl.ell[row] = ell; ctl.ref[row] = ref; }
-    }
-    tc::cp_async_wait<0>();
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    // per-row statistics. Accumulator A (tensor-memory columns 0-127) is the old term's, B (128-255) the new term's;
-    // in ECON they are streams 0 and 1 of the new term, each with its own row sum and reference.
-    float m_i = ECON ? (row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f) : ctl.mass[row];
-    float l_a = ECON ? ctl.mass[row] : 0.f, ref_a = ECON ? ctl.ref0[row] : -INFINITY;
-    float l_i = ctl.ell[row], ref_i = ctl.ref[row];
-    // warp-uniform: the tensor-memory reads below are collective
-    const bool valid_a = ok && c_hi > c_lo;
-    const bool valid_b = ok && (ECON ? c_hi > c_lo + 1 : c_hi > c_lo);
-    // ---- split problems: the CTA of the pair that finishes first leaves its partial result in the workspace, the
-    // other one adds it to its own (nobody waits for anybody: whoever finds the counter at 1 merges)
-    const float* other = nullptr;
-    float f_a = 0.f, f_b = 1.f, f_oa = 0.f, f_ob = 0.f;   // factors of accumulators A and B, own and other CTA's
-    if (split) {
-      // counter of the pair: each CTA adds 1 when its accumulation is complete (the one that finds 0 is first), the
-      // first one adds 16 once its partial result is in the workspace; the second resets it for the next launch
-      if (tid == 0) ctl.merge_role = atomicAdd(a.part_cnt + pair, 1) & 1;
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (ctl.merge_role == 0) {
-        float* mine = a.part_acc + ((size_t)pair * 2 + part) * kPartFloats;
-#pragma unroll 1
-        for (int c16 = 0; c16 < 8; ++c16) {   // accumulator A columns 0-63 of the group's half, then B: 16 at a time
-          uint32_t v[16];
-          const int col = (c16 >> 2) * kDH + grp * 64 + (c16 & 3) * 16;   // column of the [A | B] accumulator pair
-          const bool valid = (c16 >> 2) ? valid_b : valid_a;
-          if (valid) {
-            tc::tmem_ld16(tmem + lane_base + kAccOld + col, v);           // kAccNew == kAccOld + kDH
-            tc::tmem_wait_ld();
-          }
-#pragma unroll
-          for (int i = 0; i < 16; ++i) mine[(col + i) * kM + row] = valid ? __uint_as_float(v[i]) : 0.f;
-        }
-        if (grp == 0) {
-          mine[2 * kM * kDH + row] = ECON ? (valid_a ? l_a : 0.f) : (valid_a ? m_i : 0.f);
-          mine[2 * kM * kDH + 3 * kM + row] = (ECON && valid_a) ? ref_a : -INFINITY;
+      for (int n = 0; n < kPatch; ++n) {
+        if (mask[n] == 0) continue;
+        const uint32_t off = tc::sw128_offset(u + n * kPatchWarps, ch & 7);
+        if (ECON) {
+          *reinterpret_cast<uint4*>(t_old + off) = v_new[n];     // the chunk's only slot holds Xhat^(r)
         } else {
-          mine[2 * kM * kDH + kM + row] = valid_b ? l_i : 0.f;
-          mine[2 * kM * kDH + 2 * kM + row] = valid_b ? ref_i : -INFINITY;
+          if (mask[n] & ((1u << a.n_old) - 1u)) *reinterpret_cast<uint4*>(t_old + off) = v_old[n];
+          if (ck.patch) *reinterpret_cast<uint4*>(t_new + off) = v_new[n];
         }
-        __threadfence();
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (tid == 0) atomicAdd(a.part_cnt + pair, 16);
-      } else {
-        // the other CTA came first and is writing its partial result (it is resident and past its main loop: the
-        // wait is short, and bounded like every other)
-        if (tid == 0) {
-          int seen = atomicAdd(a.part_cnt + pair, 0);
-          for (int it = 0; seen < 16 && it < (1 << 16); ++it) {
-            __nanosleep(100);
-            seen = atomicAdd(a.part_cnt + pair, 0);
-          }
-          if (seen < 16) { *abort_flag = 1; ctl.merge_role = 2; }   // gave up: no output, FL_ERR_TIMEOUT
-          a.part_cnt[pair] = 0;                                     // ready for the next launch either way
-        }
-        asm volatile("bar.sync 1, 256;" ::: "memory");
-        if (ctl.merge_role == 1) {   // CTA-uniform
-          __threadfence();
-          const float* theirs = a.part_acc + ((size_t)pair * 2 + (part ^ 1)) * kPartFloats;
-          // the other CTA's accumulators (128 KB) come into the idle ring in one round of asynchronous copies
-          static_assert(2 * kM * kDH * sizeof(float) <= (size_t)kSlots * kSlotBytes, "a partial result fits in the ring");
+      }
+    }
+    tc::fence_proxy_async_smem();
+    __syncwarp();
+    if (lane == 0)
+      for (int k = 0; k < n_slots; ++k) tc::mbar_arrive(&ctl.patched[(f + k) % kSlots]);
+    return true;
+  };
+
+  // every role walks the tiles in step: main_part works on one, finish writes it out
+  auto run_tiles = [&](auto&& main_part, auto&& finish) {
 #pragma unroll 1
-          for (int i = tid; i < 2 * kM * kDH / 4; i += 256) tc::cp_async16(ring + i * 16, theirs + i * 4);
-          tc::cp_async_commit();
-          other = reinterpret_cast<const float*>(ring);
-          const float s0_o = __ldcg(theirs + 2 * kM * kDH + row), l_o = __ldcg(theirs + 2 * kM * kDH + kM + row);
-          const float ref_o = __ldcg(theirs + 2 * kM * kDH + 2 * kM + row);
-          const float ref_oa = __ldcg(theirs + 2 * kM * kDH + 3 * kM + row);
-          // products and sums rounded one by one (no fused multiply-add), the two CTAs' contributions joined by one
-          // commutative addition: the result must not depend on which of the two does the merging
-          if (ECON) {
-            const float ref_t = fmaxf(fmaxf(ref_a, ref_i), fmaxf(ref_oa, ref_o));
-            f_a = ref_a > -INFINITY ? tc::ex2(ref_a - ref_t) : 0.f;
-            f_b = ref_i > -INFINITY ? tc::ex2(ref_i - ref_t) : 0.f;
-            f_oa = ref_oa > -INFINITY ? tc::ex2(ref_oa - ref_t) : 0.f;
-            f_ob = ref_o > -INFINITY ? tc::ex2(ref_o - ref_t) : 0.f;
-            l_i = __fadd_rn(__fadd_rn(__fmul_rn(l_a, f_a), __fmul_rn(l_i, f_b)),
-                            __fadd_rn(__fmul_rn(s0_o, f_oa), __fmul_rn(l_o, f_ob)));
-            ref_i = ref_t;
-          } else {
-            const float ref_t = fmaxf(ref_i, ref_o);
-            f_b = ref_i > -INFINITY ? tc::ex2(ref_i - ref_t) : 0.f;
-            f_ob = ref_o > -INFINITY ? tc::ex2(ref_o - ref_t) : 0.f;
-            m_i = __fadd_rn(m_i, s0_o);
-            l_i = __fadd_rn(__fmul_rn(l_i, f_b), __fmul_rn(l_o, f_ob));
-            ref_i = ref_t;
-          }
-          tc::cp_async_wait<0>();
-          asm volatile("bar.sync 1, 256;" ::: "memory");
-        }
-      }
-    }
-    if (ECON && other == nullptr) {   // the CTA's own two streams on a common reference
-      const float ref_t = fmaxf(ref_a, ref_i);
-      f_a = ref_a > -INFINITY ? tc::ex2(ref_a - ref_t) : 0.f;
-      f_b = ref_i > -INFINITY ? tc::ex2(ref_i - ref_t) : 0.f;
-      l_i = __fadd_rn(__fmul_rn(l_a, f_a), __fmul_rn(l_i, f_b));
-      ref_i = ref_t;
-    }
-    const bool writer = !split || other != nullptr;       // CTA-uniform: this CTA produces the output rows
-    const bool has = valid_a && ref_i > -INFINITY && (!ECON || m_i > 0.f);   // per row: T_i is not empty
-    const float w = has ? m_i / l_i : 0.f;
-#pragma unroll 1
-    for (int c0 = 0; c0 < 64 && writer; c0 += 16) {   // 16 head-dim columns = two 16-byte cells of the staged row at a time
-      uint32_t ao[16], an[16];
-      const int col = grp * 64 + c0;
-      if (valid_a) tc::tmem_ld16(tmem + lane_base + kAccOld + col, ao);
-      if (valid_b) tc::tmem_ld16(tmem + lane_base + kAccNew + col, an);
-      tc::tmem_wait_ld();
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        if (!valid_a) ao[i] = 0u;
-        if (!valid_b) an[i] = 0u;
-      }
-      if (ECON) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          float v = __fadd_rn(__fmul_rn(__uint_as_float(ao[i]), f_a), __fmul_rn(__uint_as_float(an[i]), f_b));
-          if (other != nullptr)
-            v = __fadd_rn(v, __fadd_rn(__fmul_rn(other[(col + i) * kM + row], f_oa),
-                                       __fmul_rn(other[(kDH + col + i) * kM + row], f_ob)));
-          an[i] = __float_as_uint(v);
-        }
-      } else if (other != nullptr) {
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-          ao[i] = __float_as_uint(__fadd_rn(__uint_as_float(ao[i]), other[(col + i) * kM + row]));
-          an[i] = __float_as_uint(__fadd_rn(__fmul_rn(__uint_as_float(an[i]), f_b),
-                                            __fmul_rn(other[(kDH + col + i) * kM + row], f_ob)));
-        }
-      }
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const int off = row * 128 + (((c0 / 8 + q) ^ (row & 7)) << 4);
-        uint4* cell = reinterpret_cast<uint4*>(stage + off);
-        uint4* cell_bg = reinterpret_cast<uint4*>(stage_bg + off);
-        if (has) {
-          float pv[8];
-          unpack8(*cell, pv);
-          if (!ECON) {
-            // background of the row: what stays of its previous output once the old term is taken out
-#pragma unroll
-            for (int i = 0; i < 8; ++i) pv[i] = pv[i] - __uint_as_float(ao[q * 8 + i]);
-            if (write_bg) *cell_bg = pack8(pv);
-          }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) pv[i] = pv[i] + w * __uint_as_float(an[q * 8 + i]);
-          *cell = pack8(pv);
-        } else if (write_bg) {
-          *cell_bg = *cell;                                   // empty T_i: the row itself is its background
-        }
-      }
-    }
-    if (grp == 1 && row_ok && writer) {
-      if (has) a.lse_out[(size_t)h * a.L + pos] = (ref_i + log2f(l_i)) * kLn2 - logf(m_i);
-      else if (!ECON) a.lse_out[(size_t)h * a.L + pos] = lse2 * kLn2;
-      else if (a.lse_prev != nullptr) a.lse_out[(size_t)h * a.L + pos] = a.lse_prev[(size_t)h * a.L + pos];
-    }
-    if (write_bg && grp == 0 && row_ok && writer) a.mass[(size_t)h * a.L + pos] = has ? m_i : 0.f;
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (writer) {
-#pragma unroll 4
-      for (int k = 0; k < 8; ++k) {
-        const int rr = k * 16 + (gt >> 3), cc = gt & 7;
-        if (rr < n_rows) {
-          const size_t dst = (INDEXED ? (size_t)row_pos[rr] : (size_t)(s0 + rr)) * a.d + o_col0 + cc * 8;
-          const int off = rr * 128 + ((cc ^ (rr & 7)) << 4);
-          *reinterpret_cast<uint4*>(a.o_out + dst) = *reinterpret_cast<const uint4*>(stage + off);
-          if (write_bg) *reinterpret_cast<uint4*>(a.bg_out + dst) = *reinterpret_cast<const uint4*>(stage_bg + off);
-        }
-      }
-    }
-  }
-  if (INDEXED && split && a.q_store != nullptr) {   // CTA-uniform
+  for (; s0 < q_hi; ++tile) {
+  n_rows = min(kM, q_hi - s0);
+  g0 = g; g0_1 = g1; fill0 = fill;
+  dirty_par0 = dirty_par_cta;
+  ok = true; bad = false;
+  main_part();
+  // A row whose sum left the range in which its probabilities are exact (the reference was no estimate of its logits) sends the
+  // tile through two more passes: one finds the largest logits, one takes the probabilities against them. Nothing has been
+  // written by then; the Q tiles come again, because the rows were staged in their place
+  redo = __syncthreads_or(bad) && !ctl.abort_flag;
+  if (!redo) finish();
+  if (INDEXED && !redo && a.q_store != nullptr && ctl.split >= 0) {   // CTA-uniform
     // Both halves of a split problem gathered the previous loop's Q rows from the store; the new rows may take their
     // place only when both are done with them, which the merging CTA knows
     __syncthreads();
@@ -946,24 +486,502 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     }
   }
   // every role is done with this tile: accumulators, Q tiles and the ring bookkeeping move on together
-  if (s0 + row_step < q_hi) {   // CTA-uniform: another row tile of the block follows
+  if (redo || s0 + (a.n_share * kM) < q_hi) {   // CTA-uniform: this row tile again, or another one of the block
     if (ECON) { g += (c_hi - c_lo + 1) >> 1; g1 += (c_hi - c_lo) >> 1; }
     else g += c_hi - c_lo;
     int f = fill;
     for (int ci = c_lo; ci < c_hi; ++ci) {   // replay the tile's fills (same for every role)
-      const ChunkInfo ck = chunk_info(ci, n_plain, n_patch, n_stale);
+      const ChunkInfo ck = chunk(ci);
       const int n_slots = (ck.patch && !ECON) ? 2 : 1;
       if (ctl.chunk_mask[ci] != 0)
         for (int k = 0; k < n_slots; ++k) dirty_par_cta ^= 1u << ((f + k) % kSlots);
       f += n_slots;
     }
     fill = f;
+    tc::fence_proxy_async_smem();     // the staged rows, before the next Q tiles come into their place
     tc::tc_fence_before();
     __syncthreads();
     tc::tc_fence_after();
     if (ctl.abort_flag) break;
   }
-  }  // tiles of the block
+  if (redo) {
+    ++pass;
+  } else {
+    pass = 0;
+    s0 += (a.n_share * kM);
+  }
+  }
+  };
+
+  if (warp < kSoftmaxWarps) {
+  run_tiles([&]() {
+    // ============================================ softmax ============================================
+    // (from a copy of the thread's number that the compiler takes for another one: what is made of it stays out of the
+    // registers of the other parts)
+    const int t = opaque(tid);
+    const int grp = (t >> 7) & 1;                 // 0: old term, 1: new term (ECON: streams 0 and 1 of the new term)
+    const int row = t & (kM - 1);
+    const uint32_t lane_base = (uint32_t)(row & ~31) << 16;
+    const bool row_ok = row < n_rows;
+    pos = row_ok ? __ldg(a.active_idx + s0 + row) : -1;
+    const float c2 = a.scale * kLog2e;
+    if (row_ok && (!ECON || a.lse_prev != nullptr)) lse2 = a.lse_prev[(size_t)h * a.L + pos] * kLog2e;
+    // what the row's probabilities are taken against: the old term's are normalised by the previous loop's log-normaliser; for
+    // the new term's any number near the row's largest logit does. The log-normaliser is an upper estimate of it, 2^20 is taken
+    // off because the columns of the set need not hold the row's mass; with the mass at hand (ECON) it is taken off instead
+    float ref = lse2;
+    if (ECON) {
+      const float m_row = row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f;
+      ref = start_ref(a.lse_prev != nullptr ? lse2 + log2f(m_row) : 0.f);
+    } else if (grp == 1) {
+      ref = start_ref(lse2 - 20.f);
+    }
+    if ((ECON || grp == 1) && pass == 2) {
+      ref = ctl.top[1][row];      // -inf: no column is seen with a finite logit
+      if (ECON) ref = fmaxf(ref, ctl.top[0][row]);
+    }
+    // the epilogue reads the row's previous output (ECON: its background): have it in L2 by then (each term asks
+    // for its 128-byte half)
+    if (row_ok)
+      tc::prefetch_l2(prev_rows + (INDEXED ? (size_t)pos : (size_t)(s0 + row)) * a.d + h * kDH + grp * 64);
+    ctl.pos[grp][row] = pos;
+    asm volatile("bar.sync %0, %1;" ::"r"(2 + grp), "n"(kTermThreads) : "memory");
+    // Each term's threads finish 64 of the 128 head-dim columns. Their half of the O_prev tile (ECON: of the background rows) is
+    // staged in shared memory with coalesced asynchronous copies, which run under the term's last chunk: the staging area
+    // is the first half of the term's own Q tile (the QK^T MMAs of the term have all retired once its last S
+    // arrived); the second half takes the background rows a recomputing launch leaves for later loops. In ECON both streams
+    // read the new Q tile until the very end and the old one is never loaded: the groups stage in its two halves.
+    auto stage_rows = [&]() {
+      const int gt = opaque(tid) & (kTermThreads - 1);
+      uint8_t* stage = stage_of(grp);
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const int rr = k * 16 + (gt >> 3), cc = gt & 7;
+        if (rr < n_rows) {
+          const size_t src_row = INDEXED ? (size_t)ctl.pos[grp][rr] : (size_t)(s0 + rr);
+          tc::cp_async16(stage + rr * 128 + ((cc ^ (rr & 7)) << 4), prev_rows + src_row * a.d + h * kDH + grp * 64 + cc * 8);
+        }
+      }
+      tc::cp_async_commit();
+    };
+    bool staged = false;
+    const uint32_t s_addr = tmem + lane_base + (grp ? kSNew : kSOld);
+    const float sub = ref > -INFINITY ? ref : 0.f;
+    float2 sums = make_float2(0.f, 0.f);
+    float top = -INFINITY;
+    bool seen = false;
+    constexpr int kStep = ECON ? 2 : 1;           // ECON: a group's stream takes every other chunk
+    const int gbase = (ECON && grp) ? g0_1 : g0;
+    for (int ci = c_lo + (ECON ? grp : 0), n = 0; ci < c_hi; ci += kStep, ++n) {
+      const int gc = gbase + n, pb = gc & 1;
+      // rows of a warp that lie at or after every column of the chunk need no causal mask; rows beyond the
+      // tile's last (their results are never stored) must not force the masked path
+      const bool unmasked = __all_sync(0xffffffffu, !row_ok || ctl.chunk_last[ci] <= pos);
+      int vis = kNC;
+      if (!unmasked) {
+        // the chunk's columns ascend: the visible ones are a prefix, found by bisection; the rest read as -inf
+        const ChunkInfo ck = chunk(ci);
+        const int32_t* cp = ord_col + ck.off;
+        int lo = 0, hi = row_ok ? ck.n_valid : 0;
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (cp[mid] <= pos) lo = mid + 1; else hi = mid;
+        }
+        vis = lo;
+      }
+      seen |= vis > 0;
+      if (!warp_wait(&ctl.s_full[grp][pb], (gc >> 1) & 1, abort_flag)) { ok = false; break; }
+      tc::tc_fence_after();
+      if (ci + kStep >= c_hi && pass != 1) { staged = true; stage_rows(); }
+      // P goes over the first half of the S buffer (the QK^T issuer waited for the PV MMAs of chunk gc - 2 before it
+      // overwrote the buffer): the first 32 logits are in registers before columns 0-15 are stored, the second 32
+      // (columns 32-63) before columns 16-31 are
+      const uint32_t sp_addr = s_addr + pb * kNC;
+#pragma unroll
+      for (int hf = 0; hf < 2; ++hf) {     // (64 logits at once spill)
+        uint32_t r[32], pk[16];
+        tc::tmem_ld32(sp_addr + hf * 32, r);
+        tc::tmem_wait_ld();
+        if (!unmasked) {
+          const int lim = vis - hf * 32;
+#pragma unroll
+          for (int u = 0; u < 32; ++u) r[u] = u < lim ? r[u] : 0xff800000u;
+        }
+        if (pass == 1) top = fmaxf(top, max32(r) * c2);      // c2 > 0: scaling commutes with the maximum
+        exp32(r, c2, sub, pk, sums);
+        tc::tmem_st16(sp_addr + hf * 16, pk);
+      }
+      // P is announced at once: its PV MMAs free both the ring slot (for the gathers) and this S buffer (for the
+      // QK^T of the chunk after the next), and both are on the critical path
+      tc::tmem_wait_st();
+      tc::tc_fence_before();
+      __syncwarp();
+      if (lane == 0) tc::mbar_arrive(&ctl.p_full[grp][pb]);
+    }
+    // a tile without a single chunk (empty column set): no issuer has waited for the Q tiles, which are still on
+    // their way into the very memory the rows are staged in
+    if (ok && c_hi == c_lo) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
+    if (ok && !staged && pass != 1) stage_rows();
+    ctl.sum[grp][row] = sums.x;
+    ctl.rsum[grp][row] = sums.y;
+    if (pass == 1) ctl.top[grp][row] = top;
+    ctl.ref[grp][row] = seen ? ref : -INFINITY;
+    if (ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
+    tc::tc_fence_after();
+    tc::cp_async_wait<0>();
+    asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
+    const float total = ctl.sum[1][row] + (ECON ? ctl.sum[0][row] : 0.f);
+    const bool any = ctl.ref[1][row] > -INFINITY || (ECON && ctl.ref[0][row] > -INFINITY);
+    bad = ok && (pass == 1 || (pass == 0 && row_ok && any && !sum_in_range(total)));
+  }, [&]() {
+    // ---- epilogue ------------------------------------------------------------------------------------
+    // (from a copy of the thread's number that the compiler takes for another one: what is made of it stays out of the
+    // registers of the other parts)
+    const int t = opaque(tid);
+    const int grp = (t >> 7) & 1;                 // 0: old term, 1: new term (ECON: streams 0 and 1 of the new term)
+    const int row = t & (kM - 1);
+    const uint32_t lane_base = (uint32_t)(row & ~31) << 16;
+    const bool row_ok = row < n_rows;
+    // The staged rows are combined in place by the row-owning threads and written out coalesced again.
+    const int col_lo = grp * 64;                             // the term's half of the head dimension
+    uint8_t* stage = stage_of(grp);
+    uint8_t* stage_bg = stage + kM * 128;                    // recomputing launch with bg_out only
+    const bool write_bg = !ECON && INDEXED && a.bg_out != nullptr;   // CTA-uniform
+    // per-row statistics. Accumulator A (tensor-memory columns 0-127) is the old term's, B (128-255) the new term's;
+    // in ECON they are streams 0 and 1 of the new term, whose sums are taken against one reference.
+    const float sum_a = ctl.sum[0][row];
+    float m_i = ECON ? (row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f) : sum_a;
+    float l_i = ctl.sum[1][row], ref_i = ctl.ref[1][row];
+    // factor of the new term's accumulators that makes the weights of the rounded probabilities add up to what the unrounded do
+    float r_b = ctl.rsum[1][row];
+    if (ECON) {
+      l_i = __fadd_rn(sum_a, l_i);
+      r_b = __fadd_rn(ctl.rsum[0][row], r_b);
+      ref_i = fmaxf(ctl.ref[0][row], ref_i);
+    }
+    r_b = r_b > 0.f ? l_i / r_b : 1.f;
+    // warp-uniform: the tensor-memory reads below are collective
+    bool valid_a = ok && c_hi > c_lo;
+    bool valid_b = ok && (ECON ? c_hi > c_lo + 1 : c_hi > c_lo);
+    // ---- split problems: the CTA of the pair that finishes first leaves its partial result in the workspace, the
+    // other one adds it to its own (nobody waits for anybody: whoever finds the counter at 1 merges)
+    bool writer = true;                                   // CTA-uniform: this CTA produces the output rows
+    if (ctl.split >= 0) {
+      // counter of the pair: each CTA adds 1 when its accumulation is complete (the one that finds 0 is first), the
+      // first one adds 16 once its partial result is in the workspace; the second resets it for the next launch
+      if (tid == 0) ctl.merge_role = atomicAdd(a.part_cnt + (ctl.split >> 1), 1) & 1;
+      asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
+      writer = ctl.merge_role != 0;
+      if (!writer) {
+        float* mine = a.part_acc + (size_t)ctl.split * kPartFloats;
+#pragma unroll 1
+        for (int c8 = 0; c8 < 16; ++c8) {     // accumulator A's columns of the term's half, then B's: 8 at a time
+          uint32_t v[8];
+          const int col = (c8 >> 3) * kDH + col_lo + (c8 & 7) * 8;      // column of the [A | B] accumulator pair
+          const bool valid = (c8 >> 3) ? valid_b : valid_a;
+          if (valid) {
+            tc::tmem_ld8(tmem + lane_base + kAccOld + col, v);            // kAccNew == kAccOld + kDH
+            tc::tmem_wait_ld();
+          }
+#pragma unroll
+          for (int i = 0; i < 8; ++i) mine[(col + i) * kM + row] = valid ? __uint_as_float(v[i]) * (ECON || (c8 >> 3) ? r_b : 1.f) : 0.f;
+        }
+        if (grp == 0) {
+          mine[2 * kM * kDH + row] = valid_a ? m_i : 0.f;
+          mine[2 * kM * kDH + kM + row] = valid_a ? l_i : 0.f;
+          mine[2 * kM * kDH + 2 * kM + row] = valid_a ? ref_i : -INFINITY;
+        }
+        __threadfence();
+        asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
+        if (tid == 0) atomicAdd(a.part_cnt + (ctl.split >> 1), 16);
+      } else {
+        // the other CTA came first and is writing its partial result (it is resident and past its main loop: the
+        // wait is short, and bounded like every other)
+        if (tid == 0) {
+          int seen16 = atomicAdd(a.part_cnt + (ctl.split >> 1), 0);
+          for (int it = 0; seen16 < 16 && it < (1 << 16); ++it) {
+            __nanosleep(100);
+            seen16 = atomicAdd(a.part_cnt + (ctl.split >> 1), 0);
+          }
+          if (seen16 < 16) { *abort_flag = 1; ctl.merge_role = 2; }   // gave up: no output, FL_ERR_TIMEOUT
+          a.part_cnt[ctl.split >> 1] = 0;                                       // ready for the next launch either way
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
+        writer = ctl.merge_role == 1;
+        if (writer) {   // CTA-uniform
+          __threadfence();
+          const float* theirs = a.part_acc + (size_t)(ctl.split ^ 1) * kPartFloats;
+          // the other CTA's accumulators (128 KB) come into the idle ring in one round of asynchronous copies
+          static_assert(2 * kM * kDH * sizeof(float) <= (size_t)kSlots * kSlotBytes, "a partial result fits in the ring");
+#pragma unroll 1
+          for (int i = tid; i < 2 * kM * kDH / 4; i += kSoftmaxThreads) tc::cp_async16(ring + i * 16, theirs + i * 4);
+          tc::cp_async_commit();
+          const float l_o = __ldcg(theirs + 2 * kM * kDH + kM + row), ref_o = __ldcg(theirs + 2 * kM * kDH + 2 * kM + row);
+          // products and sums rounded one by one (no fused multiply-add), the two CTAs' contributions joined by one
+          // commutative addition: the result must not depend on which of the two does the merging
+          const float ref_t = fmaxf(ref_i, ref_o);
+          const float f = ref_i > -INFINITY ? tc::ex2(ref_i - ref_t) : 0.f;
+          const float f_o = ref_o > -INFINITY ? tc::ex2(ref_o - ref_t) : 0.f;
+          if (!ECON) m_i = __fadd_rn(m_i, __ldcg(theirs + 2 * kM * kDH + row));
+          l_i = __fadd_rn(__fmul_rn(l_i, f), __fmul_rn(l_o, f_o));
+          ref_i = ref_t;
+          tc::cp_async_wait<0>();
+          asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
+          // into the own accumulators, so that nothing of this is alive where the rows are written
+          const float* other = reinterpret_cast<const float*>(ring) + row;
+#pragma unroll 1
+          for (int c8 = 0; c8 < 16; ++c8) {
+            uint32_t v[8];
+            const int col = (c8 >> 3) * kDH + col_lo + (c8 & 7) * 8;
+            const bool valid = (c8 >> 3) ? valid_b : valid_a;
+            const bool plain = !ECON && (c8 >> 3) == 0;                  // the old term has one normaliser on both sides
+            const float fm = plain ? 1.f : f, fo = plain ? 1.f : f_o, rc = plain ? 1.f : r_b;
+            if (valid) {
+              tc::tmem_ld8(tmem + lane_base + kAccOld + col, v);
+              tc::tmem_wait_ld();
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              v[i] = __float_as_uint(__fadd_rn(__fmul_rn(valid ? __uint_as_float(v[i]) * rc : 0.f, fm), __fmul_rn(other[(col + i) * kM], fo)));
+            tc::tmem_st8(tmem + lane_base + kAccOld + col, v);
+          }
+          tc::tmem_wait_st();
+          valid_a = valid_b = true;
+          r_b = 1.f;
+        }
+      }
+    }
+    const bool has = valid_a && ref_i > -INFINITY && (!ECON || m_i > 0.f);   // per row: T_i is not empty
+    const float w = has ? m_i / l_i * r_b : 0.f;
+#pragma unroll 1
+    for (int c0 = 0; c0 < 64 && writer; c0 += 8) {   // one 16-byte cell of the staged row at a time
+      uint32_t ao[8], an[8];
+      const int col = grp * 64 + c0;
+      if (valid_a) tc::tmem_ld8(tmem + lane_base + kAccOld + col, ao);
+      if (valid_b) tc::tmem_ld8(tmem + lane_base + kAccNew + col, an);
+      tc::tmem_wait_ld();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        if (!valid_a) ao[i] = 0u;
+        if (!valid_b) an[i] = 0u;
+        if (ECON) an[i] = __float_as_uint(__fadd_rn(__uint_as_float(ao[i]), __uint_as_float(an[i])));
+      }
+      const int off = row * 128 + (((c0 / 8) ^ (row & 7)) << 4);
+      uint4* cell = reinterpret_cast<uint4*>(stage + off);
+      uint4* cell_bg = reinterpret_cast<uint4*>(stage_bg + off);
+      if (has) {
+        float pv[8];
+        unpack8(*cell, pv);
+        if (!ECON) {
+          // background of the row: what stays of its previous output once the old term is taken out
+#pragma unroll
+          for (int i = 0; i < 8; ++i) pv[i] = pv[i] - __uint_as_float(ao[i]);
+          if (write_bg) *cell_bg = pack8(pv);
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) pv[i] = pv[i] + w * __uint_as_float(an[i]);
+        *cell = pack8(pv);
+      } else if (write_bg) {
+        *cell_bg = *cell;                                   // empty T_i: the row itself is its background
+      }
+    }
+    if (grp == 1 && row_ok && writer) {
+      if (has) a.lse_out[(size_t)h * a.L + pos] = (ref_i + log2f(l_i)) * kLn2 - logf(m_i);
+      else if (!ECON) a.lse_out[(size_t)h * a.L + pos] = lse2 * kLn2;
+      else if (a.lse_prev != nullptr) a.lse_out[(size_t)h * a.L + pos] = a.lse_prev[(size_t)h * a.L + pos];
+    }
+    if (write_bg && grp == 0 && row_ok && writer) a.mass[(size_t)h * a.L + pos] = has ? m_i : 0.f;
+    asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
+    if (writer) {
+#pragma unroll 4
+      for (int k = 0; k < 8; ++k) {
+        const int rr = k * 16 + ((t & (kTermThreads - 1)) >> 3), cc = t & 7;
+        if (rr < n_rows) {
+          const size_t dst = (INDEXED ? (size_t)ctl.pos[grp][rr] : (size_t)(s0 + rr)) * a.d + h * kDH + grp * 64 + cc * 8;
+          const int off = rr * 128 + ((cc ^ (rr & 7)) << 4);
+          *reinterpret_cast<uint4*>(a.o_out + dst) = *reinterpret_cast<const uint4*>(stage + off);
+          if (write_bg) *reinterpret_cast<uint4*>(a.bg_out + dst) = *reinterpret_cast<const uint4*>(stage_bg + off);
+        }
+      }
+    }
+  });
+  } else {
+  run_tiles([&]() {
+    if (tile > 0 || !q_early) load_q(s0);
+    if (warp >= kTmaWarp) {
+    // ========================================== TMA + patch ==========================================
+    // In-order fills of the ring, the K tiles one chunk ahead of the V tiles; the lookahead is whatever the four slots
+    // allow. A step's four-row gathers (the K tiles of the next chunk, then the V tiles of this one, 32 per tile: 2 slabs x
+    // 16 groups) are dealt round robin to the six warps, one per lane; every warp announces its own share of the bytes on
+    // the tile's barrier. K and V in steps of their own, with half the lanes busy, cost launches of 2048 columns at 128K 14%;
+    // slots held as a whole until the chunk's PV cost launches of two-slot chunks 17%. Chunks whose columns carry residual
+    // payloads are then rewritten in place by the same warps (6 columns at a time, lanes 0-15 the K row, lanes 16-31 the V
+    // row).
+    const int tw = warp - kTmaWarp;
+    auto slots_of = [&](const ChunkInfo& ck) { return (ck.patch && !ECON) ? 2 : 1; };  // ECON: only the new tiles are needed
+    // one step: the K tiles of chunk ck (k_slots of them, 0: none) at ring position fk, the V tiles of chunk cv at fv
+    auto fill_tiles = [&](const ChunkInfo& ck, int fk, int k_slots, const ChunkInfo& cv, int fv, int v_slots) -> bool {
+      for (int k = 0; k < k_slots; ++k)
+        if (fk + k >= kSlots && !warp_wait(&ctl.k_done[(fk + k) % kSlots], ((fk + k) / kSlots - 1) & 1, abort_flag)) return false;
+      for (int k = 0; k < v_slots; ++k)
+        if (fv + k >= kSlots && !warp_wait(&ctl.v_done[(fv + k) % kSlots], ((fv + k) / kSlots - 1) & 1, abort_flag)) return false;
+      const int u = tw * 16 + (lane & 15);
+#pragma unroll 1
+      for (int t = 0; t < k_slots + v_slots; ++t) {
+        const bool is_v = t >= k_slots;
+        const ChunkInfo& c = is_v ? cv : ck;
+        const int second = is_v ? t - k_slots : t;
+        // columns that are active in this loop come from the materialized rows (old tile: before the loop's
+        // residual, new tile: after it), indexed by their row in the loop's stream; stale ones from the rebuilt rows, all
+        // others from the base; a row past the end of the tensor reads as zero
+        const bool from_rows = c.patch && a.use_rows;
+        const int y = u >= c.n_valid ? (from_rows ? a.n_active : a.L) : (from_rows ? (int)ord_mask[c.off + u] : ord_col[c.off + u]);
+        const void* src;
+        if (c.stale) src = is_v ? static_cast<const void*>(&a.v_stale_map) : static_cast<const void*>(&a.k_stale_map);
+        else if (!from_rows) src = is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map);
+        else if (second == 0 && !ECON) src = is_v ? static_cast<const void*>(&a.v_prev_map) : static_cast<const void*>(&a.k_prev_map);
+        else src = is_v ? static_cast<const void*>(&a.v_cur_map) : static_cast<const void*>(&a.k_cur_map);
+        const int slot = ((is_v ? fv : fk) + second) % kSlots;
+        gather_rows<4>(ring + slot * kSlotBytes + (is_v ? kTileBytes : 0) + tw * 2048, kNC * 128, src,
+                       is_v ? &ctl.v_landed[slot] : &ctl.k_landed[slot], h * kDH, y);
+      }
+      return true;
+    };
+    int f = fill0;
+    ChunkInfo ck = chunk(c_lo);
+    if (c_lo < c_hi) ok = fill_tiles(ck, f, slots_of(ck), ck, f, 0);
+#pragma unroll 1
+    for (int ci = c_lo; ci < c_hi && ok; ++ci) {
+      const int n_slots = slots_of(ck);
+      const bool dirty = ctl.chunk_mask[ci] != 0;
+      const ChunkInfo nx = chunk(ci + 1);
+      ok = fill_tiles(nx, f + n_slots, ci + 1 < c_hi ? slots_of(nx) : 0, ck, f, n_slots);
+      if (!ok) break;
+      if (dirty) ok = rebuild(ck, f, tw);
+      f += n_slots;
+      ck = nx;
+    }
+    } else {
+    // ========================================== MMA issuers ==========================================
+    // Two warps per term: one issues S = Q Khat^T of chunk after chunk (its S buffer is free once PV of the chunk before the
+    // previous one has retired), the other acc += P Vhat (V has arrived, P is written). The whole warp walks the chunks and
+    // waits, one elected thread issues: with the loop inside `if (lane == 0)` every operand went through per-lane code, ~90
+    // cycles an MMA and ~300 a wait, and one thread for both kinds was what a chunk waited for (3 k cycles).
+    const int t = __shfl_sync(0xffffffffu, (warp - kIssueWarp) >> 1, 0);      // 0: old term, 1: new term (ECON: streams 0 and 1 of the new term)
+    const bool is_pv = __shfl_sync(0xffffffffu, (warp - kIssueWarp) & 1, 0) != 0;
+    const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint32_t s_base = tmem_u + (t ? kSNew : kSOld);
+    // the chunks of this term: all of them, or (ECON) every other one starting at the stream's number
+    constexpr int kStep = ECON ? 2 : 1;
+    const int first = c_lo + (ECON ? t : 0);
+    const int n_mine = first < c_hi ? (c_hi - first + kStep - 1) / kStep : 0;
+    const int gbase = (ECON && t) ? g0_1 : g0;
+    // Descriptors differ only in their start-address field (bits 0-13, units of 16 bytes): the low word
+    // moves (no carry into the other fields: shared memory is < 256 KB), the high word stays.
+    int f = fill0;               // ring position of the chunk
+    uint32_t dirty_par = dirty_par0;
+    if (!is_pv) {
+      const uint32_t idesc = tc::make_idesc_bf16(kM, kNC, false);
+      // K-major operands (Q, Khat): 32 bytes per 16-element K step inside a 64-element slab, then the next slab.
+      const uint64_t q_desc = tc::make_desc_sw128(tc::smem_u32((t || ECON) ? q_new_tile : q_old_tile), 16, 1024);
+      const uint64_t k_desc0 = tc::make_desc_sw128(tc::smem_u32(ring), 16, 1024);
+      const uint32_t kq_hi = (uint32_t)(k_desc0 >> 32);
+      const uint32_t q_lo_w = (uint32_t)q_desc, k_lo0 = (uint32_t)k_desc0;
+      if (n_mine > 0 && !warp_wait(&ctl.q_full, tile & 1, abort_flag)) ok = false;
+#pragma unroll 1
+      for (int n = 0; n < n_mine && ok; ++n) {
+        const int ci = first + n * kStep, gc = gbase + n;
+        if (ECON) f = fill0 + (ci - c_lo);    // one slot per chunk, filled in chunk order
+        const bool two = chunk(ci).patch && !ECON;
+        const int slot0 = f % kSlots, slot1 = (f + 1) % kSlots;
+        // a term reads one slot of the chunk only (the new term of a two-slot chunk the second): it starts on it
+        // without waiting for the other
+        const int my_slot = (t && two) ? slot1 : slot0, my_fill = (t && two) ? f + 1 : f;
+        const bool dirty = ctl.chunk_mask[ci] != 0;
+        // the S buffer holds P of the chunk before the previous one until its PV MMAs have read it
+        if (gc >= 2 && !warp_wait(&ctl.p_free[t][gc & 1], ((gc >> 1) - 1) & 1, abort_flag)) break;
+        if (!warp_wait(&ctl.k_landed[my_slot], (my_fill / kSlots) & 1, abort_flag)) break;
+        if (dirty) {       // residual-carrying columns are rewritten by the patch warps, of which this is one
+          if (!rebuild(chunk(ci), f, kTmaWarps + (ECON ? 0 : t))) break;
+          // (ECON: the ring has an even number of slots and the streams alternate, so within a row tile a slot
+          // always serves the same stream, which therefore sees every phase of the slot's barrier)
+          if (!warp_wait(&ctl.patched[my_slot], (dirty_par >> my_slot) & 1, abort_flag)) break;
+          dirty_par ^= 1u << slot0;
+          if (two) dirty_par ^= 1u << slot1;
+        }
+        tc::tc_fence_after();
+        if (tc::elect_one()) {
+          const uint32_t s_dst = s_base + (gc & 1) * kNC;
+          const uint32_t k_lo = k_lo0 + my_slot * (kSlotBytes >> 4);
+#define FL_QK(KK, ACC)                                                                                       \
+  tc::mma_ss_lo<ACC>(s_dst, q_lo_w + ((((KK) >> 2) * (kM * 128) + ((KK)&3) * 32) >> 4), kq_hi,               \
+                     k_lo + ((((KK) >> 2) * (kNC * 128) + ((KK)&3) * 32) >> 4), kq_hi, idesc)
+          FL_QK(0, false); FL_QK(1, true); FL_QK(2, true); FL_QK(3, true);
+          FL_QK(4, true);  FL_QK(5, true); FL_QK(6, true); FL_QK(7, true);
+#undef FL_QK
+          tc::mma_commit(&ctl.s_full[t][gc & 1]);
+          tc::mma_commit(&ctl.k_done[slot0]);
+          if (two) tc::mma_commit(&ctl.k_done[slot1]);
+        }
+        __syncwarp();
+        f += two ? 2 : 1;
+      }
+    } else {
+      const uint32_t idesc = tc::make_idesc_bf16(kM, kDH, true);
+      // MN-major Vhat: 16 key rows = two 1024-byte row groups per K step
+      const uint64_t v_desc0 = tc::make_desc_sw128(tc::smem_u32(ring) + kTileBytes, kNC * 128, 1024);
+      const uint32_t v_hi = (uint32_t)(v_desc0 >> 32), v_lo0 = (uint32_t)v_desc0;
+      const uint32_t acc = tmem_u + (t ? kAccNew : kAccOld);
+      uint32_t accum = 0;          // the first chunk of the tile overwrites the accumulator
+#pragma unroll 1
+      for (int n = 0; n < n_mine; ++n) {
+        const int ci = first + n * kStep, gc = gbase + n, pb = gc & 1;
+        if (ECON) f = fill0 + (ci - c_lo);
+        const bool two = chunk(ci).patch && !ECON;
+        const int slot0 = f % kSlots, slot1 = (f + 1) % kSlots;
+        const int my_slot = (t && two) ? slot1 : slot0, my_fill = (t && two) ? f + 1 : f;
+        if (ctl.chunk_mask[ci] != 0) {
+          if (!warp_wait(&ctl.patched[my_slot], (dirty_par >> my_slot) & 1, abort_flag)) break;
+          dirty_par ^= 1u << slot0;
+          if (two) dirty_par ^= 1u << slot1;
+        }
+        if (!warp_wait(&ctl.v_landed[my_slot], (my_fill / kSlots) & 1, abort_flag)) break;
+        if (!warp_wait(&ctl.p_full[t][pb], (gc >> 1) & 1, abort_flag)) break;
+        tc::tc_fence_after();
+        if (tc::elect_one()) {
+          const uint32_t v_lo = v_lo0 + my_slot * (kSlotBytes >> 4);
+          const uint32_t p_src = s_base + pb * kNC;
+#pragma unroll
+          for (int kk = 0; kk < kNC / 16; ++kk)
+            tc::mma_ts_lo(acc, p_src + kk * 8, v_lo + kk * (2048 >> 4), v_hi, idesc, kk > 0 ? 1u : accum);
+          tc::mma_commit(&ctl.p_free[t][pb]);
+          tc::mma_commit(&ctl.v_done[slot0]);
+          if (two) tc::mma_commit(&ctl.v_done[slot1]);
+        }
+        __syncwarp();
+        accum = 1;
+        f += two ? 2 : 1;
+      }
+    }
+    if (is_pv && tc::elect_one()) tc::mma_commit(&ctl.acc_done);
+    __syncwarp();
+    }
+  }, [&]() {
+    if (INDEXED && a.q_store != nullptr && ok && ctl.split < 0) {
+      // The Q store rows of this (row tile, head) were read by the gathers that completed q_full and belong to
+      // no other CTA: the new rows take their place for the next loop.
+      ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
+      const int pt = tid - kSoftmaxThreads;
+#pragma unroll 1
+      for (int it = pt; ok && it < n_rows * 16; it += (kWarps - kSoftmaxWarps) * 32) {
+        const int r = it >> 4, ch = it & 15;
+        const int pos_r = __ldg(a.active_idx + s0 + r);
+        *reinterpret_cast<uint4*>(a.q_store + (size_t)pos_r * a.d + h * kDH + ch * 8) =
+            __ldg(reinterpret_cast<const uint4*>(a.q_new + (size_t)(s0 + r) * a.d + h * kDH + ch * 8));
+      }
+    }
+  });
+  }
   }  // block has active rows
   // ---- teardown ------------------------------------------------------------------------------------------
   tc::tc_fence_before();

@@ -16,6 +16,12 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kLn2 = 0.6931471805599453f;
 constexpr float kRescaleThreshold = 60.f;   // in log2 units: rescale only when the reference falls this far behind
 
+// x, as a value of its own: what is computed from it is not kept in registers from one use to the next
+__device__ __forceinline__ int opaque(int x) {
+  asm volatile("" : "+r"(x));
+  return x;
+}
+
 // Bounded wait of a fully converged warp; every lane observes the completed phase itself, so each acquires
 // what the arriving threads released. Returns a warp-uniform verdict.
 __device__ __forceinline__ bool warp_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag) {
@@ -59,6 +65,30 @@ __device__ __forceinline__ int lower_bound_warp(const int32_t* __restrict__ arr,
   return lo + cnt;
 }
 
+// n groups (at most N) of four rows of 256 bytes (lane i names row i) into two 128B-swizzled slabs of 64 elements, `slab_bytes`
+// apart: four-row gathers by ONE thread of the warp from warp-uniform row numbers, the two halves of a row one after the other.
+// Called by a converged warp; announces its bytes on the barrier. Why so: a request costs the issuing warp 42-50 cycles this
+// way, 76-95 when every lane brings its own row numbers (the lanes' operands are then taken one lane at a time), and at 512 MB of
+// rows the halves of a row asked for apart reach 29 B/clk per SM where halves asked for together reach 59.
+template <int N>
+__device__ __forceinline__ void gather_rows(uint8_t* dst, uint32_t slab_bytes, const void* map, uint64_t* bar, int x, int y,
+                                            int n = N) {
+  int r[4 * N];
+#pragma unroll
+  for (int i = 0; i < 4 * N; ++i) r[i] = __shfl_sync(0xffffffffu, y, i);
+  if (tc::elect_one()) {
+    tc::mbar_arrive_expect_tx(bar, n * 1024);
+#pragma unroll
+    for (int g = 0; g < N; ++g) {
+      if (g < n) {
+        tc::tma_gather4(dst + g * 512, map, bar, x, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+        tc::tma_gather4(dst + slab_bytes + g * 512, map, bar, x + 64, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+      }
+    }
+  }
+  __syncwarp();
+}
+
 __device__ __forceinline__ uint4 pack8(const float (&x)[8]) {
   uint4 r;
   r.x = tc::pack_bf16(x[0], x[1]);
@@ -99,13 +129,23 @@ __device__ __forceinline__ float max32(const uint32_t (&r)[32]) {
   return fmaxf(max3(m[0], m[1], m[2]), m[3]);
 }
 
-// P = 2^(s c2 - sub) of 32 logits: 16 packed bf16 pairs into p, returns the sum of the unrounded values. A softmax warp
-// shares its scheduler with one other and is bound by its own latencies: pairs (.f32x2) halve the instructions around the
-// exponentials, and the sum runs in independent chains.
-__device__ __forceinline__ float exp32(const uint32_t (&r)[32], float c2, float sub, uint32_t (&p)[16]) {
+// The reference (log2 units) that a row's probabilities 2^(s - ref) are taken against need not be its largest logit: an
+// estimate from the loop before does, which takes the maximum, the rescales and with them any order of the columns out of
+// the chunk loop. The row's sum tells afterwards whether it did: between these bounds the largest of up to 3072 terms lies
+// above 2^-76, so that what is flushed to zero (2^-126) is below 2^-38 of the sum, and nothing came near an overflow.
+__device__ __forceinline__ float start_ref(float x) { return fabsf(x) < 1e5f ? x : 0.f; }
+__device__ __forceinline__ bool sum_in_range(float sum) { return sum >= 0x1p-64f && sum <= 0x1p60f; }
+
+// P = 2^(s c2 - sub) of 32 logits: 16 packed bf16 pairs into p; adds the sum of the unrounded values (what log-normalisers and
+// masses are made of) to sum.x and the sum of the rounded ones to sum.y. The accumulator is a sum over the rounded values, so
+// its weights add up to one exactly when it is divided by theirs. A softmax warp shares its scheduler with one other and is
+// bound by its own latencies: pairs (.f32x2) halve the instructions around the exponentials, and the sums run in independent
+// chains.
+__device__ __forceinline__ void exp32(const uint32_t (&r)[32], float c2, float sub, uint32_t (&p)[16], float2& sum) {
   using namespace fl_codec;
   const f32x2 cc = pair(c2, c2), ns = pair(-sub, -sub);
   f32x2 acc[4];
+  float acr[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int u = 0; u < 16; ++u) {
     float x0, x1;
@@ -113,26 +153,75 @@ __device__ __forceinline__ float exp32(const uint32_t (&r)[32], float c2, float 
     const float p0 = tc::ex2(x0), p1 = tc::ex2(x1);
     acc[u & 3] = u < 4 ? pair(p0, p1) : add2(acc[u & 3], pair(p0, p1));
     p[u] = tc::pack_bf16(p0, p1);
+    tc::add_bf16x2(p[u], acr[2 * (u & 1)], acr[2 * (u & 1) + 1]);
   }
   float a, b;
   split(add2(add2(acc[0], acc[1]), add2(acc[2], acc[3])), a, b);
-  return a + b;
+  sum.x += a + b;
+  sum.y += (acr[0] + acr[1]) + (acr[2] + acr[3]);
 }
 
-// Dequantize-and-add for one 16-byte piece of a column that carries residual payloads (Eq. 8 chain in
-// binary32, loop order): the rare path of the gather.
+// payload_apply on pairs (.f32x2): the same roundings in half the instructions.
 template <int BITS>
-__device__ __forceinline__ void patch_piece(const DevSide& side, int n_old, uint32_t mask, int j, int elem, int d,
-                                         int group, const uint4& raw, uint4& v_old, uint4& v_new) {
-  float x[8];
-  unpack8(raw, x);
-  v_old = raw;
-#pragma unroll 1
-  for (int s = 0; s <= n_old; ++s) {
-    if (s == n_old && (mask & ((1u << n_old) - 1u))) v_old = pack8(x);
-    if ((mask >> s) & 1u) apply_stream8<__nv_bfloat16, BITS>(side.s[s], j, elem, d, group, x);
+__device__ __forceinline__ void apply_payload(const Payload8<__nv_bfloat16, BITS>& p, float (&x)[8]) {
+  if (BITS == 16) {
+    payload_apply<__nv_bfloat16, BITS>(p, x);
+    return;
   }
-  v_new = ((mask >> n_old) & 1u) ? pack8(x) : v_old;
+  using namespace fl_codec;
+  const float sc = __half2float(p.sc), zr = __half2float(p.zr);
+  const f32x2 s2 = pair(sc, sc), z2 = pair(zr, zr), m2 = pair(-8388608.f, -8388608.f);
+  auto code = [&](int i) -> uint32_t {
+    if (BITS == 8) return ((i < 4 ? p.raw.x : p.raw.y) >> (8 * (i & 3))) & 0xFFu;
+    if (BITS == 4) return (p.raw.x >> (4 * i)) & 0xFu;
+    return (p.raw.x >> (2 * i)) & 0x3u;
+  };
+#pragma unroll
+  for (int i = 0; i < 8; i += 2) {
+    // code -> float without the conversion unit: 2^23 + c is exact in binary32
+    const f32x2 cf = add2(pair_u(0x4B000000u | code(i), 0x4B000000u | code(i + 1)), m2);
+    split(add2(pair(x[i], x[i + 1]), fma2(cf, s2, z2)), x[i], x[i + 1]);
+  }
+}
+
+// Dequantize-and-add for one 16-byte piece of each of N columns that carry residual payloads (Eq. 8 chain in binary32, loop
+// order): the rare path of the gather. mask: the streams that carry the column (0: nothing to do). What three streams of all N
+// columns hold is asked for together, because a slot and the payload behind it are two trips to memory each: a warp takes a
+// 64-column share of four columns and four streams in 2 trips where one column and one stream at a time took 16.
+template <int BITS, int N>
+__device__ __forceinline__ void patch_pieces(const DevSide& side, int n_old, const uint32_t (&mask)[N], const int (&j)[N], int elem,
+                                             int d, int group, const uint4 (&raw)[N], uint4 (&v_old)[N], uint4 (&v_new)[N]) {
+  constexpr int kS = 3;
+  float x[N][8];
+#pragma unroll
+  for (int n = 0; n < N; ++n) {
+    unpack8(raw[n], x[n]);
+    v_old[n] = raw[n];
+  }
+#pragma unroll 1
+  for (int s0 = 0; s0 <= n_old; s0 += kS) {
+    int slot[N][kS];
+    Payload8<__nv_bfloat16, BITS> p[N][kS];
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+      for (int q = 0; q < kS; ++q)
+        slot[n][q] = (s0 + q <= n_old && ((mask[n] >> (s0 + q)) & 1u)) ? __ldg(side.s[s0 + q].slot + j[n]) : -1;
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+      for (int q = 0; q < kS; ++q)
+        if (slot[n][q] >= 0) payload_load<__nv_bfloat16, BITS>(side.s[s0 + q], slot[n][q], elem, d, group, p[n][q]);
+#pragma unroll
+    for (int n = 0; n < N; ++n)
+#pragma unroll
+      for (int q = 0; q < kS; ++q) {
+        if (s0 + q == n_old && (mask[n] & ((1u << n_old) - 1u))) v_old[n] = pack8(x[n]);
+        if (slot[n][q] >= 0) apply_payload<BITS>(p[n][q], x[n]);
+      }
+  }
+#pragma unroll
+  for (int n = 0; n < N; ++n) v_new[n] = ((mask[n] >> n_old) & 1u) ? pack8(x[n]) : v_old[n];
 }
 
 // chunk ci of the partitioned column list: patched chunks first, then stale ones, then plain ones. In the ordered list
@@ -165,8 +254,5 @@ __device__ __forceinline__ ChunkInfo chunk_info(int ci, int n_plain, int n_patch
   }
   return c;
 }
-
-// INDEXED: the previous loop's Q and O rows are read from, and the new O rows written to, position-indexed
-// stores (row active_idx[t] for compact row t) instead of compact buffers.
 
 }  // namespace fl_tc
