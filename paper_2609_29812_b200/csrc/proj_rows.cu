@@ -283,24 +283,27 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
 
   if (warp >= kFirstGatherWarp) {
     if (GATHER) {
-      const int gw = warp - kFirstGatherWarp;
-      const int g4 = gw * 4 + (lane & 3);            // the lane's group of four rows inside the tile
+      const int row0 = (warp - kFirstGatherWarp) * 16;               // the warp's sixteen rows of the tile
       bool ok = true;
       int g = 0;
       for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x) {
-        const int m0 = (w / a.n_tiles) * kBM + g4 * 4;
-        int r[4];
+        const int m = (w / a.n_tiles) * kBM + row0 + (lane & 15);
+        const int y = m < a.n ? __ldg(a.src_idx + m) : a.x_rows;     // a row outside X reads as zero
+        int r[16];                                                    // the same in every lane: one thread asks for all of them
 #pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] = m0 + q < a.n ? __ldg(a.src_idx + m0 + q) : a.x_rows;   // a row outside X reads as zero
+        for (int q = 0; q < 16; ++q) r[q] = __shfl_sync(0xffffffffu, y, q);
         for (int ks = 0; ks < n_slabs; ++ks, ++g) {
           const int st = g % kStages;
           if (g >= kStages) ok = warp_wait(&ctl.empty[st], ((g / kStages) - 1) & 1, abort_flag);
           if (!ok) break;
-          if (lane == 0) tc::mbar_arrive_expect_tx(&ctl.full[st], 4 * 512);
+          if (tc::elect_one()) {
+            tc::mbar_arrive_expect_tx(&ctl.full[st], 4 * 512);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              tc::tma_gather4(smem + (size_t)st * kStageBytes + row0 * 128 + q * 512, &a.x_map, &ctl.full[st], ks * kBK, r[4 * q],
+                              r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]);
+          }
           __syncwarp();
-          if (lane < 4)
-            tc::tma_gather4(smem + (size_t)st * kStageBytes + g4 * 512, &a.x_map, &ctl.full[st], ks * kBK, r[0], r[1],
-                            r[2], r[3]);
         }
       }
     }
@@ -313,7 +316,7 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
         const int st = g % kStages;
         if (g >= kStages) ok = warp_wait(&ctl.empty[st], ((g / kStages) - 1) & 1, abort_flag);
         if (!ok) break;
-        if (lane == 0) {
+        if (tc::elect_one()) {
           uint8_t* stage = smem + (size_t)st * kStageBytes;
           tc::mbar_arrive_expect_tx(&ctl.full[st], GATHER ? kBBytes : kABytes + kBBytes);
           tc::tma_tile2d(stage + kABytes, &a.w_map, &ctl.full[st], ks * kBK, n0);
@@ -323,29 +326,34 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
       }
     }
   } else if (warp == kIssueWarp) {
-    if (lane == 0) {
+    {                        // the whole warp walks the slabs and waits, one elected thread issues
       const uint32_t idesc = tc::make_idesc_bf16(kBM, kBN, false);
       const uint64_t desc0 = tc::make_desc_sw128(tc::smem_u32(smem), 16, 1024);
       const uint32_t hi = (uint32_t)(desc0 >> 32), lo0 = (uint32_t)desc0;
+      const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
       int g = 0, i = 0;
       bool ok = true;
       for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, ++i) {
         const int buf = i & 1;
-        if (i >= 2) ok = tc::mbar_wait(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
+        if (i >= 2) ok = warp_wait(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
         if (!ok) break;
         tc::tc_fence_after();
-        const uint32_t d_dst = tmem + buf * kBN;
+        const uint32_t d_dst = tmem_u + buf * kBN;
         for (int ks = 0; ks < n_slabs; ++ks, ++g) {
           const int st = g % kStages;
-          if (!tc::mbar_wait(&ctl.full[st], (g / kStages) & 1, abort_flag)) { ok = false; break; }
+          if (!warp_wait(&ctl.full[st], (g / kStages) & 1, abort_flag)) { ok = false; break; }
           tc::tc_fence_after();
           const uint32_t a_lo = lo0 + ((st * kStageBytes) >> 4), b_lo = a_lo + (kABytes >> 4);
+          if (tc::elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk)
-            mma_ss_acc(d_dst, a_lo + kk * 2, b_lo + kk * 2, hi, idesc, (ks | kk) != 0 ? 1u : 0u);
-          tc::mma_commit(&ctl.empty[st]);
+            for (int kk = 0; kk < 4; ++kk)
+              mma_ss_acc(d_dst, a_lo + kk * 2, b_lo + kk * 2, hi, idesc, (ks | kk) != 0 ? 1u : 0u);
+            tc::mma_commit(&ctl.empty[st]);
+          }
+          __syncwarp();
         }
-        if (ok) tc::mma_commit(&ctl.acc_full[buf]);
+        if (ok && tc::elect_one()) tc::mma_commit(&ctl.acc_full[buf]);
+        __syncwarp();
       }
     }
     __syncwarp();
@@ -482,24 +490,29 @@ __global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(cons
 
   if (warp >= kFirstGatherWarp) {
     if (GATHER) {
-      const int g4 = (warp - kFirstGatherWarp) * 4 + (lane & 3);     // the lane's group of four rows inside the CTA's 128
+      const int row0 = (warp - kFirstGatherWarp) * 16;               // the warp's sixteen rows of the CTA's 128
       bool ok = true;
       int g = 0;
       for (int w = pair; w < n_work && ok; w += n_pairs) {
-        const int m0 = (w / a.n_tiles) * (2 * kBM) + (int)rank * kBM + g4 * 4;
-        int r[4];
+        const int m = (w / a.n_tiles) * (2 * kBM) + (int)rank * kBM + row0 + (lane & 15);
+        const int y = m < a.n ? __ldg(a.src_idx + m) : a.x_rows;     // a row outside X reads as zero
+        int r[16];                                                    // the same in every lane: one thread asks for all of them
 #pragma unroll
-        for (int q = 0; q < 4; ++q) r[q] = m0 + q < a.n ? __ldg(a.src_idx + m0 + q) : a.x_rows;   // a row outside X reads as zero
+        for (int q = 0; q < 16; ++q) r[q] = __shfl_sync(0xffffffffu, y, q);
         for (int ks = 0; ks < n_slabs; ++ks, ++g) {
           const int st = g % kPairStages;
           if (g >= kPairStages) ok = warp_wait(&ctl.empty[st], ((g / kPairStages) - 1) & 1, abort_flag);
           if (!ok) break;
           // rank 0 announces the bytes of both (the other's may come first: the phase stays open for the announcement)
-          if (rank == 0 && lane == 0) tc::mbar_arrive_expect_tx(&ctl.full[st], 2 * 4 * 512);
+          if (tc::elect_one()) {
+            if (rank == 0) tc::mbar_arrive_expect_tx(&ctl.full[st], 2 * 4 * 512);
+            const uint32_t bar = cluster_map(&ctl.full[st], 0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              pair_gather4(smem + (size_t)st * kPairStageBytes + row0 * 128 + q * 512, &a.x_map, bar, ks * kBK, r[4 * q], r[4 * q + 1],
+                           r[4 * q + 2], r[4 * q + 3]);
+          }
           __syncwarp();
-          if (lane < 4)
-            pair_gather4(smem + (size_t)st * kPairStageBytes + g4 * 512, &a.x_map, cluster_map(&ctl.full[st], 0), ks * kBK, r[0], r[1],
-                         r[2], r[3]);
         }
       }
     }
@@ -512,7 +525,7 @@ __global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(cons
         const int st = g % kPairStages;
         if (g >= kPairStages) ok = warp_wait(&ctl.empty[st], ((g / kPairStages) - 1) & 1, abort_flag);
         if (!ok) break;
-        if (lane == 0) {
+        if (tc::elect_one()) {
           uint8_t* stage = smem + (size_t)st * kPairStageBytes;
           if (rank == 0) tc::mbar_arrive_expect_tx(&ctl.full[st], (GATHER ? 0 : 2 * kABytes) + bn * kBK * 2);
           const uint32_t bar = cluster_map(&ctl.full[st], 0);
@@ -525,29 +538,34 @@ __global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(cons
     // the MMAs' last arrivals on this CTA's barriers have come: it may leave
     for (int k = max(0, g - kPairStages); k < g && ok; ++k) ok = warp_wait(&ctl.empty[k % kPairStages], (k / kPairStages) & 1, abort_flag);
   } else if (warp == kIssueWarp) {
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {         // the whole warp walks the slabs and waits, one elected thread issues
       const uint32_t idesc = tc::make_idesc_bf16(2 * kBM, bn, false);
       const uint64_t desc0 = tc::make_desc_sw128(tc::smem_u32(smem), 16, 1024);
       const uint32_t hi = (uint32_t)(desc0 >> 32), lo0 = (uint32_t)desc0;
+      const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
       int g = 0, i = 0;
       bool ok = true;
       for (int w = pair; w < n_work && ok; w += n_pairs, ++i) {
         const int buf = i & 1;
         // the epilogue warps of both CTAs have read the accumulator: an acquire at cluster scope, once per tile
-        if (i >= 2) ok = tc::mbar_wait_cluster(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
+        if (i >= 2) ok = __all_sync(0xffffffffu, tc::mbar_wait_cluster(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag));
         if (!ok) break;
         tc::tc_fence_after();
-        const uint32_t d_dst = tmem + buf * 256;
+        const uint32_t d_dst = tmem_u + buf * 256;
         for (int ks = 0; ks < n_slabs; ++ks, ++g) {
           const int st = g % kPairStages;
-          if (!tc::mbar_wait(&ctl.full[st], (g / kPairStages) & 1, abort_flag)) { ok = false; break; }
+          if (!warp_wait(&ctl.full[st], (g / kPairStages) & 1, abort_flag)) { ok = false; break; }
           tc::tc_fence_after();
           const uint32_t a_lo = lo0 + ((st * kPairStageBytes) >> 4), b_lo = a_lo + (kABytes >> 4);
+          if (tc::elect_one()) {
 #pragma unroll
-          for (int kk = 0; kk < 4; ++kk) mma_pair(d_dst, a_lo + kk * 2, b_lo + kk * 2, hi, idesc, (ks | kk) != 0 ? 1u : 0u);
-          pair_commit(&ctl.empty[st]);
+            for (int kk = 0; kk < 4; ++kk) mma_pair(d_dst, a_lo + kk * 2, b_lo + kk * 2, hi, idesc, (ks | kk) != 0 ? 1u : 0u);
+            pair_commit(&ctl.empty[st]);
+          }
+          __syncwarp();
         }
-        if (ok) pair_commit(&ctl.acc_full[buf]);
+        if (ok && tc::elect_one()) pair_commit(&ctl.acc_full[buf]);
+        __syncwarp();
       }
     }
     __syncwarp();
