@@ -399,8 +399,7 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
 // ---- two CTAs per tile ---------------------------------------------------------------------------------------
 // The plain projection by pairs of neighbouring SMs (tcgen05 with cta_group::2): a pair computes 256 x bn output tiles, each CTA
 // brings in its own 128 rows of X and HALF of the tile's rows of W, which the MMAs of both read: a 256-column tile costs a CTA
-// 32 KB per slab where the kernel above takes 48 KB, and the slabs are what that kernel waits for (762 cycles, 846 with
-// gathered rows, for 512 of MMA).
+// 32 KB per slab where the kernel above takes 48 KB, and the slabs are what that kernel waits for (512 cycles of MMA each).
 // The CTA of rank 0 issues the MMAs; the copies of both CTAs complete on ITS barriers (with a thread of the other CTA passing its
 // own barriers on, slab by slab, a slab took 2000 cycles). Accumulators, epilogue and tile order as above, per CTA. The tile's width is
 // chosen per call by proj_plan below.
@@ -609,6 +608,8 @@ __global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(cons
 // of those sizes, up to a third, and loses more than 3% at 22 of 4323 (9% at most). Without the epilogue in the model, pairs
 // were taken for few rows and for short d_in, and 750 of them lost 3 to 75%. d = 2048, 3277 rows of 32768: Q/K/V 72.2 -> 66.0 us
 // (rows in order 67.1 -> 59.6), output projection added into the store 31.3 -> 28.2; 12000 rows: Q/K/V 243 -> 221, output 90 -> 79.
+// Since copies and MMAs go out from one elected thread of a warp, pairs take, L2 flushed, 61.4 us for 71.7 (rows in order 57.4 for
+// 63.5), 12000 rows 190.5 for 208.9; the constants are those of before.
 struct ProjPlan {
   int bn;
   bool pairs;
