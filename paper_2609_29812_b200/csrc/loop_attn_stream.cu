@@ -478,7 +478,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     if (row_ok) tc::prefetch_l2(a.rows_in + (size_t)pos * a.d + h * kDH + half_sm * 64);
     if (half_sm == 0) ctl.pos[row] = pos;
     asm volatile("bar.sync 1, %0;" ::"n"(kSmThreads) : "memory");
-    const float sub = ref > -INFINITY ? ref : 0.f;
+    // (OLD pass: a normaliser that is no number reaches the row's mass; it must not pass for another one)
+    const float sub = (MODE == kOldPass || ref > -INFINITY) ? ref : 0.f;
     const uint32_t s_addr = tmem + lane_base + kS + half_sm * (kNC / 2);
     float top = -INFINITY;
     float2 sums = make_float2(0.f, 0.f);

@@ -566,7 +566,8 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     };
     bool staged = false;
     const uint32_t s_addr = tmem + lane_base + (grp ? kSNew : kSOld);
-    const float sub = ref > -INFINITY ? ref : 0.f;
+    // (a normaliser that is no number reaches the old term's sums, and with them the row: it must not pass for another one)
+    const float sub = ((!ECON && grp == 0) || ref > -INFINITY) ? ref : 0.f;
     float2 sums = make_float2(0.f, 0.f);
     float top = -INFINITY;
     bool seen = false;

@@ -87,3 +87,45 @@ def test_reuse_without_useful_normalisers(env, rows, L, q_block, k_tok):
         assert_attn_close(to_np(st.o_store[act]), ref["loops"][1]["O_rows"], f"reuse, hint {name}", carried=1)
         seen = st.mass[:, act] > 0
         assert torch.allclose(lse_out[:, act][seen], want_lse[:, act][seen], rtol=1e-5, atol=1e-4), name
+
+
+@pytest.mark.parametrize("two_pass", [False, True], ids=["two-term kernel", "one-term kernels"])
+def test_normalisers_that_are_no_numbers(env, two_pass, monkeypatch):
+    """A row whose previous log-normaliser is NaN or -inf has no old probabilities. It must not come out as numbers: the two-term
+    kernel passes them on (output and log-normaliser are no finite numbers either), the one-term kernels leave a row without a mass
+    as it was. The other rows, those of the same tile among them, keep their bits."""
+    B, P, ctx = env
+    if two_pass:
+        monkeypatch.setenv("FL_TWO_PASS", "1")
+        ctx = B.Context(0)
+        monkeypatch.delenv("FL_TWO_PASS")
+    w = workloads.replace(small_bf16(L=1100, H=2, R=2), q_block=256)
+    x = workloads.make_layer_inputs(w, seed=77)
+    ref = run_oracle(w, x)
+    act = torch.from_numpy(ref["active"][0]).cuda()
+    bad = {(0, len(act) - 9): float("nan"), (1, len(act) // 2): float("-inf"), (1, len(act) - 40): float("nan")}
+    outs = []
+    for spoil in (False, True):
+        st = P.LayerState(ctx, w)
+        st.dense_loop(to_dev(x.Q[0], w), to_dev(x.K[0], w), to_dev(x.V[0], w))
+        st.select_columns_dense()
+        before = st.o_store.clone()
+        for (h, t), value in bad.items() if spoil else ():
+            st.lse[h, act[t]] = value
+        loop(st, w, x, P, ref, 2, carry="write")
+        outs.append((st.o_store[act].clone(), st.lse[:, act].clone(), st.mass[:, act].clone()))
+    (o, lse, mass), (o_bad, lse_bad, mass_bad) = outs
+    assert torch.isfinite(o.float()).all() and torch.isfinite(lse).all()
+    same = torch.ones(w.n_heads, len(act), dtype=torch.bool, device="cuda")
+    for (h, t), value in bad.items():
+        same[h, t] = False
+        got, m = o_bad[t, h].float(), mass_bad[h, t].item()
+        assert not (0.0 < m < float("inf")), (h, t, m)
+        if two_pass and m == 0.0:
+            assert torch.equal(o_bad[t, h], before[act[t], h]), (h, t)
+        else:
+            assert not torch.isfinite(got).any() and not torch.isfinite(lse_bad[h, t]), (h, t)
+    assert torch.equal(o_bad.transpose(0, 1)[same], o.transpose(0, 1)[same])
+    assert torch.equal(lse_bad[same], lse[same]) and torch.equal(mass_bad[same], mass[same])
+    if two_pass:
+        ctx.close()
