@@ -457,7 +457,8 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     return true;
   };
 
-  // every role walks the tiles in step: main_part works on one, finish writes it out
+  // every role walks the tiles in step: main_part works on one, finish writes it out (softmax warps and the others have a copy
+  // of this loop each: its barriers are met from both)
   auto run_tiles = [&](auto&& main_part, auto&& finish) {
 #pragma unroll 1
   for (; s0 < q_hi; ++tile) {
@@ -469,12 +470,12 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   // A row whose sum left the range in which its probabilities are exact (the reference was no estimate of its logits) sends the
   // tile through two more passes: one finds the largest logits, one takes the probabilities against them. Nothing has been
   // written by then; the Q tiles come again, because the rows were staged in their place
-  redo = __syncthreads_or(bad) && !ctl.abort_flag;
+  redo = tc::cta_sync_or(bad) && !ctl.abort_flag;
   if (!redo) finish();
   if (INDEXED && !redo && a.q_store != nullptr && ctl.split >= 0) {   // CTA-uniform
     // Both halves of a split problem gathered the previous loop's Q rows from the store; the new rows may take their
     // place only when both are done with them, which the merging CTA knows
-    __syncthreads();
+    tc::cta_sync();
     if (ctl.merge_role == 1 && !ctl.abort_flag) {
 #pragma unroll 1
       for (int it = tid; it < n_rows * 16; it += kThreads) {
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     fill = f;
     tc::fence_proxy_async_smem();     // the staged rows, before the next Q tiles come into their place
     tc::tc_fence_before();
-    __syncthreads();
+    tc::cta_sync();
     tc::tc_fence_after();
     if (ctl.abort_flag) break;
   }

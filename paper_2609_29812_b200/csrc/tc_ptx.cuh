@@ -15,6 +15,26 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
+// ---- barriers of the whole CTA for code whose roles are instantiated apart: each warp arrives as a whole, but not all of them from
+// the same instruction. `barrier` counts arrivals wherever they come from; __syncthreads() under a role's condition is undefined ----
+__device__ __forceinline__ void cta_sync() {
+  __syncwarp();
+  asm volatile("barrier.cta.sync.aligned 0;" ::: "memory");
+}
+__device__ __forceinline__ bool cta_sync_or(bool pred) {
+  __syncwarp();
+  uint32_t any;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "barrier.cta.red.or.pred.aligned p, 0, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(any)
+      : "r"((uint32_t)pred)
+      : "memory");
+  return any != 0;
+}
+
 // ---- mbarrier ------------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");

@@ -4,6 +4,7 @@ through two more passes: single tiles, several tiles of a block, shared and spli
 import numpy as np
 import pytest
 
+from oracle import flashloop_oracle as fo
 from paper_2609_29812_b200 import workloads
 from helpers import assert_attn_close, to_dev, to_np
 from test_gpu_economy import run_oracle
@@ -128,4 +129,89 @@ def test_normalisers_that_are_no_numbers(env, two_pass, monkeypatch):
     assert torch.equal(o_bad.transpose(0, 1)[same], o.transpose(0, 1)[same])
     assert torch.equal(lse_bad[same], lse[same]) and torch.equal(mass_bad[same], mass[same])
     if two_pass:
+        ctx.close()
+
+
+def spiked(w, seed, k_tok):
+    """Inputs in which one key column, and it alone, has weight in the first head dimension. Its logit is 8 in units of log2 for
+    ordinary rows and 326 for every third row of a sparse loop (another third per loop), whose other logits stay within +-100: past the
+    row's first 64 columns its largest logit grows by more than any reference chosen from them can take, so its tile needs all
+    three passes. Returns the inputs, the oracle's record and the column."""
+    x = workloads.make_layer_inputs(w, seed=seed)
+    act = run_oracle(w, x, k_tok=k_tok)["active"]
+    col = next(p for p in range(int(0.7 * w.L), w.L) if not any(p in a for a in act))
+    for r in range(w.n_loops):
+        q, k = x.Q[r], x.K[r]
+        k[:, :, 0] = 0.0
+        k[col, :, 0] = 16.0
+        q[:, :, 0] = 4.0
+        if r > 0:
+            q[r % 3::3, :, 0] = 160.0
+    ref = run_oracle(w, x, k_tok=k_tok)
+    for r, rec in enumerate(ref["loops"], start=2):
+        sent = 0
+        for (h, b), S in rec["col_sets"].items():
+            S, rows = np.asarray(S), rec["active"][rec["active"] // w.q_block == b]
+            rows = rows[(rows >= col) & (rows % 3 == (r - 1) % 3)]
+            if col not in S or len(rows) == 0:
+                continue
+            # the kernels take columns that are active in the loop first, in chunks of their own
+            assert np.isin(S, rec["active"]).any() or np.searchsorted(S, col) >= 64
+            kh = fo.round_bf16(rec["khat"])[S[S != col]][:, h].astype(np.float64)
+            logits = x.Q[r - 1][rows][:, h].astype(np.float64) @ kh.T * w.sm_scale * np.log2(np.e)
+            assert np.abs(logits).max() < 100.0 and 160.0 * 16.0 * w.sm_scale * np.log2(np.e) > 300.0
+            sent += len(rows)
+        assert sent > 0, r
+    return x, ref, col
+
+
+# "rebuilt": no materialized rows, so chunks with payloads are rewritten in the ring (two slots each where the old term is computed
+# again); "several tiles": blocks of 130 rows whose two tiles one CTA walks (112 problems on 148 SMs, 208 on 296 slots)
+PASSES = {
+    "two terms": dict(kw=dict(carry="write")),
+    "two terms, whole problems": dict(split=False, kw=dict(carry="write")),
+    "two terms, rebuilt": dict(kw=dict(rows=False)),
+    "two terms, rebuilt, whole problems, 16 bits": dict(split=False, bits=16, kw=dict(rows=False)),
+    "two terms, rebuilt, several tiles": dict(L=1792, H=16, k_tok=[930], kw=dict(rows=False, carry="write")),
+    "two terms, compact": dict(kw=dict(indexed=False)),
+    "two terms, compact, rebuilt": dict(split=False, kw=dict(indexed=False, rows=False)),
+    "two terms, shrinking sets": dict(k_tok=[400, 150, 60], kw=dict(rows=False)),
+    "two streams": dict(k_tok=[300, 300, 300], reuse=dict(rows=False)),
+    "two streams, rebuilt, shrinking sets": dict(k_tok=[400, 150, 60], split=False, reuse=dict(rows=False)),
+    "one term": dict(k_tok=[300, 300, 300], reuse=dict(rows="cur")),
+    "one term, shrinking sets": dict(k_tok=[400, 150, 60], split=False, reuse=dict(rows="cur")),
+    "one term, several tiles": dict(L=3328, H=16, k_tok=[1740, 1700], reuse=dict(rows="cur")),
+    "one term twice": dict(k_tok=[400, 150, 60], two_pass=True, kw=dict(carry="write")),
+}
+
+
+@pytest.mark.parametrize("name", list(PASSES))
+def test_three_passes(env, name, monkeypatch):
+    """Rows whose largest logit no reference from their first columns fits, in every form that a tile is worked on."""
+    B, P, ctx = env
+    c = PASSES[name]
+    if c.get("two_pass"):
+        monkeypatch.setenv("FL_TWO_PASS", "1")
+        ctx = B.Context(0)
+        monkeypatch.delenv("FL_TWO_PASS")
+    k_tok = c.get("k_tok", [300])
+    w = workloads.replace(small_bf16(L=c.get("L", 1100), H=c.get("H", 2), R=1 + len(k_tok), bits=c.get("bits", 4)),
+                          changed_fracs=tuple(k / c.get("L", 1100) for k in k_tok))
+    x, ref, col = spiked(w, 5, k_tok)
+    st = P.LayerState(ctx, w, split=c.get("split", True))
+    st.dense_loop(to_dev(x.Q[0], w), to_dev(x.K[0], w), to_dev(x.V[0], w))
+    st.select_columns_dense()
+    for r in range(2, w.n_loops + 1):
+        rec, act = ref["loops"][r - 2], ref["active"][r - 2]
+        kw = dict(indexed=True, **c["kw"]) if "kw" in c and "indexed" not in c["kw"] else dict(c.get("kw", {}))
+        if "reuse" in c:
+            kw = dict(indexed=True, carry="write") if r == 2 else dict(indexed=True, carry="reuse", **c["reuse"])
+        sel = oracle_selection(P, w, ref, r)
+        o, _ = st.sparse_loop(r, to_dev(x.Q[r - 1][act], w), to_dev(x.K[r - 1][act], w), to_dev(x.V[r - 1][act], w), sel, **kw)
+        st.check_status()
+        # (the carried output is rounded once per loop on the GPU side only; where the old term is taken over, once in all)
+        assert_attn_close(to_np(o), rec["O_rows"], f"three passes, {name}, loop {r}", carried=1 if "reuse" in c else r - 1)
+        ok = np.isfinite(rec["lse_rows"])
+        np.testing.assert_allclose(to_np(st.lse)[:, act][ok], rec["lse_rows"][ok], rtol=0, atol=5e-3 * (r - 1))
+    if c.get("two_pass"):
         ctx.close()
