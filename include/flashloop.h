@@ -281,9 +281,10 @@ FL_API int fl_loop_attention_indexed(fl_ctx* ctx, const fl_shape* shape, int loo
  *   reuse == 0: the call computes what fl_loop_attention_indexed computes and also WRITES, for every active row,
  *               B_i (rounded once to the storage type) and m_i (0 for a row with empty T_i, whose B_i is o_prev_i).
  *   reuse != 0: the call READS B_i and m_i and computes the new term only: q_store_in and o_store_in are not read, and
- *               lse_in is a hint (all three may be NULL): the row's probabilities are first taken against lse_in + log m_i,
- *               and again against their largest logit where that was no estimate of it, so that any numbers there give
- *               the same results up to rounding. Rows with m_i == 0 get o_out = B_i; their lse_out entry is copied from
+ *               lse_in is a hint (all three may be NULL): the row's probabilities are first taken against a number near
+ *               lse_in + log m_i, without it against one near the largest logit of the first columns, and again against the
+ *               largest logit of all where that was no estimate of it: any numbers there give the same results up to
+ *               rounding (numbers that are far off cost time). Rows with m_i == 0 get o_out = B_i; their lse_out entry is copied from
  *               lse_in when that is given and left alone otherwise.
  * The caller guarantees, for a reuse call: col_idx / col_cnt are those of the call that wrote the buffers, and every
  * active row was active in that call (nested token sets, Appendix D.1). After the column sets are pruned the next

@@ -34,7 +34,9 @@
 // after they are asked for, 33 B/clk per SM: rows out of DRAM and L2. 88 -> 83 us a launch, 131072 rows, c = 2048: 477 -> 416 us.
 //
 // Probabilities are taken against an estimate of the row's largest logit (NEW pass: lse_prev + log m; see start_ref), not against a
-// running maximum: the two halves of a chunk need not agree on anything, and no accumulator is rescaled.
+// running maximum: the two halves of a chunk need not agree on anything, and no accumulator is rescaled. A NEW pass without
+// log-normalisers is a build of its own (kFreshPass): the two warps of 32 rows agree on a reference where a row sees its first
+// columns (see row_ref). 2 to 4% slower, and its code alone cost calls with log-normalisers 3 to 5%, wherever it stood.
 // Every mbarrier wait is bounded; on a timeout the CTA raises a flag, drains and reports FL_ERR_TIMEOUT.
 #include "tc_attn_common.cuh"
 
@@ -56,7 +58,7 @@ constexpr uint32_t kAcc = 0, kS = 128;         // tensor-memory columns
 constexpr uint32_t kTmemCols = 256;
 static_assert(3 * kMaxCols * 4 <= 4 * kTileBytes, "prologue staging must fit in the K and V rings");
 
-enum { kOldPass = 0, kNewPass = 1 };
+enum { kOldPass = 0, kNewPass = 1, kFreshPass = 2 };   // kFreshPass: the NEW pass without log-normalisers
 
 struct alignas(64) StArgs {
   CUtensorMap k_map, v_map;            // row-gather maps of the K / V base ([L, d] bf16, box 64 x 1, 128B swizzle)
@@ -91,6 +93,7 @@ struct __align__(16) StSmemCtl {
   uint64_t p_full[2];       // softmax -> issuer: P of the chunk is in tensor memory
   uint64_t p_free[2];       // issuer -> issuer, TMA: the PV MMAs of the chunk have finished (S buffer and V tile free)
   uint64_t acc_done;        // issuer -> softmax: all accumulation of the tile finished
+  uint64_t agree[4];        // kFreshPass, the two warps of 32 rows: both halves' largest logits of a chunk are there
   uint32_t tmem_base;
   int abort_flag;
   int q_lo, q_hi, i_last;
@@ -99,7 +102,8 @@ struct __align__(16) StSmemCtl {
   int chunk_last[kMaxChunks];        // largest entry of the chunk, INT32_MAX if the chunk is padded
   int pos[kM];                       // positions of the tile's rows
   float sum[2][kM];                  // row sums of the two halves: of the probabilities,
-  float rsum[2][kM];                 // and of what is left of them in bf16 (second pass of a tile: the largest logits)
+  float rsum[2][kM];                 // and of what is left of them in bf16 (second pass of a tile: the largest logits);
+                                     // kFreshPass: before that, in turn, the largest logits of the columns that references come from
   uint32_t stale[kMaxCols / 32];     // bit u: ordered column u carries a payload from an earlier loop only
 };
 
@@ -109,6 +113,7 @@ static_assert(2 * (kStSmemBytes + 1024) <= 233472, "two CTAs share an SM's 228 K
 
 template <int BITS, int MODE>
 __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __grid_constant__ StArgs a) {
+  constexpr bool kNew = MODE != kOldPass, kFresh = MODE == kFreshPass;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* q_tile = smem;
@@ -144,6 +149,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       tc::mbar_init(&ctl.p_free[s], 1);
     }
     tc::mbar_init(&ctl.acc_done, 1);
+    if (kFresh)
+      for (int q = 0; q < 4; ++q) tc::mbar_init(&ctl.agree[q], 2);
     ctl.abort_flag = 0;
     tc::fence_barrier_init();
   }
@@ -206,7 +213,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   volatile int* abort_flag = &ctl.abort_flag;
   const int q_lo = ctl.q_lo + share * kM, q_hi = ctl.q_hi;
   auto load_q = [&](int s) {   // one warp
-    if (MODE == kNewPass) {
+    if (kNew) {
       // Q tile of this row tile: two 64-element slabs; rows past the compact list read as zero, rows of the next
       // block (past n_rows) are computed and dropped
       if (lane == 0) {
@@ -294,7 +301,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
   int g = 0;                    // chunks issued so far (all tiles): buffers = g & 1, one phase of their barriers per use
   uint32_t dirty_par_cta = 0;   // per-slot phase parity of the patched[] barriers (they only see dirty chunks)
 
-  int pass = 0;
+  int pass = 0, met = 0;        // met: agreements of the two warps of 32 rows so far
   for (int s0 = q_lo, tile = 0; s0 < q_hi; ++tile) {
   const int n_rows = min(kM, q_hi - s0);
   const int g0 = g;
@@ -468,7 +475,9 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       ref = lse2;
     } else {
       mass = row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f;
-      if (pass < 2) {
+      if (kFresh && pass < 2) {
+        ref = row_ok ? -INFINITY : 0.f;                       // until a finite logit is seen
+      } else if (pass < 2) {
         ref = start_ref(a.lse_prev != nullptr ? lse2 + log2f(mass) : 0.f);
       } else {
         ref = fmaxf(ctl.rsum[0][row], ctl.rsum[1][row]);      // -inf: no column is seen with a finite logit
@@ -479,7 +488,7 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     if (half_sm == 0) ctl.pos[row] = pos;
     asm volatile("bar.sync 1, %0;" ::"n"(kSmThreads) : "memory");
     // (OLD pass: a normaliser that is no number reaches the row's mass; it must not pass for another one)
-    const float sub = (MODE == kOldPass || ref > -INFINITY) ? ref : 0.f;
+    float sub = (MODE == kOldPass || ref > -INFINITY) ? ref : 0.f;
     const uint32_t s_addr = tmem + lane_base + kS + half_sm * (kNC / 2);
     float top = -INFINITY;
     float2 sums = make_float2(0.f, 0.f);
@@ -503,6 +512,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
         vis = lo;
       }
       seen |= vis > 0;
+      // (the same in both warps of the rows: they hold the same references and see the same columns)
+      const bool fresh = kFresh && __any_sync(0xffffffffu, ref == -INFINITY && vis > 0);
       if (!warp_wait(&ctl.s_full[pb], (gc >> 1) & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
       if (ci == n_chunks - 1 && pass != 1) stage_rows();
@@ -516,7 +527,18 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
 #pragma unroll
         for (int u = 0; u < 32; ++u) r[u] = u < lim ? r[u] : 0xff800000u;
       }
-      if (MODE == kNewPass && pass == 1) top = fmaxf(top, max32(r) * c2);      // c2 > 0: scaling commutes with the maximum
+      if (kNew && pass == 1) top = fmaxf(top, max32(r) * c2);      // c2 > 0: scaling commutes with the maximum
+      if (kFresh && fresh) {
+        // two buffers in turn: this one is written again only when the other warp has gone on from here to the next agreement
+        float* mine = &(met & 1 ? ctl.rsum : ctl.sum)[0][row];
+        mine[half_sm * kM] = max32(r) * c2;
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(&ctl.agree[warp & 3]);
+        if (!warp_wait(&ctl.agree[warp & 3], met & 1, abort_flag)) { ok = false; break; }
+        ++met;
+        const float m = fmaxf(mine[0], mine[kM]), near = row_ref(-INFINITY, m);
+        if (ref == -INFINITY && m > -INFINITY) sub = ref = near;
+      }
       exp32(r, c2, sub, pk, sums);
       tc::tmem_st16(sp_addr, pk);
       tc::tmem_wait_st();
@@ -529,21 +551,24 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       if (ok) ok = warp_wait(&ctl.q_full, tile & 1, abort_flag);
       if (ok) stage_rows();
     }
+    // (the other warp of the rows may still be about to read an agreement: it has been through all of them when all PV are done)
+    if (kFresh && ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
     ctl.sum[half_sm][row] = sums.x;
-    ctl.rsum[half_sm][row] = MODE == kNewPass && pass == 1 ? top : sums.y;
+    ctl.rsum[half_sm][row] = kNew && pass == 1 ? top : sums.y;
     if (ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
     tc::tc_fence_after();
     tc::cp_async_wait<0>();
     asm volatile("bar.sync 1, %0;" ::"n"(kSmThreads) : "memory");
     ell = ctl.sum[0][row] + ctl.sum[1][row];
-    bad = MODE == kNewPass && ok && (pass == 1 || (pass == 0 && row_ok && seen && mass > 0.f && !sum_in_range(ell)));
+    const bool fits = kFresh ? ref == -INFINITY || (ell >= kSumMin && ell <= kSumMax) : sum_in_range(ell);
+    bad = kNew && ok && (pass == 1 || (pass == 0 && row_ok && seen && mass > 0.f && !fits));
   }
   // A row whose sum left the range in which its probabilities are exact (the reference was no estimate of its logits) sends the
   // tile through two more passes: one finds the largest logits, one takes the probabilities against them.
-  const bool redo = MODE == kNewPass && __syncthreads_or(bad) && !ctl.abort_flag;
+  const bool redo = kNew && __syncthreads_or(bad) && !ctl.abort_flag;
   if (!redo) {
     if (warp >= kTmaWarp) {
-      if (MODE == kNewPass && a.q_store != nullptr && ok) {
+      if (kNew && a.q_store != nullptr && ok) {
       // the new Q rows take their place in the Q store for the next loop (this pass reads no Q row from it)
       const int pt = tid - kTmaWarp * 32;
 #pragma unroll 1
@@ -559,12 +584,12 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     // The staged rows are combined in place by the row-owning threads (each half takes half of the head dimension) and
     // written out coalesced again.
     const uint32_t acc_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kAcc;
-    const float m_i = MODE == kNewPass ? mass : ell;
+    const float m_i = kNew ? mass : ell;
     const float rsum = ctl.rsum[0][row] + ctl.rsum[1][row];
     const bool valid = ok && n_chunks > 0;                 // warp-uniform: the tensor-memory reads below are collective
     bool has;                                              // per row: T_i is not empty
     float w;
-    if (MODE == kNewPass) {
+    if (kNew) {
       has = valid && seen && ref > -INFINITY && m_i > 0.f;
       w = has ? m_i / rsum : 0.f;
     } else {
@@ -593,8 +618,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
       }
     }
     if (row_ok && half_sm == 0) {
-      if (MODE == kNewPass) {
-        if (has) a.lse_out[(size_t)h * a.L + pos] = (ref + log2f(ell)) * kLn2 - logf(m_i);
+      if (kNew) {
+        if (has) a.lse_out[(size_t)h * a.L + pos] = (kFresh ? log2_sum(ref, ell) : ref + log2f(ell)) * kLn2 - logf(m_i);
         else if (a.lse_prev != nullptr) a.lse_out[(size_t)h * a.L + pos] = a.lse_prev[(size_t)h * a.L + pos];
       } else {
         a.mass[(size_t)h * a.L + pos] = has ? m_i : 0.f;
@@ -725,5 +750,5 @@ int fl_launch_loop_attn_stream(fl_ctx* ctx, const fl_shape* s, int loop_r, const
   a.lse_out = lse_out;
   a.q_new = static_cast<const __nv_bfloat16*>(q_new);
   a.q_store = static_cast<__nv_bfloat16*>(q_store_out);
-  return launch_mode<kNewPass>(ctx, s->bits, grid, a, st);
+  return lse_in != nullptr ? launch_mode<kNewPass>(ctx, s->bits, grid, a, st) : launch_mode<kFreshPass>(ctx, s->bits, grid, a, st);
 }

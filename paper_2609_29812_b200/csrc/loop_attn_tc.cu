@@ -4,7 +4,7 @@
 //
 // Warp roles (16 warps, 512 threads):
 //   warps 0-3   softmax of the OLD term  (fixed normaliser lse_prev: p_old = exp(s_old - lse_prev), mass m_i)
-//   warps 4-7   softmax of the NEW term  (against an estimate of the row's largest logit, see start_ref)
+//   warps 4-7   softmax of the NEW term  (against a number near the row's largest logit, see row_ref)
 //   warps 8-11  MMA issuers, two warps per term: S = Q Khat^T, and acc += P Vhat. The warps wait as a whole and one elected thread
 //               issues from uniform operands. One thread per term for both kinds, inside `if (lane == 0)`, took 3 k cycles a
 //               chunk whatever the gathers and the exponentials did (~90 cycles an MMA, ~300 a wait)
@@ -50,8 +50,8 @@
 // and the cached mass m_i is the one of loop w (Eq. 6: it does not change while the set does not). A recomputing
 // launch can leave B (storage type, by position) and m_i (binary32, [H, L]) in buffers of the caller; an ECON launch
 // reads them and computes the new term only. Its two pipelines then are two STREAMS of the new term (even and odd
-// chunks of the column list, an accumulator and row sums each, taken against one reference), added up in the epilogue; the
-// previous loop's Q and O rows are not read, its log-normalisers are a hint.
+// chunks of the column list, an accumulator, row sums and a reference each), brought to the larger reference and added up in the
+// epilogue; the previous loop's Q and O rows are not read, its log-normalisers are a hint.
 #include "tc_attn_common.cuh"
 
 namespace {
@@ -144,7 +144,7 @@ struct __align__(16) TcSmemCtl {
   int pos[2][kM];            // positions of the tile's rows, one copy per term
   float sum[2][kM], rsum[2][kM];   // row sums per term: of the probabilities (old term: the mass), and of what is left of them in bf16
   float top[2][kM];          // largest logits, second pass of a tile only
-  float ref[2][kM];          // references of the two terms' sums, -inf: no column was seen
+  float ref[2][kM];          // references of the two terms' (streams') sums, -inf: no finite logit was seen
 };
 
 constexpr size_t kTcSmemBytes = 1024 /* alignment slack */ + 2 * kQTileBytes + kSlots * kSlotBytes + sizeof(TcSmemCtl) +
@@ -467,8 +467,8 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
   dirty_par0 = dirty_par_cta;
   ok = true; bad = false;
   main_part();
-  // A row whose sum left the range in which its probabilities are exact (the reference was no estimate of its logits) sends the
-  // tile through two more passes: one finds the largest logits, one takes the probabilities against them. Nothing has been
+  // A row whose sum is too large (some logit far above both the estimate and the row's first columns, see row_ref) sends the tile
+  // through two more passes: one finds the largest logits, one takes the probabilities against them. Nothing has been
   // written by then; the Q tiles come again, because the rows were staged in their place
   redo = tc::cta_sync_or(bad) && !ctl.abort_flag;
   if (!redo) finish();
@@ -527,20 +527,16 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     pos = row_ok ? __ldg(a.active_idx + s0 + row) : -1;
     const float c2 = a.scale * kLog2e;
     if (row_ok && (!ECON || a.lse_prev != nullptr)) lse2 = a.lse_prev[(size_t)h * a.L + pos] * kLog2e;
-    // what the row's probabilities are taken against: the old term's are normalised by the previous loop's log-normaliser; for
-    // the new term's any number near the row's largest logit does. The log-normaliser is an upper estimate of it, 2^20 is taken
-    // off because the columns of the set need not hold the row's mass; with the mass at hand (ECON) it is taken off instead
-    float ref = lse2;
+    // what the row's probabilities are taken against: the old term's are normalised by the previous loop's log-normaliser; the
+    // new term's reference is chosen where the row sees its first columns, near an estimate of its largest logit (the
+    // log-normaliser, less the row's mass where that is at hand). The third pass of a tile has the largest logit itself
+    float hint = lse2;
     if (ECON) {
       const float m_row = row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f;
-      ref = start_ref(a.lse_prev != nullptr ? lse2 + log2f(m_row) : 0.f);
-    } else if (grp == 1) {
-      ref = start_ref(lse2 - 20.f);
+      hint = a.lse_prev != nullptr ? lse2 + log2f(m_row) : -INFINITY;
     }
-    if ((ECON || grp == 1) && pass == 2) {
-      ref = ctl.top[1][row];      // -inf: no column is seen with a finite logit
-      if (ECON) ref = fmaxf(ref, ctl.top[0][row]);
-    }
+    float ref = !ECON && grp == 0 ? lse2 : (row_ok ? -INFINITY : 0.f);       // -inf: no finite logit seen
+    if ((ECON || grp == 1) && row_ok && pass == 2) ref = rintf(ECON ? fmaxf(ctl.top[0][row], ctl.top[1][row]) : ctl.top[1][row]);
     // the epilogue reads the row's previous output (ECON: its background): have it in L2 by then (each term asks
     // for its 128-byte half)
     if (row_ok)
@@ -568,10 +564,11 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     bool staged = false;
     const uint32_t s_addr = tmem + lane_base + (grp ? kSNew : kSOld);
     // (a normaliser that is no number reaches the old term's sums, and with them the row: it must not pass for another one)
-    const float sub = ((!ECON && grp == 0) || ref > -INFINITY) ? ref : 0.f;
+    float sub = ((!ECON && grp == 0) || ref > -INFINITY) ? ref : 0.f;
     float2 sums = make_float2(0.f, 0.f);
     float top = -INFINITY;
-    bool seen = false;
+    // some row of the warp has no reference yet, or the pass is there for the largest logits: false from the second chunk on, as a rule
+    bool open = ECON || grp == 1;
     constexpr int kStep = ECON ? 2 : 1;           // ECON: a group's stream takes every other chunk
     const int gbase = (ECON && grp) ? g0_1 : g0;
     for (int ci = c_lo + (ECON ? grp : 0), n = 0; ci < c_hi; ci += kStep, ++n) {
@@ -591,7 +588,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
         }
         vis = lo;
       }
-      seen |= vis > 0;
+      const bool look = open && (pass == 1 || __any_sync(0xffffffffu, ref == -INFINITY && vis > 0));
       if (!warp_wait(&ctl.s_full[grp][pb], (gc >> 1) & 1, abort_flag)) { ok = false; break; }
       tc::tc_fence_after();
       if (ci + kStep >= c_hi && pass != 1) { staged = true; stage_rows(); }
@@ -609,10 +606,16 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
 #pragma unroll
           for (int u = 0; u < 32; ++u) r[u] = u < lim ? r[u] : 0xff800000u;
         }
-        if (pass == 1) top = fmaxf(top, max32(r) * c2);      // c2 > 0: scaling commutes with the maximum
+        if (look) {
+          const float m = max32(r) * c2;                     // c2 > 0: scaling commutes with the maximum
+          top = fmaxf(top, m);
+          const float near = row_ref(hint, m);
+          if (ref == -INFINITY && m > -INFINITY) sub = ref = near;
+        }
         exp32(r, c2, sub, pk, sums);
         tc::tmem_st16(sp_addr + hf * 16, pk);
       }
+      if (look) open = pass == 1 || __any_sync(0xffffffffu, ref == -INFINITY);
       // P is announced at once: its PV MMAs free both the ring slot (for the gathers) and this S buffer (for the
       // QK^T of the chunk after the next), and both are on the critical path
       tc::tmem_wait_st();
@@ -627,14 +630,12 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     ctl.sum[grp][row] = sums.x;
     ctl.rsum[grp][row] = sums.y;
     if (pass == 1) ctl.top[grp][row] = top;
-    ctl.ref[grp][row] = seen ? ref : -INFINITY;
+    ctl.ref[grp][row] = ref;
     if (ok) ok = warp_wait(&ctl.acc_done, tile & 1, abort_flag);
     tc::tc_fence_after();
     tc::cp_async_wait<0>();
     asm volatile("bar.sync 1, %0;" ::"n"(kSoftmaxThreads) : "memory");
-    const float total = ctl.sum[1][row] + (ECON ? ctl.sum[0][row] : 0.f);
-    const bool any = ctl.ref[1][row] > -INFINITY || (ECON && ctl.ref[0][row] > -INFINITY);
-    bad = ok && (pass == 1 || (pass == 0 && row_ok && any && !sum_in_range(total)));
+    bad = ok && (pass == 1 || (pass == 0 && row_ok && (ECON || grp == 1) && sums.x > kSumMax));
   }, [&]() {
     // ---- epilogue ------------------------------------------------------------------------------------
     // (from a copy of the thread's number that the compiler takes for another one: what is made of it stays out of the
@@ -650,16 +651,19 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     uint8_t* stage_bg = stage + kM * 128;                    // recomputing launch with bg_out only
     const bool write_bg = !ECON && INDEXED && a.bg_out != nullptr;   // CTA-uniform
     // per-row statistics. Accumulator A (tensor-memory columns 0-127) is the old term's, B (128-255) the new term's;
-    // in ECON they are streams 0 and 1 of the new term, whose sums are taken against one reference.
+    // in ECON they are streams 0 and 1 of the new term, brought to the larger of their references by f_a and f_b.
     const float sum_a = ctl.sum[0][row];
     float m_i = ECON ? (row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f) : sum_a;
     float l_i = ctl.sum[1][row], ref_i = ctl.ref[1][row];
     // factor of the new term's accumulators that makes the weights of the rounded probabilities add up to what the unrounded do
-    float r_b = ctl.rsum[1][row];
+    float r_b = ctl.rsum[1][row], f_a = 1.f, f_b = 1.f;
     if (ECON) {
-      l_i = __fadd_rn(sum_a, l_i);
-      r_b = __fadd_rn(ctl.rsum[0][row], r_b);
-      ref_i = fmaxf(ctl.ref[0][row], ref_i);
+      const float ref_a = ctl.ref[0][row], ref_b = ref_i;
+      ref_i = fmaxf(ref_a, ref_b);
+      f_a = ref_a > -INFINITY ? tc::ex2(ref_a - ref_i) : 0.f;
+      f_b = ref_b > -INFINITY ? tc::ex2(ref_b - ref_i) : 0.f;
+      l_i = __fadd_rn(__fmul_rn(sum_a, f_a), __fmul_rn(l_i, f_b));
+      r_b = __fadd_rn(__fmul_rn(ctl.rsum[0][row], f_a), __fmul_rn(r_b, f_b));
     }
     r_b = r_b > 0.f ? l_i / r_b : 1.f;
     // warp-uniform: the tensor-memory reads below are collective
@@ -686,7 +690,8 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
             tc::tmem_wait_ld();
           }
 #pragma unroll
-          for (int i = 0; i < 8; ++i) mine[(col + i) * kM + row] = valid ? __uint_as_float(v[i]) * (ECON || (c8 >> 3) ? r_b : 1.f) : 0.f;
+          for (int i = 0; i < 8; ++i)
+            mine[(col + i) * kM + row] = valid ? __uint_as_float(v[i]) * (ECON || (c8 >> 3) ? r_b * ((c8 >> 3) ? f_b : f_a) : 1.f) : 0.f;
         }
         if (grp == 0) {
           mine[2 * kM * kDH + row] = valid_a ? m_i : 0.f;
@@ -737,7 +742,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
             const int col = (c8 >> 3) * kDH + col_lo + (c8 & 7) * 8;
             const bool valid = (c8 >> 3) ? valid_b : valid_a;
             const bool plain = !ECON && (c8 >> 3) == 0;                  // the old term has one normaliser on both sides
-            const float fm = plain ? 1.f : f, fo = plain ? 1.f : f_o, rc = plain ? 1.f : r_b;
+            const float fm = plain ? 1.f : f, fo = plain ? 1.f : f_o, rc = plain ? 1.f : r_b * ((c8 >> 3) ? f_b : f_a);
             if (valid) {
               tc::tmem_ld8(tmem + lane_base + kAccOld + col, v);
               tc::tmem_wait_ld();
@@ -749,7 +754,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
           }
           tc::tmem_wait_st();
           valid_a = valid_b = true;
-          r_b = 1.f;
+          r_b = f_a = f_b = 1.f;
         }
       }
     }
@@ -766,7 +771,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       for (int i = 0; i < 8; ++i) {
         if (!valid_a) ao[i] = 0u;
         if (!valid_b) an[i] = 0u;
-        if (ECON) an[i] = __float_as_uint(__fadd_rn(__uint_as_float(ao[i]), __uint_as_float(an[i])));
+        if (ECON) an[i] = __float_as_uint(__fadd_rn(__fmul_rn(__uint_as_float(ao[i]), f_a), __fmul_rn(__uint_as_float(an[i]), f_b)));
       }
       const int off = row * 128 + (((c0 / 8) ^ (row & 7)) << 4);
       uint4* cell = reinterpret_cast<uint4*>(stage + off);
@@ -788,7 +793,7 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
       }
     }
     if (grp == 1 && row_ok && writer) {
-      if (has) a.lse_out[(size_t)h * a.L + pos] = (ref_i + log2f(l_i)) * kLn2 - logf(m_i);
+      if (has) a.lse_out[(size_t)h * a.L + pos] = log2_sum(ref_i, l_i) * kLn2 - logf(m_i);
       else if (!ECON) a.lse_out[(size_t)h * a.L + pos] = lse2 * kLn2;
       else if (a.lse_prev != nullptr) a.lse_out[(size_t)h * a.L + pos] = a.lse_prev[(size_t)h * a.L + pos];
     }

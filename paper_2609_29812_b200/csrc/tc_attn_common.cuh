@@ -129,12 +129,36 @@ __device__ __forceinline__ float max32(const uint32_t (&r)[32]) {
   return fmaxf(max3(m[0], m[1], m[2]), m[3]);
 }
 
-// The reference (log2 units) that a row's probabilities 2^(s - ref) are taken against need not be its largest logit: an
-// estimate from the loop before does, which takes the maximum, the rescales and with them any order of the columns out of
-// the chunk loop. The row's sum tells afterwards whether it did: between these bounds the largest of up to 3072 terms lies
-// above 2^-76, so that what is flushed to zero (2^-126) is below 2^-38 of the sum, and nothing came near an overflow.
+// The reference (log2 units) that a row's probabilities 2^(s - ref) are taken against need not be its largest logit: a number near
+// it does, which takes the maximum, the rescales and with them any order of the columns out of the chunk loop. The row's sum tells
+// afterwards whether it did, and a tile with a row for which it did not is done again (three passes in all, 2.3 to 2.6 times the
+// time).
+// start_ref: an estimate from the loop before. Between the bounds of sum_in_range the largest of up to 3072 terms lies above 2^-76, so
+// that what is flushed to zero (2^-126) is below 2^-38 of the sum, and nothing came near an overflow.
 __device__ __forceinline__ float start_ref(float x) { return fabsf(x) < 1e5f ? x : 0.f; }
 __device__ __forceinline__ bool sum_in_range(float sum) { return sum >= 0x1p-64f && sum <= 0x1p60f; }
+
+// row_ref: chosen where the row sees its first columns, of which `m` is the largest logit: an estimate of the largest of all (what
+// the loop before left or, if that is more, the largest m of the warp's rows, because a row of the first block may see a single column
+// here), kept between 30 and 90 above m; an estimate that is no number counts as none. The row's largest logit is no smaller
+// than m, so its sum is no smaller than 2^-90, and what is flushed to zero is below 2^-36 of it. A sum above 2^60 (kSumMax)
+// means that a later logit was 60 above the reference, 90 to 150 above m: 62 to 104 in units of the natural logarithm. The
+// reference is a whole number, so that nothing is lost when the sum's logarithm is added to it. Called by a converged warp.
+constexpr float kRefLow = 30.f, kRefHigh = 90.f, kSumMin = 0x1p-92f, kSumMax = 0x1p60f;
+__device__ __forceinline__ float row_ref(float hint, float m) {
+  const int i = __float_as_int(fmaxf(m, -INFINITY));                                   // (in the order of whole numbers)
+  const int w = __reduce_max_sync(0xffffffffu, i ^ ((i >> 31) & 0x7fffffff));
+  const float most = __int_as_float(w ^ ((w >> 31) & 0x7fffffff));
+  return rintf(fminf(fmaxf(fmaxf(hint, most), m + kRefLow), m + kRefHigh));
+}
+
+// log2 of the sum of 2^s for a whole reference: ref + log2(l). The exponent of l is added to the reference first: log2(l) alone would
+// be rounded as coarsely as 2^-90 asks for.
+__device__ __forceinline__ float log2_sum(float ref, float l) {
+  if (!(l < INFINITY && l >= 0x1p-126f)) return ref + log2f(l);
+  const int bits = __float_as_int(l);
+  return ref + (float)((bits >> 23) - 127) + log2f(__int_as_float((bits & 0x007fffff) | 0x3f800000));
+}
 
 // P = 2^(s c2 - sub) of 32 logits: 16 packed bf16 pairs into p; adds the sum of the unrounded values (what log-normalisers and
 // masses are made of) to sum.x and the sum of the rounded ones to sum.y. The accumulator is a sum over the rounded values, so
