@@ -531,12 +531,14 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     // new term's reference is chosen where the row sees its first columns, near an estimate of its largest logit (the
     // log-normaliser, less the row's mass where that is at hand). The third pass of a tile has the largest logit itself
     float hint = lse2;
+    float ref = !ECON && grp == 0 ? lse2 : (row_ok ? -INFINITY : 0.f);       // -inf: no finite logit seen
     if (ECON) {
       const float m_row = row_ok ? a.mass[(size_t)h * a.L + pos] : 0.f;
       hint = a.lse_prev != nullptr ? lse2 + log2f(m_row) : -INFINITY;
+      // a row without a mass keeps its background whatever its logits are: no probabilities, and no second pass for them
+      if (!(m_row > 0.f)) ref = INFINITY;
     }
-    float ref = !ECON && grp == 0 ? lse2 : (row_ok ? -INFINITY : 0.f);       // -inf: no finite logit seen
-    if ((ECON || grp == 1) && row_ok && pass == 2) ref = rintf(ECON ? fmaxf(ctl.top[0][row], ctl.top[1][row]) : ctl.top[1][row]);
+    if ((ECON || grp == 1) && ref == -INFINITY && pass == 2) ref = rintf(ECON ? fmaxf(ctl.top[0][row], ctl.top[1][row]) : ctl.top[1][row]);
     // the epilogue reads the row's previous output (ECON: its background): have it in L2 by then (each term asks
     // for its 128-byte half)
     if (row_ok)
