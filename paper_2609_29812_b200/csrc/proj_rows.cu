@@ -12,9 +12,9 @@
 // main loop of the next.
 //
 //   warps 0-3  epilogue: thread = output row (TMEM lane), 32 columns at a time
-//   warp  4    MMA issuer (one thread), owner of the tensor-memory allocation
+//   warp  4    MMA issuer (the warp waits as a whole, one elected thread issues), owner of the tensor-memory allocation
 //   warp  5    W slabs (one tile copy per stage); the A slabs too when the rows are not gathered
-//   warps 6-13 A row gathers: four lanes per warp, one four-row copy each per stage
+//   warps 6-13 A row gathers: sixteen rows each, four four-row copies per stage by one elected thread
 #include "tc_attn_common.cuh"
 #include <algorithm>
 #include <cmath>
@@ -326,35 +326,34 @@ __global__ void __launch_bounds__(kThreads, 1) proj_rows_kernel(const __grid_con
       }
     }
   } else if (warp == kIssueWarp) {
-    {                        // the whole warp walks the slabs and waits, one elected thread issues
-      const uint32_t idesc = tc::make_idesc_bf16(kBM, kBN, false);
-      const uint64_t desc0 = tc::make_desc_sw128(tc::smem_u32(smem), 16, 1024);
-      const uint32_t hi = (uint32_t)(desc0 >> 32), lo0 = (uint32_t)desc0;
-      const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
-      int g = 0, i = 0;
-      bool ok = true;
-      for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, ++i) {
-        const int buf = i & 1;
-        if (i >= 2) ok = warp_wait(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
-        if (!ok) break;
+    // the whole warp walks the slabs and waits, one elected thread issues
+    const uint32_t idesc = tc::make_idesc_bf16(kBM, kBN, false);
+    const uint64_t desc0 = tc::make_desc_sw128(tc::smem_u32(smem), 16, 1024);
+    const uint32_t hi = (uint32_t)(desc0 >> 32), lo0 = (uint32_t)desc0;
+    const uint32_t tmem_u = __shfl_sync(0xffffffffu, tmem, 0);
+    int g = 0, i = 0;
+    bool ok = true;
+    for (int w = blockIdx.x; w < n_work && ok; w += gridDim.x, ++i) {
+      const int buf = i & 1;
+      if (i >= 2) ok = warp_wait(&ctl.acc_free[buf], ((i >> 1) - 1) & 1, abort_flag);
+      if (!ok) break;
+      tc::tc_fence_after();
+      const uint32_t d_dst = tmem_u + buf * kBN;
+      for (int ks = 0; ks < n_slabs; ++ks, ++g) {
+        const int st = g % kStages;
+        if (!warp_wait(&ctl.full[st], (g / kStages) & 1, abort_flag)) { ok = false; break; }
         tc::tc_fence_after();
-        const uint32_t d_dst = tmem_u + buf * kBN;
-        for (int ks = 0; ks < n_slabs; ++ks, ++g) {
-          const int st = g % kStages;
-          if (!warp_wait(&ctl.full[st], (g / kStages) & 1, abort_flag)) { ok = false; break; }
-          tc::tc_fence_after();
-          const uint32_t a_lo = lo0 + ((st * kStageBytes) >> 4), b_lo = a_lo + (kABytes >> 4);
-          if (tc::elect_one()) {
+        const uint32_t a_lo = lo0 + ((st * kStageBytes) >> 4), b_lo = a_lo + (kABytes >> 4);
+        if (tc::elect_one()) {
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)
-              mma_ss_acc(d_dst, a_lo + kk * 2, b_lo + kk * 2, hi, idesc, (ks | kk) != 0 ? 1u : 0u);
-            tc::mma_commit(&ctl.empty[st]);
-          }
-          __syncwarp();
+          for (int kk = 0; kk < 4; ++kk)
+            mma_ss_acc(d_dst, a_lo + kk * 2, b_lo + kk * 2, hi, idesc, (ks | kk) != 0 ? 1u : 0u);
+          tc::mma_commit(&ctl.empty[st]);
         }
-        if (ok && tc::elect_one()) tc::mma_commit(&ctl.acc_full[buf]);
         __syncwarp();
       }
+      if (ok && tc::elect_one()) tc::mma_commit(&ctl.acc_full[buf]);
+      __syncwarp();
     }
     __syncwarp();
   } else {
@@ -604,12 +603,14 @@ __global__ void __launch_bounds__(pair_threads(GATHER), 1) proj_pair_kernel(cons
 // wide one, 0.8 when its rows are gathered). Pairs of the best width where they gain 5% by a model of both: a tile's loads and MMAs
 // run under the epilogue of the tile before it, so that a launch takes its start, one of the two for every round, whichever is
 // longer, and the other once. Constants in us, fitted to 2490 sizes (60 to 12000 rows, d_in 256 to 8192, d_out 256 to 12288, rows
-// gathered and not, added and not, weights in L2 and not; 5% mean error). Against one CTA per tile this gains 0.9 to 3.7% in the mean
-// of those sizes, up to a third, and loses more than 3% at 22 of 4323 (9% at most). Without the epilogue in the model, pairs
-// were taken for few rows and for short d_in, and 750 of them lost 3 to 75%. d = 2048, 3277 rows of 32768: Q/K/V 72.2 -> 66.0 us
-// (rows in order 67.1 -> 59.6), output projection added into the store 31.3 -> 28.2; 12000 rows: Q/K/V 243 -> 221, output 90 -> 79.
-// Since copies and MMAs go out from one elected thread of a warp, pairs take, L2 flushed, 61.4 us for 71.7 (rows in order 57.4 for
-// 63.5), 12000 rows 190.5 for 208.9; the constants are those of before.
+// gathered and not, added and not, weights in L2 and not) before copies and MMAs went out from one elected thread of a warp. On
+// 3925 sizes drawn like these, L2 flushed, with every plan of today's kernels timed at each: the rule is 2.4% behind the best plan in
+// the mean, gains 5.3% (rows in order), 3.6% (in order, added), 3.0% (gathered) and 3.4% (gathered, added) in the mean and up to
+// 56% against its own one-CTA tiles, and loses more than 3% against them at 23 (20% at most: 9537 rows, 1024 x 1024, added);
+// of the two widths for one CTA it takes the slower by more than 3% at 251. Constants fitted anew to these times come
+// within 0.9% of the best in the mean, but are more than 3% slower than these at 40 sizes (34% at most): not taken. d = 2048, 3277 rows of 32768,
+// one CTA / pairs: Q/K/V 69.4 / 59.6 us (rows in order 69.2 / 57.0), output projection added into the store 38.9 / 32.5; 12000
+// rows: Q/K/V 246.6 / 211.1, output 104.2 / 93.9.
 struct ProjPlan {
   int bn;
   bool pairs;
