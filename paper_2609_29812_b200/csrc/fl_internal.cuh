@@ -51,7 +51,8 @@ int fl_debug_check_attn(fl_ctx* ctx, const fl_shape* s, int n_streams, const int
                         int64_t n_segments, int32_t* status, void* stream);
 
 // Layout of the loop-attention workspace: kFlMaxSplit int32 arrival counters, then per split problem two partial
-// results of kFlPartFloats binary32 values (both 128 x 128 accumulators and four statistics per row).
+// results of kFlPartFloats binary32 values (both 128 x 128 accumulators and room for four statistics per row, three of which are
+// in use: the size is the one callers have been told).
 constexpr int kFlPartFloats = 2 * 128 * 128 + 4 * 128;
 constexpr int kFlMaxSplit = 256;
 

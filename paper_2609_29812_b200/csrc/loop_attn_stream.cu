@@ -332,8 +332,8 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
     // ========================================== TMA + patch ==========================================
     // Per chunk n, in this order: the K tile of chunk n + 1 (its ring slot is free once QK^T of chunk n - 1 has
     // completed), then the V tile of chunk n (free once PV of chunk n - 2 has completed: V is needed a whole softmax
-    // later than K). The 32 four-row gathers of a tile (2 slabs x 16 groups) are dealt round robin to the warps, one
-    // per lane; every warp announces its own share of the bytes on the tile's barrier.
+    // later than K). Each warp gathers sixteen rows of a tile (see gather_rows) and announces its own share of the bytes on the
+    // tile's barrier.
     const int tw = warp - kTmaWarp;
     const int half = lane >> 4, ch = lane & 15;
     const DevSide& side = half ? a.v : a.k;
@@ -352,15 +352,14 @@ __global__ void __launch_bounds__(kThreads, 2) loop_attn_stream_kernel(const __g
                                  : (is_v ? static_cast<const void*>(&a.v_map) : static_cast<const void*>(&a.k_map));
       gather_rows<4>((is_v ? v_ring : k_ring) + (gc & 1) * kTileBytes + tw * 2048, kNC * 128, src, bar, h * kDH, y);
     };
-    const int n_mine = n_chunks;
-    if (n_mine > 0) {
+    if (n_chunks > 0) {
       if (g0 >= 2) ok = warp_wait(&ctl.s_full[g0 & 1], ((g0 >> 1) - 1) & 1, abort_flag);
       if (ok) fill(0, g0, false);
     }
 #pragma unroll 1
-    for (int ci = 0; ci < n_mine && ok; ++ci) {
+    for (int ci = 0; ci < n_chunks && ok; ++ci) {
       const int gc = g0 + ci;
-      if (ci + 1 < n_mine) {
+      if (ci + 1 < n_chunks) {
         if (gc + 1 >= 2) ok = warp_wait(&ctl.s_full[(gc + 1) & 1], (((gc + 1) >> 1) - 1) & 1, abort_flag);
         if (!ok) break;
         fill(ci + 1, gc + 1, false);

@@ -80,7 +80,7 @@ constexpr uint32_t kAccOld = 0, kAccNew = 128, kSOld = 256, kSNew = 384;   // tw
 // (column-major, so that the row-owning threads write and read coalesced) and the three per-row statistics.
 constexpr int kPartFloats = kFlPartFloats;
 constexpr int kMaxSplit = kFlMaxSplit;      // counters at the head of the workspace
-static_assert(kPartFloats == 2 * kM * kDH + 4 * kM, "partial result: two accumulators and four statistics per row");
+static_assert(kPartFloats >= 2 * kM * kDH + 3 * kM, "partial result: two accumulators and three statistics per row");
 static_assert(3 * kMaxCols * 4 <= kSlots * kSlotBytes, "prologue staging must fit in the ring");
 static_assert(kAccNew == kAccOld + kDH, "the two accumulators are adjacent in tensor memory");
 
@@ -820,12 +820,9 @@ __global__ void __launch_bounds__(kThreads, 1) loop_attn_tc_kernel(const __grid_
     if (warp >= kTmaWarp) {
     // ========================================== TMA + patch ==========================================
     // In-order fills of the ring, the K tiles one chunk ahead of the V tiles; the lookahead is whatever the four slots
-    // allow. A step's four-row gathers (the K tiles of the next chunk, then the V tiles of this one, 32 per tile: 2 slabs x
-    // 16 groups) are dealt round robin to the six warps, one per lane; every warp announces its own share of the bytes on
-    // the tile's barrier. K and V in steps of their own, with half the lanes busy, cost launches of 2048 columns at 128K 14%;
-    // slots held as a whole until the chunk's PV cost launches of two-slot chunks 17%. Chunks whose columns carry residual
-    // payloads are then rewritten in place by the same warps (6 columns at a time, lanes 0-15 the K row, lanes 16-31 the V
-    // row).
+    // allow. Each of the four warps gathers sixteen rows of a tile (see gather_rows) and announces its own share of the bytes on
+    // the tile's barrier; K and V slots are given back apart. Chunks whose columns carry residual payloads that nobody has materialized
+    // are then rewritten in place, two columns at a time, by these warps and the QK^T issuers (see rebuild).
     const int tw = warp - kTmaWarp;
     auto slots_of = [&](const ChunkInfo& ck) { return (ck.patch && !ECON) ? 2 : 1; };  // ECON: only the new tiles are needed
     // one step: the K tiles of chunk ck (k_slots of them, 0: none) at ring position fk, the V tiles of chunk cv at fv

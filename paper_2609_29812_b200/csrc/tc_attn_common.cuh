@@ -65,25 +65,23 @@ __device__ __forceinline__ int lower_bound_warp(const int32_t* __restrict__ arr,
   return lo + cnt;
 }
 
-// n groups (at most N) of four rows of 256 bytes (lane i names row i) into two 128B-swizzled slabs of 64 elements, `slab_bytes`
-// apart: four-row gathers by ONE thread of the warp from warp-uniform row numbers, the two halves of a row one after the other.
-// Called by a converged warp; announces its bytes on the barrier. Why so: a request costs the issuing warp 42-50 cycles this
-// way, 76-95 when every lane brings its own row numbers (the lanes' operands are then taken one lane at a time), and at 512 MB of
-// rows the halves of a row asked for apart reach 29 B/clk per SM where halves asked for together reach 59.
+// N groups of four rows of 256 bytes (lane i names row i) into two 128B-swizzled slabs of 64 elements, `slab_bytes` apart: four-row
+// gathers by ONE thread of the warp from warp-uniform row numbers, the two halves of a row one after the other. Called by a
+// converged warp; announces its bytes on the barrier. Why so: a request costs the issuing warp 42-50 cycles this way, 76-95 when
+// every lane brings its own row numbers (the lanes' operands are then taken one lane at a time). Twelve warps that read one head of
+// 131072 rows 4 KB apart again and again (32 MB, which L2 holds) take in 59 B/clk per SM with the halves of a row asked for
+// together and 29 with the four first halves before the second ones; where all heads are read (512 MB, out of DRAM) 26 to 27 either way.
 template <int N>
-__device__ __forceinline__ void gather_rows(uint8_t* dst, uint32_t slab_bytes, const void* map, uint64_t* bar, int x, int y,
-                                            int n = N) {
+__device__ __forceinline__ void gather_rows(uint8_t* dst, uint32_t slab_bytes, const void* map, uint64_t* bar, int x, int y) {
   int r[4 * N];
 #pragma unroll
   for (int i = 0; i < 4 * N; ++i) r[i] = __shfl_sync(0xffffffffu, y, i);
   if (tc::elect_one()) {
-    tc::mbar_arrive_expect_tx(bar, n * 1024);
+    tc::mbar_arrive_expect_tx(bar, N * 1024);
 #pragma unroll
     for (int g = 0; g < N; ++g) {
-      if (g < n) {
-        tc::tma_gather4(dst + g * 512, map, bar, x, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
-        tc::tma_gather4(dst + slab_bytes + g * 512, map, bar, x + 64, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
-      }
+      tc::tma_gather4(dst + g * 512, map, bar, x, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
+      tc::tma_gather4(dst + slab_bytes + g * 512, map, bar, x + 64, r[4 * g], r[4 * g + 1], r[4 * g + 2], r[4 * g + 3]);
     }
   }
   __syncwarp();
@@ -210,8 +208,8 @@ __device__ __forceinline__ void apply_payload(const Payload8<__nv_bfloat16, BITS
 
 // Dequantize-and-add for one 16-byte piece of each of N columns that carry residual payloads (Eq. 8 chain in binary32, loop
 // order): the rare path of the gather. mask: the streams that carry the column (0: nothing to do). What three streams of all N
-// columns hold is asked for together, because a slot and the payload behind it are two trips to memory each: a warp takes a
-// 64-column share of four columns and four streams in 2 trips where one column and one stream at a time took 16.
+// columns hold is asked for together, because a slot and the payload behind it are two trips to memory each: four columns with up to
+// three streams take 4 trips two columns at a time, where one column and one stream at a time took 24.
 template <int BITS, int N>
 __device__ __forceinline__ void patch_pieces(const DevSide& side, int n_old, const uint32_t (&mask)[N], const int (&j)[N], int elem,
                                              int d, int group, const uint4 (&raw)[N], uint4 (&v_old)[N], uint4 (&v_new)[N]) {

@@ -1,6 +1,6 @@
-"""The number that a row's new probabilities are taken against comes from the previous loop's log-normaliser. Rows for which it is
-no estimate of the new logits (queries that jump between loops, no or useless log-normalisers in a reusing call) send their tile
-through two more passes: single tiles, several tiles of a block, shared and split problems, the one-term and the two-term kernel."""
+"""What a row's new probabilities are taken against: a number near its largest logit, from the previous loop's log-normaliser (one-term
+kernel) or from the row's first columns as well. Rows for which it is none send their tile through two more passes: single
+tiles, several tiles of a block, shared and split problems, the one-term and the two-term kernel, and what that costs."""
 import numpy as np
 import pytest
 
@@ -187,7 +187,8 @@ PASSES = {
 
 @pytest.mark.parametrize("name", list(PASSES))
 def test_three_passes(env, name, monkeypatch):
-    """Rows whose largest logit no reference from their first columns fits, in every form that a tile is worked on."""
+    """Rows whose largest logit no reference from their first columns fits, in every form that a tile is worked on. (The column
+    lies in the later half of the lists: of a split problem one CTA needs the passes and the other does not.)"""
     B, P, ctx = env
     c = PASSES[name]
     if c.get("two_pass"):

@@ -187,8 +187,8 @@ def test_economy_with_shrinking_token_sets(env, rows):
 
 
 def test_economy_with_logits_far_apart(env):
-    """Queries scaled by 16 (logits tens to hundreds of nats apart): both streams of the reuse kernel rescale their
-    accumulators, in either half of a chunk, and are merged on a common reference."""
+    """Queries scaled by 16 in every loop (logits tens to hundreds of nats apart, log-normalisers that know of it): calls with a pair
+    split and without, the one-term kernel in loop 3."""
     B, P, ctx = env
     w = small_bf16(L=1500, H=2, R=3)
     x = workloads.make_layer_inputs(w, seed=7)
