@@ -31,7 +31,8 @@
 // `if (lane == 0)` the TMA warps took 1400 cycles for a tile's requests and a chunk 2.95 k cycles of a CTA, whatever the softmax
 // did (halving a softmax step from 1.9 to 0.95 k cycles changed nothing). Requests and MMAs by one elected thread from uniform
 // operands, two issuers and two softmax warps per 32 rows: 1.9 k, of which 2 are under way per SM. Then K and V arrive 2 k cycles
-// after they are asked for, 33 B/clk per SM: rows out of DRAM and L2. 88 -> 83 us a launch, 131072 rows, c = 2048: 477 -> 416 us.
+// after they are asked for, 33 B/clk per SM: rows out of DRAM and L2. 78 -> 69 us a launch (back to back, L2 flushed
+// between; 88 -> 83 by events around one), 131072 rows, c = 2048: 504 -> 428 us.
 //
 // Probabilities are taken against an estimate of the row's largest logit (NEW pass: lse_prev + log m; see start_ref), not against a
 // running maximum: the two halves of a chunk need not agree on anything, and no accumulator is rescaled. A NEW pass without

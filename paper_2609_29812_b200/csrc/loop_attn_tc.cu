@@ -13,7 +13,8 @@
 //               materialized the overwrite of the gathered base rows with the dequantize-and-add result (Eq. 8), shared with the
 //               QK^T issuers
 // A chunk now takes 2.2 k cycles, of which a softmax step (64 logits a thread) is 1.85 k: 1.0 k of the exponential unit for the two
-// warps of a scheduler, both terms in step. 157 -> 136 us a launch (32768 rows, c = 1024), 131072 rows, c = 2048: 873 -> 732 us.
+// warps of a scheduler, both terms in step. 146 -> 128 us a launch (32768 rows, c = 1024; back to back, L2 flushed between; 157 -> 136
+// by events around one), 131072 rows, c = 2048: 918 -> 780 us.
 // Measured and dropped: sixteen softmax warps with half of a chunk's columns each (a step of 1.5 k cycles, but 80 registers: what
 // spilled went through an L1 of 28 KB, and with it the gathers arrived three times as late: 295 us; with registers moved between
 // warpgroups 155); logits in four pieces, each asked for ahead (142 us).

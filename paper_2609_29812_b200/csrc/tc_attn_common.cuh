@@ -129,7 +129,7 @@ __device__ __forceinline__ float max32(const uint32_t (&r)[32]) {
 
 // The reference (log2 units) that a row's probabilities 2^(s - ref) are taken against need not be its largest logit: a number near
 // it does, which takes the maximum, the rescales and with them any order of the columns out of the chunk loop. The row's sum tells
-// afterwards whether it did, and a tile with a row for which it did not is done again (three passes in all, 2.3 to 2.6 times the
+// afterwards whether it did, and a tile with a row for which it did not is done again (three passes in all, 2.1 to 2.6 times the
 // time).
 // start_ref: an estimate from the loop before. Between the bounds of sum_in_range the largest of up to 3072 terms lies above 2^-76, so
 // that what is flushed to zero (2^-126) is below 2^-38 of the sum, and nothing came near an overflow.
