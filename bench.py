@@ -46,7 +46,7 @@ UNIT = "tokens/s"
 # a shape that is not listed reports null.
 NCU_ATTN_TRAFFIC_BYTES = {
     ("c3:L=32768", "recompute"): 169.9e6,   # loop 2: loop_attn_tc_kernel<4,1,0>
-    ("c3:L=32768", "economy"): 136.1e6,     # loops 3, 4: loop_attn_stream_kernel<4,1> (mean of 133.5 and 133.9 MB)
+    ("c3:L=32768", "economy"): 136.1e6,     # loops 3, 4: loop_attn_stream_kernel<4,1> (mean of 137.0 and 135.2 MB)
 }
 
 
